@@ -18,6 +18,7 @@
 #include "mixer.cuh"
 #include "synth.cuh"
 #include "backward.cuh"
+#include "slice.cuh"
 
 using namespace hn;
 
@@ -153,6 +154,9 @@ struct hyenand_plan {
     long long r0, r1;
     cudaStream_t copy_in, copy_out;   // streams of hyenand_forward_host's pipeline (created on first use)
     cudaEvent_t ev_in[2], ev_out;
+    // small grids of the general path: a slice's spectra fit in shared memory, one kernel does the whole forward
+    bool slice;
+    SliceGeo sg;
     // long 1-D path
     Ct1dPlan ct;
     // host-staging for hyenand_forward_host
@@ -232,7 +236,8 @@ extern "C" hyenand_plan *hyenand_create_plan(int ndim, const int *dims, int B, i
     return hyenand_create_plan_mode(ndim, dims, B, C, causal ? HYENAND_MODE_CAUSAL : HYENAND_MODE_LINEAR, dtype);
 }
 
-extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int B, int C, int mode, int dtype)
+// allow_slice: false for plans whose owner needs the stages of the general path one by one
+static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mode, int dtype, bool allow_slice)
 {
     g_err[0] = 0;
     if (mode != HYENAND_MODE_LINEAR && mode != HYENAND_MODE_CAUSAL && mode != HYENAND_MODE_CIRCULAR) {
@@ -279,6 +284,8 @@ extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int
     }
     p->XH = p->P[2] / 2 + 1;
     p->XP = (p->XH + 1) & ~1;
+    // (the switches that ask for a particular stage of the general path, or for a grouping of it, mean that path)
+    const bool slice_ok = allow_slice && !p->sw.force_generic && !p->sw.generic_rows && !p->sw.generic_core && !getenv("HYENAND_GROUP_SLICES");
     if (circular) {
         // periodic boundaries run on the general N-D passes, which transform whole lines here (nothing is
         // padded, so there is no zero half to prune and no half to crop); no plane, fused or tensor-copy kernels
@@ -316,7 +323,8 @@ extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int
         p->path = PATH_PLANES3D;
     if (ndim == 2 && p->log2p[1] == p->log2p[2] && fused2d_supported(p->log2p[2]) && !p->sw.force_generic)
         p->path = PATH_FUSED2D;
-    if (p->path == PATH_FUSED2D) {
+    p->slice = p->path == PATH_ND_GENERIC && slice_ok && slice_geo(&p->sg, p->L, causal, circular);
+    if (p->path == PATH_FUSED2D || p->slice) {
         p->ws_a_slice = p->wh_a_slice = p->ws_b_slice = p->wh_b_slice = 0;   // nothing leaves the chip
     } else if (p->path == PATH_PLANES3D) {
         // spectra [plane][XH][P_y]; the z pass works in place on the k*v spectra
@@ -335,6 +343,11 @@ extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int
 
     int gl = 1;
     for (int a = 0; a < 3; ++a) if (p->log2p[a] > gl) gl = p->log2p[a];
+    if (p->slice) {                                        // (the slice engine may pad short axes further)
+        if (p->sg.l0 > gl) gl = p->sg.l0;
+        if (p->sg.l1 > gl) gl = p->sg.l1;
+        if (p->sg.l2 > gl) gl = p->sg.l2;
+    }
     p->gtw_n = 1 << gl;
     std::vector<float2> tw(p->gtw_n);
     for (int t = 0; t < p->gtw_n; ++t) {
@@ -367,10 +380,15 @@ extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int
     return p;
 }
 
+extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int B, int C, int mode, int dtype)
+{
+    return create_plan(ndim, dims, B, C, mode, dtype, true);
+}
+
 // tensor maps of the fused core's buffers; left invalid where the TMA core does not apply
 static void make_core_maps(hyenand_plan *p)
 {
-    if (p->path != PATH_PLANES3D && p->path != PATH_ND_GENERIC) return;
+    if ((p->path != PATH_PLANES3D && p->path != PATH_ND_GENERIC) || p->slice) return;
     if (p->sw.no_tma) return;
     const long long spc = p->slices_per_chunk;
     for (int l = 0; l < p->n_lanes; ++l) {
@@ -787,12 +805,29 @@ static int forward_fused2d(hyenand_plan *p, const void *q, const void *k, const 
     return 0;
 }
 
+static int forward_slice(hyenand_plan *p, const void *q, const void *k, const void *v, const void *h,
+                         bool shared, void *y, cudaStream_t st, int *launches)
+{
+    SliceArgs a{};
+    a.q = q; a.k = k; a.v = v; a.h = h; a.y = y;
+    a.s0 = p->r0; a.s1 = p->r1; a.C = shared ? p->C : 0; a.h_bf16 = p->h_dtype != HYENAND_F32;
+    a.g = p->sg; a.gtw = p->gtw; a.gtw_n = p->gtw_n;
+    p->prof.begin(KID_SLICE, st);
+    const int c = launch_slice(a, p->dtype, st);
+    p->prof.end(st);
+    if (c < 0) return -1;
+    *launches += c;
+    return 0;
+}
+
 static int run_forward(hyenand_plan *p, const void *q, const void *k, const void *v, const void *h,
                        bool shared, void *y, cudaStream_t st, int *launches)
 {
     int rc;
     if (p->path == PATH_FUSED2D)
         rc = forward_fused2d(p, q, k, v, h, shared, y, st, launches);
+    else if (p->slice)
+        rc = forward_slice(p, q, k, v, h, shared, y, st, launches);
     else if (p->path == PATH_PLANES3D)
         rc = forward_planes3d(p, (const char *)q, (const char *)k, (const char *)v, (const char *)h, shared,
                               (char *)y, st, launches);
@@ -981,7 +1016,7 @@ extern "C" int hyenand_plan_launches(const hyenand_plan *p, int h_shared)
     const long long S = (long long)p->B * p->C;
     const long long chunks = (S + p->slices_per_chunk - 1) / p->slices_per_chunk;
     const int three = p->P[0] > 1;
-    if (p->path == PATH_FUSED2D) return 1;
+    if (p->path == PATH_FUSED2D || p->slice) return 1;
     if (p->path == PATH_PLANES3D) return (int)(h_shared ? 1 + chunks * 3 : chunks * 4);
     const int filt = 1 + three, body = 3 + 2 * three;
     return (int)(h_shared ? filt + chunks * body : chunks * (filt + body));
@@ -991,7 +1026,7 @@ extern "C" int hyenand_plan_groups(const hyenand_plan *p, long long *slices_per_
 {
     g_err[0] = 0;
     if (!p) return fail(HYENAND_ERR_INVALID_ARG, "plan is NULL");
-    if (slices_per_group) *slices_per_group = p->path == PATH_CT1D ? p->ct.slices_per_chunk : p->path == PATH_FUSED2D ? (long long)p->B * p->C : p->slices_per_chunk;
+    if (slices_per_group) *slices_per_group = p->path == PATH_CT1D ? p->ct.slices_per_chunk : (p->path == PATH_FUSED2D || p->slice) ? (long long)p->B * p->C : p->slices_per_chunk;
     if (lanes) *lanes = p->path == PATH_CT1D || p->path == PATH_FUSED2D ? 1 : p->n_lanes;
     return HYENAND_OK;
 }
@@ -1007,7 +1042,7 @@ extern "C" const char *hyenand_plan_path(const hyenand_plan *p)
 
 const char *const hn::kKernelNames[KID_COUNT] = {
     "rows_fwd(h)", "axis_fwd(h)", "rows_fwd(k*v)", "axis_fwd(k*v)", "axis_core", "axis_inv", "rows_inv",
-    "ct_cols_fwd(h)", "ct_cols_fwd(k*v)", "ct_core", "ct_cols_inv", "plane_fwd(h)", "plane_fwd(k*v)", "plane_inv", "fused2d", "ct_hspec"};
+    "ct_cols_fwd(h)", "ct_cols_fwd(k*v)", "ct_core", "ct_cols_inv", "plane_fwd(h)", "plane_fwd(k*v)", "plane_inv", "fused2d", "ct_hspec", "slice_fused"};
 
 static double fft_flops(double lines, int log2n) { return lines * 5.0 * ldexp(1.0, log2n) * log2n; }
 
@@ -1058,6 +1093,15 @@ extern "C" int hyenand_plan_kernel_info(const hyenand_plan *p, int kid, int h_sh
     }
     const bool three = p->P[0] > 1;
     const double chunks = ceil(S / (double)p->slices_per_chunk);
+    if (p->slice) {
+        if (kid == KID_SLICE) {
+            const int lm = p->sg.l0 + p->sg.l1 + p->sg.l2;
+            *launches = 1;
+            *bytes = 4.0 * S * p->vol * es + Sh * (double)p->kvol * es;
+            *flops = fft_flops(2.0 * S + Sh, lm) + 36.0 * S * ldexp(1.0, lm);
+        }
+        return HYENAND_OK;
+    }
     if (p->path == PATH_FUSED2D) {
         if (kid == KID_FUSED2D) {
             const double PP = p->P[2], XHd = p->XH;
@@ -1489,25 +1533,25 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
     if (nb > B) nb = B;
     g->nb = (int)nb;
     const long long S = nb * C;
-    g->main = hyenand_create_plan_mode(ndim, dims, (int)nb, C, mode, HYENAND_F32);
+    g->main = create_plan(ndim, dims, (int)nb, C, mode, HYENAND_F32, false);
     if (!g->main) { delete g; return nullptr; }
     g->two_gate = g->main->path == PATH_FUSED2D && mode == HYENAND_MODE_LINEAR;
     if (g->two_gate && dtype != HYENAND_F32) {
         hyenand_destroy_plan(g->main);
-        g->main = hyenand_create_plan_mode(ndim, dims, (int)nb, C, mode, dtype);
+        g->main = create_plan(ndim, dims, (int)nb, C, mode, dtype, false);
         if (!g->main) { delete g; return nullptr; }
     }
     g->adj = g->main;
     g->pair = g->main->path == PATH_PLANES3D || g->main->path == PATH_ND_GENERIC;
     // (a long causal 1-D grid gets du from the causal plan and reversed signals, see hyenand_backward)
     if (mode == HYENAND_MODE_CAUSAL && !g->pair && !g->long1d) {
-        g->adj = hyenand_create_plan_mode(ndim, dims, (int)nb, C, HYENAND_MODE_LINEAR, HYENAND_F32);
+        g->adj = create_plan(ndim, dims, (int)nb, C, HYENAND_MODE_LINEAR, HYENAND_F32, false);
         if (!g->adj) { g->adj = g->main; hyenand_backward_destroy(g); return nullptr; }
     }
     if (g->long1d) {
         g->caus = g->main;
         if (mode != HYENAND_MODE_CAUSAL) {
-            g->caus = hyenand_create_plan_mode(ndim, dims, (int)nb, C, HYENAND_MODE_CAUSAL, HYENAND_F32);
+            g->caus = create_plan(ndim, dims, (int)nb, C, HYENAND_MODE_CAUSAL, HYENAND_F32, false);
             if (!g->caus) { hyenand_backward_destroy(g); return nullptr; }
         }
     } else if (mode != HYENAND_MODE_CIRCULAR) {

@@ -1,0 +1,44 @@
+// Slice-fused path: which grids it takes and how they are padded.
+#include "slice_fwd.cuh"
+
+namespace hn {
+
+bool slice_geo(SliceGeo *g, const int *L, int causal, int circular)
+{
+    const bool one_d = L[0] == 1 && L[1] == 1;
+    int l[3];
+    for (int a = 0; a < 3; ++a) {
+        const int need = circular ? L[a] : 2 * L[a] - 1;
+        int b = 0;
+        while ((1 << b) < need) ++b;
+        if (circular && (1 << b) != L[a]) return false;
+        // zero-padded axes may be padded further, to the smallest instance; an axis of one point is no axis
+        if (!circular && a < 2 && L[a] > 1 && b < 4) b = 4;
+        if (!circular && a == 2 && b < (one_d ? 7 : 5)) b = one_d ? 7 : 5;
+        l[a] = b;
+    }
+    g->l0 = l[0]; g->l1 = l[1]; g->l2 = l[2] - 1;
+    bool known = false;
+#define HN_SLICE_KNOWN(A, B, C) known = known || (g->l0 == A && g->l1 == B && g->l2 == C);
+    HN_SLICE_1D(HN_SLICE_KNOWN) HN_SLICE_2D(HN_SLICE_KNOWN) HN_SLICE_3D(HN_SLICE_KNOWN)
+#undef HN_SLICE_KNOWN
+    if (!known) return false;
+    g->vol = g->kvol = 1;
+    g->full = circular;
+    for (int a = 0; a < 3; ++a) {
+        g->L[a] = L[a];
+        g->K[a] = (causal || circular) ? L[a] : 2 * L[a] - 1;
+        g->shift[a] = (causal || circular) ? 0 : L[a] - 1;
+        g->vol *= g->L[a]; g->kvol *= g->K[a];
+    }
+    return true;
+}
+
+int launch_slice(const SliceArgs &a, int dtype, cudaStream_t st)
+{
+    if (a.g.l0 > 0) return dtype == 0 ? launch_slice_3d_f32(a, st) : launch_slice_3d_bf16(a, st);
+    if (a.g.l1 > 0) return dtype == 0 ? launch_slice_2d_f32(a, st) : launch_slice_2d_bf16(a, st);
+    return dtype == 0 ? launch_slice_1d_f32(a, st) : launch_slice_1d_bf16(a, st);
+}
+
+}  // namespace hn
