@@ -191,6 +191,27 @@ __global__ void batch_sum_kernel(const float *src, long long nb, long long C, lo
     }
 }
 
+// the last pass of the sum: acc (earlier passes; nullptr: none) plus this pass's entries, rounded once to the taps' type
+template <typename T> __global__ void batch_sum_cast_kernel(const float *src, long long nb, long long total, const float *acc, T *dst)
+{
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        if (acc) HN_G(acc + e, 4);
+        float s = acc ? acc[e] : 0.f;
+#pragma unroll 8
+        for (long long b = 0; b < nb; ++b) { HN_G(src + b * total + e, 4); s += __ldg(src + b * total + e); }
+        IO<T>::st(dst, e, s);
+    }
+}
+
+int launch_batch_sum_cast(const float *src, long long nb, long long C, long long kvol, const float *acc, int dtype, void *dst, cudaStream_t st)
+{
+    const int grid = bwd_grid(C * kvol);
+    if (grid <= 0) return 0;
+    if (dtype == 0) batch_sum_cast_kernel<float><<<grid, kBwdThreads, 0, st>>>(src, nb, C * kvol, acc, (float *)dst);
+    else batch_sum_cast_kernel<bf16><<<grid, kBwdThreads, 0, st>>>(src, nb, C * kvol, acc, (bf16 *)dst);
+    return 1;
+}
+
 int launch_remap(const RemapArgs &r, cudaStream_t st)
 {
     const long long rows = r.slices * r.G[0] * r.G[1];

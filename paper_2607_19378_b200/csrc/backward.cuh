@@ -26,6 +26,7 @@ int launch_fill(float *dst, float value, long long n, cudaStream_t st);
 // dst (I/O dtype) = a * (b ? b : 1); b holds elements of b_dtype (0: fp32, else bf16)
 int launch_mul_cast(const float *a, const void *b, int b_dtype, long long n, int dtype, void *dst, cudaStream_t st);
 // acc[c][t] (+)= sum over nb of src[(b * C + c)][t]   (set = true overwrites)
+int launch_batch_sum_cast(const float *src, long long nb, long long C, long long kvol, const float *acc, int dtype, void *dst, cudaStream_t st);
 int launch_batch_sum(const float *src, long long nb, long long C, long long kvol, bool set, float *acc, cudaStream_t st);
 
 }  // namespace hn

@@ -1362,6 +1362,8 @@ struct hyenand_grad {
                                       // they are, dq leaves its forward as bf16 (only the fp32 intermediates have scratch)
     bool two_gate;                    // fused 2-D path, linear mode: the plan runs in the caller's element type; dq is a forward
                                       // gated by dy, dk and dv are the two results of one forward gated by v and by k
+    bool slice;                       // a slice's spectra fit in shared memory: one kernel does the whole backward (slice_bwd.cuh)
+    SliceGeo sg;
     bool native;                      // bf16 I/O on the multi-kernel paths and with two_gate: every kernel reads the caller's bf16 tensors itself and
                                       // dq leaves its pass as bf16 (no widened copies of q, k, v, dy)
     int nb;                           // batch entries per pass
@@ -1526,6 +1528,30 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
         fail(HYENAND_ERR_UNSUPPORTED, "a padded axis exceeds %d points (only 1-D linear and causal grids may)", 1 << kMaxLineLog2);
         delete g; return nullptr;
     }
+    {
+        const Switches sw = read_switches();
+        g->slice = !g->long1d && !sw.force_generic && !sw.generic_rows && !sw.generic_core && !getenv("HYENAND_GROUP_SLICES") &&
+                   !getenv("HYENAND_BACKWARD_RING_SLICES") && slice_geo(&g->sg, g->L, mode == HYENAND_MODE_CAUSAL, mode == HYENAND_MODE_CIRCULAR);
+    }
+    if (g->slice) {
+        // a plan for the twiddle table and the device, no workspace; the taps' gradients of a pass in fp32 (within 2 GiB) for
+        // a kernel shared over the batch
+        long long nb = (2ll << 30) / (4ll * C * g->kvol);
+        if (const char *e = getenv("HYENAND_BACKWARD_MAX_BATCH")) { const long long v = atoll(e); if (v > 0 && v < nb) nb = v; }   // development aid
+        g->nb = (int)(nb < 1 ? 1 : nb > B ? B : nb);
+        g->main = create_plan(ndim, dims, 1, 1, mode, dtype, true);
+        if (!g->main) { delete g; return nullptr; }
+        g->adj = g->main;
+        cudaError_t ce = guarded_alloc(&g->allocs, (void **)&g->dhs, (size_t)g->nb * C * g->kvol * sizeof(float));
+        if (ce == cudaSuccess && g->nb < B) ce = guarded_alloc(&g->allocs, (void **)&g->dh32, (size_t)C * g->kvol * sizeof(float));
+        if (ce != cudaSuccess) {
+            cudaGetLastError();
+            fail(HYENAND_ERR_ALLOC, "scratch of the backward pass: %s", cudaGetErrorString(ce));
+            hyenand_backward_destroy(g);
+            return nullptr;
+        }
+        return g;
+    }
     // batch entries per pass: nine fp32 tensors of nb*C*vol elements (+ kernels) within about 4 GiB
     long long nb = (4ll << 30) / (4ll * C * (8 * g->vol + g->kopp + 3 * g->kvol));
     if (const char *e = getenv("HYENAND_BACKWARD_MAX_BATCH")) { const long long v = atoll(e); if (v > 0 && v < nb) nb = v; }   // development aid
@@ -1631,6 +1657,33 @@ static int grad_forward_pair(hyenand_plan *p, long long n, const void *q, const 
     return e;
 }
 
+// The whole backward in one kernel per pass.  Kernel shared over the batch: per-slice tap gradients in fp32, summed over the
+// batch entries in a fixed order.
+static int backward_slice(hyenand_grad *g, const void *q, const void *k, const void *v, const void *h, bool shared, const void *dy,
+                          void *dq, void *dk, void *dv, void *dh, cudaStream_t st)
+{
+    const size_t es = elsize(g->dtype);
+    const long long C = g->C, vol = g->vol, kvol = g->kvol;
+    SliceBwdArgs a{};
+    a.g = g->sg; a.gtw = g->main->gtw; a.gtw_n = g->main->gtw_n;
+    for (int b0 = 0; b0 < g->B; b0 += shared ? g->nb : g->B) {
+        const long long n = !shared ? g->B : g->B - b0 < g->nb ? g->B - b0 : g->nb, off = (long long)b0 * C * vol * es;
+        a.q = (const char *)q + off; a.k = (const char *)k + off; a.v = (const char *)v + off; a.dy = (const char *)dy + off;
+        a.dq = (char *)dq + off; a.dk = (char *)dk + off; a.dv = (char *)dv + off;
+        a.h = h; a.dh = shared ? (void *)g->dhs : dh; a.dh_f32 = shared || g->dtype == HYENAND_F32;
+        a.slices = n * C; a.C = shared ? (int)C : 0;
+        if (launch_slice_bwd(a, g->dtype, st) < 0) return fail(HYENAND_ERR_CUDA, "internal launch dispatch failed");
+        if (shared) {
+            const bool last = b0 + g->nb >= g->B;
+            if (last) launch_batch_sum_cast(g->dhs, n, C, kvol, b0 == 0 ? nullptr : g->dh32, g->dtype, dh, st);
+            else launch_batch_sum(g->dhs, n, C, kvol, b0 == 0, g->dh32, st);
+        }
+    }
+    const cudaError_t ce = cudaGetLastError();
+    if (ce != cudaSuccess) return fail(HYENAND_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(ce));
+    return HYENAND_OK;
+}
+
 extern "C" int hyenand_backward(hyenand_grad *g, const void *q, const void *k, const void *v, const void *h,
                                 long long h_batch_stride_elems, const void *dy, void *dq, void *dk, void *dv, void *dh,
                                 void *cuda_stream)
@@ -1672,6 +1725,7 @@ extern "C" int hyenand_backward(hyenand_grad *g, const void *q, const void *k, c
         d.commit();
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    if (g->slice) return backward_slice(g, q, k, v, h, shared, dy, dq, dk, dv, dh, st);
     const size_t es = elsize(g->dtype);
     const bool widen = g->dtype == HYENAND_BF16;
     const long long C = g->C, vol = g->vol, kvol = g->kvol;

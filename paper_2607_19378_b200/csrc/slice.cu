@@ -1,5 +1,5 @@
 // Slice-fused path: which grids it takes and how they are padded.
-#include "slice_fwd.cuh"
+#include "slice_bwd.cuh"
 
 namespace hn {
 
@@ -32,6 +32,27 @@ bool slice_geo(SliceGeo *g, const int *L, int causal, int circular)
         g->vol *= g->L[a]; g->kvol *= g->K[a];
     }
     return true;
+}
+
+int slice_resident(int (&cache)[64], const void *fn, int threads, size_t smem)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
+    if (!cache[dev]) {
+        int sms = 0, per = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return -1;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem) != cudaSuccess) return -1;
+        cache[dev] = sms * per;
+    }
+    return cache[dev];
+}
+
+int launch_slice_bwd(const SliceBwdArgs &a, int dtype, cudaStream_t st)
+{
+    if (a.g.l0 > 0) return dtype == 0 ? launch_slice_bwd_3d_f32(a, st) : launch_slice_bwd_3d_bf16(a, st);
+    if (a.g.l1 > 0) return dtype == 0 ? launch_slice_bwd_2d_f32(a, st) : launch_slice_bwd_2d_bf16(a, st);
+    return dtype == 0 ? launch_slice_bwd_1d_f32(a, st) : launch_slice_bwd_1d_bf16(a, st);
 }
 
 int launch_slice(const SliceArgs &a, int dtype, cudaStream_t st)

@@ -31,4 +31,21 @@ struct SliceArgs {
 
 int launch_slice(const SliceArgs &a, int dtype, cudaStream_t st);
 
+// Gradients of `slices` slices (backward pass).
+struct SliceBwdArgs {
+    const void *q, *k, *v, *h, *dy;
+    void *dq, *dk, *dv;
+    void *dh;                 // one set of taps per slice
+    int dh_f32;               // taps leave in fp32 (they are summed over the batch afterwards), else in the tensors' type
+    long long slices;
+    int C;                    // channels, for a filter shared over the batch (slices start at a batch entry); 0: one per slice
+    SliceGeo g;
+    const float2 *gtw;
+    int gtw_n;
+};
+int launch_slice_bwd(const SliceBwdArgs &a, int dtype, cudaStream_t st);
+
+// resident CTAs of a kernel on the current device (cached in `cache`, one entry per device); sets its shared-memory limit
+int slice_resident(int (&cache)[64], const void *fn, int threads, size_t smem);
+
 }  // namespace hn

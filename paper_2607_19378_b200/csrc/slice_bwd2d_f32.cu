@@ -1,0 +1,13 @@
+// Instances of the slice-fused backward for 2-D grids of fp32 tensors.
+#include "slice_bwd.cuh"
+#define HN_SLICE_T float
+
+namespace hn {
+
+int launch_slice_bwd_2d_f32(const SliceBwdArgs &a, cudaStream_t st)
+{
+    HN_SLICE_2D(HN_SLICE_BWD_CASE)
+    return -1;
+}
+
+}  // namespace hn

@@ -187,7 +187,17 @@ template <int L0_, int L1_, int L2_> struct SliceFft {
             }
         }
     }
-    template <int AX, int D> static __device__ __forceinline__ void fwd_pass(float2 *buf, const Tw &tw, int t)
+    // NB buffers one after the other (in a loop: one copy of the code, one barrier for all of them)
+    template <int AX, int D, int NB = 1> static __device__ __forceinline__ void fwd_pass(float2 *buf, const Tw &tw, int t)
+    {
+        if constexpr (NB > 1) {
+#pragma unroll 1
+            for (int b = 0; b < NB; ++b) fwd_one<AX, D>(buf + b * BUF, tw, t);
+        } else {
+            fwd_one<AX, D>(buf, tw, t);
+        }
+    }
+    template <int AX, int D> static __device__ __forceinline__ void fwd_one(float2 *buf, const Tw &tw, int t)
     {
         using P = Pass<AX, D>;
 #pragma unroll
@@ -206,7 +216,16 @@ template <int L0_, int L1_, int L2_> struct SliceFft {
             }
         }
     }
-    template <int AX, int D> static __device__ __forceinline__ void inv_pass(float2 *buf, const Tw &tw, int t)
+    template <int AX, int D, int NB = 1> static __device__ __forceinline__ void inv_pass(float2 *buf, const Tw &tw, int t)
+    {
+        if constexpr (NB > 1) {
+#pragma unroll 1
+            for (int b = 0; b < NB; ++b) inv_one<AX, D>(buf + b * BUF, tw, t);
+        } else {
+            inv_one<AX, D>(buf, tw, t);
+        }
+    }
+    template <int AX, int D> static __device__ __forceinline__ void inv_one(float2 *buf, const Tw &tw, int t)
     {
         using P = Pass<AX, D>;
 #pragma unroll
@@ -249,34 +268,34 @@ template <int L0_, int L1_, int L2_> struct SliceFft {
     }
     // all forward passes between the first and the last one, and the inverse ones; sync() separates passes (called before
     // each of them)
-    template <class Sync> static __device__ __forceinline__ void fwd_mid(float2 *buf, const Tw &tw, int t, Sync sync)
+    template <int NB = 1, class Sync> static __device__ __forceinline__ void fwd_mid(float2 *buf, const Tw &tw, int t, Sync sync)
     {
-        fwd_from<first_axis(), 1>(buf, tw, t, sync);
+        fwd_from<first_axis(), 1, NB>(buf, tw, t, sync);
     }
-    template <int AX, int D, class Sync> static __device__ __forceinline__ void fwd_from(float2 *buf, const Tw &tw, int t, Sync sync)
+    template <int AX, int D, int NB, class Sync> static __device__ __forceinline__ void fwd_from(float2 *buf, const Tw &tw, int t, Sync sync)
     {
         if constexpr (AX < 3) {
-            if constexpr (D >= sl_ndig(bits(AX))) fwd_from<AX + 1, 0>(buf, tw, t, sync);
+            if constexpr (D >= sl_ndig(bits(AX))) fwd_from<AX + 1, 0, NB>(buf, tw, t, sync);
             else if constexpr (!(AX == 2 && D == sl_ndig(L2) - 1)) {
                 sync();
-                fwd_pass<AX, D>(buf, tw, t);
-                fwd_from<AX, D + 1>(buf, tw, t, sync);
+                fwd_pass<AX, D, NB>(buf, tw, t);
+                fwd_from<AX, D + 1, NB>(buf, tw, t, sync);
             }
         }
     }
-    template <class Sync> static __device__ __forceinline__ void inv_mid(float2 *buf, const Tw &tw, int t, Sync sync)
+    template <int NB = 1, class Sync> static __device__ __forceinline__ void inv_mid(float2 *buf, const Tw &tw, int t, Sync sync)
     {
-        inv_from<2, sl_ndig(L2) - 2>(buf, tw, t, sync);
+        inv_from<2, sl_ndig(L2) - 2, NB>(buf, tw, t, sync);
     }
-    template <int AX, int D, class Sync> static __device__ __forceinline__ void inv_from(float2 *buf, const Tw &tw, int t, Sync sync)
+    template <int AX, int D, int NB, class Sync> static __device__ __forceinline__ void inv_from(float2 *buf, const Tw &tw, int t, Sync sync)
     {
         if constexpr (AX >= first_axis()) {
             if constexpr (D < 0) {
-                if constexpr (AX > first_axis()) inv_from<AX - 1, sl_ndig(bits(AX - 1)) - 1>(buf, tw, t, sync);
+                if constexpr (AX > first_axis()) inv_from<AX - 1, sl_ndig(bits(AX - 1)) - 1, NB>(buf, tw, t, sync);
             } else if constexpr (!(AX == first_axis() && D == 0)) {
                 sync();
-                inv_pass<AX, D>(buf, tw, t);
-                inv_from<AX, D - 1>(buf, tw, t, sync);
+                inv_pass<AX, D, NB>(buf, tw, t);
+                inv_from<AX, D - 1, NB>(buf, tw, t, sync);
             }
         }
     }

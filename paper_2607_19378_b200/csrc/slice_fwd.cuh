@@ -172,6 +172,19 @@ __device__ __forceinline__ void slice_signal(const T *k, const T *v, const Slice
     }
 }
 
+// the pair of tap gradients at array index idx: the inverse of the placement above
+template <class S, typename T> __device__ __forceinline__ void slice_tap_store(T *dh, const SliceGeo &g, int idx, bool on, float2 w)
+{
+    const SliceIdx<S> c(idx);
+    const int m0 = S::L0 ? (c.i0 + g.shift[0]) & ((1 << S::L0) - 1) : 0;
+    const int m1 = S::L1 ? (c.i1 + g.shift[1]) & ((1 << S::L1) - 1) : 0;
+    const int ma = (c.x + g.shift[2]) & ((2 << S::L2) - 1), mb = (c.x + 1 + g.shift[2]) & ((2 << S::L2) - 1);
+    const bool row = on && (S::L0 == 0 || m0 < g.K[0]) && (S::L1 == 0 || m1 < g.K[1]);
+    T *p = dh + ((S::L0 ? m0 * g.K[1] * g.K[2] : 0) + (S::L1 ? m1 * g.K[2] : 0));
+    if (row && ma < g.K[2]) IO<T>::st(p, ma, w.x);
+    if (row && mb < g.K[2]) IO<T>::st(p, mb, w.y);
+}
+
 // Mirrored frequency of a last-digit item: where the 16 legs of its partner sit.  Leg r's partner is leg (16 - r) mod 16
 // of the partner item where the lower digits of k2 are zero, else leg 15 - r.
 template <class S> struct SliceMirror {
@@ -201,6 +214,15 @@ __device__ __forceinline__ float2 sl_odd(float2 z, float2 m) { return make_float
 
 // a * exp(-2 pi i R / 16), R a compile-time leg
 template <int R> struct SlLeg { static __device__ __forceinline__ float2 rot(float2 a) { return mul_w16<R, false>(a); } };
+
+// w * exp(-2 pi i r / 16) for a leg r known after unrolling
+__device__ __forceinline__ float2 sl_rot16(float2 w, int r)
+{
+    switch (r) {
+    case 1: return SlLeg<1>::rot(w); case 2: return SlLeg<2>::rot(w); case 3: return SlLeg<3>::rot(w); case 4: return SlLeg<4>::rot(w);
+    case 5: return SlLeg<5>::rot(w); case 6: return SlLeg<6>::rot(w); case 7: return SlLeg<7>::rot(w); default: return w;
+    }
+}
 
 template <int R, class F> __device__ __forceinline__ void sl_legs(F f)
 {
@@ -338,19 +360,11 @@ template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN> int launch_s
     using CT = SliceCta<S>;
     constexpr size_t sm = CT::smem(2);
     auto fn = slice_fwd_kernel<T, L0, L1, L2, FULL, EVEN>;
-    // resident CTAs of this kernel, per device
     static int resident[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
-    if (!resident[dev]) {
-        int sms = 0, per = 0;
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, CT::CT, sm) != cudaSuccess || per < 1 || sms < 1) return -1;
-        resident[dev] = sms * per;
-    }
+    const int ctas_fit = slice_resident(resident, (const void *)fn, CT::CT, sm);
+    if (ctas_fit <= 0) return -1;
     SliceArgs a = a0;
-    const long long n = a.s1 - a.s0, slots = (long long)resident[dev] * CT::NG;
+    const long long n = a.s1 - a.s0, slots = (long long)ctas_fit * CT::NG;
     if (n <= 0) return 0;
     long long units = n;
     a.nb = 1;
@@ -366,7 +380,7 @@ template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN> int launch_s
         }
     }
     const long long ctas = (units + CT::NG - 1) / CT::NG;
-    const int grid = (int)(ctas < resident[dev] ? ctas : resident[dev]);
+    const int grid = (int)(ctas < ctas_fit ? ctas : ctas_fit);
     fn<<<grid, CT::CT, sm, st>>>(a);
     return 1;
 }

@@ -8,6 +8,7 @@ from paper_2607_19378_b200 import workloads as W
 pytestmark = pytest.mark.gpu
 
 from parity_util import check
+from test_gpu_backward import check_backward
 
 # smallest and largest extents of each padded length, odd and even rows; 2-D and 3-D: both ends of every axis instance
 LINES = [64, 65, 127, 128, 129, 256, 257, 511, 512, 1023, 1025, 2047, 2048, 2049, 4095, 4096]
@@ -43,3 +44,19 @@ def test_many_slices_shared_filter():
     """More units of work than the GPU has room for: every batch entry of every channel is written once."""
     w, (q, k, v, h) = W.random_problem((100,), B=37, C=211, dtype="bf16", causal=True, h_shared=True, seed=104)
     check(w, q, k, v, h)
+
+
+@pytest.mark.parametrize("dtype,shared", [("f32", True), ("bf16", False), ("bf16", True)])
+@pytest.mark.parametrize("dims,causal", [((64,), False), ((65,), True), ((257,), True), ((512,), False), ((1025,), True), ((2048,), False),
+                                         ((3000,), True), ((4096,), True), ((2, 1), False), ((8, 16), False), ((16, 17), False),
+                                         ((17, 16), False), ((33, 15), False), ((33, 64), False), ((64, 33), False), ((128, 32), False),
+                                         ((8, 8, 16), False), ((7, 9, 15), False), ((8, 7, 17), False)], ids=str)
+def test_backward(dims, causal, dtype, shared):
+    w, (q, k, v, h) = W.random_problem(dims, B=3, C=5, dtype=dtype, causal=causal, h_shared=shared, seed=105)
+    check_backward(w, q, k, v, h, seed=105)
+
+
+@pytest.mark.parametrize("dims", [(128,), (16, 32), (16, 16, 32)], ids=str)
+def test_backward_periodic(dims):
+    w, (q, k, v, h) = W.random_problem(dims, B=2, C=3, dtype="f32", seed=106, circular=True)
+    check_backward(w, q, k, v, h, seed=106)
