@@ -118,6 +118,7 @@ extern "C" long long hyenand_debug_selftest(void)
 
 enum Path { PATH_ND_GENERIC = 0, PATH_CT1D = 1, PATH_PLANES3D = 2, PATH_FUSED2D = 3 };
 constexpr int kMaxLanes = 4;
+constexpr long long kFusedPlanesMax = 148;               // slices of 64-point planes that find an SM each
 
 struct hyenand_plan {
     int ndim, B, C, causal, dtype;
@@ -323,7 +324,13 @@ static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mo
         p->path = PATH_PLANES3D;
     if (ndim == 2 && p->log2p[1] == p->log2p[2] && fused2d_supported(p->log2p[2]) && !p->sw.force_generic)
         p->path = PATH_FUSED2D;
-    p->slice = p->path == PATH_ND_GENERIC && slice_ok && slice_geo(&p->sg, p->L, causal, circular);
+    // 64-point planes: the fused 2-D kernel gives a slice 17 warps of an SM of its own, the slice engine four, several slices to
+    // an SM.  As long as every slice has an SM the former is faster (8 slices of 32x32: 5.9 against 7.7 us), beyond that the
+    // latter (3072 slices: 83 against 65 us).  128-point planes leave the slice engine one CTA per SM: 776 against 1139 us
+    // for 12288 slices of 64x64, they stay with the fused kernel.
+    const bool slice_plane = p->path == PATH_FUSED2D && p->log2p[2] == 6 && (long long)B * C > kFusedPlanesMax;
+    p->slice = (p->path == PATH_ND_GENERIC || slice_plane) && slice_ok && slice_geo(&p->sg, p->L, causal, circular);
+    if (p->slice) p->path = PATH_ND_GENERIC;
     if (p->path == PATH_FUSED2D || p->slice) {
         p->ws_a_slice = p->wh_a_slice = p->ws_b_slice = p->wh_b_slice = 0;   // nothing leaves the chip
     } else if (p->path == PATH_PLANES3D) {

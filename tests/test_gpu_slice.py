@@ -60,3 +60,14 @@ def test_backward(dims, causal, dtype, shared):
 def test_backward_periodic(dims):
     w, (q, k, v, h) = W.random_problem(dims, B=2, C=3, dtype="f32", seed=106, circular=True)
     check_backward(w, q, k, v, h, seed=106)
+
+
+@pytest.mark.parametrize("C,path", [(37, "fused2d"), (38, "nd_generic")])
+def test_many_planes_of_64_points(C, path):
+    """Either side of the number of slices from which 64-point planes leave the fused 2-D kernel."""
+    from paper_2607_19378_b200 import hyenand as hn
+    w, (q, k, v, h) = W.random_problem((30, 20), B=4, C=C, dtype="bf16", seed=107)
+    plan = hn.Plan(w.dims, w.B, w.C, dtype=w.torch_dtype)
+    assert hn.hyenand_plan_path(plan.handle) == path
+    plan.close()
+    check(w, q, k, v, h)
