@@ -430,7 +430,7 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
             if (!shared && ct1d_w_filter(c, (const char *)h + (size_t)s0 * c->K * eh, n, staged_ok, st, launches, prof, filter_pass))
                 return -1;
             if (ct1d_w_body(c, (const char *)q + (size_t)s0 * c->L * eo, (const char *)k + (size_t)s0 * c->L * ei,
-                            (const char *)v + (size_t)s0 * c->L * ei, n, shared, s0, (char *)y + (size_t)s0 * c->L * eo,
+                            v ? (const char *)v + (size_t)s0 * c->L * ei : nullptr, n, shared, s0, (char *)y + (size_t)s0 * c->L * eo,
                             st, launches, prof))
                 return -1;
         }
@@ -441,7 +441,7 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
         const long long n = c->r1 - s0 < c->slices_per_chunk ? c->r1 - s0 : c->slices_per_chunk;
         if (!shared && filter_pass(c, (const char *)h + (size_t)s0 * c->K * eh, n, st, launches, prof)) return -1;
         ColsFwdArgs a{};
-        a.a = (const char *)k + (size_t)s0 * c->L * ei; a.b = (const char *)v + (size_t)s0 * c->L * ei;
+        a.a = (const char *)k + (size_t)s0 * c->L * ei; a.b = v ? (const char *)v + (size_t)s0 * c->L * ei : nullptr;
         a.out = c->wu; a.slices = n; a.in_slice = c->L; a.len = c->L; a.shift = 0;
         a.log2p2 = c->log2p2; a.tw1 = c->tw1; a.tw1_n = 1 << c->log2p1; a.twp = twp;
         prof->begin(KID_CT_COLS_U, st);

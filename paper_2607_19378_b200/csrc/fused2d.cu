@@ -16,8 +16,22 @@
 #include "common.cuh"
 #include "fused2d.cuh"
 #include "plane_util.cuh"
+#include "mix.cuh"
 
 namespace hn {
+
+// VEC results as 16-byte stores: in the tensors' type, or in fp32
+template <typename T> __device__ __forceinline__ void store_vec(T *p, const float (&a)[Vec16<T>::VEC])
+{
+    HN_G(p, 16);
+    *reinterpret_cast<uint4 *>(p) = Vec16<T>::pack(a);
+}
+template <typename T, typename = typename std::enable_if<sizeof(T) == 2>::type> __device__ __forceinline__ void store_vec(float *p, const float (&a)[Vec16<T>::VEC])
+{
+    HN_G(p, 32);
+    *reinterpret_cast<float4 *>(p) = make_float4(a[0], a[1], a[2], a[3]);
+    *reinterpret_cast<float4 *>(p + 4) = make_float4(a[4], a[5], a[6], a[7]);
+}
 
 constexpr int kF2Threads = kPlaneThreads + 32;               // 68 groups of 8 lanes: one per column kx = 0 .. 64 of a 128-point plane
 
@@ -44,8 +58,10 @@ template <int LOG2P> struct F2Cfg {
 // so every phase keeps all groups busy; the k*v store is double buffered.
 // VST: rows are whole numbers of 16-byte vectors and q, y are 16-byte aligned: gate values arrive as 16-byte loads, the
 // cropped rows go through the line once more and leave as 16-byte stores; else one element per lane and leg.
-// TWO: a second gate and result, y2 = q2 * (the same convolution) (the backward pass: dk = v du and dv = k du).
-template <typename T, int LOG2P, bool VST, bool TWO>
+// MIX: Eq. 2 around the convolution.  k and v are then the operator's raw q and k, and q its raw v: the signal is
+// q scale g_in SiLU(k) with one scale per token (the l2 norm and the inner RMSNorm, mixer.cu), the outer gate Sigmoid(v), and
+// the result leaves in fp32 for the outer RMSNorm.
+template <typename T, int LOG2P, bool VST, bool MIX>
 __global__ void __launch_bounds__(kF2Threads, 1) fused2d_kernel(Fused2dArgs p)     // 96 registers: one scheduler hosts 5 of the 17 warps
 {
     using C = F2Cfg<LOG2P>;
@@ -73,9 +89,9 @@ __global__ void __launch_bounds__(kF2Threads, 1) fused2d_kernel(Fused2dArgs p)  
     const unsigned char *hb = (const unsigned char *)p.h;
     const unsigned char *ke = kb + p.kv_elems * sizeof(T), *ve = vb + p.kv_elems * sizeof(T), *he = hb + p.h_elems * sizeof(T);
     const T *pq = (const T *)p.q;
-    T *py = (T *)p.y;
-    const T *pq2 = (const T *)p.q2;
-    T *py2 = (T *)p.y2;
+    using TO = typename MixOut<T, MIX>::type;
+    TO *py = (TO *)p.y;
+    auto gate = [](float x) { return MIX ? mix_sigmoid(x) : x; };
     const int Lx = p.lx, Ly = p.ly, Kx = 2 * Lx - 1, Ky = 2 * Ly - 1;
     const long long vol = (long long)Lx * Ly, kvol = (long long)Kx * Ky;
     using PL = typename F::LastPass;
@@ -118,34 +134,11 @@ __global__ void __launch_bounds__(kF2Threads, 1) fused2d_kernel(Fused2dArgs p)  
 #pragma unroll
                         for (int e = 0; e < VEC; ++e) {
                             const float2 z = line[FI::ph(x0 + e)];
-                            a[e] = z.x * ga[e];
-                            b[e] = z.y * gb[e];
+                            a[e] = z.x * gate(ga[e]);
+                            b[e] = z.y * gate(gb[e]);
                         }
-                        HN_G(py + o0 + x0, 16);
-                        *reinterpret_cast<uint4 *>(py + o0 + x0) = Vec16<T>::pack(a);
-                        if (has1) { HN_G(py + o1 + x0, 16); *reinterpret_cast<uint4 *>(py + o1 + x0) = Vec16<T>::pack(b); }
-                    }
-                }
-                if constexpr (TWO) {
-#pragma unroll
-                    for (int j = 0; j < NV; ++j) {
-                        const int x0 = (l + j * TPL) * VEC;
-                        if (x0 < Lx) {
-                            float a[VEC], b[VEC], ga[VEC], gb[VEC];
-                            HN_G(pq2 + o0 + x0, 16);
-                            Vec16<T>::unpack(__ldg(reinterpret_cast<const uint4 *>(pq2 + o0 + x0)), ga);
-                            if (has1) HN_G(pq2 + o1 + x0, 16);
-                            Vec16<T>::unpack(has1 ? __ldg(reinterpret_cast<const uint4 *>(pq2 + o1 + x0)) : make_uint4(0u, 0u, 0u, 0u), gb);
-#pragma unroll
-                            for (int e = 0; e < VEC; ++e) {
-                                const float2 z = line[FI::ph(x0 + e)];
-                                a[e] = z.x * ga[e];
-                                b[e] = z.y * gb[e];
-                            }
-                            HN_G(py2 + o0 + x0, 16);
-                            *reinterpret_cast<uint4 *>(py2 + o0 + x0) = Vec16<T>::pack(a);
-                            if (has1) { HN_G(py2 + o1 + x0, 16); *reinterpret_cast<uint4 *>(py2 + o1 + x0) = Vec16<T>::pack(b); }
-                        }
+                        store_vec<T>(py + o0 + x0, a);
+                        if (has1) store_vec<T>(py + o1 + x0, b);
                     }
                 }
             } else {
@@ -163,13 +156,8 @@ __global__ void __launch_bounds__(kF2Threads, 1) fused2d_kernel(Fused2dArgs p)  
                 FI::template run<PRUNE_OUT>(l, m, twi, line, spectrum,
                     [&](int i, int r, int idx, float2 v) {
                         if (idx < Lx) {
-                            IO<T>::st(py, o0 + idx, v.x * (float)q0[i * (PIL::R / 2) + r]);
-                            if (has1) IO<T>::st(py, o1 + idx, v.y * (float)q1[i * (PIL::R / 2) + r]);
-                            if constexpr (TWO) {
-                                HN_G(pq2 + o0 + idx, ES);
-                                IO<T>::st(py2, o0 + idx, v.x * IO<T>::ld(pq2, o0 + idx));
-                                if (has1) { HN_G(pq2 + o1 + idx, ES); IO<T>::st(py2, o1 + idx, v.y * IO<T>::ld(pq2, o1 + idx)); }
-                            }
+                            IO<TO>::st(py, o0 + idx, v.x * gate((float)q0[i * (PIL::R / 2) + r]));
+                            if (has1) IO<TO>::st(py, o1 + idx, v.y * gate((float)q1[i * (PIL::R / 2) + r]));
                         }
                     });
             }
@@ -247,7 +235,30 @@ __global__ void __launch_bounds__(kF2Threads, 1) fused2d_kernel(Fused2dArgs p)  
                     const T *k1 = reinterpret_cast<const T *>(sk1 + ((unsigned long long)gk1 & 15ull)) + l;
                     const T *v1p = reinterpret_cast<const T *>(sv1 + ((unsigned long long)gv1 & 15ull)) + l;
                     auto keep = [&](int, int, int kk, float2 z) { ucs[kk * UCS + rp] = z; };
-                    if (Lx == HP && has1) {
+                    if constexpr (MIX) {
+                        // the operator's token scales of the two rows, and its channel weight
+                        const long long sb = s / p.C;
+                        HN_G(p.g_in + (s - sb * p.C), 4);
+                        const float gin = __ldg(p.g_in + (s - sb * p.C));
+                        const float *t0 = p.token_scale + sb * vol + (long long)rp * Lx + l, *t1 = t0 + (long long)QP * Lx;
+                        auto gated = [&](float a, float b, const float *t) { HN_G(t, 4); return a * (__ldg(t) * gin) * (b * mix_sigmoid(b)); };
+                        if (Lx == HP && has1) {
+                            F::template run<PRUNE_IN, true>(l, m, twf, line, [&](int i, int r, int) {
+                                const int x = i * TPL + r * (P / PF0::R);
+                                return make_float2(gated((float)k0[x], (float)v0p[x], t0 + x), gated((float)k1[x], (float)v1p[x], t1 + x));
+                            }, keep);
+                        } else {
+                            F::template run<PRUNE_IN, true>(l, m, twf, line, [&](int i, int r, int idx) {
+                                const int x = i * TPL + r * (P / PF0::R);
+                                float a = 0.f, b = 0.f;
+                                if (idx < Lx) {
+                                    a = gated((float)k0[x], (float)v0p[x], t0 + x);
+                                    if (has1) b = gated((float)k1[x], (float)v1p[x], t1 + x);
+                                }
+                                return make_float2(a, b);
+                            }, keep);
+                        }
+                    } else if (Lx == HP && has1) {
                         // full rows: no bounds tests in the input functor
                         F::template run<PRUNE_IN, true>(l, m, twf, line, [&](int i, int r, int) {
                             const int x = i * TPL + r * (P / PF0::R);
@@ -351,13 +362,12 @@ template <typename T, int LOG2P> static int launch_fused2d_t(const Fused2dArgs &
         if (sms <= 0) sms = 148;
     }
     // 16-byte gate loads and result stores where every row is a whole number of vectors on a 16-byte boundary
-    const bool two = a.q2 != nullptr && a.y2 != nullptr;
-    const bool vst = a.lx % Vec16<T>::VEC == 0 &&
-                     (((uintptr_t)a.q | (uintptr_t)a.y | (uintptr_t)a.q2 | (uintptr_t)a.y2) & 15) == 0;
+    const bool mix = a.token_scale != nullptr;
+    const bool vst = a.lx % Vec16<T>::VEC == 0 && (((uintptr_t)a.q | (uintptr_t)a.y) & 15) == 0;
     static DevOnce attr[4];
-    void (*fn)(Fused2dArgs) = two ? (vst ? fused2d_kernel<T, LOG2P, true, true> : fused2d_kernel<T, LOG2P, false, true>)
+    void (*fn)(Fused2dArgs) = mix ? (vst ? fused2d_kernel<T, LOG2P, true, true> : fused2d_kernel<T, LOG2P, false, true>)
                                   : (vst ? fused2d_kernel<T, LOG2P, true, false> : fused2d_kernel<T, LOG2P, false, false>);
-    if (attr[(two ? 2 : 0) + (vst ? 1 : 0)].first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    if (attr[(mix ? 2 : 0) + (vst ? 1 : 0)].first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     const int grid = (int)(a.slices < sms ? a.slices : sms);
     if (grid <= 0) return 0;
     fn<<<grid, kF2Threads, C::SMEM, st>>>(a);

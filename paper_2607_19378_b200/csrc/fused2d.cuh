@@ -7,8 +7,10 @@ namespace hn {
 struct Fused2dArgs {
     const void *q, *k, *v, *h;
     void *y;
-    const void *q2;           // optional second gate and result of the same convolution: y2 = q2 * (h conv (k v)); both or none
-    void *y2;
+    // Eq. 2 around the convolution (nullptr: none): k, v, q are the operator's q, k, v, y is fp32
+    const float *token_scale; // [B][ly][lx]
+    const float *g_in;        // [C]
+    int C;
     long long slices;         // B*C
     int lx, ly;               // grid extent along x (contiguous) and y
     long long h_mod, h_off;   // filter slice = h_mod ? (s + h_off) % h_mod : s

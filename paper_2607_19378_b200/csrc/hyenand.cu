@@ -173,8 +173,11 @@ struct hyenand_plan {
     // the group has just computed.  Unused (nullptr) in an ordinary forward.
     const char *q2, *k2, *v2;
     char *y2;
-    const char *qg2;                  // a second gate and result of the same convolution, yg2 = qg2 * (h conv (k v)): of the one
-    char *yg2;                        // forward on the fused 2-D path, of the second signal side on the multi-kernel paths
+    const char *qg2;                  // a second gate and result of the second signal side, yg2 = qg2 * (h' conv (k2 v2))
+    char *yg2;
+    // Eq. 2 inside the convolution's kernel (one-kernel paths): token scales and channel weights of the next forward, whose
+    // q, k, v are then the operator's and whose result is fp32.  nullptr in an ordinary forward.
+    const float *mix_scale, *mix_gin;
     size_t ws_bytes;
     Prof prof;
 };
@@ -645,9 +648,9 @@ static int forward_generic(hyenand_plan *p, const char *q, const char *k, const 
                         const char *sq2, char *sy2) -> int {
             const size_t ei = elsize(dt_in), eo = elsize(dt_out);
             RowsArgs r{};
-            r.a = sk + (size_t)s0 * p->vol * ei; r.b = sv + (size_t)s0 * p->vol * ei; r.out = ln.ws_a; r.pitch = p->XP;
+            r.a = sk + (size_t)s0 * p->vol * ei; r.b = sv ? sv + (size_t)s0 * p->vol * ei : nullptr; r.out = ln.ws_a; r.pitch = p->XP;
             r.rows = n * p->L[0] * p->L[1]; r.len = p->L[2]; r.shift = 0; r.log2p = p->log2p[2];
-            r.prune_in = 1; r.full_in = p->circular; r.gtw = p->gtw; r.gtw_n = p->gtw_n;
+            r.prune_in = !p->circular; r.full_in = p->circular; r.gtw = p->gtw; r.gtw_n = p->gtw_n;
             p->prof.begin(KID_ROWS_U, st);
             const bool roww = rows_w_supported(r.log2p) && !p->sw.generic_rows;
             int c = roww ? launch_rows_fwd_w(r, dt_in, st) : launch_rows_fwd(r, dt_in, st);
@@ -800,7 +803,7 @@ static int forward_fused2d(hyenand_plan *p, const void *q, const void *k, const 
     a.slices = p->r1 - p->r0; a.lx = p->L[2]; a.ly = p->L[1];
     a.h_mod = shared ? p->C : 0; a.h_off = shared ? p->r0 % p->C : 0;
     a.scale = (float)(1.0 / ((double)p->P[1] * p->P[2]));
-    if (p->yg2) { a.q2 = p->qg2 + off; a.y2 = p->yg2 + off; }
+    a.token_scale = p->mix_scale; a.g_in = p->mix_gin; a.C = p->C;
     a.gtw = p->gtw; a.gtw_n = p->gtw_n;
     a.kv_elems = a.slices * p->vol;
     a.h_elems = (shared ? p->C : a.slices) * p->kvol;
@@ -818,6 +821,7 @@ static int forward_slice(hyenand_plan *p, const void *q, const void *k, const vo
     SliceArgs a{};
     a.q = q; a.k = k; a.v = v; a.h = h; a.y = y;
     a.s0 = p->r0; a.s1 = p->r1; a.C = shared ? p->C : 0; a.h_bf16 = p->h_dtype != HYENAND_F32;
+    a.token_scale = p->mix_scale; a.g_in = p->mix_gin; a.mix_C = p->C;
     a.g = p->sg; a.gtw = p->gtw; a.gtw_n = p->gtw_n;
     p->prof.begin(KID_SLICE, st);
     const int c = launch_slice(a, p->dtype, st);
@@ -1195,16 +1199,19 @@ extern "C" int hyenand_plan_kernel_time(hyenand_plan *p, int kid, double *total_
 
 // ---- the full HyenaND operator (Eq. 2): pointwise stages around the long convolution -----------------
 //
-// The long convolution runs on an fp32 plan whatever the I/O type, so that nothing between the first read of
-// q, k, v and the final store of y is rounded below fp32: the pre-stage writes its three results in fp32, the
-// kernel h is widened once per call when the I/O type is bf16, and the post-stage reads the gated convolution
-// in fp32.  Batches are worked off in groups of batch entries that bound the fp32 scratch.
+// Nothing between the first read of q, k, v and the final store of y is rounded below fp32.  Where the convolution is one
+// kernel (fused 2-D, slice-fused) it reads the operator's q, k, v and taps in their own type, evaluates the gates as it
+// loads and writes fp32 for the outer norm.  Elsewhere the gates are written out in fp32 and the convolution runs on an
+// fp32 plan whatever the I/O type; the kernel h is widened once per call where that plan cannot read bf16 taps.  Batches
+// are worked off in groups of batch entries that bound the fp32 scratch.
 
 struct hyenand_mixer {
     hyenand_plan *plan;               // fp32 plan over nb batch entries
     int B, C, dtype, nb;              // nb: batch entries per pass
     long long L, kvol;
     float eps;
+    bool fused;                       // the convolution's kernel evaluates the gates itself
+    float *scale;                     // scratch, fp32: one number per token of a pass
     float *qz, *kz, *vz, *oz, *h32;   // scratch, fp32 (h32: widened bf16 taps, only where the inner plan cannot read them itself)
     bool h_native;                    // the inner plan reads the taps in the caller's element type
     GuardedAllocs allocs;
@@ -1223,6 +1230,15 @@ extern "C" void hyenand_mixer_destroy(hyenand_mixer *m)
     delete m;
 }
 
+// grids whose forward is one kernel (paths PATH_FUSED2D and slice)
+static bool one_kernel_grid(int ndim, const int *dims, int mode)
+{
+    int L[3] = {1, 1, 1};
+    for (int a = 0; a < ndim; ++a) L[3 - ndim + a] = dims[a];
+    SliceGeo g;
+    return slice_geo(&g, L, mode == HYENAND_MODE_CAUSAL, mode == HYENAND_MODE_CIRCULAR);
+}
+
 extern "C" hyenand_mixer *hyenand_mixer_create(int ndim, const int *dims, int B, int C, int mode, int dtype, float eps)
 {
     g_err[0] = 0;
@@ -1239,17 +1255,30 @@ extern "C" hyenand_mixer *hyenand_mixer_create(int ndim, const int *dims, int B,
     if (const char *e = getenv("HYENAND_MIXER_MAX_BATCH")) { const long long v = atoll(e); if (v > 0 && v < nb) nb = v; }   // development aid
     if (nb < 1) nb = 1;
     if (nb > B) nb = B;
-    hyenand_plan *plan = hyenand_create_plan_mode(ndim, dims, (int)nb, C, mode, HYENAND_F32);
+    hyenand_plan *plan = hyenand_create_plan_mode(ndim, dims, (int)nb, C, mode, one_kernel_grid(ndim, dims, mode) ? dtype : HYENAND_F32);
     if (!plan) return nullptr;
+    const bool fused = plan->path == PATH_FUSED2D || plan->slice;
+    if (!fused && plan->dtype != HYENAND_F32) {            // (a development switch took the one-kernel paths away)
+        hyenand_destroy_plan(plan);
+        plan = hyenand_create_plan_mode(ndim, dims, (int)nb, C, mode, HYENAND_F32);
+        if (!plan) return nullptr;
+    }
     hyenand_mixer *m = new hyenand_mixer();
     memset(m, 0, sizeof(*m));
+    m->fused = fused;
     m->plan = plan; m->B = B; m->C = C; m->dtype = dtype; m->nb = (int)nb; m->L = L; m->kvol = plan->kvol; m->eps = eps;
     m->device = plan->device;
     m->h_native = plan_set_filter_dtype(plan, dtype);      // else bf16 taps are widened into h32 first
     const size_t n = (size_t)nb * C * L * sizeof(float);
-    cudaError_t e = guarded_alloc(&m->allocs, (void **)&m->qz, n);
-    if (e == cudaSuccess) e = guarded_alloc(&m->allocs, (void **)&m->kz, n);
-    if (e == cudaSuccess) e = guarded_alloc(&m->allocs, (void **)&m->vz, n);
+    cudaError_t e = cudaSuccess;
+    if (fused) {
+        e = guarded_alloc(&m->allocs, (void **)&m->scale, (size_t)nb * L * sizeof(float));
+    } else {
+        e = guarded_alloc(&m->allocs, (void **)&m->qz, n);
+        if (e == cudaSuccess) e = guarded_alloc(&m->allocs, (void **)&m->kz, n);
+        // (the row and column kernels of the multi-kernel paths take the gated product as one tensor; the plane kernels two)
+        if (e == cudaSuccess && plan->path == PATH_PLANES3D) e = guarded_alloc(&m->allocs, (void **)&m->vz, n);
+    }
     if (e == cudaSuccess) e = guarded_alloc(&m->allocs, (void **)&m->oz, n);
     if (e == cudaSuccess && dtype == HYENAND_BF16 && !m->h_native)
         e = guarded_alloc(&m->allocs, (void **)&m->h32, (size_t)nb * C * m->kvol * sizeof(float));
@@ -1310,7 +1339,8 @@ extern "C" int hyenand_mixer_forward(hyenand_mixer *m, const void *q, const void
         const int n = m->B - b0 < m->nb ? m->B - b0 : m->nb;
         const char *qb = (const char *)q + (size_t)b0 * slab * es, *kb = (const char *)k + (size_t)b0 * slab * es,
                    *vb = (const char *)v + (size_t)b0 * slab * es;
-        launch_mixer_pre(qb, kb, vb, g_in, m->eps, m->dtype, n, m->C, m->L, m->qz, m->kz, m->vz, st);
+        if (m->fused) launch_token_scale(qb, kb, m->eps, m->dtype, n, m->C, m->L, m->scale, st);
+        else launch_mixer_gates(qb, kb, vb, g_in, m->eps, m->dtype, n, m->C, m->L, m->qz, m->kz, m->vz, st);
         const float *hb = hf;
         if (!shared) {
             if (widen_h) {
@@ -1322,7 +1352,13 @@ extern "C" int hyenand_mixer_forward(hyenand_mixer *m, const void *q, const void
         }
         int launches = 0;
         p->r0 = 0; p->r1 = (long long)n * m->C;
-        e = run_forward(p, m->qz, m->kz, m->vz, hb, shared, m->oz, st, &launches);
+        if (m->fused) {
+            p->mix_scale = m->scale; p->mix_gin = g_in;
+            e = run_forward(p, vb, qb, kb, hb, shared, m->oz, st, &launches);
+            p->mix_scale = p->mix_gin = nullptr;
+        } else {
+            e = run_forward(p, m->qz, m->kz, m->vz, hb, shared, m->oz, st, &launches);
+        }
         p->r0 = 0; p->r1 = (long long)p->B * p->C;
         if (e) return e;
         launch_mixer_post(m->oz, g_out, m->eps, m->dtype, n, m->C, m->L, (char *)y + (size_t)b0 * slab * es, st);
@@ -1367,11 +1403,9 @@ struct hyenand_grad {
     bool pair;                        // dq and du come out of one pass over the groups (one filter spectrum serves both)
     bool ct_native;                   // long causal 1-D grid with bf16 I/O whose kernels take bf16 rows: k, v, dy, q, h are read as
                                       // they are, dq leaves its forward as bf16 (only the fp32 intermediates have scratch)
-    bool two_gate;                    // fused 2-D path, linear mode: the plan runs in the caller's element type; dq is a forward
-                                      // gated by dy, dk and dv are the two results of one forward gated by v and by k
     bool slice;                       // a slice's spectra fit in shared memory: one kernel does the whole backward (slice_bwd.cuh)
     SliceGeo sg;
-    bool native;                      // bf16 I/O on the multi-kernel paths and with two_gate: every kernel reads the caller's bf16 tensors itself and
+    bool native;                      // bf16 I/O on the multi-kernel paths: every kernel reads the caller's bf16 tensors itself and
                                       // dq leaves its pass as bf16 (no widened copies of q, k, v, dy)
     int nb;                           // batch entries per pass
     long long ns;                     // slices per pass of the dh correlation (0: not on that path)
@@ -1568,12 +1602,6 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
     const long long S = nb * C;
     g->main = create_plan(ndim, dims, (int)nb, C, mode, HYENAND_F32, false);
     if (!g->main) { delete g; return nullptr; }
-    g->two_gate = g->main->path == PATH_FUSED2D && mode == HYENAND_MODE_LINEAR;
-    if (g->two_gate && dtype != HYENAND_F32) {
-        hyenand_destroy_plan(g->main);
-        g->main = create_plan(ndim, dims, (int)nb, C, mode, dtype, false);
-        if (!g->main) { delete g; return nullptr; }
-    }
     g->adj = g->main;
     g->pair = g->main->path == PATH_PLANES3D || g->main->path == PATH_ND_GENERIC;
     // (a long causal 1-D grid gets du from the causal plan and reversed signals, see hyenand_backward)
@@ -1599,8 +1627,8 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
     auto reads_bf16 = [](const hyenand_plan *q) { return q->path == PATH_PLANES3D || q->path == PATH_ND_GENERIC; };
     g->ct_native = widen && g->long1d && mode == HYENAND_MODE_CAUSAL && g->main->path == PATH_CT1D &&
                    ct1d_takes_dtype(&g->main->ct, HYENAND_BF16);
-    g->h_native = widen && ((reads_bf16(g->main) && reads_bf16(g->adj)) || g->two_gate || g->ct_native);
-    g->native = widen && ((g->pair && mode != HYENAND_MODE_CIRCULAR && !g->long1d) || g->two_gate || g->ct_native);
+    g->h_native = widen && ((reads_bf16(g->main) && reads_bf16(g->adj)) || g->ct_native);
+    g->native = widen && ((g->pair && mode != HYENAND_MODE_CIRCULAR && !g->long1d) || g->ct_native);
     cudaError_t e = cudaSuccess;
     auto get = [&](float **ptr, long long elems) {
         if (e == cudaSuccess) e = guarded_alloc(&g->allocs, (void **)ptr, (size_t)elems * sizeof(float));
@@ -1759,22 +1787,7 @@ extern "C" int hyenand_backward(hyenand_grad *g, const void *q, const void *k, c
         // the caller's tensors of this pass, in their own element type
         const char *qn = (const char *)q + off * es, *kn = (const char *)k + off * es, *vn = (const char *)v + off * es,
                    *dyn = (const char *)dy + off * es;
-        if (g->two_gate) {
-            // the plan runs in the caller's element type: dq = dy * (h conv (k v)) is a forward gated by dy; the forward of
-            // dy q against the kernel at the opposite displacement leaves through two gates, dk = v * du and dv = k * du
-            char *dqn = (char *)dq + off * es, *dkn = (char *)dk + off * es, *dvn = (char *)dv + off * es;
-            if ((e = grad_forward(g->main, S, (const float *)dyn, (const float *)kn, (const float *)vn, h32, shared, (float *)dqn, st, g->dtype)))
-                return e;
-            RemapArgs r{};
-            r.a = h32; r.b = nullptr; r.out = g->hopp; r.slices = Sh;
-            r.a_bf16 = r.out_bf16 = widen;
-            for (int a = 0; a < 3; ++a) { r.Ls[a] = K[a]; r.G[a] = K[a]; r.mode[a] = REMAP_REV; }
-            launch_remap(r, st);
-            g->main->qg2 = kn; g->main->yg2 = dvn;
-            e = grad_forward(g->main, S, (const float *)vn, (const float *)dyn, (const float *)qn, g->hopp, shared, (float *)dkn, st, g->dtype);
-            g->main->qg2 = nullptr; g->main->yg2 = nullptr;
-            if (e) return e;
-        } else if (g->native && g->pair) {
+        if (g->native && g->pair) {
             // as below, on the caller's bf16 tensors: the first side is a bf16 forward with dy as its gate and dq as its
             // result, the second reads dy and q and leaves through two gates, dk = v * du and dv = k * du
             g->main->qg2 = kn; g->main->yg2 = (char *)dv + off * es;

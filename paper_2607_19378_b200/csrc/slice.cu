@@ -57,9 +57,10 @@ int launch_slice_bwd(const SliceBwdArgs &a, int dtype, cudaStream_t st)
 
 int launch_slice(const SliceArgs &a, int dtype, cudaStream_t st)
 {
-    if (a.g.l0 > 0) return dtype == 0 ? launch_slice_3d_f32(a, st) : launch_slice_3d_bf16(a, st);
-    if (a.g.l1 > 0) return dtype == 0 ? launch_slice_2d_f32(a, st) : launch_slice_2d_bf16(a, st);
-    return dtype == 0 ? launch_slice_1d_f32(a, st) : launch_slice_1d_bf16(a, st);
+    const bool f = dtype == 0, m = a.token_scale != nullptr;
+    if (a.g.l0 > 0) return m ? (f ? launch_slice_mix_3d_f32(a, st) : launch_slice_mix_3d_bf16(a, st)) : (f ? launch_slice_3d_f32(a, st) : launch_slice_3d_bf16(a, st));
+    if (a.g.l1 > 0) return m ? (f ? launch_slice_mix_2d_f32(a, st) : launch_slice_mix_2d_bf16(a, st)) : (f ? launch_slice_2d_f32(a, st) : launch_slice_2d_bf16(a, st));
+    return m ? (f ? launch_slice_mix_1d_f32(a, st) : launch_slice_mix_1d_bf16(a, st)) : (f ? launch_slice_1d_f32(a, st) : launch_slice_1d_bf16(a, st));
 }
 
 }  // namespace hn

@@ -24,6 +24,10 @@ struct SliceArgs {
     int C;                    // channels, for a filter shared over the batch; 0: one filter per slice
     int nb;                   // batch entries per unit of work (shared filter)
     int h_bf16;               // element type of the taps
+    // Eq. 2 around the convolution (nullptr: none): k, v, q are the operator's q, k, v, y is fp32
+    const float *token_scale; // [B][grid]
+    const float *g_in;        // [mix_C]
+    int mix_C;
     SliceGeo g;
     const float2 *gtw;
     int gtw_n;

@@ -9,6 +9,7 @@
 #pragma once
 #include "slice.cuh"
 #include "slice_fft.cuh"
+#include "mix.cuh"
 
 namespace hn {
 
@@ -172,6 +173,25 @@ __device__ __forceinline__ void slice_signal(const T *k, const T *v, const Slice
     }
 }
 
+// the operator's signal of an item's legs: q scale g_in SiLU(k)
+template <class S, int NIN, bool EVEN, typename T>
+__device__ __forceinline__ void slice_mixed(const T *q, const T *k, const float *ts, float gin, const SliceLegs<S> &g, float2 *x)
+{
+    SlPair<T, EVEN> a[NIN], b[NIN];
+    SlPair<float, EVEN> c[NIN];
+#pragma unroll
+    for (int r = 0; r < NIN; ++r) {
+        a[r].load(q + g.at(r), r < g.na, r < g.nb);
+        b[r].load(k + g.at(r), r < g.na, r < g.nb);
+        c[r].load(ts + g.at(r), r < g.na, r < g.nb);
+    }
+#pragma unroll
+    for (int r = 0; r < NIN; ++r) {
+        const float2 u = a[r].get(), w = b[r].get(), sc = c[r].get();
+        x[r] = make_float2(u.x * (sc.x * gin) * (w.x * mix_sigmoid(w.x)), u.y * (sc.y * gin) * (w.y * mix_sigmoid(w.y)));
+    }
+}
+
 // the pair of tap gradients at array index idx: the inverse of the placement above
 template <class S, typename T> __device__ __forceinline__ void slice_tap_store(T *dh, const SliceGeo &g, int idx, bool on, float2 w)
 {
@@ -240,7 +260,10 @@ template <class S, typename T> __device__ __forceinline__ void slice_prefetch(co
 }
 
 // FULL: circular mode, else the upper half of the signal's first axis is padding.  EVEN: rows of whole pairs.
-template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN>
+// MIX: Eq. 2 around the convolution.  k, v, q are then the operator's raw q, k, v: the signal is q scale g_in SiLU(k) with
+// one scale per token (the l2 norm and the inner RMSNorm, mixer.cu), the outer gate Sigmoid(v), the result fp32 for the
+// outer RMSNorm.
+template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN, bool MIX>
 __global__ void __launch_bounds__(SliceCta<SliceFft<L0, L1, L2>>::CT, SliceCta<SliceFft<L0, L1, L2>>::PER_SM) slice_fwd_kernel(SliceArgs p)
 {
     using S = SliceFft<L0, L1, L2>;
@@ -290,7 +313,14 @@ __global__ void __launch_bounds__(SliceCta<SliceFft<L0, L1, L2>>::CT, SliceCta<S
             const bool on = live && s >= p.s0 && s < p.s1;
             if (!CT::WARP && !on) continue;                  // (the same for the whole CTA)
             const T *k = (const T *)p.k + s * g.vol, *v = (const T *)p.v + s * g.vol;
-            S::template fwd_first<!FULL>(bu, tw, t, [&](int, int base, float2 *x) { slice_signal<S, NU, EVEN>(k, v, SliceLegs<S>(g, base, on), x); });
+            if constexpr (MIX) {
+                const float *ts = p.token_scale + (s / p.mix_C) * g.vol;
+                HN_G(p.g_in + s % p.mix_C, 4);
+                const float gin = on ? __ldg(p.g_in + s % p.mix_C) : 0.f;
+                S::template fwd_first<!FULL>(bu, tw, t, [&](int, int base, float2 *x) { slice_mixed<S, NU, EVEN>(k, v, ts, gin, SliceLegs<S>(g, base, on), x); });
+            } else {
+                S::template fwd_first<!FULL>(bu, tw, t, [&](int, int base, float2 *x) { slice_signal<S, NU, EVEN>(k, v, SliceLegs<S>(g, base, on), x); });
+            }
             {
                 // what this group reads next travels to L2 under this slice's transforms
                 const bool last = bi + 1 == nbu;
@@ -336,7 +366,8 @@ __global__ void __launch_bounds__(SliceCta<SliceFft<L0, L1, L2>>::CT, SliceCta<S
             S::inv_mid(bu, tw, t, sync);
             // the gate values are requested before the last barrier
             const T *q = (const T *)p.q + s * g.vol;
-            T *y = (T *)p.y + s * g.vol;
+            using TO = typename MixOut<T, MIX>::type;
+            TO *y = (TO *)p.y + s * g.vol;
             SlPair<T, EVEN> gate[S::First::IPT][NU];
 #pragma unroll
             for (int i = 0; i < S::First::IPT; ++i) {
@@ -347,19 +378,20 @@ __global__ void __launch_bounds__(SliceCta<SliceFft<L0, L1, L2>>::CT, SliceCta<S
             sync();
             S::template inv_last<!FULL>(bu, tw, t, [&](int i, int r, int, float2 w) {
                 const SliceLegs<S> lg(g, S::First::base(t + i * S::T), on);
-                const float2 a = gate[i][r].get();
-                SlPair<T, EVEN>::store(y + lg.at(r), make_float2(w.x * sc * a.x, w.y * sc * a.y), r < lg.na, r < lg.nb);
+                float2 a = gate[i][r].get();
+                if constexpr (MIX) a = make_float2(mix_sigmoid(a.x), mix_sigmoid(a.y));
+                SlPair<TO, EVEN>::store(y + lg.at(r), make_float2(w.x * sc * a.x, w.y * sc * a.y), r < lg.na, r < lg.nb);
             });
         }
     }
 }
 
-template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN> int launch_slice_t(const SliceArgs &a0, cudaStream_t st)
+template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN, bool MIX> int launch_slice_t(const SliceArgs &a0, cudaStream_t st)
 {
     using S = SliceFft<L0, L1, L2>;
     using CT = SliceCta<S>;
     constexpr size_t sm = CT::smem(2);
-    auto fn = slice_fwd_kernel<T, L0, L1, L2, FULL, EVEN>;
+    auto fn = slice_fwd_kernel<T, L0, L1, L2, FULL, EVEN, MIX>;
     static int resident[64];
     const int ctas_fit = slice_resident(resident, (const void *)fn, CT::CT, sm);
     if (ctas_fit <= 0) return -1;
@@ -387,19 +419,25 @@ template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN> int launch_s
 
 // (l1, l2) / (l0, l1, l2) instances of the 1-D, 2-D and 3-D translation units; -1: none
 int launch_slice_1d_f32(const SliceArgs &a, cudaStream_t st);
+int launch_slice_mix_1d_f32(const SliceArgs &a, cudaStream_t st);
 int launch_slice_1d_bf16(const SliceArgs &a, cudaStream_t st);
+int launch_slice_mix_1d_bf16(const SliceArgs &a, cudaStream_t st);
 int launch_slice_2d_f32(const SliceArgs &a, cudaStream_t st);
+int launch_slice_mix_2d_f32(const SliceArgs &a, cudaStream_t st);
 int launch_slice_2d_bf16(const SliceArgs &a, cudaStream_t st);
+int launch_slice_mix_2d_bf16(const SliceArgs &a, cudaStream_t st);
 int launch_slice_3d_f32(const SliceArgs &a, cudaStream_t st);
+int launch_slice_mix_3d_f32(const SliceArgs &a, cudaStream_t st);
 int launch_slice_3d_bf16(const SliceArgs &a, cudaStream_t st);
+int launch_slice_mix_3d_bf16(const SliceArgs &a, cudaStream_t st);
 
-template <typename T, int A, int B, int C> int launch_slice_d(const SliceArgs &a, cudaStream_t st)
+template <typename T, int A, int B, int C, bool MIX> int launch_slice_d(const SliceArgs &a, cudaStream_t st)
 {
-    if (a.g.full) return launch_slice_t<T, A, B, C, true, true>(a, st);          // (power-of-two rows)
-    return (a.g.L[2] & 1) ? launch_slice_t<T, A, B, C, false, false>(a, st) : launch_slice_t<T, A, B, C, false, true>(a, st);
+    if (a.g.full) return launch_slice_t<T, A, B, C, true, true, MIX>(a, st);          // (power-of-two rows)
+    return (a.g.L[2] & 1) ? launch_slice_t<T, A, B, C, false, false, MIX>(a, st) : launch_slice_t<T, A, B, C, false, true, MIX>(a, st);
 }
 #define HN_SLICE_CASE(A, B, C)                                                                             \
-    if (a.g.l0 == A && a.g.l1 == B && a.g.l2 == C) return launch_slice_d<HN_SLICE_T, A, B, C>(a, st);
+    if (a.g.l0 == A && a.g.l1 == B && a.g.l2 == C) return launch_slice_d<HN_SLICE_T, A, B, C, HN_SLICE_MIX>(a, st);
 
 // instances of the engine: 1-D lines of 128 .. 8192 reals; 2-D and 3-D grids of up to 8192 complex points
 #define HN_SLICE_1D(X) X(0, 0, 6) X(0, 0, 7) X(0, 0, 8) X(0, 0, 9) X(0, 0, 10) X(0, 0, 11) X(0, 0, 12)

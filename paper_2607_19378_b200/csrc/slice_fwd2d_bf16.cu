@@ -1,6 +1,7 @@
 // Instances of the slice-fused forward for 2-D grids of bf16 tensors.
 #include "slice_fwd.cuh"
 #define HN_SLICE_T bf16
+#define HN_SLICE_MIX false
 
 namespace hn {
 
