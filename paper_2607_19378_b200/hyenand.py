@@ -8,6 +8,7 @@ library has not been built, loading raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import torch
@@ -118,7 +119,7 @@ def _check(code: int):
 
 
 def hyenand_create_plan(ndim: int, dims, B: int, C: int, causal: int, dtype: int) -> int:
-    arr = (ctypes.c_int * max(1, len(dims)))(*[int(d) for d in dims])
+    arr = _dims_array(tuple(map(int, dims)))
     h = lib().hyenand_create_plan(int(ndim), arr, int(B), int(C), int(causal), int(dtype))
     if not h:
         msg = hyenand_last_error()
@@ -128,7 +129,7 @@ def hyenand_create_plan(ndim: int, dims, B: int, C: int, causal: int, dtype: int
 
 
 def hyenand_create_plan_mode(ndim: int, dims, B: int, C: int, mode: int, dtype: int) -> int:
-    arr = (ctypes.c_int * max(1, len(dims)))(*[int(d) for d in dims])
+    arr = _dims_array(tuple(map(int, dims)))
     h = lib().hyenand_create_plan_mode(int(ndim), arr, int(B), int(C), int(mode), int(dtype))
     if not h:
         msg = hyenand_last_error()
@@ -141,8 +142,23 @@ def hyenand_destroy_plan(plan: int) -> None:
     lib().hyenand_destroy_plan(plan)
 
 
+@functools.lru_cache(maxsize=64)
+def _dims_array(dims: tuple):
+    """dims as a C int array (read only: the library copies what it keeps)."""
+    return (ctypes.c_int * max(1, len(dims)))(*dims)
+
+
+# The calls below are the launch path of small problems, whose kernels take a few microseconds: no tensor views, no stream
+# objects, shapes compared with tuples worked out when the object was created (one 32x32x8 forward: 15.2 us a call when the
+# filter's stride came from h[0, 0].numel() and the stream from torch.cuda.current_stream(), 8 now).
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -255,14 +271,14 @@ def hyenand_forward_noalloc(dims, B: int, C: int, causal: int, dtype: int, q, k,
                             h_batch_stride_elems: int, y, stream=None) -> None:
     """Forward through the entry point that allocates no device memory (fixed workspace inside
     the library; see include/hyenand.h for its limits and the rule about overlapping calls)."""
-    arr = (ctypes.c_int * max(1, len(dims)))(*[int(d) for d in dims])
+    arr = _dims_array(tuple(map(int, dims)))
     _check(lib().hyenand_forward_noalloc(len(dims), arr, int(B), int(C), int(causal), int(dtype),
                                          q.data_ptr(), k.data_ptr(), v.data_ptr(), h.data_ptr(),
                                          int(h_batch_stride_elems), y.data_ptr(), _stream_ptr(stream)))
 
 
 def hyenand_mixer_create(ndim: int, dims, B: int, C: int, mode: int, dtype: int, eps: float) -> int:
-    arr = (ctypes.c_int * max(1, len(dims)))(*[int(d) for d in dims])
+    arr = _dims_array(tuple(map(int, dims)))
     h = lib().hyenand_mixer_create(int(ndim), arr, int(B), int(C), int(mode), int(dtype), float(eps))
     if not h:
         raise HyenaNDError(hyenand_last_error_code() or HYENAND_ERR_INVALID_ARG, hyenand_last_error())
@@ -291,7 +307,7 @@ def hyenand_synthesize_kernel(dims, mode: int, B: int, C: int, hidden: int, laye
                               bout, gamma, beta, window, dtype: int, h, stream=None) -> None:
     """K(x) on the tap grid of `dims` into h (device tensor [B, C, K..]); parameters: fp32 device tensors, gamma and
     beta may both be None (static kernel), Wh and bh may be None when layers == 1."""
-    arr = (ctypes.c_int * max(1, len(dims)))(*[int(d) for d in dims])
+    arr = _dims_array(tuple(map(int, dims)))
     ptr = lambda t: None if t is None else t.data_ptr()
     _check(lib().hyenand_synthesize_kernel(len(dims), arr, int(mode), int(B), int(C), int(hidden), int(layers),
                                            ptr(W1), ptr(b1), ptr(omega0), ptr(Wh), ptr(bh), ptr(Wout), ptr(bout),
@@ -299,7 +315,7 @@ def hyenand_synthesize_kernel(dims, mode: int, B: int, C: int, hidden: int, laye
 
 
 def hyenand_backward_create(ndim: int, dims, B: int, C: int, mode: int, dtype: int) -> int:
-    arr = (ctypes.c_int * max(1, len(dims)))(*[int(d) for d in dims])
+    arr = _dims_array(tuple(map(int, dims)))
     h = lib().hyenand_backward_create(int(ndim), arr, int(B), int(C), int(mode), int(dtype))
     if not h:
         raise HyenaNDError(hyenand_last_error_code() or HYENAND_ERR_INVALID_ARG, hyenand_last_error())
@@ -319,6 +335,30 @@ def hyenand_backward_destroy(grad: int) -> None:
     lib().hyenand_backward_destroy(grad)
 
 
+def _check_tensors(tensors, dtype, what):
+    for t in tensors:
+        if not (t.is_cuda and t.is_contiguous() and t.dtype == dtype):
+            raise ValueError(f"inputs must be contiguous CUDA tensors of the {what}'s dtype")
+
+
+class _FilterShape:
+    """h's shape -> batch stride: 0 for one filter per channel [C, K..], C K.. for one per sample [B, C, K..]."""
+
+    def __init__(self, B, C, taps):
+        self.shared, self.full = (C,) + taps, (B, C) + taps
+        self.stride = C
+        for K in taps:
+            self.stride *= K
+
+    def __call__(self, h) -> int:
+        shape = h.shape
+        if shape == self.full:
+            return self.stride
+        if shape == self.shared:
+            return 0
+        raise ValueError(f"h has shape {tuple(shape)}")
+
+
 class Backward:
     """Owner of a hyenand_grad handle: dq, dk, dv, dh of the gated long convolution."""
 
@@ -326,19 +366,12 @@ class Backward:
         self.dims = tuple(int(d) for d in dims)
         self.B, self.C, self.mode, self.dtype = B, C, mode, dtype
         code = {"linear": HYENAND_MODE_LINEAR, "causal": HYENAND_MODE_CAUSAL, "circular": HYENAND_MODE_CIRCULAR}[mode]
+        self._filter = _FilterShape(B, C, tuple(2 * L - 1 if mode == "linear" else L for L in self.dims))
         self.handle = hyenand_backward_create(len(self.dims), self.dims, B, C, code, _DTYPES[dtype])
 
     def __call__(self, q, k, v, h, dy, stream=None):
-        taps = tuple(2 * L - 1 if self.mode == "linear" else L for L in self.dims)
-        if tuple(h.shape) == (self.C,) + taps:
-            stride = 0
-        elif tuple(h.shape) == (self.B, self.C) + taps:
-            stride = self.C * h[0, 0].numel()
-        else:
-            raise ValueError(f"h has shape {tuple(h.shape)}")
-        for t in (q, k, v, h, dy):
-            if not (t.is_cuda and t.is_contiguous() and t.dtype == self.dtype):
-                raise ValueError("inputs must be contiguous CUDA tensors of the handle's dtype")
+        stride = self._filter(h)
+        _check_tensors((q, k, v, h, dy), self.dtype, "handle")
         dq, dk, dv, dh = torch.empty_like(q), torch.empty_like(q), torch.empty_like(q), torch.empty_like(h)
         hyenand_backward(self.handle, q, k, v, h, stride, dy, dq, dk, dv, dh, stream)
         return dq, dk, dv, dh
@@ -362,19 +395,12 @@ class Mixer:
         self.dims = tuple(int(d) for d in dims)
         self.B, self.C, self.mode, self.dtype = B, C, mode, dtype
         code = {"linear": HYENAND_MODE_LINEAR, "causal": HYENAND_MODE_CAUSAL, "circular": HYENAND_MODE_CIRCULAR}[mode]
+        self._filter = _FilterShape(B, C, tuple(2 * L - 1 if mode == "linear" else L for L in self.dims))
         self.handle = hyenand_mixer_create(len(self.dims), self.dims, B, C, code, _DTYPES[dtype], eps)
 
     def forward(self, q, k, v, h, g_in, g_out, y=None, stream=None):
-        taps = tuple(2 * L - 1 if self.mode == "linear" else L for L in self.dims)
-        if tuple(h.shape) == (self.C,) + taps:
-            stride = 0
-        elif tuple(h.shape) == (self.B, self.C) + taps:
-            stride = self.C * h[0, 0].numel()
-        else:
-            raise ValueError(f"h has shape {tuple(h.shape)}")
-        for t in (q, k, v, h):
-            if not (t.is_cuda and t.is_contiguous() and t.dtype == self.dtype):
-                raise ValueError("inputs must be contiguous CUDA tensors of the mixer's dtype")
+        stride = self._filter(h)
+        _check_tensors((q, k, v, h), self.dtype, "mixer")
         for g in (g_in, g_out):
             if not (g.is_cuda and g.is_contiguous() and g.dtype == torch.float32 and g.numel() == self.C):
                 raise ValueError("g_in, g_out must be contiguous fp32 CUDA tensors of C elements")
@@ -401,6 +427,7 @@ class Plan:
     def __init__(self, dims, B: int, C: int, causal: bool = False, dtype=torch.float32, circular: bool = False):
         self.dims = tuple(int(d) for d in dims)
         self.B, self.C, self.causal, self.dtype, self.circular = B, C, bool(causal), dtype, bool(circular)
+        self._stride = _FilterShape(B, C, tuple(L if (self.causal or self.circular) else 2 * L - 1 for L in self.dims))
         if self.circular:
             if self.causal:
                 raise ValueError("a plan is causal or circular, not both")
@@ -408,19 +435,9 @@ class Plan:
         else:
             self.handle = hyenand_create_plan(len(self.dims), self.dims, B, C, int(self.causal), _DTYPES[dtype])
 
-    def _stride(self, h) -> int:
-        taps = tuple(L if (self.causal or self.circular) else 2 * L - 1 for L in self.dims)
-        if tuple(h.shape) == (self.C,) + taps:
-            return 0
-        if tuple(h.shape) == (self.B, self.C) + taps:
-            return self.C * h[0, 0].numel()
-        raise ValueError(f"h has shape {tuple(h.shape)}")
-
     def forward(self, q, k, v, h, y=None, stream=None):
         """Device tensors in, device tensor out (enqueued on the current stream)."""
-        for t in (q, k, v, h):
-            if not (t.is_cuda and t.is_contiguous() and t.dtype == self.dtype):
-                raise ValueError("inputs must be contiguous CUDA tensors of the plan's dtype")
+        _check_tensors((q, k, v, h), self.dtype, "plan")
         if y is None:
             y = torch.empty_like(q)
         hyenand_forward_ex(self.handle, q, k, v, h, self._stride(h), y, stream)
