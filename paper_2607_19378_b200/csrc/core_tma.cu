@@ -1,8 +1,8 @@
-// Fused spectral core along a strided axis for 256- and 1024-point lines, tiles moved by TMA.
+// Fused spectral core along a strided axis for 64- to 1024-point lines, tiles moved by TMA.
 //
 // Same arithmetic as core_w.cu (forward transform of the filter lines, forward transform of the
 // k*v lines, spectral product of Eq. 12 of the paper, inverse, cropped half written back in
-// place), but the tiles -- 8 adjacent bins by all rows of the axis -- travel as tensor copies:
+// place), but the tiles -- 8 or 16 adjacent bins by all rows of the axis -- travel as tensor copies:
 //
 //   cp.async.bulk.tensor loads   filter tile (boxes of up to 256 rows; the wrapped placement of the
 //                                taps is two row ranges) and k*v tile (one box; rows past the data
@@ -25,39 +25,46 @@
 
 namespace hn {
 
-// Threads per CTA: 256-point lines run as 4 CTAs of 128 threads per SM (8 lines per tile), 1024-point lines as one
-// CTA of 256 threads (8 lines per tile).  A CTA synchronises at two barriers per tile; more, smaller CTAs per SM
-// keep the schedulers busy while one of them waits.
-template <int LOG2P> struct TmaCta {
+// Threads per CTA: 128, several CTAs per SM (a CTA synchronises at two barriers per tile; more, smaller CTAs keep the
+// schedulers busy while one of them waits), but one CTA of 256 threads for 1024-point lines.
+// FULL (periodic axis: N rows in, N rows out) at 512 points: the result tile takes the k*v tile's buffer, which keeps two
+// CTAs per SM; the next k*v tile is then asked for after the result has left, under the next filter tile's transforms.
+template <int LOG2P, bool FULL> struct TmaCta {
     static constexpr int THREADS = LOG2P >= 10 ? 256 : 128;
-    static constexpr int PER_SM = LOG2P >= 10 ? 1 : 4;
+    static constexpr int PER_SM = LOG2P >= 10 ? 1 : LOG2P == 9 ? 2 : FULL && LOG2P >= 7 ? 3 : 4;
+    static constexpr bool SHARE = FULL && LOG2P >= 9;
 };
 
 // Geometry of a tile for LOG2P-point lines: one line per group of TPL lanes, so TX = THREADS / TPL bins
-// per tile and TX * 8 bytes per tile row (64 here: the swizzle span of the tensor maps).  A box holds at
+// per tile and TX * 8 bytes per tile row (64 or 128: the swizzle span of the tensor maps).  A box holds at
 // most 256 rows.
-template <int LOG2P> struct TmaGeo {
+template <int LOG2P, bool FULL> struct TmaGeo {
     using F = WF<LOG2P, false>;
     static constexpr int N = 1 << LOG2P, HALF = N / 2;
-    static constexpr int THREADS = TmaCta<LOG2P>::THREADS;
+    using CTA = TmaCta<LOG2P, FULL>;
+    static constexpr int THREADS = CTA::THREADS;
     static constexpr int TX = THREADS / F::TPL;
     static constexpr unsigned ROWB = TX * 8;
     static constexpr int BOXR = HALF < 256 ? HALF : 256;             // rows per box
     static constexpr int NB = HALF / BOXR;                           // boxes per half line
     static constexpr unsigned BOXB = BOXR * ROWB;
     static constexpr unsigned HALFB = HALF * ROWB;
-    // 16-lane groups (two lines per warp): the lanes of a half warp belong to both lines (see the kernel), whose
+    static constexpr unsigned UB = FULL ? 2 * HALFB : HALFB;         // k*v tile and result tile
+    static constexpr int NBU = FULL ? 2 * NB : NB;                   // their boxes
+    // 8- and 16-lane groups (several lines per warp): a half warp works on two lines (see the kernel), whose
     // strides are therefore 8 mod 16 entries, i.e. half a bank row apart
-    static constexpr int LS = F::TPL == 16 ? plane_ls(N) : ((F::ph(N - 1) + 1 + 15) / 16 * 16 + 2);
+    static constexpr int LS = F::TPL <= 16 ? plane_ls(N) : ((F::ph(N - 1) + 1 + 15) / 16 * 16 + 2);
     static_assert(ROWB == 128 || ROWB == 64, "tile rows match a swizzle span");
+    static constexpr int TWTAB = N + PlaneTw<LOG2P, false>::TABLE + PlaneTw<LOG2P, true>::TABLE;
     // shared memory: tile buffers first (1024-byte aligned, as the swizzle pattern repeats every 1024 bytes)
     static constexpr size_t TH = 0;                                  // filter tile, N rows
-    static constexpr size_t TU = TH + 2 * HALFB;                     // k*v tile, N/2 rows
-    static constexpr size_t TO = TU + HALFB;                         // result tile, N/2 rows
-    static constexpr size_t LINES = TO + HALFB;                      // one skewed line per group
+    static constexpr size_t TU = TH + 2 * HALFB;                     // k*v tile
+    static constexpr size_t TO = CTA::SHARE ? TU : TU + UB;          // result tile
+    static constexpr size_t LINES = TO + UB;                         // one skewed line per group
     static constexpr size_t TW = LINES + sizeof(float2) * TX * LS;
-    static constexpr size_t BARS = TW + sizeof(float2) * N;
+    static constexpr size_t BARS = TW + sizeof(float2) * TWTAB;
     static constexpr size_t TOTAL = BARS + 2 * sizeof(uint64_t) + 1024;    // + room to align the start
+    static_assert(CTA::PER_SM * (TOTAL + 1024) <= 228 * 1024, "resident CTAs");
 };
 
 struct CoreTmaParams {
@@ -72,19 +79,24 @@ struct CoreTmaParams {
     int *status;              // device word: 0 ok, else which wait gave up
 };
 
-template <int LOG2P>
-__global__ void __launch_bounds__(TmaCta<LOG2P>::THREADS, TmaCta<LOG2P>::PER_SM)
+template <int LOG2P, bool FULL>
+__global__ void __launch_bounds__(TmaCta<LOG2P, FULL>::THREADS, TmaCta<LOG2P, FULL>::PER_SM)
 axis_core_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_constant__ CUtensorMap map_h, CoreTmaParams p)
 {
-    using G = TmaGeo<LOG2P>;
+    using G = TmaGeo<LOG2P, FULL>;
     using F = WF<LOG2P, false>;
     using FI = WF<LOG2P, true>;
     constexpr int N = G::N, TPL = F::TPL, NP = F::NP, kTmaThreads = G::THREADS;
-    static_assert(NP == 2 && F::radix(0) == F::radix(1), "two equal passes: one register set of twiddles serves both directions");
+    // two equal passes: the twiddles depend on the lane only and live in registers; the inverse uses the same values
+    // conjugated, so one set serves both directions
+    constexpr bool EQUAL = NP == 2 && F::radix(0) == F::radix(1);
+    static_assert(NP == 2, "two passes");
     using PL = typename F::template Pass<NP - 1>;
     using P0 = typename F::template Pass<0>;
-    static_assert(P0::IPL == 1 && PL::IPL == 1, "one item per lane and pass");
-    constexpr int RSTEP = (N / P0::R) * (int)G::ROWB / 8;            // float2 between legs r and r+1 of a lane in a tile
+    using PE = typename FI::template Pass<NP - 1>;
+    // float2 between a lane's first point and leg r of item i in a tile: multiples of 8 rows, which the swizzle repeats after
+    constexpr int RF2 = (int)G::ROWB / 8;
+    static_assert(TPL % 8 == 0 && (N / P0::R) % 8 == 0 && (N / PE::R) % 8 == 0, "legs keep the swizzle");
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     // the swizzle pattern is a function of the shared-memory address: start on a 1024-byte boundary
     unsigned char *smem_raw = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
@@ -111,11 +123,14 @@ axis_core_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_con
         fence_mbar_init();
     }
     __syncthreads();
-    // two equal passes: the twiddles depend on the lane only and live in registers; the inverse uses the
-    // same values conjugated, so one set serves both directions
     PlaneTw<LOG2P, false> tw;
-    static_assert(PlaneTw<LOG2P, false>::HOIST, "register twiddles");
-    tw.init(l, twt, twt, tid, kTmaThreads);
+    tw.init(l, twt, twt + N, tid, kTmaThreads);
+    PlaneTw<LOG2P, true> twi_own;
+    if constexpr (!EQUAL) {
+        twi_own.init(l, twt, twt + N + PlaneTw<LOG2P, false>::TABLE, tid, kTmaThreads);
+        __syncthreads();
+    }
+    const auto &twi = [&]() -> const auto & { if constexpr (EQUAL) return tw; else return twi_own; }();
     // Row z = l + TPL*r of bin `gid` inside a swizzled tile.  A row is ROWB bytes; the 16-byte chunk index
     // of an address is XORed with address bits 7 and up (3 bits for the 128-byte swizzle, 2 for the 64-byte
     // one), i.e. with a function of z that TPL*r does not change: every leg r is the same per-lane offset
@@ -131,23 +146,23 @@ axis_core_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_con
         mbar_expect_tx(bar_h, 2 * G::HALFB);
 #pragma unroll
         for (int b = 0; b < G::NB; ++b) {
-            // positions [0, N/2) hold filter rows from h_shift on, positions [N/2, N) the rows before it
+            // positions [0, N/2) hold filter rows from h_shift on, positions [N/2, N) the rows before it (periodic: all in order)
             tma_load_3d(th + b * G::BOXB, &map_h, bar_h, x, p.h_shift + b * G::BOXR, (int)oh);
-            tma_load_3d(th + G::HALFB + b * G::BOXB, &map_h, bar_h, x, p.h_shift - G::HALF + b * G::BOXR, (int)oh);
+            tma_load_3d(th + G::HALFB + b * G::BOXB, &map_h, bar_h, x, (FULL ? G::HALF : p.h_shift - G::HALF) + b * G::BOXR, (int)oh);
         }
     };
     auto issue_u = [&](long long t) {
         const long long o = t / p.tiles_per_outer;
         const int x = (int)(t % p.tiles_per_outer) * G::TX * 2;
-        mbar_expect_tx(bar_u, G::HALFB);
+        mbar_expect_tx(bar_u, G::UB);
 #pragma unroll
-        for (int b = 0; b < G::NB; ++b) tma_load_3d(tu + b * G::BOXB, &map_u, bar_u, x, b * G::BOXR, (int)o);
+        for (int b = 0; b < G::NBU; ++b) tma_load_3d(tu + b * G::BOXB, &map_u, bar_u, x, b * G::BOXR, (int)o);
     };
     auto store_tile = [&](long long t) {               // one thread
         const long long o = t / p.tiles_per_outer;
         const int x = (int)(t % p.tiles_per_outer) * G::TX * 2;
 #pragma unroll
-        for (int b = 0; b < G::NB; ++b) tma_store_3d(&map_u, to + b * G::BOXB, x, b * G::BOXR, (int)o);
+        for (int b = 0; b < G::NBU; ++b) tma_store_3d(&map_u, to + b * G::BOXB, x, b * G::BOXR, (int)o);
         tma_commit();
     };
     long long t = blockIdx.x, tprev = 0;
@@ -157,13 +172,13 @@ axis_core_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_con
     int failed = 0;
     for (; t < tiles; t += gridDim.x, phase ^= 1u) {
         const long long tn = t + gridDim.x;
-        float2 H[PL::R];
+        float2 H[PL::IPL][PL::R];
         // ---- filter lines: tile -> registers ------------------------------------------------------
         if (!mbar_wait(bar_h, phase)) failed = 1;
         {
             const float2 *src = reinterpret_cast<const float2 *>(th + tile_off);
             F::template pass<0, PRUNE_NONE>(l, tw,
-                [&](int, int r, int) { return src[r * RSTEP]; },
+                [&](int i, int r, int) { return src[(i * TPL + r * (N / P0::R)) * RF2]; },
                 [&](int, int, int idx, float2 v) { line[F::ph(idx)] = v; });
         }
         if (__syncthreads_or(failed)) break;           // the filter tile buffer is free again; the previous result tile is complete
@@ -173,33 +188,37 @@ axis_core_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_con
         }
         F::template pass<NP - 1, PRUNE_NONE>(l, tw,
             [&](int, int, int idx) { return line[F::ph(idx)]; },
-            [&](int, int r, int, float2 v) { H[r] = make_float2(v.x * p.scale, v.y * p.scale_im); });
+            [&](int i, int r, int, float2 v) { H[i][r] = make_float2(v.x * p.scale, v.y * p.scale_im); });
         __syncwarp(m);
+        if constexpr (G::CTA::SHARE) {
+            // the previous result tile has left the buffer it shares with the k*v tile
+            if (tid == 0 && have_prev) { tma_wait_read0(); issue_u(t); }
+        }
         // ---- k*v lines: tile -> spectrum, product, inverse ----------------------------------------
         if (!mbar_wait(bar_u, phase)) failed = 2;
         {
             const float2 *src = reinterpret_cast<const float2 *>(tu + tile_off);
-            F::template pass<0, PRUNE_IN>(l, tw,
-                [&](int, int r, int) { return src[r * RSTEP]; },
+            F::template pass<0, FULL ? PRUNE_NONE : PRUNE_IN>(l, tw,
+                [&](int i, int r, int) { return src[(i * TPL + r * (N / P0::R)) * RF2]; },
                 [&](int, int, int idx, float2 v) { line[F::ph(idx)] = v; });
         }
-        if (tid == 0) tma_wait_read0();                // the previous result tile has left its buffer
+        if (!G::CTA::SHARE && tid == 0) tma_wait_read0();      // the previous result tile has left its buffer
         if (__syncthreads_or(failed)) break;           // the k*v tile buffer is free again
-        if (tid == 0 && tn < tiles) issue_u(tn);
-        float2 Y[PL::R];
+        if (!G::CTA::SHARE && tid == 0 && tn < tiles) issue_u(tn);
+        float2 Y[PL::IPL][PL::R];
         F::template pass<NP - 1, PRUNE_NONE>(l, tw,
             [&](int, int, int idx) { return line[F::ph(idx)]; },
-            [&](int, int r, int, float2 v) { Y[r] = cmul(v, H[r]); });
+            [&](int i, int r, int, float2 v) { Y[i][r] = cmul(v, H[i][r]); });
         __syncwarp(m);
-        FI::template pass<0, PRUNE_NONE>(l, tw,
-            [&](int, int r, int) { return Y[r]; },
+        FI::template pass<0, PRUNE_NONE>(l, twi,
+            [&](int i, int r, int) { return Y[i][r]; },
             [&](int, int, int idx, float2 v) { line[FI::ph(idx)] = v; });
         __syncwarp(m);
         {
             float2 *dst = reinterpret_cast<float2 *>(to + tile_off);
-            FI::template pass<NP - 1, PRUNE_OUT>(l, tw,
+            FI::template pass<NP - 1, FULL ? PRUNE_NONE : PRUNE_OUT>(l, twi,
                 [&](int, int, int idx) { return line[FI::ph(idx)]; },
-                [&](int, int r, int, float2 v) { dst[r * RSTEP] = v; });
+                [&](int i, int r, int, float2 v) { dst[(i * TPL + r * (N / PE::R)) * RF2] = v; });
         }
         __syncwarp(m);
         fence_async_smem();                            // generic-proxy writes visible to the copy engine
@@ -234,24 +253,27 @@ static bool make_map(CUtensorMap *map, const float2 *base, long long outer, int 
     return tma_encode_3d(map, base, /*bf16=*/false, dims, strides, box, tx * 8);
 }
 
-static bool tma_log2p_ok(int log2p) { return log2p == 8 || log2p == 10; }
-
 bool core_tma_supported(const AxisArgs &a)
 {
-    if (!tma_log2p_ok(a.log2p)) return false;
+    if (a.log2p < 6 || a.log2p > 10) return false;
     const int n = 1 << a.log2p;
-    return a.in == a.out && a.in_outer == a.out_outer && a.n_in == a.n_out && a.n_in >= 1 && a.n_in <= n / 2 &&
-           a.h_n_in >= 1 && a.h_n_in <= n && a.shift == 0 && a.h_shift >= 0 && a.h_shift < n && (a.nc % 2) == 0 &&
-           a.n_outer < (1ll << 31) && tma_available();
+    const bool rows = a.full ? a.n_in == n && a.h_n_in == n && a.h_shift == 0 && a.log2p <= 9
+                             : a.n_in >= 1 && a.n_in <= n / 2 && a.h_n_in >= 1 && a.h_n_in <= n;
+    return rows && a.in == a.out && a.in_outer == a.out_outer && a.n_in == a.n_out && a.shift == 0 && a.h_shift >= 0 && a.h_shift < n &&
+           (a.nc % 2) == 0 && a.n_outer < (1ll << 31) && tma_available();
 }
+
+#define HN_TMA_CASES(X) X(6) X(7) X(8) X(9) X(10)
 
 bool core_tma_make(CoreTmaMaps *m, const AxisArgs &a, long long max_outer, long long h_outer_count)
 {
     m->valid = false;
     if (!core_tma_supported(a)) return false;
     static_assert(sizeof(m->u) >= sizeof(CUtensorMap) && sizeof(m->h) >= sizeof(CUtensorMap), "room for a tensor map");
-    const int tx = a.log2p == 8 ? TmaGeo<8>::TX : TmaGeo<10>::TX;
-    const int br = a.log2p == 8 ? TmaGeo<8>::BOXR : TmaGeo<10>::BOXR;
+    int tx = 0, br = 0;                                    // (tile width and box height do not depend on FULL)
+#define HN_TMA_GEO(L) if (a.log2p == L) { tx = TmaGeo<L, false>::TX; br = TmaGeo<L, false>::BOXR; }
+    HN_TMA_CASES(HN_TMA_GEO)
+#undef HN_TMA_GEO
     if (!make_map(reinterpret_cast<CUtensorMap *>(m->u), a.in, max_outer, a.n_in, a.nc, a.in_outer, tx, br)) return false;
     if (!make_map(reinterpret_cast<CUtensorMap *>(m->h), a.h, h_outer_count, a.h_n_in, a.nc, a.h_outer, tx, br)) return false;
     m->in = a.in; m->h_base = a.h; m->nc = a.nc; m->n_in = a.n_in; m->h_n_in = a.h_n_in; m->log2p = a.log2p;
@@ -260,9 +282,9 @@ bool core_tma_make(CoreTmaMaps *m, const AxisArgs &a, long long max_outer, long 
     return true;
 }
 
-template <int LOG2P> static int launch_core_tma_t(const CoreTmaParams &p0, const CoreTmaMaps &m, int nc, cudaStream_t st)
+template <int LOG2P, bool FULL> static int launch_core_tma_t(const CoreTmaParams &p0, const CoreTmaMaps &m, int nc, cudaStream_t st)
 {
-    using G = TmaGeo<LOG2P>;
+    using G = TmaGeo<LOG2P, FULL>;
     CoreTmaParams p = p0;
     p.tiles_per_outer = (nc + G::TX - 1) / G::TX;
     static int sms = 0;
@@ -274,12 +296,12 @@ template <int LOG2P> static int launch_core_tma_t(const CoreTmaParams &p0, const
     }
     static DevOnce attr;
     if (attr.first())
-        cudaFuncSetAttribute(axis_core_tma_kernel<LOG2P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::TOTAL);
+        cudaFuncSetAttribute(axis_core_tma_kernel<LOG2P, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::TOTAL);
     const long long tiles = p.n_outer * p.tiles_per_outer;
-    const long long res = (long long)sms * TmaCta<LOG2P>::PER_SM;    // resident CTAs
+    const long long res = (long long)sms * G::CTA::PER_SM;           // resident CTAs
     const int grid = (int)(tiles < res ? tiles : res);
     if (grid <= 0) return 0;
-    axis_core_tma_kernel<LOG2P><<<grid, G::THREADS, G::TOTAL, st>>>(
+    axis_core_tma_kernel<LOG2P, FULL><<<grid, G::THREADS, G::TOTAL, st>>>(
         *reinterpret_cast<const CUtensorMap *>(m.u), *reinterpret_cast<const CUtensorMap *>(m.h), p);
     return 1;
 }
@@ -297,7 +319,13 @@ int launch_core_tma(const AxisArgs &a, const CoreTmaMaps &m, int *status, cudaSt
     p.n_outer = a.n_outer;
     p.h_shift = a.h_shift; p.h_mod = a.h_mod; p.h_off = a.h_off;
     p.scale = a.scale; p.scale_im = a.h_conj ? -a.scale : a.scale; p.gtw = a.gtw; p.gtw_n = a.gtw_n; p.status = status;
-    return a.log2p == 8 ? launch_core_tma_t<8>(p, m, a.nc, st) : launch_core_tma_t<10>(p, m, a.nc, st);
+    switch (a.log2p) {
+    case 6: return a.full ? launch_core_tma_t<6, true>(p, m, a.nc, st) : launch_core_tma_t<6, false>(p, m, a.nc, st);
+    case 7: return a.full ? launch_core_tma_t<7, true>(p, m, a.nc, st) : launch_core_tma_t<7, false>(p, m, a.nc, st);
+    case 8: return a.full ? launch_core_tma_t<8, true>(p, m, a.nc, st) : launch_core_tma_t<8, false>(p, m, a.nc, st);
+    case 9: return a.full ? launch_core_tma_t<9, true>(p, m, a.nc, st) : launch_core_tma_t<9, false>(p, m, a.nc, st);
+    default: return launch_core_tma_t<10, false>(p, m, a.nc, st);
+    }
 }
 
 }  // namespace hn

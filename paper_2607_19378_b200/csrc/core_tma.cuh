@@ -16,7 +16,7 @@ struct CoreTmaMaps {
     bool valid;
 };
 
-// true if `a` is a case the TMA core handles (256- or 1024-point axis, in place, even number of bins) and the
+// true if `a` is a case the TMA core handles (64- to 1024-point axis, periodic up to 512, in place, even number of bins) and the
 // driver offers tensor-map encoding
 bool core_tma_supported(const AxisArgs &a);
 // builds the maps for buffers a.in (max_outer outer entries) and a.h (h_outer_count entries)

@@ -292,8 +292,8 @@ static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mo
     const bool slice_ok = allow_slice && !p->sw.force_generic && !p->sw.generic_rows && !p->sw.generic_core && !getenv("HYENAND_GROUP_SLICES");
     if (circular) {
         // periodic boundaries run on the general N-D passes, which transform whole lines here (nothing is
-        // padded, so there is no zero half to prune and no half to crop); no plane, fused or tensor-copy kernels
-        p->sw.force_generic = p->sw.no_tma = true;
+        // padded, so there is no zero half to prune and no half to crop); no plane or fused kernels
+        p->sw.force_generic = true;
     }
 
     if (ndim == 1 && p->log2p[2] > kMaxLineLog2 && !circular) {
@@ -399,7 +399,7 @@ extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int
 static void make_core_maps(hyenand_plan *p)
 {
     if ((p->path != PATH_PLANES3D && p->path != PATH_ND_GENERIC) || p->slice) return;
-    if (p->sw.no_tma) return;
+    if (p->sw.no_tma || p->sw.generic_core) return;
     const long long spc = p->slices_per_chunk;
     for (int l = 0; l < p->n_lanes; ++l) {
         hyenand_plan::Lane &ln = p->lane[l];
