@@ -216,6 +216,7 @@ struct RowsInvArgs {
     const float2 *gtw;
     int gtw_n;
     int full_out;         // 1: no output half is cropped away, the first len <= P outputs of a row are kept (circular mode: len == P)
+    int shift;            // full_out only: element n of a row is position (n - shift) mod P (rows of taps)
 };
 
 // A family of strided lines: line (o, c), element a at base[o*outer + a*nc + c].
@@ -229,7 +230,8 @@ struct AxisArgs {
     int nc;                   // contiguous lines per outer index (= element stride along the axis)
     int n_in;                 // valid input entries along the axis
     int n_out;                // entries written along the axis
-    int shift;                // input entry m goes to position (m - shift) mod P
+    int shift;                // forward: input entry m goes to position (m - shift) mod P; inverse with `full`: entry m is position
+                              // (m - shift) mod P
     int log2p;
     int prune_in;
     // core only: filter lines, outer index oh = h_shared ? o % h_mod : o

@@ -249,6 +249,7 @@ __global__ void __launch_bounds__(core_threads(LOG2P), (LOG2P >= 10 ? 1 : 2)) ax
     __syncthreads();
     const long long tpo = (p.nc + TX - 1) / TX;
     const long long tiles = p.n_outer * tpo;
+    const int shift = INV ? 0 : p.shift;                   // (of the input; an inverse without crop shifts its output)
     constexpr int RPS = kCoreThreads / TX;                 // rows per step
     const int x = tid % TX, r0 = tid / TX;
     const unsigned bu_x = (unsigned)__cvta_generic_to_shared(bu + x * LS);
@@ -262,15 +263,15 @@ __global__ void __launch_bounds__(core_threads(LOG2P), (LOG2P >= 10 ? 1 : 2)) ax
         if (inside) {
             // position pos holds entry (pos + shift) mod N: entries [shift, n_in) sit at [0, n_in - shift), entries
             // [0, shift) at [N - shift, N), the gap is zero
-            const int head = p.n_in - p.shift, tail0 = N - p.shift;
-            const float2 *src = us + (long long)(p.shift + r0) * p.nc;
+            const int head = p.n_in - shift, tail0 = N - shift;
+            const float2 *src = us + (long long)(shift + r0) * p.nc;
             for (int pos = r0; pos < head && pos < NFILL; pos += RPS, src += step) cp_async8_s(bu_x + 8u * (unsigned)F::ph(pos), src);
-            if (p.shift) {
+            if (shift) {
                 int pos = tail0 + ((r0 - tail0) & (RPS - 1));
                 src = us + (long long)(pos - tail0) * p.nc;
                 for (; pos < NFILL; pos += RPS, src += step) cp_async8_s(bu_x + 8u * (unsigned)F::ph(pos), src);
             }
-            const int z1 = p.shift ? tail0 : N;
+            const int z1 = shift ? tail0 : N;
             for (int z = (head > 0 ? head : 0) + ((r0 - (head > 0 ? head : 0)) & (RPS - 1)); z < z1 && z < NFILL; z += RPS)
                 bu[x * LS + F::ph(z)] = make_float2(0.f, 0.f);
         } else {
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__(core_threads(LOG2P), (LOG2P >= 10 ? 1 : 2)) ax
         __syncthreads();
         if (inside) {
             float2 *dst = p.out + o * p.out_outer + c0 + x + (long long)r0 * p.nc;
-            for (int pos = r0; pos < p.n_out; pos += RPS, dst += step) { HN_G(dst, 8); *dst = bu[x * LS + F::ph(pos)]; }
+            for (int pos = r0; pos < p.n_out; pos += RPS, dst += step) { HN_G(dst, 8); *dst = bu[x * LS + F::ph(INV && !PRUNE ? (pos - p.shift) & (N - 1) : pos)]; }
         }
         __syncthreads();
     }
@@ -319,7 +320,7 @@ int launch_axis_w(const AxisArgs &a, bool inverse, cudaStream_t st)
     const int n = 1 << a.log2p;
     if (a.in == a.out) return -1;
     if (!inverse && (a.n_in > (a.prune_in ? n / 2 : n) || a.n_out > n || a.shift < 0 || a.shift >= n || (a.prune_in && a.shift))) return -1;
-    if (inverse && (a.n_in > n || a.shift || a.n_out > (a.full ? n : n / 2))) return -1;
+    if (inverse && (a.n_in > n || (a.shift && !a.full) || a.n_out > (a.full ? n : n / 2))) return -1;
 #define HN_AXW(L)                                                                                       \
     case L:                                                                                             \
         if (!inverse) return a.prune_in ? launch_axis_w_t<L, false, true>(a, st) : launch_axis_w_t<L, false, false>(a, st); \

@@ -13,6 +13,7 @@
 #include "ct1d.cuh"
 #include "planes.cuh"
 #include "core_tma.cuh"
+#include "core3_tma.cuh"
 #include "tma_util.cuh"
 #include "fused2d.cuh"
 #include "mixer.cuh"
@@ -1405,6 +1406,11 @@ struct hyenand_grad {
                                       // they are, dq leaves its forward as bf16 (only the fp32 intermediates have scratch)
     bool slice;                       // a slice's spectra fit in shared memory: one kernel does the whole backward (slice_bwd.cuh)
     SliceGeo sg;
+    // Grids whose spectral core has a three-product kernel (core3_tma.cuh): one pass over groups of ns slices, see backward_spectral.
+    bool spec;
+    Core3Maps maps, maps_sh;          // per-sample filters (tap gradients replace the filter's spectra); shared filters
+    float2 *fu, *fg, *fh, *fa, *fha;  // spectra of k v, of dy q, of the filter; 3-D general path: rows before the middle axis
+    float2 *fd, *fhc;                 // shared filters, from their first use on: tap gradients of a group, spectra of all C filters
     bool native;                      // bf16 I/O on the multi-kernel paths: every kernel reads the caller's bf16 tensors itself and
                                       // dq leaves its pass as bf16 (no widened copies of q, k, v, dy)
     int nb;                           // batch entries per pass
@@ -1540,6 +1546,203 @@ static int corr_dh(hyenand_grad *g, long long m, const void *gy, const void *gq,
     return HYENAND_OK;
 }
 
+// ---- all gradients from one set of spectra (2-D and 3-D grids) -------------------------------------------------------------
+// The filter, k v and dy q are transformed once; the core forms the three spectral products and brings each back along its
+// axis (core3_tma.cu); dq leaves through the gate dy, dk and dv through v and k, and the taps' gradients as rows of taps (3-D
+// planes: the transpose of the filter-plane kernel).  Nothing but spectra and, for a filter shared over the batch, fp32 taps per
+// slice is stored in between.  (Before: two signal sides that each ended in a core of their own, then a third convolution for
+// dh on the general kernels from transforms of its own.)
+struct SpecGeo {
+    bool three, planes;
+    long long u, h, mid_u, mid_h;     // float2 elements per slice
+    int nc, L, K, log2p;              // core axis
+};
+static SpecGeo spec_geo(const hyenand_plan *p)
+{
+    SpecGeo s{};
+    s.planes = p->path == PATH_PLANES3D;
+    s.three = p->P[0] > 1;
+    const int ax = s.three ? 0 : 1;
+    s.nc = s.planes ? p->XH * p->P[1] : s.three ? p->P[1] * p->XP : p->XP;
+    s.L = p->L[ax]; s.K = p->K[ax]; s.log2p = p->log2p[ax];
+    s.u = (long long)s.L * s.nc; s.h = (long long)s.K * s.nc;
+    if (s.three && !s.planes) { s.mid_u = (long long)p->L[0] * p->L[1] * p->XP; s.mid_h = (long long)p->K[0] * p->K[1] * p->XP; }
+    return s;
+}
+
+static Core3Args spec_core_args(const hyenand_grad *g, bool shared)
+{
+    const hyenand_plan *p = g->main;
+    const SpecGeo s = spec_geo(p);
+    Core3Args a{};
+    a.u = g->fu; a.g = g->fg; a.h = shared ? g->fhc : g->fh; a.dh = shared ? g->fd : g->fh;
+    a.u_outer = s.u; a.h_outer = s.h; a.nc = s.nc; a.L = s.L; a.K = s.K;
+    a.h_shift = p->circular ? 0 : s.L - 1; a.log2p = s.log2p; a.full = p->circular;
+    // 1/P of the inverses; the plane kernels leave a factor 2 in each operand
+    a.scale = (float)((s.planes ? 0.25 : 1.0) / ((double)p->P[0] * p->P[1] * p->P[2]));
+    a.gtw = p->gtw; a.gtw_n = p->gtw_n;
+    return a;
+}
+
+// true: the grid is this path's (g->spec), or an error was recorded (!g->spec); false: another path takes it
+static bool spec_create(hyenand_grad *g)
+{
+    const Switches sw = read_switches();
+    if (g->ndim < 2 || sw.force_generic || sw.generic_rows || sw.generic_core || sw.no_tma) return false;
+    // geometry, twiddle table and status word: a plan of one slice
+    hyenand_plan *p = create_plan(g->ndim, g->dims, 1, 1, g->mode, g->dtype, false);
+    if (!p) return true;
+    const SpecGeo s = spec_geo(p);
+    if ((p->path != PATH_PLANES3D && p->path != PATH_ND_GENERIC) || !core3_tma_supported(s.log2p, p->circular, s.nc)) {
+        hyenand_destroy_plan(p);
+        return false;
+    }
+    g->main = g->adj = p;
+    const long long S = (long long)g->B * g->C;
+    long long ns = (2ll << 30) / (8ll * (2 * s.u + s.h + s.mid_u + s.mid_h));
+    if (const char *e = getenv("HYENAND_BACKWARD_RING_SLICES")) { const long long v = atoll(e); if (v > 0 && v < ns) ns = v; }   // development aid
+    g->ns = ns < 1 ? 1 : ns > S ? S : ns;
+    // shared filters: fp32 tap gradients of nb batch entries within 2 GiB
+    long long nb = (2ll << 30) / (4ll * g->C * g->kvol);
+    if (const char *e = getenv("HYENAND_BACKWARD_MAX_BATCH")) { const long long v = atoll(e); if (v > 0 && v < nb) nb = v; }   // development aid
+    g->nb = (int)(nb < 1 ? 1 : nb > g->B ? g->B : nb);
+    cudaError_t e = cudaSuccess;
+    auto get = [&](float2 **ptr, long long elems) {
+        if (e == cudaSuccess && elems) e = guarded_alloc(&g->allocs, (void **)ptr, (size_t)elems * g->ns * sizeof(float2));
+    };
+    get(&g->fu, s.u); get(&g->fg, s.u); get(&g->fh, s.h); get(&g->fa, s.mid_u); get(&g->fha, s.mid_h);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        fail(HYENAND_ERR_ALLOC, "scratch of the backward pass: %s", cudaGetErrorString(e));
+        return true;
+    }
+    if (!core3_tma_make(&g->maps, spec_core_args(g, false), g->ns, g->ns)) {
+        fail(HYENAND_ERR_CUDA, "tensor maps of the backward pass");
+        return true;
+    }
+    g->spec = true;
+    return true;
+}
+
+// room a filter shared over the batch needs, taken the first time one is used
+static int spec_shared_room(hyenand_grad *g)
+{
+    if (g->maps_sh.valid) return HYENAND_OK;
+    const SpecGeo s = spec_geo(g->main);
+    cudaError_t e = cudaSuccess;
+    auto get = [&](void **ptr, long long bytes) {
+        if (e == cudaSuccess && !*ptr) e = guarded_alloc(&g->allocs, ptr, (size_t)bytes);
+    };
+    get((void **)&g->fd, s.h * g->ns * 8); get((void **)&g->fhc, s.h * g->C * 8);
+    get((void **)&g->dhs, 4ll * g->nb * g->C * g->kvol);
+    if (g->nb < g->B) get((void **)&g->dh32, 4ll * g->C * g->kvol);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(HYENAND_ERR_ALLOC, "scratch of the backward pass: %s", cudaGetErrorString(e));
+    }
+    if (!core3_tma_make(&g->maps_sh, spec_core_args(g, true), g->ns, g->C)) return fail(HYENAND_ERR_CUDA, "tensor maps of the backward pass");
+    return HYENAND_OK;
+}
+
+static int backward_spectral(hyenand_grad *g, const void *q, const void *k, const void *v, const void *h, bool shared, const void *dy,
+                             void *dq, void *dk, void *dv, void *dh, cudaStream_t st)
+{
+    hyenand_plan *p = g->main;
+    const SpecGeo s = spec_geo(p);
+    const size_t es = elsize(g->dtype);
+    const long long C = g->C, vol = g->vol, kvol = g->kvol;
+    const int *L = p->L, *K = p->K, *P = p->P;
+    const int circ = p->circular, hsh[2] = {circ ? 0 : L[1] - 1, circ ? 0 : L[2] - 1};
+    const bool roww = rows_w_supported(p->log2p[2]);
+    auto bad = [] { return fail(HYENAND_ERR_CUDA, "internal launch dispatch failed"); };
+    auto rows = [&](const void *a, const void *b, long long n_rows, int len, int shift, bool prune, float2 *dst) {
+        RowsArgs r{};
+        r.a = a; r.b = b; r.out = dst; r.pitch = p->XP; r.rows = n_rows; r.len = len; r.shift = shift; r.log2p = p->log2p[2];
+        r.prune_in = prune && !circ; r.full_in = circ; r.gtw = p->gtw; r.gtw_n = p->gtw_n;
+        return (roww ? launch_rows_fwd_w(r, g->dtype, st) : launch_rows_fwd(r, g->dtype, st)) >= 0;
+    };
+    auto middle = [&](const float2 *src, float2 *dst, long long outer, int n_in, int n_out, int shift, bool prune, bool inverse) {
+        AxisArgs a{};
+        a.in = src; a.out = dst; a.n_outer = outer; a.nc = p->XP;
+        a.in_outer = (long long)n_in * p->XP; a.out_outer = (long long)n_out * p->XP;
+        a.n_in = n_in; a.n_out = n_out; a.shift = shift; a.log2p = p->log2p[1];
+        a.prune_in = !inverse && prune && !circ; a.full = inverse && (!prune || circ);
+        a.gtw = p->gtw; a.gtw_n = p->gtw_n;
+        return launch_axis_any(p->sw, a, inverse ? AXIS_INV : AXIS_FWD, st) >= 0;
+    };
+    // spectra of n filters (taps at hp) into dst
+    auto filter = [&](const char *hp, long long n, float2 *dst) {
+        if (s.planes) {
+            PlaneArgs a{};
+            a.a = hp; a.out = dst; a.planes = n * K[0]; a.a_elems = n * kvol; a.lx = L[2]; a.ly = L[1]; a.gtw = p->gtw; a.gtw_n = p->gtw_n;
+            return launch_plane(a, PLANE_H, p->log2p[2], g->dtype, st) >= 0;
+        }
+        if (!rows(hp, nullptr, n * K[0] * K[1], K[2], hsh[1], false, s.three ? g->fha : dst)) return false;
+        return !s.three || middle(g->fha, dst, n * K[0], K[1], P[1], hsh[0], false, false);
+    };
+    auto signal = [&](const char *a, const char *b, long long n, float2 *dst) {
+        if (s.planes) {
+            PlaneArgs u{};
+            u.a = a; u.b = b; u.out = dst; u.a_elems = n * vol; u.planes = n * L[0]; u.lx = L[2]; u.ly = L[1]; u.gtw = p->gtw; u.gtw_n = p->gtw_n;
+            return launch_plane(u, PLANE_U, p->log2p[2], g->dtype, st) >= 0;
+        }
+        if (!rows(a, b, n * L[0] * L[1], L[2], 0, true, s.three ? g->fa : dst)) return false;
+        return !s.three || middle(g->fa, dst, n * L[0], L[1], P[1], 0, true, false);
+    };
+    // y = gate * back(src), and y2 = gate2 * back(src)
+    auto back = [&](const float2 *src, long long n, const char *gate, char *y, const char *gate2, char *y2) {
+        if (s.planes) {
+            PlaneArgs iv{};
+            iv.a = gate; iv.y = y; iv.in = src; iv.q2 = gate2; iv.y2 = y2;
+            iv.planes = n * L[0]; iv.lx = L[2]; iv.ly = L[1]; iv.gtw = p->gtw; iv.gtw_n = p->gtw_n;
+            return launch_plane(iv, PLANE_INV, p->log2p[2], g->dtype, st) >= 0;
+        }
+        if (s.three && !middle(src, g->fa, n * L[0], P[1], L[1], 0, true, true)) return false;
+        RowsInvArgs ri{};
+        ri.in = s.three ? g->fa : src; ri.pitch = p->XP; ri.q = gate; ri.y = y; ri.q2 = gate2; ri.y2 = y2;
+        ri.rows = n * L[0] * L[1]; ri.len = L[2]; ri.log2p = p->log2p[2]; ri.gtw = p->gtw; ri.gtw_n = p->gtw_n; ri.full_out = circ;
+        return (roww ? launch_rows_inv_w(ri, g->dtype, st) : launch_rows_inv(ri, g->dtype, st)) >= 0;
+    };
+    auto taps = [&](const float2 *src, long long n, void *out, int dt) {
+        if (s.planes) {
+            PlaneArgs iv{};
+            iv.y = out; iv.in = src; iv.planes = n * K[0]; iv.lx = L[2]; iv.ly = L[1]; iv.gtw = p->gtw; iv.gtw_n = p->gtw_n;
+            return launch_plane(iv, PLANE_H_INV, p->log2p[2], dt, st) >= 0;
+        }
+        if (s.three && !middle(src, g->fha, n * K[0], P[1], K[1], hsh[0], false, true)) return false;
+        RowsInvArgs ri{};
+        ri.in = s.three ? g->fha : src; ri.pitch = p->XP; ri.y = out; ri.rows = n * K[0] * K[1]; ri.len = K[2]; ri.log2p = p->log2p[2];
+        ri.gtw = p->gtw; ri.gtw_n = p->gtw_n; ri.full_out = 1; ri.shift = hsh[1];
+        return (roww ? launch_rows_inv_w(ri, dt, st) : launch_rows_inv(ri, dt, st)) >= 0;
+    };
+    if (shared)
+        for (long long c0 = 0; c0 < C; c0 += g->ns)
+            if (!filter((const char *)h + c0 * kvol * es, C - c0 < g->ns ? C - c0 : g->ns, g->fhc + c0 * s.h)) return bad();
+    Core3Args ca = spec_core_args(g, shared);
+    const long long S = (long long)g->B * C, pass = shared ? g->nb * C : S;
+    for (long long p0 = 0; p0 < S; p0 += pass) {
+        const long long p1 = p0 + pass < S ? p0 + pass : S;
+        for (long long s0 = p0; s0 < p1; s0 += g->ns) {
+            const long long n = p1 - s0 < g->ns ? p1 - s0 : g->ns;
+            const size_t o = (size_t)s0 * vol * es;
+            if (!shared && !filter((const char *)h + s0 * kvol * es, n, g->fh)) return bad();
+            if (!signal((const char *)k + o, (const char *)v + o, n, g->fu) || !signal((const char *)dy + o, (const char *)q + o, n, g->fg)) return bad();
+            ca.n_outer = n; ca.h_mod = shared ? C : 0; ca.h_off = shared ? s0 % C : 0;
+            if (launch_core3_tma(ca, shared ? g->maps_sh : g->maps, p->dev_status, st) < 0) return bad();
+            if (!back(g->fu, n, (const char *)dy + o, (char *)dq + o, nullptr, nullptr) ||
+                !back(g->fg, n, (const char *)v + o, (char *)dk + o, (const char *)k + o, (char *)dv + o)) return bad();
+            if (!taps(ca.dh, n, shared ? (void *)(g->dhs + (s0 - p0) * kvol) : (void *)((char *)dh + s0 * kvol * es), shared ? HYENAND_F32 : g->dtype)) return bad();
+        }
+        if (shared) {
+            if (p1 == S) launch_batch_sum_cast(g->dhs, (p1 - p0) / C, C, kvol, p0 == 0 ? nullptr : g->dh32, g->dtype, dh, st);
+            else launch_batch_sum(g->dhs, (p1 - p0) / C, C, kvol, p0 == 0, g->dh32, st);
+        }
+    }
+    const cudaError_t ce = cudaGetLastError();
+    if (ce != cudaSuccess) return fail(HYENAND_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(ce));
+    return HYENAND_OK;
+}
+
 extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int B, int C, int mode, int dtype)
 {
     g_err[0] = 0;
@@ -1592,6 +1795,11 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
             return nullptr;
         }
         return g;
+    }
+    if (spec_create(g)) {
+        if (g->spec) return g;
+        hyenand_backward_destroy(g);
+        return nullptr;
     }
     // batch entries per pass: nine fp32 tensors of nb*C*vol elements (+ kernels) within about 4 GiB
     long long nb = (4ll << 30) / (4ll * C * (8 * g->vol + g->kopp + 3 * g->kvol));
@@ -1748,6 +1956,7 @@ extern "C" int hyenand_backward(hyenand_grad *g, const void *q, const void *k, c
                     return fail(HYENAND_ERR_INVALID_ARG, "output %d overlaps pointer %d", o, i);
             }
     }
+    if (g->spec && shared && (e = spec_shared_room(g))) return e;
     {
         DbgScope d;
         const size_t nbytes = (size_t)g->B * g->C * g->vol * elsize(g->dtype);
@@ -1760,6 +1969,7 @@ extern "C" int hyenand_backward(hyenand_grad *g, const void *q, const void *k, c
         d.commit();
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    if (g->spec) return backward_spectral(g, q, k, v, h, shared, dy, dq, dk, dv, dh, st);
     if (g->slice) return backward_slice(g, q, k, v, h, shared, dy, dq, dk, dv, dh, st);
     const size_t es = elsize(g->dtype);
     const bool widen = g->dtype == HYENAND_BF16;

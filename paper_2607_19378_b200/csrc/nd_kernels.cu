@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kThreads) rows_inv_kernel(RowsInvArgs p)
             for (int idx = tid; idx < G * p.len; idx += kThreads) {
                 const int g = idx / p.len, n = idx % p.len;
                 const long long r0 = 2 * (ch * G + g), r1 = r0 + 1;
-                const float2 z = buf[g * LS + phys(n)];
+                const float2 z = buf[g * LS + phys(FULL ? (n - p.shift) & (N - 1) : n)];
                 if (r0 < p.rows) IO<T>::st(py, r0 * p.len + n, z.x * IO<T>::ld(pq, r0 * p.len + n));
                 if (r1 < p.rows) IO<T>::st(py, r1 * p.len + n, z.y * IO<T>::ld(pq, r1 * p.len + n));
             }
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kThreads) rows_inv_kernel(RowsInvArgs p)
             for (int idx = tid; idx < G * p.len; idx += kThreads) {
                 const int g = idx / p.len, n = idx % p.len;
                 const long long r0 = 2 * (ch * G + g), r1 = r0 + 1;
-                const float2 z = buf[g * LS + phys(n)];
+                const float2 z = buf[g * LS + phys(FULL ? (n - p.shift) & (N - 1) : n)];
                 if (r0 < p.rows) IO<T>::st(py, r0 * p.len + n, z.x);
                 if (r1 < p.rows) IO<T>::st(py, r1 * p.len + n, z.y);
             }
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kThreads) rows_inv_kernel(RowsInvArgs p)
             for (int idx = tid; idx < G * p.len; idx += kThreads) {
                 const int g = idx / p.len, n = idx % p.len;
                 const long long r0 = 2 * (ch * G + g), r1 = r0 + 1;
-                const float2 z = buf[g * LS + phys(n)];
+                const float2 z = buf[g * LS + phys(FULL ? (n - p.shift) & (N - 1) : n)];
                 if (r0 < p.rows) IO<T>::st(py2, r0 * p.len + n, z.x * IO<T>::ld(pq2, r0 * p.len + n));
                 if (r1 < p.rows) IO<T>::st(py2, r1 * p.len + n, z.y * IO<T>::ld(pq2, r1 * p.len + n));
             }
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kThreads) axis_kernel(AxisArgs p)
         const long long o = t / tpo;
         const int c0 = (int)(t % tpo) * TX;
         const int width = p.nc - c0 < TX ? p.nc - c0 : TX;
-        fill_tile<N, NFILL_U>(bu, LS, TX, p.in + o * p.in_outer + c0, p.nc, width, p.n_in, p.shift, tid);
+        fill_tile<N, NFILL_U>(bu, LS, TX, p.in + o * p.in_outer + c0, p.nc, width, p.n_in, MODE == AXIS_INV ? 0 : p.shift, tid);
         if (MODE == AXIS_CORE) {
             const long long oh = p.h_mod ? (o + p.h_off) % p.h_mod : o;
             fill_tile<N, N>(bh, LS, TX, p.h + oh * p.h_outer + c0, p.nc, width, p.h_n_in, p.h_shift, tid);
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kThreads) axis_kernel(AxisArgs p)
         float2 *dst = p.out + o * p.out_outer + c0;
         for (int idx = tid; idx < TX * p.n_out; idx += kThreads) {
             const int x = idx % TX, a = idx / TX;
-            if (x < width) { HN_G(dst + (long long)a * p.nc + x, 8); dst[(long long)a * p.nc + x] = bu[x * LS + phys(a)]; }
+            if (x < width) { HN_G(dst + (long long)a * p.nc + x, 8); dst[(long long)a * p.nc + x] = bu[x * LS + phys(MODE == AXIS_INV && !PRUNE ? (a - p.shift) & (N - 1) : a)]; }
         }
         __syncthreads();
     }

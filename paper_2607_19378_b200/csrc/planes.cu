@@ -633,6 +633,168 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_inv_kernel(PlaneArgs p
     }
 }
 
+// ---- inverse filter planes ---------------------------------------------------------------------------------------------
+
+// The transpose of hplane_kernel: spectra of a plane of tap gradients back to its 2Ly-1 rows of 2Lx-1 taps.  The even and the
+// odd bins along x are brought back one after the other, each half through a store [bin][row pair y, y + P/2] of lines
+// G = A + iB that the column transforms leave behind (as in plane_inv_kernel), and a row of each half is one half-length
+// inverse: with E and O those of the even and of the odd bins, f[x] = E[x] + W_P^-x O[x], f[x + P/2] = E[x] - W_P^-x O[x].
+// E waits in tensor memory until O is there.
+template <typename T, int LOG2P>
+__global__ void __launch_bounds__(kPlaneThreads, 1) hplane_inv_kernel(PlaneArgs p)
+{
+    using C = PlaneCfg<LOG2P>;
+    using FI = typename C::FI;
+    using FH = WF<LOG2P - 1, true>;
+    constexpr int P = C::P, HP = C::HP, QP = P / 4, TPL = FI::TPL, TPLH = FH::TPL;
+    constexpr int CS2 = HP + 1;
+    constexpr unsigned FULL = 0xffffffffu;                   // every warp runs the loops below in step: whole-warp barriers
+    extern __shared__ float2 smem[];
+    float2 *cs = smem;
+    float2 *wbuf = cs + C::CSN;
+    float2 *tw = wbuf + C::WBUF;
+    float2 *twh = tw + P;
+    const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL, lh = tid % TPLH, gidh = tid / TPLH;
+    float2 *line = wbuf + gid * C::LS, *lineh = wbuf + gidh * C::LSH;
+    using P0 = typename FI::template Pass<0>;
+    using P1 = typename FI::template Pass<1>;
+    using PE = typename FH::LastPass;
+    static_assert(FI::NP == 2, "two-pass plans");
+    constexpr int NPT = 2 * PE::IPL * PE::R;                 // parked values per thread and row pair
+    constexpr int ROUNDS = HP / C::NGH, TCOLS = 4 * ROUNDS * NPT;
+    static_assert(HP % C::NGH == 0 && TCOLS >= 32 && TCOLS <= 512 && (TCOLS & (TCOLS - 1)) == 0, "tensor-memory columns");
+    static_assert(QP % C::NG == 0 || C::NG % QP == 0, "whole warps take part in the column loop");
+    const int warp = tid >> 5;
+    unsigned *tslot = reinterpret_cast<unsigned *>(smem + C::TMP + P);
+    if (warp == 0) tmem_alloc((unsigned)__cvta_generic_to_shared(tslot), TCOLS);
+    load_plane_twiddles<LOG2P>(tw, twh, p.gtw, p.gtw_n, tid);
+    tmem_fence_before_sync();
+    __syncthreads();
+    tmem_fence_after_sync();
+    const unsigned tbase = *tslot;
+    const unsigned tpark = tmem_addr(tbase, warp, (warp >> 2) * ROUNDS * NPT);
+    PlaneTw<LOG2P, true> twp;
+    twp.init(l, tw, twh + HP, tid, kPlaneThreads);
+    PassTw<LOG2P - 1, true> twr;                             // half-length rows
+    twr.base = twh + HP + P;
+    PassTw<LOG2P - 1, true>::build(twh + HP + P, p.gtw, p.gtw_n, tid, kPlaneThreads);
+    __syncthreads();
+    T *py = (T *)p.y;
+    const int Lx = p.lx, Ly = p.ly, Kx = 2 * Lx - 1, Ky = 2 * Ly - 1, J0 = HP + 1 - Lx;
+    for (long long pl = blockIdx.x; pl < p.planes; pl += gridDim.x) {
+        const float2 *src = p.in + pl * (long long)C::XH * P;
+        T *out = py + pl * (long long)Ky * Kx;
+        for (int e = 0; e < 2; ++e) {
+            // columns kx = 2k + e: bins k and H - k (even half; k = 0 packs kx = 0 and kx = P/2, whose bins are 0 and H/2), k and
+            // H - 1 - k (odd half)
+            for (int k = gid; k < QP; k += C::NG) {
+                const bool packed = e == 0 && k == 0;
+                const float2 *s = src + (long long)(2 * k + e) * P;
+                float2 x[P0::IPL][P0::R];
+#pragma unroll
+                for (int i = 0; i < P0::IPL; ++i)
+#pragma unroll
+                    for (int r = 0; r < P0::R; ++r) {
+                        const int idx = l + i * TPL + r * (P / P0::R);
+                        HN_G(s + idx, 8);
+                        x[i][r] = __ldcg(s + idx);
+                    }
+                if (packed) {
+                    const float2 *sn = src + (long long)HP * P;
+#pragma unroll
+                    for (int i = 0; i < P0::IPL; ++i)
+#pragma unroll
+                        for (int r = 0; r < P0::R; ++r) {
+                            const int idx = l + i * TPL + r * (P / P0::R);
+                            HN_G(sn + idx, 8);
+                            const float2 gn = __ldcg(sn + idx);
+                            x[i][r] = make_float2(x[i][r].x - gn.y, x[i][r].y + gn.x);
+                        }
+                }
+                __syncwarp();
+                float2 *lo = cs + k * CS2, *hi = cs + (packed ? HP / 2 : (e == 0 ? HP - k : HP - 1 - k)) * CS2;
+                FI::template pass<0, PRUNE_NONE>(l, twp, [&](int i, int r, int) { return x[i][r]; },
+                    [&](int, int, int idx, float2 v) { line[FI::ph(idx)] = v; });
+                __syncwarp();
+                float2 first[P1::IPL][P1::R / 2];
+                FI::template pass<1, PRUNE_NONE>(l, twp, [&](int, int, int idx) { return line[FI::ph(idx)]; },
+                    [&](int i, int r, int idx, float2 B) {
+                        if (r < P1::R / 2) { first[i][r] = B; return; }
+                        const float2 A = first[i][r - P1::R / 2];
+                        lo[idx - HP] = make_float2(A.x - B.y, A.y + B.x);
+                        hi[idx - HP] = make_float2(A.x + B.y, B.x - A.y);
+                    });
+                __syncwarp();
+            }
+            __syncthreads();
+            if (e == 1 && pl + gridDim.x < p.planes)
+                prefetch_l2(p.in + (pl + gridDim.x) * (long long)C::XH * P, (long long)C::XH * P * sizeof(float2), tid);
+            int round = 0;
+            for (int rp = spread_pair<8>(gidh); rp < HP; rp += C::NGH, ++round) {
+                const unsigned tcol = tpark + round * NPT;
+                const float2 *g = cs + rp;
+                float2 nyq = make_float2(0.f, 0.f);
+                auto spectrum = [&](int, int, int idx) {
+                    float2 v = g[idx * CS2];
+                    if (e == 0) {
+                        if (idx == 0) {
+                            // the packed column's two bins (both lane 0's): see plane_inv_kernel
+                            const float2 w = g[(HP / 2) * CS2];
+                            nyq = make_float2(0.5f * (v.y - w.y), 0.5f * (w.x - v.x));
+                            v = make_float2(0.5f * (v.x + w.x), 0.5f * (v.y + w.y));
+                        }
+                        if (idx == HP / 2) v = nyq;
+                    }
+                    return v;
+                };
+                float dd[NPT], oo[NPT];
+                if (e == 0) {
+                    FH::template run<PRUNE_NONE>(lh, FULL, twr, lineh, spectrum,
+                        [&](int i, int r, int, float2 z) { dd[2 * (i * PE::R + r)] = z.x; dd[2 * (i * PE::R + r) + 1] = z.y; });
+                    __syncwarp();
+                    TmemIO<NPT>::st(tcol, dd);
+                    tmem_wait_st();
+                } else {
+                    FH::template run<PRUNE_NONE>(lh, FULL, twr, lineh, spectrum,
+                        [&](int i, int r, int idx, float2 z) {
+                            const float2 w = cmulc(z, tw[idx]);
+                            oo[2 * (i * PE::R + r)] = w.x;
+                            oo[2 * (i * PE::R + r) + 1] = w.y;
+                        });
+                    __syncwarp();
+                    TmemIO<NPT>::ld(dd, tcol);
+                    tmem_wait_ld();
+                    // padded rows rp and rp + P/2 are tap rows my0 and my0 ^ P/2 (at most one lies in the zero band)
+                    const int my0 = (rp + Ly - 1) & (P - 1), my1 = my0 ^ HP;
+                    const bool v0 = my0 < Ky, v1 = my1 < Ky;
+                    T *o0 = out + (long long)my0 * Kx, *o1 = out + (long long)my1 * Kx;
+#pragma unroll
+                    for (int i = 0; i < PE::IPL; ++i)
+#pragma unroll
+                        for (int r = 0; r < PE::R; ++r) {
+                            const int x = lh + i * TPLH + r * (HP / PE::R), j = 2 * (i * PE::R + r);
+                            const int ta = x + Lx - 1, tb = x - J0;
+                            if (ta < Kx) {
+                                if (v0) IO<T>::st(o0, ta, dd[j] + oo[j]);
+                                if (v1) IO<T>::st(o1, ta, dd[j + 1] + oo[j + 1]);
+                            }
+                            if (tb >= 0) {
+                                if (v0) IO<T>::st(o0, tb, dd[j] - oo[j]);
+                                if (v1) IO<T>::st(o1, tb, dd[j + 1] - oo[j + 1]);
+                            }
+                        }
+                }
+                __syncwarp();
+            }
+            __syncthreads();
+        }
+    }
+    // every warp's last tensor-memory read was waited for before the barrier above; the allocating warp frees
+    tmem_fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tbase, TCOLS);
+}
+
 // ---- launchers --------------------------------------------------------------------------------------------
 
 static int plane_sms()
@@ -658,15 +820,17 @@ template <typename T, int LOG2P> static int launch_plane_t(const PlaneArgs &a, i
     using C = PlaneCfg<LOG2P>;
     const int grid = plane_grid(a.planes);
     if (grid <= 0) return 0;
-    static DevOnce attr[6];
+    static DevOnce attr[7];
     // 16-byte gate loads and result stores where every row is a whole number of vectors on a 16-byte boundary
     const bool two = which == PLANE_INV && a.q2 != nullptr && a.y2 != nullptr;
     const bool vst = which == PLANE_INV && a.lx % Vec16<T>::VEC == 0 &&
                      (((uintptr_t)a.a | (uintptr_t)a.y | (uintptr_t)a.q2 | (uintptr_t)a.y2) & 15) == 0;
     void (*fn)(PlaneArgs) = which == PLANE_U ? uplane_kernel<T, LOG2P>
                           : which == PLANE_H ? hplane_kernel<T, LOG2P>
+                          : which == PLANE_H_INV ? hplane_inv_kernel<T, LOG2P>
                           : two ? (vst ? plane_inv_kernel<T, LOG2P, true, true> : plane_inv_kernel<T, LOG2P, false, true>)
                                 : (vst ? plane_inv_kernel<T, LOG2P, true, false> : plane_inv_kernel<T, LOG2P, false, false>);
+    if (which == PLANE_H_INV) which = 6;
     if (vst) which = 3;
     if (two) which = vst ? 5 : 4;
     if (attr[which].first()) {

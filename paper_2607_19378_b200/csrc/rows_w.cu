@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
             const float sg = (r == RH && idx == HP) ? 1.f : -1.f;
             return make_float2(fmaf(-sg, B.y, A.x), fmaf(sg, A.y, B.x));
         });
+        auto at = [&](int n) { return line[FI::ph(FULL ? (n - p.shift) & (P - 1) : n)]; };
         if (!FULL && p.len == HP && has1 && pq) {
             // full rows: all gate loads of the pair are in flight together (they were asked into L2 above)
             float qa[HP / TPL], qb[HP / TPL];
@@ -214,14 +215,14 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
             if (pq) {
                 // (a loop of its own: the read-only gate loads of several iterations go out together)
                 for (int n = l; n < p.len; n += TPL) {
-                    const float2 z = line[FI::ph(n)];
+                    const float2 z = at(n);
                     IO<T>::st(py, r0 * p.len + n, z.x * IO<T>::ld(pq, r0 * p.len + n));
                     if (has1) IO<T>::st(py, r1 * p.len + n, z.y * IO<T>::ld(pq, r1 * p.len + n));
                 }
             } else {
                 // no gate tensor: the rows leave as they are
                 for (int n = l; n < p.len; n += TPL) {
-                    const float2 z = line[FI::ph(n)];
+                    const float2 z = at(n);
                     IO<T>::st(py, r0 * p.len + n, z.x);
                     if (has1) IO<T>::st(py, r1 * p.len + n, z.y);
                 }
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
             const T *pq2 = (const T *)p.q2;
             T *py2 = (T *)p.y2;
             for (int n = l; n < p.len; n += TPL) {
-                const float2 z = line[FI::ph(n)];
+                const float2 z = at(n);
                 IO<T>::st(py2, r0 * p.len + n, z.x * IO<T>::ld(pq2, r0 * p.len + n));
                 if (has1) IO<T>::st(py2, r1 * p.len + n, z.y * IO<T>::ld(pq2, r1 * p.len + n));
             }
