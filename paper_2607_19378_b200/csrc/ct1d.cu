@@ -471,26 +471,9 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
     return 0;
 }
 
-// the warp-engine kernels serve a forward when they take every element type it uses
-bool ct1d_uses_w(const Ct1dPlan *c)
-{
-    if (c->sw.force_generic) return false;
-    const int dts[4] = {c->dtype, c->dt_in, c->dt_out, c->dt_h};
-    for (int i = 0; i < 4; ++i)
-        if (!ct1d_w_supported(c->log2p1, c->log2p2, c->L, c->K, c->causal, dts[i])) return false;
-    return true;
-}
-
-// The warp-engine kernels need 16-byte rows in the given type; the block-wide kernels take either type as it is.  A plan
-// must not change kernel family between forwards (the filter workspace layouts differ), so a type is accepted when it
-// leaves the family the plan's own type selects.
-bool ct1d_takes_dtype(const Ct1dPlan *c, int dtype)
-{
-    if (dtype == c->dtype) return true;
-    const bool w_own = !c->sw.force_generic && ct1d_w_supported(c->log2p1, c->log2p2, c->L, c->K, c->causal, c->dtype);
-    if (!w_own) return true;
-    return ct1d_w_supported(c->log2p1, c->log2p2, c->L, c->K, c->causal, dtype);
-}
+// Both kernel families take either element type in every stage; the warp-engine kernels serve every length they have an
+// instance for (padded 2^14 .. 2^20), longer ones and the development switch take the block-wide kernels.
+bool ct1d_uses_w(const Ct1dPlan *c) { return !c->sw.force_generic && ct1d_w_supported(c->log2p1, c->log2p2); }
 
 int ct1d_launches(const Ct1dPlan *c, bool shared)
 {

@@ -35,11 +35,9 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
                  void *y, cudaStream_t st, int *launches, Prof *prof);
 int ct1d_launches(const Ct1dPlan *c, bool shared);
 bool ct1d_uses_w(const Ct1dPlan *c);
-// true when a forward of this plan may read/write tensors of element type `dtype` (0: fp32, else bf16) in any stage
-bool ct1d_takes_dtype(const Ct1dPlan *c, int dtype);
 
 // warp-engine kernels (ct1d_w.cu)
-bool ct1d_w_supported(int log2p1, int log2p2, int L, int K, int causal, int dtype);
+bool ct1d_w_supported(int log2p1, int log2p2);
 int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
                   int (*fallback)(Ct1dPlan *, const char *, long long, cudaStream_t, int *, Prof *));
 int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, long long s0,

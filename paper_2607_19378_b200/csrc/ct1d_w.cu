@@ -1,7 +1,8 @@
 // Long 1-D path, warp-engine kernels (same decomposition as ct1d.cu: P = P1*P2,
 // t = t1*P2 + t2, f = f1 + P1*f2; Appendix B.3 of the paper).
 //
-//   cols_fwd_w   tile of adjacent column pairs fetched with 16-byte asynchronous copies,
+//   cols_fwd_w   tile of adjacent column pairs fetched with tensor copies, 8-byte asynchronous copies or, where a
+//                slice starts off their boundaries, element by element (eight loads in flight),
 //                one warp-group per column pair: transform along t1 (upper half of the
 //                padded input is zero), separate the two real columns, multiply by the
 //                inter-pass twiddle, coalesced store of [f1][t2].
@@ -64,7 +65,8 @@ struct ColsFwdWArgs {
     const void *a, *b;        // k, v (b == nullptr: plain copy of a, used for a causal filter)
     float2 *out;              // [slices][P1/2+1][P2]
     long long slices;
-    long long in_slice;       // elements per slice of the input (multiple of 16 bytes)
+    long long in_slice;       // elements per slice of the input
+    bool vec;                 // every pair of column pairs starts on an 8-byte boundary
     int len;                  // valid elements (<= P/2)
     int *status;              // device word set when a bounded wait on a tensor copy gives up (may be NULL)
     int log2p2;
@@ -147,6 +149,7 @@ ct_cols_fwd_w_kernel(ColsFwdWArgs p, const __grid_constant__ CUtensorMap map_a, 
         if constexpr (TMA) {
             if (!mbar_wait(bar, phase)) failed = 1;
         } else {
+        if (p.vec) {
         for (int idx = tid; idx < HP1 * (TX / PG); idx += kCtThreads) {
             const int t1 = idx / (TX / PG), xg = idx % (TX / PG);
             const long long e0 = (long long)t1 * P2 + 2 * (c0 + PG * xg);
@@ -162,6 +165,32 @@ ct_cols_fwd_w_kernel(ColsFwdWArgs p, const __grid_constant__ CUtensorMap map_a, 
                     reinterpret_cast<T *>(d)[e] = ok ? reinterpret_cast<const T *>(ab)[base + e0 + e] : T(0.f);
                     if (HAS_B)
                         reinterpret_cast<T *>(d + (size_t)HP1 * RS)[e] = ok ? reinterpret_cast<const T *>(bb)[base + e0 + e] : T(0.f);
+                }
+            }
+        }
+        } else {
+            // slices of any length: neighbouring elements by neighbouring threads, eight loads of each tensor in flight
+            constexpr int EPR = 2 * TX, U = 8;                 // elements per row of the tile
+            static_assert(HP1 * EPR % (U * kCtThreads) == 0, "whole rounds");
+            const T *ta = reinterpret_cast<const T *>(ab) + base, *tb = reinterpret_cast<const T *>(bb) + base;
+            for (int i0 = tid; i0 < HP1 * EPR; i0 += U * kCtThreads) {
+                T va[U], vb[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = i0 + u * kCtThreads;
+                    const long long e = (long long)(i / EPR) * P2 + 2 * c0 + i % EPR;
+                    const bool ok = e < p.len;
+                    if (ok) HN_G(ta + e, sizeof(T));
+                    if (ok && HAS_B) HN_G(tb + e, sizeof(T));
+                    va[u] = ok ? __ldg(ta + e) : T(0.f);
+                    if (HAS_B) vb[u] = ok ? __ldg(tb + e) : T(0.f);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int i = i0 + u * kCtThreads;
+                    unsigned char *d = raw + (size_t)(i / EPR) * RS + (i % EPR) * sizeof(T);
+                    *reinterpret_cast<T *>(d) = va[u];
+                    if (HAS_B) *reinterpret_cast<T *>(d + (size_t)HP1 * RS) = vb[u];
                 }
             }
         }
@@ -400,7 +429,8 @@ struct ColsInvWArgs {
     const void *q;
     void *y;
     long long slices;
-    int len;                  // L (multiple of 16 bytes worth of elements)
+    int len;                  // L
+    bool pair;                // slices of whole pairs: two elements per access
     int log2p2;
     const float2 *tw1;
     int *status;              // device word set when a bounded wait on a tensor copy gives up (may be NULL)
@@ -515,6 +545,27 @@ ct_cols_inv_w_kernel(ColsInvWArgs p, const __grid_constant__ CUtensorMap map_q, 
         }
         // gate values first (all requests in flight together), then products and stores
         const long long ox = base + 2 * x;
+        if (!p.pair) {
+            T qa[NE], qb[NE];
+#pragma unroll
+            for (int e = 0; e < NE; ++e) {
+                const int t1 = tb + e * TSTEP;
+                const long long tt = (long long)t1 * P2 + 2 * (c0 + x), o = ox + (long long)t1 * P2;
+                if (tt < p.len) HN_G(pq + o, sizeof(T));
+                if (tt + 1 < p.len) HN_G(pq + o + 1, sizeof(T));
+                qa[e] = tt < p.len ? __ldg(pq + o) : T(0.f);
+                qb[e] = tt + 1 < p.len ? __ldg(pq + o + 1) : T(0.f);
+            }
+#pragma unroll
+            for (int e = 0; e < NE; ++e) {
+                const int t1 = tb + e * TSTEP;
+                const long long tt = (long long)t1 * P2 + 2 * (c0 + x), o = ox + (long long)t1 * P2;
+                const float2 z = lines[x * LS + FI::ph(t1)];
+                if (tt < p.len) IO<T>::st(py, o, z.x * (float)qa[e]);
+                if (tt + 1 < p.len) IO<T>::st(py, o + 1, z.y * (float)qb[e]);
+            }
+            continue;
+        }
         Q2 qv[NE];
 #pragma unroll
         for (int e = 0; e < NE; ++e) {
@@ -563,12 +614,9 @@ static int ctw_sms()
     return n;
 }
 
-bool ct1d_w_supported(int log2p1, int log2p2, int L, int K, int causal, int dtype)
+bool ct1d_w_supported(int log2p1, int log2p2)
 {
-    const int es = dtype == 0 ? 4 : 2;
     if (log2p1 < 7 || log2p1 > 10 || log2p2 < 7 || log2p2 > 10) return false;
-    if (((long long)L * es) % 16 != 0) return false;               // 16-byte copies of whole chunks
-    if (causal && ((long long)K * es) % 16 != 0) return false;
     const int tx = ct_tx(log2p1 >= 10 ? 32 : (log2p1 >= 8 ? 16 : 8));
     if (((1 << log2p2) / 2) % tx != 0) return false;
     return true;
@@ -584,8 +632,10 @@ static void launch_cols_fwd_w_tt(const ColsFwdWArgs &a, const CUtensorMap &ma, c
     ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, TMA><<<grid, kCtThreads, sm, st>>>(a, ma, mb, mo);
 }
 
-template <typename T, int LOG2P1> static int launch_cols_fwd_w_t(const ColsFwdWArgs &a, cudaStream_t st)
+template <typename T, int LOG2P1> static int launch_cols_fwd_w_t(const ColsFwdWArgs &a0, cudaStream_t st)
 {
+    ColsFwdWArgs a = a0;
+    a.vec = a.in_slice * sizeof(T) % 8 == 0 && (((uintptr_t)a.a | (uintptr_t)a.b) & 7) == 0;
     using F = WF<LOG2P1, false>;
     constexpr int P1 = 1 << LOG2P1, TX = ct_tx(F::TPL), LS = ct_ls(phys_max(P1) + 2);
     const size_t sm = sizeof(float2) * ((size_t)TX * LS + P1) + (size_t)2 * (P1 / 2) * (2 * TX * sizeof(T) + 8);
@@ -636,8 +686,10 @@ static void launch_cols_inv_w_tt(const ColsInvWArgs &a, const CUtensorMap &mq, c
     ct_cols_inv_w_kernel<T, LOG2P1, TMA><<<grid, kCtInvThreads, sm, st>>>(a, mq, my);
 }
 
-template <typename T, int LOG2P1> static int launch_cols_inv_w_t(const ColsInvWArgs &a, cudaStream_t st)
+template <typename T, int LOG2P1> static int launch_cols_inv_w_t(const ColsInvWArgs &a0, cudaStream_t st)
 {
+    ColsInvWArgs a = a0;
+    a.pair = a.len % 2 == 0 && (((uintptr_t)a.q | (uintptr_t)a.y) & (2 * sizeof(T) - 1)) == 0;
     using F = WF<LOG2P1, true>;
     constexpr int P1 = 1 << LOG2P1, HP1 = P1 / 2, TX = ct_inv_tx(F::TPL), LS = ct_ls(phys_max(P1) + 2);
     constexpr unsigned QROW = TX * 2 * sizeof(T);

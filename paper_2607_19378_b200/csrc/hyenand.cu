@@ -421,11 +421,7 @@ static void make_core_maps(hyenand_plan *p)
 static bool plan_set_filter_dtype(hyenand_plan *p, int dtype)
 {
     if (dtype == p->dtype) { p->h_dtype = dtype; return true; }
-    if (p->path == PATH_CT1D) {
-        if (!ct1d_takes_dtype(&p->ct, dtype)) return false;
-    } else if (p->path != PATH_PLANES3D && p->path != PATH_ND_GENERIC) {
-        return false;
-    }
+    if (p->path == PATH_FUSED2D) return false;
     p->h_dtype = dtype;
     return true;
 }
@@ -1402,7 +1398,7 @@ struct hyenand_grad {
     bool long1d;
     bool h_native;                    // bf16 I/O: the forwards for dq and du read bf16 taps themselves (no widened kernel)
     bool pair;                        // dq and du come out of one pass over the groups (one filter spectrum serves both)
-    bool ct_native;                   // long causal 1-D grid with bf16 I/O whose kernels take bf16 rows: k, v, dy, q, h are read as
+    bool ct_native;                   // long causal 1-D grid with bf16 I/O: k, v, dy, q, h are read as
                                       // they are, dq leaves its forward as bf16 (only the fp32 intermediates have scratch)
     bool slice;                       // a slice's spectra fit in shared memory: one kernel does the whole backward (slice_bwd.cuh)
     SliceGeo sg;
@@ -1833,8 +1829,7 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
     }
     const bool widen = dtype == HYENAND_BF16;
     auto reads_bf16 = [](const hyenand_plan *q) { return q->path == PATH_PLANES3D || q->path == PATH_ND_GENERIC; };
-    g->ct_native = widen && g->long1d && mode == HYENAND_MODE_CAUSAL && g->main->path == PATH_CT1D &&
-                   ct1d_takes_dtype(&g->main->ct, HYENAND_BF16);
+    g->ct_native = widen && g->long1d && mode == HYENAND_MODE_CAUSAL && g->main->path == PATH_CT1D;
     g->h_native = widen && ((reads_bf16(g->main) && reads_bf16(g->adj)) || g->ct_native);
     g->native = widen && ((g->pair && mode != HYENAND_MODE_CIRCULAR && !g->long1d) || g->ct_native);
     cudaError_t e = cudaSuccess;

@@ -26,3 +26,12 @@ def test_padded(dims, dtype, shared):
 def test_periodic(dims, dtype, shared):
     w, (q, k, v, h) = W.random_problem(dims, B=2, C=3, dtype=dtype, h_shared=shared, seed=122, circular=True)
     check(w, q, k, v, h)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("causal,shared", [(True, True), (False, False)])
+@pytest.mark.parametrize("L", [4097, 8191, 8194, 20001, 65539, 131071, 262146], ids=str)
+def test_long_lines_of_any_length(L, causal, shared, dtype):
+    """Long 1-D grids whose slices start on no particular boundary, on the warp-engine kernels."""
+    w, (q, k, v, h) = W.random_problem((L,), B=2, C=2, dtype=dtype, causal=causal, h_shared=shared, seed=123)
+    check(w, q, k, v, h)
