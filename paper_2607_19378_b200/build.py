@@ -15,7 +15,7 @@ OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libhyenand.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-         "-Xcompiler", "-fPIC", "--use_fast_math", "-Xptxas", "-v"]
+         "-Xcompiler", "-fPIC", "--use_fast_math", "-Xptxas", "-v", "--compress-mode=size"]
 # --use_fast_math only affects division/transcendental intrinsics and denormal flushing;
 # the transform kernels use neither divisions nor sin/cos on the data path (twiddles come from
 # tables computed in double on the host).  Sources that evaluate sines and exponentials of the data
