@@ -180,6 +180,9 @@ void guarded_free_all(GuardedAllocs *g);
 long long guard_damage(const GuardedAllocs *g);       // damaged guard bytes, -1 if a copy failed
 
 constexpr int kMaxLineLog2 = 13;          // longest line transformed in shared memory: 8192 points
+// Line lengths travel as an id (log2p, LOG2P): log2 of a power of two, 16 + k for 3 * 2^k.
+__host__ __device__ constexpr int len_of(int id) { return id < 16 ? 1 << id : 3 << (id - 16); }
+constexpr int kLen192 = 22, kLen384 = 23, kLen768 = 24;
 constexpr int kThreads = 256;             // threads per CTA of the generic kernels
 
 // ---- generic N-D path (nd_kernels.cu) ---------------------------------------------

@@ -20,18 +20,20 @@ namespace hn {
 
 template <int LOG2P, bool FULL> struct Core3Geo {
     using F = WF<LOG2P, false>;
-    static constexpr int N = 1 << LOG2P, HALF = N / 2;
-    static constexpr int THREADS = LOG2P >= 10 ? 256 : 128;
-    static constexpr int PER_SM = LOG2P >= 10 ? 1 : LOG2P == 9 ? (FULL ? 1 : 2) : LOG2P == 6 || (LOG2P == 8 && !FULL) ? 4 : 3;
+    static constexpr int N = len_of(LOG2P), HALF = N / 2;
+    static constexpr int THREADS = N >= 768 ? 256 : N == 192 ? 64 : 128;     // (192: 468 us with 64 threads, 498 with 128, 12 volumes of 96^3)
+    static constexpr int PER_SM = N >= 768 ? 1 : N == 192 ? 5 : N % 3 == 0 ? 2 : LOG2P == 9 ? (FULL ? 1 : 2) : LOG2P == 6 || (LOG2P == 8 && !FULL) ? 4 : 3;
     static constexpr int TX = THREADS / F::TPL;
     static constexpr unsigned ROWB = TX * 8;
     static_assert(ROWB == 128 || ROWB == 64, "tile rows match a swizzle span");
-    static constexpr int BOXR = HALF < 256 ? HALF : 256;             // rows per box
+    static constexpr int BOXR = HALF <= 256 ? HALF : HALF / 2;       // rows per box
     static constexpr int NB = HALF / BOXR;                           // boxes per half line
     static constexpr unsigned BOXB = BOXR * ROWB, HALFB = HALF * ROWB;
     static constexpr unsigned UB = FULL ? 2 * HALFB : HALFB;         // k*v and dy*q tiles
     static constexpr int NBU = FULL ? 2 * NB : NB;
-    static constexpr int LS = F::TPL <= 16 ? plane_ls(N) : ((F::ph(N - 1) + 1 + 15) / 16 * 16 + 2);
+    static constexpr int PHN = F::ph(N - 1) > WF<LOG2P, true>::ph(N - 1) ? F::ph(N - 1) : WF<LOG2P, true>::ph(N - 1);
+    static constexpr int LS = F::TPL <= 16 ? plane_ls(N) : ((PHN + 1 + 15) / 16 * 16 + 2);
+    static_assert(PHN < LS, "a skewed line fits");
     static constexpr int TWTAB = N + PlaneTw<LOG2P, false>::TABLE + PlaneTw<LOG2P, true>::TABLE;
     static constexpr size_t TH = 0, TU = TH + 2 * HALFB, TG = TU + UB, LINES = TG + UB;
     static constexpr size_t TW = LINES + sizeof(float2) * TX * LS;
@@ -167,7 +169,7 @@ axis_core3_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_co
         FI::template pass<NP - 1, PRUNE_NONE>(l, twi, [&](int, int, int idx) { return line[FI::ph(idx)]; },
             [&](int i, int r, int idx, float2 v) {
                 if constexpr (FULL) ch[(i * TPL + r * (N / PE::R)) * RF2] = v;
-                else *reinterpret_cast<float2 *>(th + row_off((unsigned)((idx + p.h_shift) & (N - 1)))) = v;
+                else *reinterpret_cast<float2 *>(th + row_off((unsigned)ring<N>(idx + p.h_shift))) = v;
             });
         fence_async_smem();                            // generic-proxy writes visible to the copy engine
         if (__syncthreads_or(failed)) break;
@@ -199,11 +201,12 @@ axis_core3_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_co
 
 // ---- host side -------------------------------------------------------------------------------------------
 
-#define HN_CORE3_CASES(X) X(6, false) X(7, false) X(8, false) X(9, false) X(10, false) X(6, true) X(7, true) X(8, true) X(9, true)
+#define HN_CORE3_CASES(X) X(6, false) X(7, false) X(8, false) X(9, false) X(10, false) X(kLen192, false) X(kLen384, false) X(kLen768, false) X(6, true) X(7, true) X(8, true) X(9, true)
 
 bool core3_tma_supported(int log2p, int full, int nc)
 {
-    return log2p >= 6 && log2p <= (full ? 9 : 10) && nc % 2 == 0 && tma_available();
+    const bool len = (log2p >= 6 && log2p <= (full ? 9 : 10)) || (log2p >= kLen192 && log2p <= kLen768 && !full);
+    return len && nc % 2 == 0 && tma_available();
 }
 
 static bool map_lines(unsigned char *map, const float2 *base, long long outer, int rows, int nc, long long outer_elems, int tx, int box_rows)

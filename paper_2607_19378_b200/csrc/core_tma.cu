@@ -30,9 +30,9 @@ namespace hn {
 // FULL (periodic axis: N rows in, N rows out) at 512 points: the result tile takes the k*v tile's buffer, which keeps two
 // CTAs per SM; the next k*v tile is then asked for after the result has left, under the next filter tile's transforms.
 template <int LOG2P, bool FULL> struct TmaCta {
-    static constexpr int THREADS = LOG2P >= 10 ? 256 : 128;
-    static constexpr int PER_SM = LOG2P >= 10 ? 1 : LOG2P == 9 ? 2 : FULL && LOG2P >= 7 ? 3 : 4;
-    static constexpr bool SHARE = FULL && LOG2P >= 9;
+    static constexpr int THREADS = len_of(LOG2P) >= 768 ? 256 : 128;
+    static constexpr int PER_SM = len_of(LOG2P) >= 768 ? 1 : LOG2P == kLen192 || LOG2P == kLen384 ? 3 : LOG2P == 9 ? 2 : FULL && LOG2P >= 7 ? 3 : 4;
+    static constexpr bool SHARE = (FULL && LOG2P >= 9) || LOG2P == kLen192 || LOG2P == kLen384;
 };
 
 // Geometry of a tile for LOG2P-point lines: one line per group of TPL lanes, so TX = THREADS / TPL bins
@@ -40,12 +40,12 @@ template <int LOG2P, bool FULL> struct TmaCta {
 // most 256 rows.
 template <int LOG2P, bool FULL> struct TmaGeo {
     using F = WF<LOG2P, false>;
-    static constexpr int N = 1 << LOG2P, HALF = N / 2;
+    static constexpr int N = len_of(LOG2P), HALF = N / 2;
     using CTA = TmaCta<LOG2P, FULL>;
     static constexpr int THREADS = CTA::THREADS;
     static constexpr int TX = THREADS / F::TPL;
     static constexpr unsigned ROWB = TX * 8;
-    static constexpr int BOXR = HALF < 256 ? HALF : 256;             // rows per box
+    static constexpr int BOXR = HALF <= 256 ? HALF : HALF / 2;       // rows per box
     static constexpr int NB = HALF / BOXR;                           // boxes per half line
     static constexpr unsigned BOXB = BOXR * ROWB;
     static constexpr unsigned HALFB = HALF * ROWB;
@@ -53,7 +53,9 @@ template <int LOG2P, bool FULL> struct TmaGeo {
     static constexpr int NBU = FULL ? 2 * NB : NB;                   // their boxes
     // 8- and 16-lane groups (several lines per warp): a half warp works on two lines (see the kernel), whose
     // strides are therefore 8 mod 16 entries, i.e. half a bank row apart
-    static constexpr int LS = F::TPL <= 16 ? plane_ls(N) : ((F::ph(N - 1) + 1 + 15) / 16 * 16 + 2);
+    static constexpr int PHN = F::ph(N - 1) > WF<LOG2P, true>::ph(N - 1) ? F::ph(N - 1) : WF<LOG2P, true>::ph(N - 1);
+    static constexpr int LS = F::TPL <= 16 ? plane_ls(N) : ((PHN + 1 + 15) / 16 * 16 + 2);
+    static_assert(PHN < LS, "a skewed line fits");
     static_assert(ROWB == 128 || ROWB == 64, "tile rows match a swizzle span");
     static constexpr int TWTAB = N + PlaneTw<LOG2P, false>::TABLE + PlaneTw<LOG2P, true>::TABLE;
     // shared memory: tile buffers first (1024-byte aligned, as the swizzle pattern repeats every 1024 bytes)
@@ -255,15 +257,15 @@ static bool make_map(CUtensorMap *map, const float2 *base, long long outer, int 
 
 bool core_tma_supported(const AxisArgs &a)
 {
-    if (a.log2p < 6 || a.log2p > 10) return false;
-    const int n = 1 << a.log2p;
+    if (!((a.log2p >= 6 && a.log2p <= 10) || (a.log2p >= kLen192 && a.log2p <= kLen768 && !a.full))) return false;
+    const int n = len_of(a.log2p);
     const bool rows = a.full ? a.n_in == n && a.h_n_in == n && a.h_shift == 0 && a.log2p <= 9
                              : a.n_in >= 1 && a.n_in <= n / 2 && a.h_n_in >= 1 && a.h_n_in <= n;
     return rows && a.in == a.out && a.in_outer == a.out_outer && a.n_in == a.n_out && a.shift == 0 && a.h_shift >= 0 && a.h_shift < n &&
            (a.nc % 2) == 0 && a.n_outer < (1ll << 31) && tma_available();
 }
 
-#define HN_TMA_CASES(X) X(6) X(7) X(8) X(9) X(10)
+#define HN_TMA_CASES(X) X(6) X(7) X(8) X(9) X(10) X(kLen192) X(kLen384) X(kLen768)
 
 bool core_tma_make(CoreTmaMaps *m, const AxisArgs &a, long long max_outer, long long h_outer_count)
 {
@@ -324,6 +326,9 @@ int launch_core_tma(const AxisArgs &a, const CoreTmaMaps &m, int *status, cudaSt
     case 7: return a.full ? launch_core_tma_t<7, true>(p, m, a.nc, st) : launch_core_tma_t<7, false>(p, m, a.nc, st);
     case 8: return a.full ? launch_core_tma_t<8, true>(p, m, a.nc, st) : launch_core_tma_t<8, false>(p, m, a.nc, st);
     case 9: return a.full ? launch_core_tma_t<9, true>(p, m, a.nc, st) : launch_core_tma_t<9, false>(p, m, a.nc, st);
+    case kLen192: return launch_core_tma_t<kLen192, false>(p, m, a.nc, st);
+    case kLen384: return launch_core_tma_t<kLen384, false>(p, m, a.nc, st);
+    case kLen768: return launch_core_tma_t<kLen768, false>(p, m, a.nc, st);
     default: return launch_core_tma_t<10, false>(p, m, a.nc, st);
     }
 }

@@ -36,7 +36,7 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 template <int LOG2P> __host__ __device__ constexpr int core_ls()
 {
     using F = WF<LOG2P, false>;
-    constexpr int N = 1 << LOG2P, TX = core_threads(LOG2P) / F::TPL;
+    constexpr int N = len_of(LOG2P), TX = core_threads(LOG2P) / F::TPL;
     if (TX >= 16) return line_stride(N);
     int n = (F::ph(N - 1) > WF<LOG2P, true>::ph(N - 1) ? F::ph(N - 1) : WF<LOG2P, true>::ph(N - 1)) + 1;
     while (n % 16 != 2) ++n;
@@ -229,11 +229,11 @@ template <int LOG2P, bool FULL> static int launch_core_w_t(const AxisArgs &a, cu
 // n_out entries (PRUNE: only the lower half is produced, n_out <= N/2).  Lines are read from `in` and written to `out`
 // (different buffers, their own outer strides).
 template <int LOG2P, bool INV, bool PRUNE>
-__global__ void __launch_bounds__(core_threads(LOG2P), (LOG2P >= 10 ? 1 : 2)) axis_w_kernel(AxisArgs p)
+__global__ void __launch_bounds__(core_threads(LOG2P), (len_of(LOG2P) >= 768 ? 1 : 2)) axis_w_kernel(AxisArgs p)
 {
     constexpr int kCoreThreads = core_threads(LOG2P);
     using F = WF<LOG2P, INV>;
-    constexpr int N = 1 << LOG2P, TPL = F::TPL;
+    constexpr int N = len_of(LOG2P), TPL = F::TPL;
     constexpr int TX = kCoreThreads / TPL;
     constexpr int LS = core_ls<LOG2P>();
     extern __shared__ float2 smem[];
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(core_threads(LOG2P), (LOG2P >= 10 ? 1 : 2)) ax
         __syncthreads();
         if (inside) {
             float2 *dst = p.out + o * p.out_outer + c0 + x + (long long)r0 * p.nc;
-            for (int pos = r0; pos < p.n_out; pos += RPS, dst += step) { HN_G(dst, 8); *dst = bu[x * LS + F::ph(INV && !PRUNE ? (pos - p.shift) & (N - 1) : pos)]; }
+            for (int pos = r0; pos < p.n_out; pos += RPS, dst += step) { HN_G(dst, 8); *dst = bu[x * LS + F::ph(INV && !PRUNE ? ring<N>(pos + N - p.shift) : pos)]; }
         }
         __syncthreads();
     }
@@ -295,7 +295,7 @@ template <int LOG2P, bool INV, bool PRUNE> static int launch_axis_w_t(const Axis
 {
     using F = WF<LOG2P, INV>;
     constexpr int kCoreThreads = core_threads(LOG2P);
-    constexpr int N = 1 << LOG2P, TX = kCoreThreads / F::TPL;
+    constexpr int N = len_of(LOG2P), TX = kCoreThreads / F::TPL;
     const size_t sm = sizeof(float2) * ((size_t)TX * core_ls<LOG2P>() + N + PlaneTw<LOG2P, INV>::TABLE);
     static int sms = 0;
     if (!sms) {
@@ -307,7 +307,7 @@ template <int LOG2P, bool INV, bool PRUNE> static int launch_axis_w_t(const Axis
     static DevOnce attr;
     if (attr.first()) cudaFuncSetAttribute(axis_w_kernel<LOG2P, INV, PRUNE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const long long tiles = a.n_outer * ((a.nc + TX - 1) / TX);
-    const long long res = (long long)sms * (LOG2P >= 10 ? 1 : 4);
+    const long long res = (long long)sms * (len_of(LOG2P) >= 768 ? 1 : 4);
     const int grid = (int)(tiles < res ? tiles : res);
     if (grid <= 0) return 0;
     axis_w_kernel<LOG2P, INV, PRUNE><<<grid, kCoreThreads, sm, st>>>(a);
@@ -317,7 +317,7 @@ template <int LOG2P, bool INV, bool PRUNE> static int launch_axis_w_t(const Axis
 // forward: a.prune_in selects the pruned first pass; inverse: a.full keeps every output, else the lower half
 int launch_axis_w(const AxisArgs &a, bool inverse, cudaStream_t st)
 {
-    const int n = 1 << a.log2p;
+    const int n = len_of(a.log2p);
     if (a.in == a.out) return -1;
     if (!inverse && (a.n_in > (a.prune_in ? n / 2 : n) || a.n_out > n || a.shift < 0 || a.shift >= n || (a.prune_in && a.shift))) return -1;
     if (inverse && (a.n_in > n || (a.shift && !a.full) || a.n_out > (a.full ? n : n / 2))) return -1;
@@ -326,7 +326,7 @@ int launch_axis_w(const AxisArgs &a, bool inverse, cudaStream_t st)
         if (!inverse) return a.prune_in ? launch_axis_w_t<L, false, true>(a, st) : launch_axis_w_t<L, false, false>(a, st); \
         return a.full ? launch_axis_w_t<L, true, false>(a, st) : launch_axis_w_t<L, true, true>(a, st);
     switch (a.log2p) {
-        HN_AXW(6) HN_AXW(7) HN_AXW(8) HN_AXW(9) HN_AXW(10)
+        HN_AXW(6) HN_AXW(7) HN_AXW(8) HN_AXW(9) HN_AXW(10) HN_AXW(kLen192) HN_AXW(kLen384) HN_AXW(kLen768)
     default: return -1;
     }
 #undef HN_AXW

@@ -23,8 +23,8 @@ enum { PRUNE_NONE = 0, PRUNE_IN = 1, PRUNE_OUT = 2 };
 __host__ __device__ __forceinline__ constexpr int phys(int i) { return i + (i >> 4); }
 // shared-memory floats2 needed for one line of n points (odd, so lines do not alias banks)
 // largest skewed position + 1 of an n-point line under any engine (the warp engine skews short
-// lines by i >> 3)
-__host__ __device__ __forceinline__ constexpr int phys_max(int n) { return n <= 128 ? n + (n >> 3) : n + (n >> 4); }
+// lines, and lines with a factor 3, by i >> 3)
+__host__ __device__ __forceinline__ constexpr int phys_max(int n) { return n <= 128 || n % 3 == 0 ? n + (n >> 3) : n + (n >> 4); }
 __host__ __device__ __forceinline__ constexpr int line_stride(int n) { return (phys_max(n) + 1) | 1; }
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
@@ -292,12 +292,55 @@ template <bool INV, int PR> __device__ __forceinline__ void dft32(float2 (&x)[32
     column(std::integral_constant<int, 2>{}); column(std::integral_constant<int, 3>{});
 }
 
+// 24 = 3 x 8 with coprime factors: n = 3 n2 + 8 n1, k = 9 k2 + 16 k1 (mod 24) makes n k = 3 n2 k2 + 8 n1 k1 (mod 24), so the
+// 3-point and the 8-point transforms meet without twiddles (Good 1958).
+template <bool INV> __device__ __forceinline__ void dft24(float2 (&x)[24])
+{
+    float2 a[3][8];                                  // a[k1][n2]
+#pragma unroll
+    for (int n2 = 0; n2 < 8; ++n2) {
+        const float2 x0 = x[3 * n2], x1 = x[(3 * n2 + 8) % 24], x2 = x[(3 * n2 + 16) % 24];
+        const float2 t = cadd(x1, x2), s = rot90<INV>(csub(x1, x2)), m = fma2(-0.5f, t, x0);
+        a[0][n2] = cadd(x0, t);
+        a[1][n2] = fma2(0.86602540378443864676f, s, m);      // sin(pi/3)
+        a[2][n2] = fma2(-0.86602540378443864676f, s, m);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+        dft8<INV, PRUNE_NONE>(a[k1]);
+#pragma unroll
+        for (int k2 = 0; k2 < 8; ++k2) x[(9 * k2 + 16 * k1) % 24] = a[k1][k2];
+    }
+}
+
+// 12 = 3 x 4 likewise: n = 3 n2 + 4 n1, k = 9 k2 + 4 k1 (mod 12).
+template <bool INV> __device__ __forceinline__ void dft12(float2 (&x)[12])
+{
+    float2 a[3][4];                                  // a[k1][n2]
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+        const float2 x0 = x[3 * n2], x1 = x[(3 * n2 + 4) % 12], x2 = x[(3 * n2 + 8) % 12];
+        const float2 t = cadd(x1, x2), s = rot90<INV>(csub(x1, x2)), m = fma2(-0.5f, t, x0);
+        a[0][n2] = cadd(x0, t);
+        a[1][n2] = fma2(0.86602540378443864676f, s, m);      // sin(pi/3)
+        a[2][n2] = fma2(-0.86602540378443864676f, s, m);
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+        dft4<INV, PRUNE_NONE>(a[k1][0], a[k1][1], a[k1][2], a[k1][3]);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) x[(9 * k2 + 4 * k1) % 12] = a[k1][k2];
+    }
+}
+
 template <int R, bool INV, int PR> __device__ __forceinline__ void dft(float2 (&x)[R])
 {
     if constexpr (R == 2) dft2<INV, PR>(x[0], x[1]);
     else if constexpr (R == 4) dft4<INV, PR>(x[0], x[1], x[2], x[3]);
     else if constexpr (R == 8) dft8<INV, PR>(x);
     else if constexpr (R == 16) dft16<INV, PR>(x);
+    else if constexpr (R == 12) { static_assert(PR == PRUNE_NONE, "radix 12 runs on whole lines"); dft12<INV>(x); }
+    else if constexpr (R == 24) { static_assert(PR == PRUNE_NONE, "radix 24 runs on whole lines"); dft24<INV>(x); }
     else dft32<INV, PR>(x);
 }
 

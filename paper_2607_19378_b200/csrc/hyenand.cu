@@ -190,6 +190,14 @@ static int next_pow2_log(int x)
     return l;
 }
 
+// id of 3 * 2^k points where those hold `need` points and the warp engine has them, else 0
+static int len3_id(int need)
+{
+    for (int id : {kLen192, kLen384, kLen768})
+        if (need > 2 * len_of(id) / 3 && need <= len_of(id)) return id;
+    return 0;
+}
+
 static size_t elsize(int dtype) { return dtype == HYENAND_F32 ? 4 : 2; }
 
 static int dev_alloc(hyenand_plan *p, void **ptr, size_t bytes)
@@ -242,7 +250,7 @@ extern "C" hyenand_plan *hyenand_create_plan(int ndim, const int *dims, int B, i
 }
 
 // allow_slice: false for plans whose owner needs the stages of the general path one by one
-static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mode, int dtype, bool allow_slice)
+static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mode, int dtype, bool allow_slice, bool allow_len3)
 {
     g_err[0] = 0;
     if (mode != HYENAND_MODE_LINEAR && mode != HYENAND_MODE_CAUSAL && mode != HYENAND_MODE_CIRCULAR) {
@@ -335,6 +343,23 @@ static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mo
     const bool slice_plane = p->path == PATH_FUSED2D && p->log2p[2] == 6 && (long long)B * C > kFusedPlanesMax;
     p->slice = (p->path == PATH_ND_GENERIC || slice_plane) && slice_ok && slice_geo(&p->sg, p->L, causal, circular);
     if (p->slice) p->path = PATH_ND_GENERIC;
+    // Axes that 3 * 2^k points hold take those instead of the next power of two: every pass moves and transforms three quarters
+    // per axis (us with powers of two -> now: 2x96 slices of 180x150 228 -> 183, 32 of 300x280 f32 167 -> 135, 2x192 of 40x90
+    // 64 -> 58; with one such axis of three 80x128x128 970 -> 922).  Planes whose axes both fit 192 points stay on chip at that
+    // size (12 volumes of 96^3: 792 -> 512, the general passes at 192 points 818); planes with one such axis stay at
+    // 256 x 256, because the general passes cost a third trip through memory (100x90x120: 558 either way).
+    const bool len3_ok = allow_len3 && !circular && !p->slice && !p->sw.force_generic && !p->sw.generic_rows && !p->sw.generic_core &&
+                         !p->sw.no_tma && tma_available();
+    if (len3_ok && (p->path == PATH_ND_GENERIC || p->path == PATH_PLANES3D)) {
+        int id[3];
+        for (int a = 0; a < 3; ++a) id[a] = len3_id(2 * p->L[a] - 1);
+        if (three && id[1] == kLen192 && id[2] == kLen192) p->path = PATH_PLANES3D;
+        else if (p->path == PATH_PLANES3D) id[1] = id[2] = 0;      // the planes stay on chip at their power of two
+        for (int a = 0; a < 3; ++a)
+            if (id[a]) { p->log2p[a] = id[a]; p->P[a] = len_of(id[a]); }
+        p->XH = p->P[2] / 2 + 1;
+        p->XP = (p->XH + 1) & ~1;
+    }
     if (p->path == PATH_FUSED2D || p->slice) {
         p->ws_a_slice = p->wh_a_slice = p->ws_b_slice = p->wh_b_slice = 0;   // nothing leaves the chip
     } else if (p->path == PATH_PLANES3D) {
@@ -352,14 +377,19 @@ static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mo
     choose_groups(p, per_slice);
     const long long spc = p->slices_per_chunk;
 
-    int gl = 1;
-    for (int a = 0; a < 3; ++a) if (p->log2p[a] > gl) gl = p->log2p[a];
+    int gl = 1, three_k = 0;                               // the table serves every length of the plan: 2^gl or 3 * 2^gl points
+    for (int a = 0; a < 3; ++a) {
+        const bool t3 = p->P[a] % 3 == 0;
+        const int e2 = t3 ? p->log2p[a] - 16 : p->log2p[a];
+        if (e2 > gl) gl = e2;
+        three_k |= t3;
+    }
     if (p->slice) {                                        // (the slice engine may pad short axes further)
         if (p->sg.l0 > gl) gl = p->sg.l0;
         if (p->sg.l1 > gl) gl = p->sg.l1;
         if (p->sg.l2 > gl) gl = p->sg.l2;
     }
-    p->gtw_n = 1 << gl;
+    p->gtw_n = (three_k ? 3 : 1) << gl;
     std::vector<float2> tw(p->gtw_n);
     for (int t = 0; t < p->gtw_n; ++t) {
         const double ang = -2.0 * M_PI * (double)t / (double)p->gtw_n;
@@ -393,7 +423,7 @@ static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mo
 
 extern "C" hyenand_plan *hyenand_create_plan_mode(int ndim, const int *dims, int B, int C, int mode, int dtype)
 {
-    return create_plan(ndim, dims, B, C, mode, dtype, true);
+    return create_plan(ndim, dims, B, C, mode, dtype, true, true);
 }
 
 // tensor maps of the fused core's buffers; left invalid where the TMA core does not apply
@@ -542,7 +572,7 @@ static int lanes_join(hyenand_plan *p, cudaStream_t st)
 // one transform along the middle axis: warp-engine kernel where it applies, else the block-wide one
 static int launch_axis_any(const Switches &sw, const AxisArgs &a, int mode, cudaStream_t st)
 {
-    if (core_w_supported(a.log2p) && !sw.generic_core) {
+    if (!sw.generic_core) {
         const int c = launch_axis_w(a, mode == AXIS_INV, st);
         if (c >= 0) return c;
     }
@@ -1052,7 +1082,7 @@ const char *const hn::kKernelNames[KID_COUNT] = {
     "rows_fwd(h)", "axis_fwd(h)", "rows_fwd(k*v)", "axis_fwd(k*v)", "axis_core", "axis_inv", "rows_inv",
     "ct_cols_fwd(h)", "ct_cols_fwd(k*v)", "ct_core", "ct_cols_inv", "plane_fwd(h)", "plane_fwd(k*v)", "plane_inv", "fused2d", "ct_hspec", "slice_fused"};
 
-static double fft_flops(double lines, int log2n) { return lines * 5.0 * ldexp(1.0, log2n) * log2n; }
+static double fft_flops(double lines, int id) { return lines * 5.0 * len_of(id) * log2((double)len_of(id)); }
 
 extern "C" int hyenand_plan_kernel_count(const hyenand_plan *p) { return p ? KID_COUNT : 0; }
 
@@ -1586,7 +1616,7 @@ static bool spec_create(hyenand_grad *g)
     const Switches sw = read_switches();
     if (g->ndim < 2 || sw.force_generic || sw.generic_rows || sw.generic_core || sw.no_tma) return false;
     // geometry, twiddle table and status word: a plan of one slice
-    hyenand_plan *p = create_plan(g->ndim, g->dims, 1, 1, g->mode, g->dtype, false);
+    hyenand_plan *p = create_plan(g->ndim, g->dims, 1, 1, g->mode, g->dtype, false, true);
     if (!p) return true;
     const SpecGeo s = spec_geo(p);
     if ((p->path != PATH_PLANES3D && p->path != PATH_ND_GENERIC) || !core3_tma_supported(s.log2p, p->circular, s.nc)) {
@@ -1779,7 +1809,7 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
         long long nb = (2ll << 30) / (4ll * C * g->kvol);
         if (const char *e = getenv("HYENAND_BACKWARD_MAX_BATCH")) { const long long v = atoll(e); if (v > 0 && v < nb) nb = v; }   // development aid
         g->nb = (int)(nb < 1 ? 1 : nb > B ? B : nb);
-        g->main = create_plan(ndim, dims, 1, 1, mode, dtype, true);
+        g->main = create_plan(ndim, dims, 1, 1, mode, dtype, true, false);
         if (!g->main) { delete g; return nullptr; }
         g->adj = g->main;
         cudaError_t ce = guarded_alloc(&g->allocs, (void **)&g->dhs, (size_t)g->nb * C * g->kvol * sizeof(float));
@@ -1804,19 +1834,19 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
     if (nb > B) nb = B;
     g->nb = (int)nb;
     const long long S = nb * C;
-    g->main = create_plan(ndim, dims, (int)nb, C, mode, HYENAND_F32, false);
+    g->main = create_plan(ndim, dims, (int)nb, C, mode, HYENAND_F32, false, false);
     if (!g->main) { delete g; return nullptr; }
     g->adj = g->main;
     g->pair = g->main->path == PATH_PLANES3D || g->main->path == PATH_ND_GENERIC;
     // (a long causal 1-D grid gets du from the causal plan and reversed signals, see hyenand_backward)
     if (mode == HYENAND_MODE_CAUSAL && !g->pair && !g->long1d) {
-        g->adj = create_plan(ndim, dims, (int)nb, C, HYENAND_MODE_LINEAR, HYENAND_F32, false);
+        g->adj = create_plan(ndim, dims, (int)nb, C, HYENAND_MODE_LINEAR, HYENAND_F32, false, false);
         if (!g->adj) { g->adj = g->main; hyenand_backward_destroy(g); return nullptr; }
     }
     if (g->long1d) {
         g->caus = g->main;
         if (mode != HYENAND_MODE_CAUSAL) {
-            g->caus = create_plan(ndim, dims, (int)nb, C, HYENAND_MODE_CAUSAL, HYENAND_F32, false);
+            g->caus = create_plan(ndim, dims, (int)nb, C, HYENAND_MODE_CAUSAL, HYENAND_F32, false, false);
             if (!g->caus) { hyenand_backward_destroy(g); return nullptr; }
         }
     } else if (mode != HYENAND_MODE_CIRCULAR) {

@@ -15,10 +15,10 @@ __host__ __device__ constexpr int plane_ls(int n) { return ((phys_max(n) + 1 + 7
 // the CTA's threads (a handful of plain prefetch instructions per thread; a bulk prefetch per thread is executed lane
 // by lane and held the issuing warps up for thousands of cycles).  The CTA issues it for the plane it will work on
 // next, so that plane's loads hit L2.
-__device__ __forceinline__ void prefetch_l2(const void *ptr, long long bytes, int tid)
+__device__ __forceinline__ void prefetch_l2(const void *ptr, long long bytes, int tid, int nthr = kPlaneThreads)
 {
     const char *b = reinterpret_cast<const char *>(ptr);
-    for (long long o = (long long)tid * 128; o < bytes; o += (long long)kPlaneThreads * 128) {
+    for (long long o = (long long)tid * 128; o < bytes; o += (long long)nthr * 128) {
         HN_G(b + o, 1);
         asm volatile("prefetch.global.L2 [%0];\n" ::"l"(b + o) : "memory");
     }
@@ -153,7 +153,7 @@ template <int LOG2P, bool INV> struct PlaneTw {
                 const int ns = F::ns(s), rad = F::radix(s), off = PassTw<LOG2P, INV>::offset(s);
                 for (int e = tid; e < (rad - 1) * ns; e += nthr) {
                     const int r = e / ns + 1, k = e % ns;
-                    tab[off + e] = full[r * k * ((1 << LOG2P) / (ns * rad))];
+                    tab[off + e] = full[r * k * (len_of(LOG2P) / (ns * rad))];
                 }
             }
         }

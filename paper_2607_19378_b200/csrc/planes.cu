@@ -30,13 +30,14 @@
 namespace hn {
 
 template <int LOG2P> struct PlaneCfg {
-    static constexpr int P = 1 << LOG2P, HP = P / 2, XH = HP + 1;
+    static constexpr int P = len_of(LOG2P), HP = P / 2, XH = HP + 1;
+    static constexpr int NT = P % 3 ? kPlaneThreads : 384;   // 192 points: 48 groups, which the 48 row pairs and 96 columns deal evenly
     static constexpr int CSS = HP + 1;                       // filter planes: store stride (odd), P/2 bins of P/2 row pairs per half
     using F = WF<LOG2P, false>;
     using FI = WF<LOG2P, true>;
     using FH = WF<LOG2P - 1, false>;                         // half-length rows of hplane
-    static constexpr int NG = kPlaneThreads / F::TPL;        // groups working on P-point lines
-    static constexpr int NGH = kPlaneThreads / FH::TPL;      // groups working on P/2-point lines
+    static constexpr int NG = NT / F::TPL;        // groups working on P-point lines
+    static constexpr int NGH = NT / FH::TPL;      // groups working on P/2-point lines
     static constexpr int LS = plane_ls(P);
     static constexpr int LSH = plane_ls(HP);
     static constexpr int WBUF = (NG * LS > NGH * LSH) ? NG * LS : NGH * LSH;
@@ -48,16 +49,16 @@ template <int LOG2P> struct PlaneCfg {
 
 template <int LOG2P> __device__ __forceinline__ void load_plane_twiddles(float2 *tw, float2 *twh, const float2 *gtw, int gtw_n, int tid)
 {
-    constexpr int P = 1 << LOG2P;
-    const int step = gtw_n >> LOG2P;
-    for (int t = tid; t < P; t += kPlaneThreads) { HN_G(gtw + t * step, 8); tw[t] = gtw[t * step]; }
-    for (int t = tid; t < P / 2; t += kPlaneThreads) { HN_G(gtw + 2 * t * step, 8); twh[t] = gtw[2 * t * step]; }
+    constexpr int P = len_of(LOG2P), NT = PlaneCfg<LOG2P>::NT;
+    const int step = gtw_n / P;
+    for (int t = tid; t < P; t += NT) { HN_G(gtw + t * step, 8); tw[t] = gtw[t * step]; }
+    for (int t = tid; t < P / 2; t += NT) { HN_G(gtw + 2 * t * step, 8); twh[t] = gtw[2 * t * step]; }
 }
 
 // ---- k*v planes ---------------------------------------------------------------------------------
 
 template <typename T, int LOG2P>
-__global__ void __launch_bounds__(kPlaneThreads, 1) uplane_kernel(PlaneArgs p)
+__global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) uplane_kernel(PlaneArgs p)
 {
     using C = PlaneCfg<LOG2P>;
     using F = typename C::F;
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) uplane_kernel(PlaneArgs p)
     load_plane_twiddles<LOG2P>(tw, twh, p.gtw, p.gtw_n, tid);
     __syncthreads();
     PlaneTw<LOG2P, false> twp;
-    twp.init(l, tw, twh + HP, tid, kPlaneThreads);
+    twp.init(l, tw, twh + HP, tid, C::NT);
     __syncthreads();
     const T *pk = (const T *)p.a;
     const T *pv = (const T *)p.b;
@@ -155,8 +156,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) uplane_kernel(PlaneArgs p)
         if (pl + gridDim.x < p.planes) {
             // the next plane's rows travel to L2 during the column phase, which loads nothing from global memory
             const long long nb = (pl + gridDim.x) * (long long)Ly * Lx;
-            prefetch_l2(pk + nb, (long long)Ly * Lx * sizeof(T), tid);
-            prefetch_l2(pv + nb, (long long)Ly * Lx * sizeof(T), tid);
+            prefetch_l2(pk + nb, (long long)Ly * Lx * sizeof(T), tid, C::NT);
+            prefetch_l2(pv + nb, (long long)Ly * Lx * sizeof(T), tid, C::NT);
         }
         for (int kx = gid; kx < HP; kx += C::NG) {
             // Column 0 packs bins kx = 0 and kx = P/2 of every row as one complex number; it runs the same transform as
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) uplane_kernel(PlaneArgs p)
             // C = raw transform of the packed column: bins kx = 0 and kx = P/2 are (C[ky] + conj C[-ky]) / 2 and
             // -i (C[ky] - conj C[-ky]) / 2.  (The line is next written after the next CTA barrier.)
             const int ky = tid;
-            const float2 c1 = tmp[ky], c2 = tmp[(P - ky) & (P - 1)];
+            const float2 c1 = tmp[ky], c2 = tmp[ring<P>(P - ky)];
             float2 *dn = dst + (long long)HP * P;
             HN_G(dst + ky, 8);
             HN_G(dn + ky, 8);
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) uplane_kernel(PlaneArgs p)
 // for it; its raw transform goes to a shared-memory line, which the whole CTA unpacks into lines 0 and P/2 of the
 // output after the column phase.
 template <typename T, int LOG2P>
-__global__ void __launch_bounds__(kPlaneThreads, 1) hplane_kernel(PlaneArgs p)
+__global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) hplane_kernel(PlaneArgs p)
 {
     using C = PlaneCfg<LOG2P>;
     using F = typename C::F;
@@ -244,8 +245,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_kernel(PlaneArgs p)
     using PC0 = typename F::template Pass<0>;
     constexpr int NPT = 2 * PH0::IPL * PH0::R;               // parked values per thread and row pair
     constexpr int ROUNDS = HP / C::NGH;                      // row pairs per lane group and half
-    constexpr int TCOLS = 4 * ROUNDS * NPT;                  // four warps share each 32-lane quadrant
-    static_assert(HP % C::NGH == 0 && TCOLS >= 32 && TCOLS <= 512 && (TCOLS & (TCOLS - 1)) == 0, "tensor-memory columns");
+    constexpr int TUSE = C::NT / 128 * ROUNDS * NPT, TCOLS = TUSE <= 128 ? 128 : TUSE <= 256 ? 256 : 512;      // NT / 128 warps share each 32-lane quadrant
+    static_assert(HP % C::NGH == 0 && TUSE <= 512, "tensor-memory columns");
     static_assert(QP % C::NG == 0 || C::NG % QP == 0, "whole warps take part in the column loop");
     const int warp = tid >> 5;
     unsigned *tslot = reinterpret_cast<unsigned *>(smem + C::TMP + P);
@@ -257,10 +258,10 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_kernel(PlaneArgs p)
     const unsigned tbase = *tslot;
     const unsigned tpark = tmem_addr(tbase, warp, (warp >> 2) * ROUNDS * NPT);
     PlaneTw<LOG2P, false> twp;
-    twp.init(l, tw, twh + HP, tid, kPlaneThreads);
+    twp.init(l, tw, twh + HP, tid, C::NT);
     PassTw<LOG2P - 1, false> twr;                            // half-length rows
     twr.base = twh + HP + P;
-    PassTw<LOG2P - 1, false>::build(twh + HP + P, p.gtw, p.gtw_n, tid, kPlaneThreads);
+    PassTw<LOG2P - 1, false>::build(twh + HP + P, p.gtw, p.gtw_n, tid, C::NT);
     __syncthreads();
     const unsigned char *hb = (const unsigned char *)p.a;
     const int Lx = p.lx, Ly = p.ly, Kx = 2 * Lx - 1, Ky = 2 * Ly - 1;
@@ -273,13 +274,13 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_kernel(PlaneArgs p)
         for (int e = 0; e < 2; ++e) {
             // the next plane's taps travel to L2 during the second half, when this plane's are on chip
             if (e == 1 && pl + gridDim.x < p.planes)
-                prefetch_l2(hb + (pl + gridDim.x) * (long long)Ky * Kx * sizeof(T), (long long)Ky * Kx * sizeof(T), tid);
+                prefetch_l2(hb + (pl + gridDim.x) * (long long)Ky * Kx * sizeof(T), (long long)Ky * Kx * sizeof(T), tid, C::NT);
             if (e == 1 && tid < P) {
                 // the raw transform C of the packed column (bins kx = 0 and kx = P/2 of every row) waits in a shared-memory
                 // line since the column phase that has just ended: the two bins are (C[ky] + conj C[-ky]) / 2 and
                 // -i (C[ky] - conj C[-ky]) / 2.  (The line is next written two CTA barriers from here.)
                 const int ky = tid;
-                const float2 c1 = tmp[ky], c2 = tmp[(P - ky) & (P - 1)];
+                const float2 c1 = tmp[ky], c2 = tmp[ring<P>(P - ky)];
                 float2 *dn = dst + (long long)HP * P;
                 HN_G(dst + ky, 8);
                 HN_G(dn + ky, 8);
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_kernel(PlaneArgs p)
             // the two groups of a half warp take row pairs 8 apart, so their stores (one row pair per group, consecutive
             // bins per lane) fall into different banks
             for (int rp = spread_pair<8>(gidh); rp < HP; rp += C::NGH, ++round) {
-                const int my0 = (rp + Ly - 1) & (P - 1), my1 = my0 ^ HP;
+                const int my0 = rp + Ly - 1, my1 = ring<P>(my0 + HP);      // (my0 < P)
                 const bool v0 = my0 < Ky, v1 = my1 < Ky;
                 // STAGED: both tap rows are fetched with 16-byte copies into the line itself, which
                 // the first pass reads before anything is written to it; 4-byte taps do not fit the
@@ -389,7 +390,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_kernel(PlaneArgs p)
             // columns: P-point transforms over y of the bins kx = 2k + e
             for (int k = gid; k < QP; k += C::NG) {
                 const bool packed = e == 0 && k == 0;
-                const int km = packed ? HP / 2 : (e == 0 ? ((HP - k) & (HP - 1)) : HP - 1 - k);
+                const int km = packed ? HP / 2 : (e == 0 ? ring<HP>(HP - k) : HP - 1 - k);
                 const float2 *ca = cs + k * CS2, *cb = cs + km * CS2;
                 float2 *d = packed ? tmp : dst + (long long)(2 * k + e) * P;
                 float2 second[PC0::IPL][PC0::R / 2] = {};     // inputs y + P/2, formed with their partners y
@@ -419,7 +420,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_kernel(PlaneArgs p)
 // once more and leave as 16-byte stores (gate values arrive as 16-byte loads); else one element per lane and leg.
 // TWO: a second gate and result of the same planes, y2 = q2 * planes (the backward pass: dk = v du, dv = k du)
 template <typename T, int LOG2P, bool VST, bool TWO>
-__global__ void __launch_bounds__(kPlaneThreads, 1) plane_inv_kernel(PlaneArgs p)
+__global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) plane_inv_kernel(PlaneArgs p)
 {
     using C = PlaneCfg<LOG2P>;
     using FI = typename C::FI;
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_inv_kernel(PlaneArgs p
     load_plane_twiddles<LOG2P>(tw, twh, p.gtw, p.gtw_n, tid);
     __syncthreads();
     PlaneTw<LOG2P, true> twp;
-    twp.init(l, tw, twh + HP, tid, kPlaneThreads);
+    twp.init(l, tw, twh + HP, tid, C::NT);
     __syncthreads();
     const T *pq = (const T *)p.a;
     T *py = (T *)p.y;
@@ -546,8 +547,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_inv_kernel(PlaneArgs p
         __syncthreads();
         if (pl + gridDim.x < p.planes) {
             // while the rows are transformed, bring the next plane's spectra and gate into L2
-            prefetch_l2(p.in + (pl + gridDim.x) * (long long)C::XH * P, (long long)C::XH * P * sizeof(float2), tid);
-            if (gated) prefetch_l2(pq + (pl + gridDim.x) * (long long)Ly * Lx, (long long)Ly * Lx * sizeof(T), tid);
+            prefetch_l2(p.in + (pl + gridDim.x) * (long long)C::XH * P, (long long)C::XH * P * sizeof(float2), tid, C::NT);
+            if (gated) prefetch_l2(pq + (pl + gridDim.x) * (long long)Ly * Lx, (long long)Ly * Lx * sizeof(T), tid, C::NT);
         }
 #pragma unroll
         for (int it = 0; it < RIT; ++it) {
@@ -641,7 +642,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_inv_kernel(PlaneArgs p
 // inverse: with E and O those of the even and of the odd bins, f[x] = E[x] + W_P^-x O[x], f[x + P/2] = E[x] - W_P^-x O[x].
 // E waits in tensor memory until O is there.
 template <typename T, int LOG2P>
-__global__ void __launch_bounds__(kPlaneThreads, 1) hplane_inv_kernel(PlaneArgs p)
+__global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) hplane_inv_kernel(PlaneArgs p)
 {
     using C = PlaneCfg<LOG2P>;
     using FI = typename C::FI;
@@ -661,8 +662,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_inv_kernel(PlaneArgs 
     using PE = typename FH::LastPass;
     static_assert(FI::NP == 2, "two-pass plans");
     constexpr int NPT = 2 * PE::IPL * PE::R;                 // parked values per thread and row pair
-    constexpr int ROUNDS = HP / C::NGH, TCOLS = 4 * ROUNDS * NPT;
-    static_assert(HP % C::NGH == 0 && TCOLS >= 32 && TCOLS <= 512 && (TCOLS & (TCOLS - 1)) == 0, "tensor-memory columns");
+    constexpr int ROUNDS = HP / C::NGH, TUSE = C::NT / 128 * ROUNDS * NPT, TCOLS = TUSE <= 128 ? 128 : TUSE <= 256 ? 256 : 512;
+    static_assert(HP % C::NGH == 0 && TUSE <= 512, "tensor-memory columns");
     static_assert(QP % C::NG == 0 || C::NG % QP == 0, "whole warps take part in the column loop");
     const int warp = tid >> 5;
     unsigned *tslot = reinterpret_cast<unsigned *>(smem + C::TMP + P);
@@ -674,10 +675,10 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_inv_kernel(PlaneArgs 
     const unsigned tbase = *tslot;
     const unsigned tpark = tmem_addr(tbase, warp, (warp >> 2) * ROUNDS * NPT);
     PlaneTw<LOG2P, true> twp;
-    twp.init(l, tw, twh + HP, tid, kPlaneThreads);
+    twp.init(l, tw, twh + HP, tid, C::NT);
     PassTw<LOG2P - 1, true> twr;                             // half-length rows
     twr.base = twh + HP + P;
-    PassTw<LOG2P - 1, true>::build(twh + HP + P, p.gtw, p.gtw_n, tid, kPlaneThreads);
+    PassTw<LOG2P - 1, true>::build(twh + HP + P, p.gtw, p.gtw_n, tid, C::NT);
     __syncthreads();
     T *py = (T *)p.y;
     const int Lx = p.lx, Ly = p.ly, Kx = 2 * Lx - 1, Ky = 2 * Ly - 1, J0 = HP + 1 - Lx;
@@ -728,7 +729,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_inv_kernel(PlaneArgs 
             }
             __syncthreads();
             if (e == 1 && pl + gridDim.x < p.planes)
-                prefetch_l2(p.in + (pl + gridDim.x) * (long long)C::XH * P, (long long)C::XH * P * sizeof(float2), tid);
+                prefetch_l2(p.in + (pl + gridDim.x) * (long long)C::XH * P, (long long)C::XH * P * sizeof(float2), tid, C::NT);
             int round = 0;
             for (int rp = spread_pair<8>(gidh); rp < HP; rp += C::NGH, ++round) {
                 const unsigned tcol = tpark + round * NPT;
@@ -764,14 +765,15 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) hplane_inv_kernel(PlaneArgs 
                     __syncwarp();
                     TmemIO<NPT>::ld(dd, tcol);
                     tmem_wait_ld();
-                    // padded rows rp and rp + P/2 are tap rows my0 and my0 ^ P/2 (at most one lies in the zero band)
-                    const int my0 = (rp + Ly - 1) & (P - 1), my1 = my0 ^ HP;
+                    // padded rows rp and rp + P/2 are tap rows my0 and my0 + P/2 mod P (at most one lies in the zero band)
+                    const int my0 = rp + Ly - 1, my1 = ring<P>(my0 + HP);      // (my0 < P)
                     const bool v0 = my0 < Ky, v1 = my1 < Ky;
                     T *o0 = out + (long long)my0 * Kx, *o1 = out + (long long)my1 * Kx;
 #pragma unroll
                     for (int i = 0; i < PE::IPL; ++i)
 #pragma unroll
                         for (int r = 0; r < PE::R; ++r) {
+                            if (PE::idle(lh + i * TPLH)) break;
                             const int x = lh + i * TPLH + r * (HP / PE::R), j = 2 * (i * PE::R + r);
                             const int ta = x + Lx - 1, tb = x - J0;
                             if (ta < Kx) {
@@ -836,17 +838,18 @@ template <typename T, int LOG2P> static int launch_plane_t(const PlaneArgs &a, i
     if (attr[which].first()) {
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     }
-    fn<<<grid, kPlaneThreads, C::SMEM, st>>>(a);
+    fn<<<grid, C::NT, C::SMEM, st>>>(a);
     return 1;
 }
 
 int launch_plane(const PlaneArgs &a, int which, int log2p, int dtype, cudaStream_t st)
 {
     if (log2p == 8) return dtype == 0 ? launch_plane_t<float, 8>(a, which, st) : launch_plane_t<bf16, 8>(a, which, st);
+    if (log2p == kLen192) return dtype == 0 ? launch_plane_t<float, kLen192>(a, which, st) : launch_plane_t<bf16, kLen192>(a, which, st);
     if (log2p == 7) return dtype == 0 ? launch_plane_t<float, 7>(a, which, st) : launch_plane_t<bf16, 7>(a, which, st);
     return -1;
 }
 
-bool plane_supported(int log2p) { return log2p == 7 || log2p == 8; }
+bool plane_supported(int log2p) { return log2p == 7 || log2p == 8 || log2p == kLen192; }
 
 }  // namespace hn

@@ -1,4 +1,4 @@
-// Contiguous-axis passes of the N-D path, warp-engine version (padded row length 64..1024).
+// Contiguous-axis passes of the N-D path, warp-engine version (padded row length 64..1024, 192, 384, 768).
 //
 //   rows_fwd_w   one group of lanes per pair of rows: the rows are fetched with 16-byte
 //                asynchronous copies into the group's line, gated (k*v) and zero-padded on the
@@ -28,7 +28,7 @@ template <typename T, int LOG2P, int MODE>
 __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
 {
     using F = WF<LOG2P, false>;
-    constexpr int P = 1 << LOG2P, HP = P / 2, TPL = F::TPL, G = kRowThreads / TPL, LS = plane_ls(P);
+    constexpr int P = len_of(LOG2P), HP = P / 2, TPL = F::TPL, G = kRowThreads / TPL, LS = plane_ls(P);
     constexpr int PR = (MODE == 1 || MODE == 3) ? PRUNE_NONE : PRUNE_IN;
     constexpr int NT = MODE == 0 ? 2 : 1;                                       // tensors per row
     constexpr int ROWMAX = (MODE == 1 ? P - 1 : HP) * (int)sizeof(T);           // longest row in bytes
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
     const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL;
     const unsigned m = F::group_mask(tid);
     float2 *line = smem + gid * LS;
-    for (int t = tid; t < P; t += kRowThreads) { HN_G(p.gtw + t * (p.gtw_n >> LOG2P), 8); twt[t] = p.gtw[t * (p.gtw_n >> LOG2P)]; }
+    for (int t = tid; t < P; t += kRowThreads) { HN_G(p.gtw + t * (p.gtw_n / P), 8); twt[t] = p.gtw[t * (p.gtw_n / P)]; }
     __syncthreads();
     PlaneTw<LOG2P, false> tw;
     tw.init(l, twt, twt + P, tid, kRowThreads);
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
             });
             float2 *o0 = p.out + r0 * p.pitch, *o1 = p.out + r1 * p.pitch;
             for (int kx = l; kx <= HP; kx += TPL) {
-                const float2 z1 = line[F::ph(kx)], z2 = line[F::ph((P - kx) & (P - 1))];
+                const float2 z1 = line[F::ph(kx)], z2 = line[F::ph(ring<P>(P - kx))];
                 HN_G(o0 + kx, 8);
                 if (has1) HN_G(o1 + kx, 8);
                 o0[kx] = make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
@@ -102,9 +102,9 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
             zero_staged<T, TPL>(s, f0, p.len, P, l);
             zero_staged<T, TPL>(s + SLOT, f1, has1 ? p.len : 0, P, l);
             __syncwarp(m);
-            const int cw = (l + p.shift) & (P - 1);
+            const int cw = ring<P>(l + p.shift);
             F::template run_to_line<PR, true>(l, m, tw, line, [&](int i, int r, int) {
-                const int mm = (cw + i * TPL + r * (P / F::template Pass<0>::R)) & (P - 1);
+                const int mm = ring<P>(cw + i * TPL + r * (P / F::template Pass<0>::R));
                 return make_float2(staged<T>(s, f0, mm), staged<T>(s + SLOT, f1, mm));
             });
         } else if (p.len == HP && has1) {
@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
         }
         float2 *o0 = p.out + r0 * p.pitch, *o1 = p.out + r1 * p.pitch;
         for (int kx = l; kx <= HP; kx += TPL) {
-            const float2 z1 = line[F::ph(kx)], z2 = line[F::ph((P - kx) & (P - 1))];
+            const float2 z1 = line[F::ph(kx)], z2 = line[F::ph(ring<P>(P - kx))];
             HN_G(o0 + kx, 8);
             if (has1) HN_G(o1 + kx, 8);
             o0[kx] = make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
@@ -148,7 +148,7 @@ template <typename T, int LOG2P, bool FULL>
 __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs p)
 {
     using FI = WF<LOG2P, true>;
-    constexpr int P = 1 << LOG2P, HP = P / 2, TPL = FI::TPL, G = kRowThreads / TPL, LS = plane_ls(P);
+    constexpr int P = len_of(LOG2P), HP = P / 2, TPL = FI::TPL, G = kRowThreads / TPL, LS = plane_ls(P);
     constexpr int RS = HP + 2;                                   // slot of one staged half spectrum
     static_assert(2 * RS <= LS, "staged spectra must fit the line");
     extern __shared__ float2 smem[];
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
     const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL;
     const unsigned m = FI::group_mask(tid);
     float2 *line = smem + gid * LS;
-    for (int t = tid; t < P; t += kRowThreads) { HN_G(p.gtw + t * (p.gtw_n >> LOG2P), 8); twt[t] = p.gtw[t * (p.gtw_n >> LOG2P)]; }
+    for (int t = tid; t < P; t += kRowThreads) { HN_G(p.gtw + t * (p.gtw_n / P), 8); twt[t] = p.gtw[t * (p.gtw_n / P)]; }
     __syncthreads();
     PlaneTw<LOG2P, true> tw;
     tw.init(l, twt, twt + P, tid, kRowThreads);
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
             const float sg = (r == RH && idx == HP) ? 1.f : -1.f;
             return make_float2(fmaf(-sg, B.y, A.x), fmaf(sg, A.y, B.x));
         });
-        auto at = [&](int n) { return line[FI::ph(FULL ? (n - p.shift) & (P - 1) : n)]; };
+        auto at = [&](int n) { return line[FI::ph(FULL ? ring<P>(n + P - p.shift) : n)]; };
         if (!FULL && p.len == HP && has1 && pq) {
             // full rows: all gate loads of the pair are in flight together (they were asked into L2 above)
             float qa[HP / TPL], qb[HP / TPL];
@@ -254,12 +254,12 @@ static int rows_sms()
     return n;
 }
 
-bool rows_w_supported(int log2p) { return log2p >= 6 && log2p <= 10; }
+bool rows_w_supported(int log2p) { return (log2p >= 6 && log2p <= 10) || (log2p >= kLen192 && log2p <= kLen768); }
 
 template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &a, cudaStream_t st)
 {
     using F = WF<LOG2P, false>;
-    constexpr int P = 1 << LOG2P, G = kRowThreads / F::TPL, LS = plane_ls(P);
+    constexpr int P = len_of(LOG2P), G = kRowThreads / F::TPL, LS = plane_ls(P);
     const size_t sm = sizeof(float2) * ((size_t)G * LS + 2 * P);
     const long long want = ((a.rows + 1) / 2 + G - 1) / G;
     const int grid = (int)(want < 2ll * rows_sms() ? want : 2ll * rows_sms());
@@ -272,7 +272,9 @@ template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &
         }                                                                                                \
         rows_fwd_w_kernel<T, LOG2P, MODE><<<grid, kRowThreads, sm, st>>>(a);                             \
     } while (0)
-    if (a.full_in) HN_LAUNCH(3);
+    if (a.full_in) {
+        if constexpr ((P & (P - 1)) == 0) HN_LAUNCH(3); else return -1;      // (periodic grids are powers of two)
+    }
     else if (a.b) HN_LAUNCH(0);
     else if (a.prune_in) HN_LAUNCH(2);
     else HN_LAUNCH(1);
@@ -283,7 +285,7 @@ template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &
 template <typename T, int LOG2P> static int launch_rows_inv_w_t(const RowsInvArgs &a, cudaStream_t st)
 {
     using F = WF<LOG2P, true>;
-    constexpr int P = 1 << LOG2P, G = kRowThreads / F::TPL, LS = plane_ls(P);
+    constexpr int P = len_of(LOG2P), G = kRowThreads / F::TPL, LS = plane_ls(P);
     const size_t sm = sizeof(float2) * ((size_t)G * LS + 2 * P);
     const long long want = ((a.rows + 1) / 2 + G - 1) / G;
     const int grid = (int)(want < 2ll * rows_sms() ? want : 2ll * rows_sms());
@@ -299,6 +301,7 @@ template <typename T, int LOG2P> static int launch_rows_inv_w_t(const RowsInvArg
     switch (x) {                                                                               \
     case 6: CALL(6); break; case 7: CALL(7); break; case 8: CALL(8); break;                    \
     case 9: CALL(9); break; case 10: CALL(10); break;                                          \
+    case kLen192: CALL(kLen192); break; case kLen384: CALL(kLen384); break; case kLen768: CALL(kLen768); break;     \
     default: return -1;                                                                        \
     }
 

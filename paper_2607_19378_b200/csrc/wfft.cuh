@@ -16,6 +16,13 @@
 
 namespace hn {
 
+// position v in [0, 2N) on a ring of N points
+template <int N> __device__ __forceinline__ int ring(int v)
+{
+    if constexpr ((N & (N - 1)) == 0) return v & (N - 1);
+    else return v >= N ? v - N : v;
+}
+
 template <int LOG2N> struct WPlan;
 template <> struct WPlan<5>  { static constexpr int NP = 2, TPL = 4; static constexpr int R[3] = {8, 4, 1};
     __host__ __device__ static constexpr int r(int s) { return s == 0 ? 8 : s == 1 ? 4 : 1; } };
@@ -30,6 +37,17 @@ template <> struct WPlan<9>  { static constexpr int NP = 2, TPL = 16; static con
 template <> struct WPlan<10>  { static constexpr int NP = 2, TPL = 32; static constexpr int R[3] = {32, 32, 1};
     __host__ __device__ static constexpr int r(int s) { return s == 0 ? 32 : s == 1 ? 32 : 1; } };
 
+// 3 * 2^k: the factor 3 sits in a radix-24 (96: radix-12) pass, last of the forward and first of the inverse transform, so that the pruned
+// passes keep their power-of-two radix.  (96, 384 and 768 leave a quarter of the lanes idle in the other pass.)
+template <> struct WPlan<21>  { static constexpr int NP = 2, TPL = 8; static constexpr int R[3] = {8, 12, 1};
+    __host__ __device__ static constexpr int r(int s) { return s == 0 ? 8 : s == 1 ? 12 : 1; } };
+template <> struct WPlan<22>  { static constexpr int NP = 2, TPL = 8; static constexpr int R[3] = {8, 24, 1};
+    __host__ __device__ static constexpr int r(int s) { return s == 0 ? 8 : s == 1 ? 24 : 1; } };
+template <> struct WPlan<23>  { static constexpr int NP = 2, TPL = 16; static constexpr int R[3] = {16, 24, 1};
+    __host__ __device__ static constexpr int r(int s) { return s == 0 ? 16 : s == 1 ? 24 : 1; } };
+template <> struct WPlan<24>  { static constexpr int NP = 2, TPL = 32; static constexpr int R[3] = {32, 24, 1};
+    __host__ __device__ static constexpr int r(int s) { return s == 0 ? 32 : s == 1 ? 24 : 1; } };
+
 // Twiddle sources.  A source answers get<S>(i, r, k, t) for pass S: item i of the lane, leg r,
 // k = position of the item inside its sub-transform, t = index into a full N-point table (the
 // twiddle wanted is exp(-2 pi i t / N); the engine conjugates it for inverse transforms).
@@ -40,7 +58,7 @@ template <int N> struct TableTw {               // full table of N entries in sh
 
 template <int LOG2N, bool INV> struct WF {
     using P = WPlan<LOG2N>;
-    static constexpr int N = 1 << LOG2N;
+    static constexpr int N = len_of(LOG2N);
     static constexpr int NP = P::NP;
     static constexpr int TPL = P::TPL;
     static constexpr int LPW = 32 / TPL;                  // lines per warp
@@ -59,14 +77,15 @@ template <int LOG2N, bool INV> struct WF {
     // Lines are stored skewed: position i sits at ph(i).  The shift follows the radix of the first
     // pass, whose results land R points apart per lane: with it the groups of a warp that work on
     // neighbouring lines never meet in a bank.
-    static constexpr int SKEW = (LOG2N <= 7 && radix(0) == 8) ? 3 : radix(0) == 32 ? 5 : 4;
+    static constexpr int SKEW = (radix(0) == 8 || radix(0) == 12 || radix(0) == 24) ? 3 : radix(0) == 32 ? 5 : 4;
     __host__ __device__ static constexpr int ph(int i) { return i + (i >> SKEW); }
     template <int S> struct Pass {
         static constexpr int R = radix(S);
         static constexpr int NS = ns(S);
         static constexpr int ITEMS = N / R;
-        static constexpr int IPL = ITEMS >= TPL ? ITEMS / TPL : 1;   // items per lane
-        static constexpr bool PARTIAL = ITEMS < TPL;                 // only lanes < ITEMS work
+        static constexpr int IPL = (ITEMS + TPL - 1) / TPL;          // items per lane
+        static constexpr bool PARTIAL = ITEMS % TPL != 0;            // the last item of the lanes beyond ITEMS does not exist
+        static __device__ __forceinline__ bool idle(int j) { return PARTIAL && j >= ITEMS; }
     };
 
     // One pass.  in(i, r, idx) -> float2 gives the point at position idx (item i of this
@@ -81,17 +100,17 @@ template <int LOG2N, bool INV> struct WF {
         constexpr int R = PS::R, NS = PS::NS;
         constexpr int NIN = (PR == PRUNE_IN) ? R / 2 : R;
         constexpr int NOUT = (PR == PRUNE_OUT) ? R / 2 : R;
-        if (PS::PARTIAL && l >= PS::ITEMS) return;
 #pragma unroll
         for (int i = 0; i < PS::IPL; ++i) {
             const int j = l + i * TPL;
+            if (PS::idle(j)) break;
             float2 x[R];
 #pragma unroll
             for (int r = 0; r < NIN; ++r) x[r] = in(i, r, j + r * (N / R));
 #pragma unroll
             for (int r = NIN; r < R; ++r) x[r] = make_float2(0.f, 0.f);
             if constexpr (NS > 1) {
-                const int k = j & (NS - 1);
+                const int k = j % NS;
 #pragma unroll
                 for (int r = 1; r < NIN; ++r) {
                     const float2 w = tw.template get<S>(i, r, k, r * k * (N / (NS * R)));
@@ -99,7 +118,7 @@ template <int LOG2N, bool INV> struct WF {
                 }
             }
             dft<R, INV, PR>(x);
-            const int k = j & (NS - 1);
+            const int k = j % NS;
             const int base = (j - k) * R + k;
 #pragma unroll
             for (int r = 0; r < NOUT; ++r) out(i, r, base + r * NS, x[r]);
@@ -120,11 +139,12 @@ template <int LOG2N, bool INV> struct WF {
                 [&](int, int, int idx) { return line[ph(idx)]; },
                 [&](int i, int r, int, float2 v) { keep[i][r] = v; });
             __syncwarp(m);
-            if (!(PS::PARTIAL && l >= PS::ITEMS)) {
+            {
 #pragma unroll
                 for (int i = 0; i < PS::IPL; ++i) {
                     const int j = l + i * TPL;
-                    const int k = j & (PS::NS - 1);
+                    if (PS::idle(j)) break;
+                    const int k = j % PS::NS;
                     const int base = (j - k) * R + k;
 #pragma unroll
                     for (int r = 0; r < R; ++r) line[ph(base + r * PS::NS)] = keep[i][r];
@@ -149,11 +169,11 @@ template <int LOG2N, bool INV> struct WF {
             float2 keep[P0::IPL][P0::R];
             pass<0, PF>(l, tw, in, [&](int i, int r, int, float2 v) { keep[i][r] = v; });
             __syncwarp(m);
-            if (!(P0::PARTIAL && l >= P0::ITEMS)) {
 #pragma unroll
-                for (int i = 0; i < P0::IPL; ++i)
+            for (int i = 0; i < P0::IPL; ++i) {
+                if (P0::idle(l + i * TPL)) break;
 #pragma unroll
-                    for (int r = 0; r < P0::R; ++r) line[ph((l + i * TPL) * P0::R + r)] = keep[i][r];
+                for (int r = 0; r < P0::R; ++r) line[ph((l + i * TPL) * P0::R + r)] = keep[i][r];
             }
         } else {
             pass<0, PF>(l, tw, in, [&](int, int, int idx, float2 v) { line[ph(idx)] = v; });
@@ -175,7 +195,7 @@ template <int LOG2N, bool INV> struct WF {
         {
 #pragma unroll
             for (int i = 0; i < PS::IPL; ++i) {
-                const int k = (l + i * TPL) & (PS::NS - 1);
+                const int k = (l + i * TPL) % PS::NS;
 #pragma unroll
                 for (int r = 1; r < PS::R; ++r) w[i][r] = table[r * k * (N / (PS::NS * PS::R))];
             }
@@ -192,11 +212,12 @@ template <int LOG2N, bool INV> struct WF {
         float2 keep[PS::IPL][PS::R];
         run<PR, ALIAS>(l, m, tw, line, in, [&](int i, int r, int, float2 v) { keep[i][r] = v; });
         __syncwarp(m);
-        if (!(PS::PARTIAL && l >= PS::ITEMS)) {
+        {
             constexpr int NOUT = (PR == PRUNE_OUT) ? PS::R / 2 : PS::R;
 #pragma unroll
             for (int i = 0; i < PS::IPL; ++i) {
                 const int j = l + i * TPL;
+                if (PS::idle(j)) break;
 #pragma unroll
                 for (int r = 0; r < NOUT; ++r) line[ph(j + r * (N / PS::R))] = keep[i][r];
             }
@@ -221,8 +242,8 @@ template <int LOG2N, bool INV> struct PassTw {
     // gtw: global table of gtw_n >= N points; all nthr threads take part; caller synchronises
     static __device__ __forceinline__ void build(float2 *dst, const float2 *gtw, int gtw_n, int tid, int nthr)
     {
-        constexpr int N = 1 << LOG2N;
-        const int step = gtw_n >> LOG2N;
+        constexpr int N = len_of(LOG2N);
+        const int step = gtw_n / N;
         for (int s = 1; s < F::NP; ++s) {
             const int ns = F::ns(s), rad = F::radix(s), off = offset(s);
             for (int e = tid; e < (rad - 1) * ns; e += nthr) {
