@@ -117,6 +117,7 @@ axis_core3_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_co
             tma_load_3d(tg + b * G::BOXB, &map_g, bar, x, b * G::BOXR, (int)o);
         }
     };
+    pdl_join();
     if (tid == 0 && (long long)blockIdx.x < tiles) issue(blockIdx.x);
     unsigned phase = 0;
     int failed = 0;
@@ -248,7 +249,7 @@ template <int LOG2P, bool FULL> static int launch_core3_t(Core3Params p, const C
     const int grid = (int)(tiles < res ? tiles : res);
     if (grid <= 0) return 0;
     auto map = [](const unsigned char *b) -> const CUtensorMap & { return *reinterpret_cast<const CUtensorMap *>(b); };
-    axis_core3_tma_kernel<LOG2P, FULL><<<grid, G::THREADS, G::TOTAL, st>>>(map(m.u), map(m.g), map(m.h), map(m.dh), p);
+    launch_pdl(axis_core3_tma_kernel<LOG2P, FULL>, grid, G::THREADS, G::TOTAL, st, map(m.u), map(m.g), map(m.h), map(m.dh), p);
     return 1;
 }
 

@@ -169,6 +169,7 @@ axis_core_tma_kernel(const __grid_constant__ CUtensorMap map_u, const __grid_con
     };
     long long t = blockIdx.x, tprev = 0;
     bool have_prev = false;
+    pdl_join();
     if (tid == 0 && t < tiles) { issue_h(t); issue_u(t); }
     unsigned phase = 0;
     int failed = 0;
@@ -303,7 +304,7 @@ template <int LOG2P, bool FULL> static int launch_core_tma_t(const CoreTmaParams
     const long long res = (long long)sms * G::CTA::PER_SM;           // resident CTAs
     const int grid = (int)(tiles < res ? tiles : res);
     if (grid <= 0) return 0;
-    axis_core_tma_kernel<LOG2P, FULL><<<grid, G::THREADS, G::TOTAL, st>>>(
+    launch_pdl(axis_core_tma_kernel<LOG2P, FULL>, grid, G::THREADS, G::TOTAL, st,
         *reinterpret_cast<const CUtensorMap *>(m.u), *reinterpret_cast<const CUtensorMap *>(m.h), p);
     return 1;
 }

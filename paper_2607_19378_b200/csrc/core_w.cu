@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(core_threads(LOG2P), (LOG2P >= 10 ? 1 : 2)) ax
     PlaneTw<LOG2P, true> twi;
     twi.init(l, twt, twt + N + PlaneTw<LOG2P, false>::TABLE, tid, kCoreThreads);
     __syncthreads();
+    pdl_join();
     const long long tpo = (p.nc + TX - 1) / TX;
     const long long tiles = p.n_outer * tpo;
     // Tile loads are asynchronous copies (one complex bin per thread and row) straight into the
@@ -219,7 +220,7 @@ template <int LOG2P, bool FULL> static int launch_core_w_t(const AxisArgs &a, cu
     const long long res = (long long)sms * 2;
     const int grid = (int)(tiles < res ? tiles : res);
     if (grid <= 0) return 0;
-    axis_core_w_kernel<LOG2P, FULL><<<grid, kCoreThreads, sm, st>>>(a);
+    launch_pdl(axis_core_w_kernel<LOG2P, FULL>, grid, kCoreThreads, sm, st, a);
     return 1;
 }
 
@@ -247,6 +248,7 @@ __global__ void __launch_bounds__(core_threads(LOG2P), (len_of(LOG2P) >= 768 ? 1
     PlaneTw<LOG2P, INV> tw;
     tw.init(l, twt, twt + N, tid, kCoreThreads);
     __syncthreads();
+    pdl_join();
     const long long tpo = (p.nc + TX - 1) / TX;
     const long long tiles = p.n_outer * tpo;
     const int shift = INV ? 0 : p.shift;                   // (of the input; an inverse without crop shifts its output)
@@ -310,7 +312,7 @@ template <int LOG2P, bool INV, bool PRUNE> static int launch_axis_w_t(const Axis
     const long long res = (long long)sms * (len_of(LOG2P) >= 768 ? 1 : 4);
     const int grid = (int)(tiles < res ? tiles : res);
     if (grid <= 0) return 0;
-    axis_w_kernel<LOG2P, INV, PRUNE><<<grid, kCoreThreads, sm, st>>>(a);
+    launch_pdl(axis_w_kernel<LOG2P, INV, PRUNE>, grid, kCoreThreads, sm, st, a);
     return 1;
 }
 

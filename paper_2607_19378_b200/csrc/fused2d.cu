@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(kF2Threads, 1) fused2d_kernel(Fused2dArgs p)  
     PlaneTw<LOG2P, true> twi;
     twi.init(l, tw, tw + 2 * P, tid, kF2Threads);
     __syncthreads();
+    pdl_join();
     const unsigned char *kb = (const unsigned char *)p.k, *vb = (const unsigned char *)p.v;
     const unsigned char *hb = (const unsigned char *)p.h;
     const unsigned char *ke = kb + p.kv_elems * sizeof(T), *ve = vb + p.kv_elems * sizeof(T), *he = hb + p.h_elems * sizeof(T);
@@ -370,7 +371,7 @@ template <typename T, int LOG2P> static int launch_fused2d_t(const Fused2dArgs &
     if (attr[(mix ? 2 : 0) + (vst ? 1 : 0)].first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     const int grid = (int)(a.slices < sms ? a.slices : sms);
     if (grid <= 0) return 0;
-    fn<<<grid, kF2Threads, C::SMEM, st>>>(a);
+    launch_pdl(fn, grid, kF2Threads, C::SMEM, st, a);
     return 1;
 }
 

@@ -164,6 +164,7 @@ struct hyenand_plan {
     // host-staging for hyenand_forward_host
     void *stage[5];
     size_t stage_bytes[5];
+    bool gtw_fresh;                   // the twiddle table is written by a kernel of each call (allocation-free entry point)
     int h_dtype;                      // element type of the filter taps (differs from dtype only inside the mixer)
     // Element types per signal side on the multi-kernel paths, which take them per launch (the backward pass reads the
     // caller's bf16 tensors and writes a bf16 gradient on one side, an fp32 intermediate on the other): k and v are
@@ -591,7 +592,7 @@ static int filter_spectrum_generic(hyenand_plan *p, int l, const char *h, long l
     r.log2p = p->log2p[2];
     r.prune_in = p->causal && p->P[2] >= 2;
     r.full_in = p->circular;
-    r.gtw = p->gtw; r.gtw_n = p->gtw_n;
+    r.gtw = p->gtw; r.gtw_n = p->gtw_n; r.gtw_fresh = p->gtw_fresh;
     p->prof.begin(KID_ROWS_H, st);
     const bool roww = rows_w_supported(r.log2p) && !p->sw.generic_rows;
     int n = roww ? launch_rows_fwd_w(r, p->h_dtype, st) : launch_rows_fwd(r, p->h_dtype, st);
@@ -677,7 +678,7 @@ static int forward_generic(hyenand_plan *p, const char *q, const char *k, const 
             RowsArgs r{};
             r.a = sk + (size_t)s0 * p->vol * ei; r.b = sv ? sv + (size_t)s0 * p->vol * ei : nullptr; r.out = ln.ws_a; r.pitch = p->XP;
             r.rows = n * p->L[0] * p->L[1]; r.len = p->L[2]; r.shift = 0; r.log2p = p->log2p[2];
-            r.prune_in = !p->circular; r.full_in = p->circular; r.gtw = p->gtw; r.gtw_n = p->gtw_n;
+            r.prune_in = !p->circular; r.full_in = p->circular; r.gtw = p->gtw; r.gtw_n = p->gtw_n; r.gtw_fresh = p->gtw_fresh;
             p->prof.begin(KID_ROWS_U, st);
             const bool roww = rows_w_supported(r.log2p) && !p->sw.generic_rows;
             int c = roww ? launch_rows_fwd_w(r, dt_in, st) : launch_rows_fwd(r, dt_in, st);
@@ -2362,6 +2363,7 @@ extern "C" int hyenand_forward_noalloc(int ndim, const int *dims, int B, int C, 
     unsigned char *base = (unsigned char *)g_noalloc_ptr[dev];
     unsigned long long off = 0;
     p->gtw = (float2 *)(base + off); off += tw_b;
+    p->gtw_fresh = true;
     ln.ws_a = (float2 *)(base + off); off += ua * spc;
     ln.ws_b = three ? (float2 *)(base + off) : nullptr; off += ub * spc;
     ln.wh_a = (float2 *)(base + off); off += ha * (unsigned long long)ln.wh_slices;

@@ -56,7 +56,9 @@ __global__ void __launch_bounds__(kThreads) rows_fwd_kernel(RowsArgs p)
     const int tid = threadIdx.x;
     const T *pa = (const T *)p.a;
     const T *pb = (const T *)p.b;
+    if (p.gtw_fresh) pdl_wait();
     if (N >= 4) load_twiddles(tw, p.gtw, N, p.gtw_n, tid, kThreads);
+    pdl_join();
     const long long pairs = (p.rows + 1) / 2;
     const long long chunks = (pairs + G - 1) / G;
     for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
@@ -107,7 +109,7 @@ static int launch_rows_fwd_t(const RowsArgs &a, cudaStream_t st)
             cudaFuncSetAttribute(rows_fwd_kernel<T, LOG2P, HASB, PR>,                           \
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);         \
         }                                                                                       \
-        rows_fwd_kernel<T, LOG2P, HASB, PR><<<grid, kThreads, sm, st>>>(a);                     \
+        launch_pdl(rows_fwd_kernel<T, LOG2P, HASB, PR>, grid, kThreads, sm, st, a);             \
     } while (0)
     if (a.b && a.full_in) HN_LAUNCH(true, false);
     else if (a.b) HN_LAUNCH(true, true);
@@ -153,6 +155,7 @@ __global__ void __launch_bounds__(kThreads) rows_inv_kernel(RowsInvArgs p)
     const T *pq = (const T *)p.q;
     T *py = (T *)p.y;
     if (N >= 4) load_twiddles(tw, p.gtw, N, p.gtw_n, tid, kThreads);
+    pdl_join();
     const long long pairs = (p.rows + 1) / 2;
     const long long chunks = (pairs + G - 1) / G;
     for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
@@ -215,7 +218,7 @@ static int launch_rows_inv_t(const RowsInvArgs &a, cudaStream_t st)
     static DevOnce attr[2];
     void (*fn)(RowsInvArgs) = a.full_out ? rows_inv_kernel<T, LOG2P, true> : rows_inv_kernel<T, LOG2P, false>;
     if (attr[a.full_out ? 1 : 0].first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    fn<<<grid, kThreads, sm, st>>>(a);
+    launch_pdl(fn, grid, kThreads, sm, st, a);
     return 1;
 }
 
@@ -260,6 +263,7 @@ __global__ void __launch_bounds__(kThreads) axis_kernel(AxisArgs p)
     float2 *tw = smem + (MODE == AXIS_CORE ? 2 : 1) * TX * LS;
     const int tid = threadIdx.x;
     if (N >= 4) load_twiddles(tw, p.gtw, N, p.gtw_n, tid, kThreads);
+    pdl_join();
     const long long tpo = (p.nc + TX - 1) / TX;
     const long long tiles = p.n_outer * tpo;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -309,7 +313,7 @@ static int launch_axis_t(const AxisArgs &a, cudaStream_t st)
     if (attr.first()) {
         cudaFuncSetAttribute(axis_kernel<MODE, LOG2P, PRUNE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     }
-    axis_kernel<MODE, LOG2P, PRUNE><<<grid, kThreads, sm, st>>>(a);
+    launch_pdl(axis_kernel<MODE, LOG2P, PRUNE>, grid, kThreads, sm, st, a);
     return 1;
 }
 

@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) uplane_kernel(PlaneArg
     const unsigned char *kb = (const unsigned char *)p.a, *vb = (const unsigned char *)p.b;
     const unsigned char *ke = kb + p.a_elems * sizeof(T), *ve = vb + p.a_elems * sizeof(T);
     const int Lx = p.lx, Ly = p.ly;
+    pdl_join();
     for (long long pl = blockIdx.x; pl < p.planes; pl += gridDim.x) {
         const long long ib = pl * (long long)Ly * Lx;
         // rows: y and y + P/4 share a transform (rows P/4 .. Ly-1 exist, Ly > P/4; a missing partner is a zero row)
@@ -268,6 +269,7 @@ __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) hplane_kernel(PlaneArg
     constexpr int R0 = PH0::R;
     const int J0 = HP + 1 - Lx;                              // window position of tap 0
     const int RU = (J0 * (int)sizeof(T) + 15) & ~15;         // bytes kept free before the first copied chunk
+    pdl_join();
     for (long long pl = blockIdx.x; pl < p.planes; pl += gridDim.x) {
         const long long ib = pl * (long long)Ky * Kx;
         float2 *dst = p.out + pl * (long long)C::XH * P;
@@ -453,6 +455,7 @@ __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) plane_inv_kernel(Plane
         for (int e = 0; e < Vec16<T>::VEC; ++e) f[e] = gated ? 0.f : 1.f;
         qvfill = Vec16<T>::pack(f);
     }
+    pdl_join();
     for (long long pl = blockIdx.x; pl < p.planes; pl += gridDim.x) {
         const float2 *src = p.in + pl * (long long)C::XH * P;
         // Column kx + NG is requested (into registers) between the two passes of column kx: the loads
@@ -682,6 +685,7 @@ __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) hplane_inv_kernel(Plan
     __syncthreads();
     T *py = (T *)p.y;
     const int Lx = p.lx, Ly = p.ly, Kx = 2 * Lx - 1, Ky = 2 * Ly - 1, J0 = HP + 1 - Lx;
+    pdl_join();
     for (long long pl = blockIdx.x; pl < p.planes; pl += gridDim.x) {
         const float2 *src = p.in + pl * (long long)C::XH * P;
         T *out = py + pl * (long long)Ky * Kx;
@@ -838,7 +842,7 @@ template <typename T, int LOG2P> static int launch_plane_t(const PlaneArgs &a, i
     if (attr[which].first()) {
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     }
-    fn<<<grid, C::NT, C::SMEM, st>>>(a);
+    launch_pdl(fn, grid, C::NT, C::SMEM, st, a);
     return 1;
 }
 

@@ -39,11 +39,13 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
     const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL;
     const unsigned m = F::group_mask(tid);
     float2 *line = smem + gid * LS;
+    if (p.gtw_fresh) pdl_wait();
     for (int t = tid; t < P; t += kRowThreads) { HN_G(p.gtw + t * (p.gtw_n / P), 8); twt[t] = p.gtw[t * (p.gtw_n / P)]; }
     __syncthreads();
     PlaneTw<LOG2P, false> tw;
     tw.init(l, twt, twt + P, tid, kRowThreads);
     __syncthreads();
+    pdl_join();
     const unsigned char *ab = (const unsigned char *)p.a, *bb = (const unsigned char *)p.b;
     const unsigned char *ahi = ab + p.rows * (long long)p.len * sizeof(T);
     const unsigned char *bhi = bb + p.rows * (long long)p.len * sizeof(T);
@@ -161,6 +163,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
     PlaneTw<LOG2P, true> tw;
     tw.init(l, twt, twt + P, tid, kRowThreads);
     __syncthreads();
+    pdl_join();
     const T *pq = (const T *)p.q;
     T *py = (T *)p.y;
     const long long pairs = (p.rows + 1) / 2;
@@ -270,7 +273,7 @@ template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &
         if (attr.first()) {                                                                                     \
             cudaFuncSetAttribute(rows_fwd_w_kernel<T, LOG2P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
         }                                                                                                \
-        rows_fwd_w_kernel<T, LOG2P, MODE><<<grid, kRowThreads, sm, st>>>(a);                             \
+        launch_pdl(rows_fwd_w_kernel<T, LOG2P, MODE>, grid, kRowThreads, sm, st, a);                     \
     } while (0)
     if (a.full_in) {
         if constexpr ((P & (P - 1)) == 0) HN_LAUNCH(3); else return -1;      // (periodic grids are powers of two)
@@ -293,7 +296,7 @@ template <typename T, int LOG2P> static int launch_rows_inv_w_t(const RowsInvArg
     static DevOnce attr[2];
     void (*fn)(RowsInvArgs) = a.full_out ? rows_inv_w_kernel<T, LOG2P, true> : rows_inv_w_kernel<T, LOG2P, false>;
     if (attr[a.full_out ? 1 : 0].first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    fn<<<grid, kRowThreads, sm, st>>>(a);
+    launch_pdl(fn, grid, kRowThreads, sm, st, a);
     return 1;
 }
 

@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(SliceCta<SliceFft<L0, L1, L2>>::CT, SliceCta<S
     extern __shared__ float2 smem[];
     const int tid = threadIdx.x, t = tid % S::T, grp = CT::WARP ? tid / S::T : 0;
     float2 *bu = smem + (size_t)grp * 3 * S::BUF, *bh = bu + S::BUF, *bg = bh + S::BUF;
+    pdl_join();
     typename S::Tw tw;
     S::init(tw, smem + (size_t)CT::NG * 3 * S::BUF, p.gtw, p.gtw_n, tid, CT::CT, t);
     __syncthreads();
@@ -166,7 +167,7 @@ template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN> int launch_s
     if (slots <= 0) return -1;
     const long long ctas = (a.slices + CT::NG - 1) / CT::NG;
     if (ctas <= 0) return 0;
-    fn<<<(int)(ctas < slots ? ctas : slots), CT::CT, sm, st>>>(a);
+    launch_pdl(fn, (unsigned)(ctas < slots ? ctas : slots), CT::CT, sm, st, a);
     return 1;
 }
 

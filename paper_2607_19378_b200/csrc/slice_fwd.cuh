@@ -274,6 +274,7 @@ __global__ void __launch_bounds__(SliceCta<SliceFft<L0, L1, L2>>::CT, SliceCta<S
     typename S::Tw tw;
     S::init(tw, smem + (size_t)CT::NG * 2 * S::BUF, p.gtw, p.gtw_n, tid, CT::CT, t);
     __syncthreads();
+    pdl_join();
     auto sync = [] { CT::sync(); };
     const SliceGeo &g = p.g;
     const float sc = 0.25f / (float)S::M;                    // 1/M of the inverse, 1/4 of the two separations
@@ -413,7 +414,7 @@ template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN, bool MIX> in
     }
     const long long ctas = (units + CT::NG - 1) / CT::NG;
     const int grid = (int)(ctas < ctas_fit ? ctas : ctas_fit);
-    fn<<<grid, CT::CT, sm, st>>>(a);
+    launch_pdl(fn, grid, CT::CT, sm, st, a);
     return 1;
 }
 
