@@ -37,7 +37,7 @@ DbgReport dbg_collect();                           // sums and clears the counte
 static __device__ hn::DbgRanges hn_dbg_ranges;
 static __device__ unsigned long long hn_dbg_bad[4];        // count, first address, first line
 namespace hn {
-__device__ __forceinline__ void dbg_check(const void *p, unsigned bytes, int line)
+static __device__ __noinline__ void dbg_check(const void *p, unsigned bytes, int line)      // (inlined, the checks take 20 minutes to compile)
 {
     if (!__isGlobal(p)) return;                            // generic pointers into shared memory are not this check's business
     const unsigned long long a = (unsigned long long)p;
