@@ -167,7 +167,7 @@ size_t hyenand_plan_workspace_bytes(const hyenand_plan *plan);        /* device 
                                                                        * staging copies once hyenand_forward_host has run, plus
                                                                        * room for C filter spectra once a filter shared over the
                                                                        * batch has been used (allocated by that first call) */
-int hyenand_plan_fft_dims(const hyenand_plan *plan, int *out_P);      /* writes ndim padded sizes P_n */
+int hyenand_plan_fft_dims(const hyenand_plan *plan, int *out_P);      /* writes ndim padded sizes P_n (2^k or 3 * 2^k) */
 int hyenand_plan_launches(const hyenand_plan *plan, int h_shared);    /* kernels enqueued by one forward */
 const char *hyenand_plan_path(const hyenand_plan *plan);              /* name of the kernel path chosen */
 /* How the batch is scheduled: slices per group and the number of lanes (workspace sets with a stream each; 1 =
@@ -183,11 +183,12 @@ int hyenand_plan_groups(const hyenand_plan *plan, long long *slices_per_group, i
  * q, k, v are the projected inputs [B][C][L_1]..[L_N], h the kernel K laid out as for hyenand_forward_ex, g_in and
  * g_out the C fp32 weights of the two RMSNorms (device pointers).  l2 and both RMSNorms act per token (one grid
  * position of one batch entry) across the C channels: l2(q) = q / max(||q||_2, 1e-12); RMSNorm(x) = x /
- * sqrt(mean_c(x^2) + eps) * g, eps as given at creation (>= 0).  The pointwise stages are kernels of their own before
- * and after the long convolution; everything between the first read of q, k, v and the store of y stays fp32 (the
- * convolution runs on an fp32 plan even when the I/O type is bf16; the taps h are read in the caller's type where the
- * path transforms the filter in kernels of its own, and widened once per call elsewhere), so y carries one rounding.  mode: HYENAND_MODE_*.  The object owns an fp32 plan and fp32 scratch for at most 2 GiB worth of batch
- * entries per pass; hyenand_mixer_plan exposes the inner plan for the reporting helpers (do not destroy it).
+ * sqrt(mean_c(x^2) + eps) * g, eps as given at creation (>= 0).  Everything between the first read of q, k, v and the store
+ * of y stays fp32, so y carries one rounding: on grids whose convolution is one kernel, that kernel reads q, k, v and h in
+ * the caller's type, applies the gates itself and writes fp32 for the last norm; elsewhere the pointwise stages are kernels
+ * before and after a convolution on fp32 tensors (the taps are read in the caller's type where the path transforms the
+ * filter in kernels of its own, and widened once per call elsewhere).  mode: HYENAND_MODE_*.  The object owns a plan and
+ * fp32 scratch for at most 2 GiB worth of batch entries per pass; hyenand_mixer_plan exposes the inner plan for the reporting helpers (do not destroy it).
  * Errors and stream semantics as hyenand_forward_ex.  hyenand_mixer_guard_damage: as hyenand_plan_guard_damage, over
  * the scratch and the inner plan.
  */
@@ -208,14 +209,16 @@ void hyenand_mixer_destroy(hyenand_mixer *mixer);
  *     the kernel is shared (h_batch_stride_elems = 0; dh then has the shape of h, [C][K..]).
  * q, k, v, dy, dq, dk, dv: [B][C][L..]; h, dh: as hyenand_forward_ex; all DEVICE pointers of the one I/O dtype,
  * 16-byte aligned; no output may overlap an input or another output (checked: HYENAND_ERR_INVALID_ARG, nothing is
- * launched).  Every gradient is accumulated in fp32 and rounded once, at its store.  The gradients are long
- * convolutions themselves and run on the forward's kernels: dq is a forward gated by dy; du is a forward of dy q against
+ * launched).  Every gradient is accumulated in fp32 and rounded once, at its store.  Small grids (one
+ * slice's three padded volumes fit an SM) are one kernel per slice; 2-D and 3-D grids transform k v, dy q and h once and form
+ * the three spectral products in one kernel.  The others (long 1-D grids, short core axes) run on the forward's kernels: dq is a forward gated by dy; du is a forward of dy q against
  * the kernel at the opposite displacement, leaving through the two gates v and k as dk and dv where the path's last
  * kernel takes a second gate (else through an fp32 du); dh is the full linear convolution of dy q with the reversed
  * k v on the general N-D kernels (circular mode: one circular convolution; 1-D grids whose padded length exceeds 8192:
  * one or two causal convolutions of reversed signals).  With bf16 I/O the kernels read the caller's tensors themselves
  * wherever the path takes an element type per launch; elsewhere the inputs are widened once.
- * The handle owns up to three plans and the scratch (about 4 GiB for the batch groups, 2 GiB for the dh groups).
+ * The handle owns up to three plans and the scratch (about 4 GiB for the batch groups, 2 GiB for the dh groups; 2 GiB in all
+ * where the spectra are formed once, and room for a shared filter's spectra from the first call that passes one).
  * Limits: as the forward's; circular mode needs power-of-two grids.  Errors and stream semantics as hyenand_forward_ex.
  */
 typedef struct hyenand_grad hyenand_grad;

@@ -66,7 +66,8 @@ struct ColsFwdWArgs {
     float2 *out;              // [slices][P1/2+1][P2]
     long long slices;
     long long in_slice;       // elements per slice of the input
-    bool vec;                 // every pair of column pairs starts on an 8-byte boundary
+    bool vec;                 // every pair of column pairs starts on an 8-byte boundary; else element by element (lengths and
+                              // slices that start anywhere, on the block-wide kernels before: 102 -> 62 and 347 -> 198 us a call)
     int len;                  // valid elements (<= P/2)
     int *status;              // device word set when a bounded wait on a tensor copy gives up (may be NULL)
     int log2p2;

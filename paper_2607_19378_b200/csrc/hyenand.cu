@@ -1611,6 +1611,9 @@ static Core3Args spec_core_args(const hyenand_grad *g, bool shared)
     return a;
 }
 
+// 2-D and 3-D grids whose core axis the tensor-copy core takes (64 points and up): training steps, forward included, on 96^3
+// 3483 -> 2583 us, 15x35x55 f32 600 -> 392, 29x51x70 118 -> 57 against the forward's kernels run twice and the full convolution
+// for dh.  Shorter core axes have no such core and stay there.
 // true: the grid is this path's (g->spec), or an error was recorded (!g->spec); false: another path takes it
 static bool spec_create(hyenand_grad *g)
 {

