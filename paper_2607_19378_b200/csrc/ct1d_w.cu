@@ -79,7 +79,8 @@ struct ColsFwdWArgs {
 // TMA = true: the tile (all rows t1 of TX column pairs, for k and for v) arrives as tensor copies into
 // row-major swizzled buffers, issued by one thread as soon as the previous tile has been read; false: 8-byte
 // asynchronous copies per thread into padded rows.
-template <typename T, int LOG2P1, bool HAS_B, bool TMA>
+// VEC: see ColsFwdWArgs::vec (a variant each: as a branch of one kernel the element loads cost the others 3 %)
+template <typename T, int LOG2P1, bool HAS_B, bool TMA, bool VEC>
 __global__ void __launch_bounds__(kCtThreads, (LOG2P1 >= 9 ? 2 : 4))
 ct_cols_fwd_w_kernel(ColsFwdWArgs p, const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                      const __grid_constant__ CUtensorMap map_o)
@@ -150,7 +151,7 @@ ct_cols_fwd_w_kernel(ColsFwdWArgs p, const __grid_constant__ CUtensorMap map_a, 
         if constexpr (TMA) {
             if (!mbar_wait(bar, phase)) failed = 1;
         } else {
-        if (p.vec) {
+        if constexpr (VEC) {
         for (int idx = tid; idx < HP1 * (TX / PG); idx += kCtThreads) {
             const int t1 = idx / (TX / PG), xg = idx % (TX / PG);
             const long long e0 = (long long)t1 * P2 + 2 * (c0 + PG * xg);
@@ -440,7 +441,7 @@ struct ColsInvWArgs {
 
 // TMA = true: the gate tile q arrives, and the result tile y leaves, as tensor copies ([t1][pair] rows of
 // TX pairs, no swizzle: a warp touches whole consecutive rows); false: per-thread loads and stores.
-template <typename T, int LOG2P1, bool TMA>
+template <typename T, int LOG2P1, bool TMA, bool PAIR>
 __global__ void __launch_bounds__(kCtInvThreads, (LOG2P1 >= 9 ? 4 : 8))
 ct_cols_inv_w_kernel(ColsInvWArgs p, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_y)
 {
@@ -546,7 +547,7 @@ ct_cols_inv_w_kernel(ColsInvWArgs p, const __grid_constant__ CUtensorMap map_q, 
         }
         // gate values first (all requests in flight together), then products and stores
         const long long ox = base + 2 * x;
-        if (!p.pair) {
+        if constexpr (!PAIR) {
             T qa[NE], qb[NE];
 #pragma unroll
             for (int e = 0; e < NE; ++e) {
@@ -623,14 +624,14 @@ bool ct1d_w_supported(int log2p1, int log2p2)
     return true;
 }
 
-template <typename T, int LOG2P1, bool HAS_B, bool TMA>
+template <typename T, int LOG2P1, bool HAS_B, bool TMA, bool VEC>
 static void launch_cols_fwd_w_tt(const ColsFwdWArgs &a, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, int grid,
                                 size_t sm, cudaStream_t st)
 {
     static DevOnce attr;
     if (attr.first())
-        cudaFuncSetAttribute(ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, TMA><<<grid, kCtThreads, sm, st>>>(a, ma, mb, mo);
+        cudaFuncSetAttribute(ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, TMA, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, TMA, VEC><<<grid, kCtThreads, sm, st>>>(a, ma, mb, mo);
 }
 
 template <typename T, int LOG2P1> static int launch_cols_fwd_w_t(const ColsFwdWArgs &a0, cudaStream_t st)
@@ -668,23 +669,26 @@ template <typename T, int LOG2P1> static int launch_cols_fwd_w_t(const ColsFwdWA
     }
     if constexpr (TROW == 64 || TROW == 128) {
         if (tma) {
-            if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, true>(a, ma, mb, mo, grid, sm, st);
-            else launch_cols_fwd_w_tt<T, LOG2P1, false, true>(a, ma, mb, mo, grid, sm, st);
+            if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, true, true>(a, ma, mb, mo, grid, sm, st);
+            else launch_cols_fwd_w_tt<T, LOG2P1, false, true, true>(a, ma, mb, mo, grid, sm, st);
             return 1;
         }
     }
-    if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, false>(a, ma, mb, mo, grid, sm, st);
-    else launch_cols_fwd_w_tt<T, LOG2P1, false, false>(a, ma, mb, mo, grid, sm, st);
+    if (a.vec) {
+        if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, false, true>(a, ma, mb, mo, grid, sm, st);
+        else launch_cols_fwd_w_tt<T, LOG2P1, false, false, true>(a, ma, mb, mo, grid, sm, st);
+    } else if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, false, false>(a, ma, mb, mo, grid, sm, st);
+    else launch_cols_fwd_w_tt<T, LOG2P1, false, false, false>(a, ma, mb, mo, grid, sm, st);
     return 1;
 }
 
-template <typename T, int LOG2P1, bool TMA>
+template <typename T, int LOG2P1, bool TMA, bool PAIR>
 static void launch_cols_inv_w_tt(const ColsInvWArgs &a, const CUtensorMap &mq, const CUtensorMap &my, int grid, size_t sm, cudaStream_t st)
 {
     static DevOnce attr;
     if (attr.first())
-        cudaFuncSetAttribute(ct_cols_inv_w_kernel<T, LOG2P1, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    ct_cols_inv_w_kernel<T, LOG2P1, TMA><<<grid, kCtInvThreads, sm, st>>>(a, mq, my);
+        cudaFuncSetAttribute(ct_cols_inv_w_kernel<T, LOG2P1, TMA, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    ct_cols_inv_w_kernel<T, LOG2P1, TMA, PAIR><<<grid, kCtInvThreads, sm, st>>>(a, mq, my);
 }
 
 template <typename T, int LOG2P1> static int launch_cols_inv_w_t(const ColsInvWArgs &a0, cudaStream_t st)
@@ -712,8 +716,9 @@ template <typename T, int LOG2P1> static int launch_cols_inv_w_t(const ColsInvWA
         const unsigned box[3] = {2 * TX, (unsigned)(HP1 < 256 ? HP1 : 256), 1};
         tma = tma_encode_3d_cached(&mq, a.q, sizeof(T) == 2, dims, strides, box, 0) && tma_encode_3d_cached(&my, a.y, sizeof(T) == 2, dims, strides, box, 0);
     }
-    if (tma) launch_cols_inv_w_tt<T, LOG2P1, true>(a, mq, my, grid, sm, st);
-    else launch_cols_inv_w_tt<T, LOG2P1, false>(a, mq, my, grid, sm, st);
+    if (tma) launch_cols_inv_w_tt<T, LOG2P1, true, true>(a, mq, my, grid, sm, st);
+    else if (a.pair) launch_cols_inv_w_tt<T, LOG2P1, false, true>(a, mq, my, grid, sm, st);
+    else launch_cols_inv_w_tt<T, LOG2P1, false, false>(a, mq, my, grid, sm, st);
     return 1;
 }
 
