@@ -71,3 +71,21 @@ def test_many_planes_of_64_points(C, path):
     assert hn.hyenand_plan_path(plan.handle) == path
     plan.close()
     check(w, q, k, v, h)
+
+
+@pytest.mark.parametrize("dims,B,C,dtype,causal", [((2000,), 4, 2048, "f32", True), ((31, 64), 3, 6000, "bf16", False)], ids=str)
+def test_shared_filter_over_ranges_inside_a_batch_entry(dims, B, C, dtype, causal):
+    """hyenand_forward_host works off a large batch in ranges of slices that start and end inside a batch entry: channels
+    without a slice in the range sit next to channels with one, in more units than the GPU has room for."""
+    from paper_2607_19378_b200 import hyenand as hn
+    w = W.Workload("ranges", dims, B, C, dtype, seed=108, causal=causal, h_shared=True)
+    q, k, v, h = (t.cpu() for t in W.make_inputs(w, device="cuda"))
+    plan = hn.Plan(dims, B, C, causal=causal, dtype=w.torch_dtype)
+    try:
+        y_dev = plan.forward(*(t.cuda() for t in (q, k, v, h)))
+        host = [t.contiguous().pin_memory() for t in (q, k, v, h)]
+        y = torch.full_like(q, float("nan")).pin_memory()
+        plan.forward_host(*host, y)
+    finally:
+        plan.close()
+    assert torch.equal(y, y_dev.cpu())
