@@ -24,21 +24,25 @@ Switches read_switches()
 }
 
 // ---- checked build: hooks of the translation units ----------------------------------------------------------
-static DbgHook g_dbg_hooks[32];
-static const char *g_dbg_files[32];
-static int g_dbg_n = 0;
-
-void dbg_register(DbgHook hook, const char *file)
+struct DbgUnit {
+    DbgHook hook;
+    const char *file;
+};
+static std::vector<DbgUnit> &dbg_list()                      // (a local static: units register before this file's statics exist)
 {
-    if (g_dbg_n < 32) { g_dbg_hooks[g_dbg_n] = hook; g_dbg_files[g_dbg_n] = file; ++g_dbg_n; }
+    static std::vector<DbgUnit> v;
+    return v;
 }
+
+void dbg_register(DbgHook hook, const char *file) { dbg_list().push_back({hook, file}); }
+int dbg_units() { return (int)dbg_list().size(); }
 
 static DbgRanges g_dbg_last;
 
 void dbg_set_ranges(const DbgRanges &r)
 {
     g_dbg_last = r;
-    for (int i = 0; i < g_dbg_n; ++i) g_dbg_hooks[i](&r, nullptr);
+    for (const DbgUnit &u : dbg_list()) u.hook(&r, nullptr);
 }
 
 void dbg_append_range(const void *ptr, size_t bytes)
@@ -53,10 +57,10 @@ void dbg_append_range(const void *ptr, size_t bytes)
 DbgReport dbg_collect()
 {
     DbgReport rep{0, 0, 0, nullptr};
-    for (int i = 0; i < g_dbg_n; ++i) {
+    for (const DbgUnit &u : dbg_list()) {
         unsigned long long c[4] = {0, 0, 0, 0};
-        g_dbg_hooks[i](nullptr, c);
-        if (c[0] && !rep.count) { rep.first_address = c[1]; rep.first_line = (int)c[2]; rep.file = g_dbg_files[i]; }
+        u.hook(nullptr, c);
+        if (c[0] && !rep.count) { rep.first_address = c[1]; rep.first_line = (int)c[2]; rep.file = u.file; }
         rep.count += c[0];
     }
     return rep;

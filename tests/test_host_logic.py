@@ -83,3 +83,15 @@ def test_cufft_composition_reference_matches_oracle():
         y = torch.from_numpy(yref).to(q.dtype)
         r = bench.cufft_composition(w, (q, k, v, h, y), reps=1)
         assert r["rel_l2_vs_ours_first_16M"] < (1e-5 if w.dtype == "f32" else 4e-3), (w.name, r)
+
+
+def test_every_kernel_source_registers_with_the_checked_build():
+    """The checked build compares accesses only in translation units whose list of ranges and counters it knows."""
+    from paper_2607_19378_b200 import build as bld
+
+    def includes_checks(name):
+        found = re.findall(r'^#include "(\w+\.cuh)"', open(os.path.join(bld.CSRC, name)).read(), flags=re.M)
+        return "common.cuh" in found or any(includes_checks(f) for f in found)
+
+    units = [s for s in bld._sources() if includes_checks(s)]
+    assert ctypes.CDLL(bld.build(debug=True))._ZN2hn9dbg_unitsEv() == len(units)
