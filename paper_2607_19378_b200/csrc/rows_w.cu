@@ -24,7 +24,12 @@ __device__ __forceinline__ void prefetch_rows_l2(const unsigned char *lo, const 
     if (a1 > a0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(a0), "r"((unsigned)(a1 - a0)) : "memory");
 }
 
-template <typename T, int LOG2P, int MODE>
+// LATE: the twiddles a lane keeps in registers are read after the wait for the preceding kernel instead of before it.  The
+// compiler sinks such reads to where they are used when registers run out, but not past the wait: at 1024 points (32 x 32, 62
+// registers of twiddles, 128 in all) reading them early costs spills in every row pair (fp32, bytes of spill loads per thread:
+// k v rows 200 -> 256, rows back 136 -> 184; a forward of 512 x 512 grids 2654 -> 2701 us, late 2656).  Grids of fewer CTAs than SMs
+// start while their predecessor runs and gain more from early reads: one 500 x 500 grid 38.0 us late, 33.7 early.
+template <typename T, int LOG2P, int MODE, bool LATE>
 __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
 {
     using F = WF<LOG2P, false>;
@@ -43,9 +48,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
     for (int t = tid; t < P; t += kRowThreads) { HN_G(p.gtw + t * (p.gtw_n / P), 8); twt[t] = p.gtw[t * (p.gtw_n / P)]; }
     __syncthreads();
     PlaneTw<LOG2P, false> tw;
+    if constexpr (LATE) pdl_join();
     tw.init(l, twt, twt + P, tid, kRowThreads);
     __syncthreads();
-    pdl_join();
+    if constexpr (!LATE) pdl_join();
     const unsigned char *ab = (const unsigned char *)p.a, *bb = (const unsigned char *)p.b;
     const unsigned char *ahi = ab + p.rows * (long long)p.len * sizeof(T);
     const unsigned char *bhi = bb + p.rows * (long long)p.len * sizeof(T);
@@ -145,10 +151,13 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
     }
 }
 
-// FULL (circular mode): all P outputs of a row are kept.
-template <typename T, int LOG2P, bool FULL>
+// OUT: which outputs of a row are kept.  ROW_CROP the first len <= P/2; ROW_FULL (circular mode) all of them; ROW_SHIFT (rows of
+// taps) positions (n - shift) mod P, n < len.
+enum { ROW_CROP = 0, ROW_FULL = 1, ROW_SHIFT = 2 };
+template <typename T, int LOG2P, int OUT, bool LATE>
 __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs p)
 {
+    constexpr bool FULL = OUT != ROW_CROP;
     using FI = WF<LOG2P, true>;
     constexpr int P = len_of(LOG2P), HP = P / 2, TPL = FI::TPL, G = kRowThreads / TPL, LS = plane_ls(P);
     constexpr int RS = HP + 2;                                   // slot of one staged half spectrum
@@ -161,9 +170,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
     for (int t = tid; t < P; t += kRowThreads) { HN_G(p.gtw + t * (p.gtw_n / P), 8); twt[t] = p.gtw[t * (p.gtw_n / P)]; }
     __syncthreads();
     PlaneTw<LOG2P, true> tw;
+    if constexpr (LATE) pdl_join();
     tw.init(l, twt, twt + P, tid, kRowThreads);
     __syncthreads();
-    pdl_join();
+    if constexpr (!LATE) pdl_join();
     const T *pq = (const T *)p.q;
     T *py = (T *)p.y;
     const long long pairs = (p.rows + 1) / 2;
@@ -199,7 +209,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
             const float sg = (r == RH && idx == HP) ? 1.f : -1.f;
             return make_float2(fmaf(-sg, B.y, A.x), fmaf(sg, A.y, B.x));
         });
-        auto at = [&](int n) { return line[FI::ph(FULL ? ring<P>(n + P - p.shift) : n)]; };
+        auto at = [&](int n) { return line[FI::ph(OUT == ROW_SHIFT ? ring<P>(n + P - p.shift) : n)]; };
         if (!FULL && p.len == HP && has1 && pq) {
             // full rows: all gate loads of the pair are in flight together (they were asked into L2 above)
             float qa[HP / TPL], qb[HP / TPL];
@@ -257,6 +267,10 @@ static int rows_sms()
     return n;
 }
 
+// length and grid size from which the kernels take their LATE variant
+template <int LOG2P> constexpr bool kLateRows = LOG2P == 10;
+static bool late_rows(int grid) { return grid >= rows_sms(); }
+
 bool rows_w_supported(int log2p) { return (log2p >= 6 && log2p <= 10) || (log2p >= kLen192 && log2p <= kLen768); }
 
 template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &a, cudaStream_t st)
@@ -267,21 +281,22 @@ template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &
     const long long want = ((a.rows + 1) / 2 + G - 1) / G;
     const int grid = (int)(want < 2ll * rows_sms() ? want : 2ll * rows_sms());
     if (grid <= 0) return 0;
-#define HN_LAUNCH(MODE)                                                                                  \
-    do {                                                                                                 \
-        static DevOnce attr;                                                                        \
-        if (attr.first()) {                                                                                     \
-            cudaFuncSetAttribute(rows_fwd_w_kernel<T, LOG2P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
-        }                                                                                                \
-        launch_pdl(rows_fwd_w_kernel<T, LOG2P, MODE>, grid, kRowThreads, sm, st, a);                     \
-    } while (0)
+    auto go = [&](auto mode, auto late) {
+        auto fn = rows_fwd_w_kernel<T, LOG2P, decltype(mode)::value, decltype(late)::value>;
+        static DevOnce attr;
+        if (attr.first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        launch_pdl(fn, grid, kRowThreads, sm, st, a);
+    };
+    auto launch = [&](auto mode) {
+        if constexpr (kLateRows<LOG2P>) { if (late_rows(grid)) return go(mode, std::true_type{}); }
+        go(mode, std::false_type{});
+    };
     if (a.full_in) {
-        if constexpr ((P & (P - 1)) == 0) HN_LAUNCH(3); else return -1;      // (periodic grids are powers of two)
+        if constexpr ((P & (P - 1)) == 0) launch(std::integral_constant<int, 3>{}); else return -1;      // (periodic grids are powers of two)
     }
-    else if (a.b) HN_LAUNCH(0);
-    else if (a.prune_in) HN_LAUNCH(2);
-    else HN_LAUNCH(1);
-#undef HN_LAUNCH
+    else if (a.b) launch(std::integral_constant<int, 0>{});
+    else if (a.prune_in) launch(std::integral_constant<int, 2>{});
+    else launch(std::integral_constant<int, 1>{});
     return 1;
 }
 
@@ -293,10 +308,20 @@ template <typename T, int LOG2P> static int launch_rows_inv_w_t(const RowsInvArg
     const long long want = ((a.rows + 1) / 2 + G - 1) / G;
     const int grid = (int)(want < 2ll * rows_sms() ? want : 2ll * rows_sms());
     if (grid <= 0) return 0;
-    static DevOnce attr[2];
-    void (*fn)(RowsInvArgs) = a.full_out ? rows_inv_w_kernel<T, LOG2P, true> : rows_inv_w_kernel<T, LOG2P, false>;
-    if (attr[a.full_out ? 1 : 0].first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    launch_pdl(fn, grid, kRowThreads, sm, st, a);
+    auto go = [&](auto out, auto late) {
+        auto fn = rows_inv_w_kernel<T, LOG2P, decltype(out)::value, decltype(late)::value>;
+        static DevOnce attr;
+        if (attr.first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        launch_pdl(fn, grid, kRowThreads, sm, st, a);
+    };
+    auto launch = [&](auto out) {
+        if constexpr (kLateRows<LOG2P>) { if (late_rows(grid)) return go(out, std::true_type{}); }
+        go(out, std::false_type{});
+    };
+    if (!a.full_out) launch(std::integral_constant<int, ROW_CROP>{});
+    else if constexpr (P % 3 == 0) launch(std::integral_constant<int, ROW_SHIFT>{});      // (periodic grids are powers of two)
+    else if (a.shift) launch(std::integral_constant<int, ROW_SHIFT>{});
+    else launch(std::integral_constant<int, ROW_FULL>{});
     return 1;
 }
 

@@ -1,0 +1,33 @@
+"""Register spills of kernels that run at their register limit, as ptxas reported them when the library was built (no GPU).
+The bounds are what the kernels need by themselves: twiddles held in registers across a wait, or a second copy of a row's first
+pass, showed as two to forty times as much and cost measured time."""
+import os
+import re
+
+import pytest
+
+
+def spill_loads(source):
+    """mangled kernel name -> bytes of spill loads, from the build's ptxas output"""
+    from paper_2607_19378_b200 import build as bld
+    bld.build()
+    log = os.path.join(bld.OBJ, source + ".ptxas.log")
+    if not os.path.exists(log):
+        pytest.skip("the objects were built elsewhere")
+    out, name = {}, None
+    for line in open(log):
+        m = re.search(r"Compiling entry function '(\S+)'", line)
+        name = m.group(1) if m else name
+        m = re.search(r"(\d+) bytes spill loads", line)
+        if m and name:
+            out[name] = int(m.group(1))
+    assert out
+    return out
+
+
+@pytest.mark.parametrize("kernel,limit", [("rows_fwd_w_kernelIfLi10ELi0ELb1E", 200), ("rows_fwd_w_kernelIfLi10ELi1ELb1E", 112),
+                                          ("rows_inv_w_kernelIfLi10ELi0ELb1E", 136), ("rows_inv_w_kernelIfLi10ELi1ELb1E", 144)])
+def test_rows_of_1024_points(kernel, limit):
+    """Grids that fill the GPU: no more than before the kernels waited for their predecessors (dependent launches)."""
+    found = [v for k, v in spill_loads("rows_w").items() if kernel in k]
+    assert len(found) == 1 and found[0] <= limit, found
