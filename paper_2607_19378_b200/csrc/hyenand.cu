@@ -349,6 +349,8 @@ static hyenand_plan *create_plan(int ndim, const int *dims, int B, int C, int mo
     // 64 -> 58; with one such axis of three 80x128x128 970 -> 922).  Planes whose axes both fit 192 points stay on chip at that
     // size (12 volumes of 96^3: 792 -> 512, the general passes at 192 points 818); planes with one such axis stay at
     // 256 x 256, because the general passes cost a third trip through memory (100x90x120: 558 either way).
+    // 768 against 1024 points at both ends of 257 .. 384 (us, 128 slices of N x N fp32, then 512 of 40 x N): N = 257 503 -> 381 and
+    // 240 -> 194, N = 383 614 -> 475 and 251 -> 206; as core axis alone (N x 40) 281 -> 268 and 333 -> 319.
     const bool len3_ok = allow_len3 && !circular && !p->slice && !p->sw.force_generic && !p->sw.generic_rows && !p->sw.generic_core &&
                          !p->sw.no_tma && tma_available();
     if (len3_ok && (p->path == PATH_ND_GENERIC || p->path == PATH_PLANES3D)) {

@@ -115,8 +115,9 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_fwd_w_kernel(RowsArgs p)
                 const int mm = ring<P>(cw + i * TPL + r * (P / F::template Pass<0>::R));
                 return make_float2(staged<T>(s, f0, mm), staged<T>(s + SLOT, f1, mm));
             });
-        } else if (p.len == HP && has1) {
-            // full rows: no bounds tests in the input functor
+        } else if (P % 3 != 0 && p.len == HP && has1) {
+            // full rows: no bounds tests in the input functor (3 * 2^k points have few full rows, and with two copies of the first
+            // pass 768 points spill 300 bytes per thread: 384x384 grids, 128 slices fp32, 470 -> 453 us with one, 257x257 393 -> 381)
             F::template run_to_line<PR, true>(l, m, tw, line, [&](int, int, int idx) {
                 float a = staged<T>(s, f0, idx), b = staged<T>(s + SLOT, f1, idx);
                 if (MODE == 0) {

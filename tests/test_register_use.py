@@ -31,3 +31,8 @@ def test_rows_of_1024_points(kernel, limit):
     """Grids that fill the GPU: no more than before the kernels waited for their predecessors (dependent launches)."""
     found = [v for k, v in spill_loads("rows_w").items() if kernel in k]
     assert len(found) == 1 and found[0] <= limit, found
+
+
+def test_rows_of_three_times_a_power_of_two():
+    rows = {k: v for k, v in spill_loads("rows_w").items() if re.search(r"Li2[234]E", k)}
+    assert len(rows) == 2 * 3 * 5 and max(rows.values()) <= 16, {k: v for k, v in rows.items() if v > 16}
