@@ -67,6 +67,13 @@ template <> struct MixVec<bf16, 4> {
     }
 };
 
+// a token's scale from sum_c q^2 and sum_c (q SiLU(k))^2: mean_c (l2(q) SiLU(k))^2 = s2 / (C ||q||^2)
+__device__ __forceinline__ float token_factor(float s1, float s2, int C, float eps)
+{
+    const float inv = 1.f / fmaxf(sqrtf(s1), kL2Floor);
+    return inv * rsqrtf(s2 * inv * inv / (float)C + eps);
+}
+
 // 32 * VEC tokens per CTA of NW warps; channels c = warp, warp + NW, ... in rounds of U.
 // GATES: the kernel also writes qz = Sigmoid(v) and the gated signal, kz = q scale g_in with vz = SiLU(k), or the product of
 // both as kz where vz is nullptr; q and k are read once more (from the caches) where a thread's channels need several rounds.
@@ -106,9 +113,7 @@ __global__ void __launch_bounds__(NW * 32) token_scale_kernel(const T *q, const 
 #pragma unroll
         for (int j = 0; j < NW; ++j) { a += red[0][j][t]; d += red[1][j][t]; }       // (red[0][0][t] is this thread's alone to replace)
         const long long tok = (long long)blockIdx.x * 32 * VEC + t;
-        // mean_c (l2(q) SiLU(k))^2 = d / (C ||q||^2)
-        const float inv = 1.f / fmaxf(sqrtf(a), kL2Floor);
-        const float sc = inv * rsqrtf(d * inv * inv / (float)C + eps);
+        const float sc = token_factor(a, d, C, eps);
         if constexpr (GATES) red[0][0][t] = sc;
         else if (tok < L) { HN_G(scale + b * L + tok, 4); scale[b * L + tok] = sc; }
     }
@@ -218,6 +223,111 @@ __global__ void __launch_bounds__(NW * 32) mixer_post_kernel(const float *o, con
     }
 }
 
+// Few channels and many tokens: a thread owns VEC tokens and walks their channels, four at a time and the rest one by one; no
+// shared memory, no barrier.  (A tile of four warps has less than a channel per warp and loop slot there and is gone before it has
+// paid for its start: operator on 16 x 512 x 512 tokens of 2 channels, fp32, 1066 us with tiles, here 881.)
+template <typename T, int VEC, bool GATES>
+__global__ void __launch_bounds__(kMixThreads) token_solo_kernel(const T *q, const T *k, const T *v, const float *g_in, float eps, int C, long long L,
+                                                                 float *scale, float *qz, float *kz, float *vz)
+{
+    constexpr int U = 4;
+    const long long i = ((long long)blockIdx.x * kMixThreads + threadIdx.x) * VEC, b = blockIdx.y, base = b * C * L + i;
+    if (i >= L) return;                                      // (VEC > 1 only where it divides L)
+    float s1[VEC] = {}, s2[VEC] = {}, sc[VEC];
+    auto sums = [&](int c, auto n) {
+        constexpr int N = decltype(n)::value;
+        float x[N][VEC], y[N][VEC];
+#pragma unroll
+        for (int u = 0; u < N; ++u) { MixVec<T, VEC>::ld(q + base + (c + u) * L, x[u]); MixVec<T, VEC>::ld(k + base + (c + u) * L, y[u]); }
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                const float qs = x[u][e] * (y[u][e] * mix_sigmoid(y[u][e]));
+                s1[e] = fmaf(x[u][e], x[u][e], s1[e]);
+                s2[e] = fmaf(qs, qs, s2[e]);
+            }
+    };
+    auto write = [&](int c, auto n) {
+        constexpr int N = decltype(n)::value;
+        float a[N][VEC], x[N][VEC], z[N][VEC];
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            MixVec<T, VEC>::ld(q + base + (c + u) * L, a[u]); MixVec<T, VEC>::ld(k + base + (c + u) * L, x[u]); MixVec<T, VEC>::ld(v + base + (c + u) * L, z[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            HN_G(g_in + c + u, 4);
+            const float g = __ldg(g_in + c + u);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) {
+                a[u][e] *= sc[e] * g;
+                x[u][e] *= mix_sigmoid(x[u][e]);
+                z[u][e] = mix_sigmoid(z[u][e]);
+                if (!vz) a[u][e] *= x[u][e];
+            }
+            MixVec<float, VEC>::st(kz + base + (c + u) * L, a[u]);
+            if (vz) MixVec<float, VEC>::st(vz + base + (c + u) * L, x[u]);
+            MixVec<float, VEC>::st(qz + base + (c + u) * L, z[u]);
+        }
+    };
+    const std::integral_constant<int, U> several{};
+    const std::integral_constant<int, 1> one{};
+    int c = 0;
+    for (; c + U <= C; c += U) sums(c, several);
+    for (; c < C; ++c) sums(c, one);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) sc[e] = token_factor(s1[e], s2[e], C, eps);
+    if constexpr (GATES) {
+        for (c = 0; c + U <= C; c += U) write(c, several);
+        for (; c < C; ++c) write(c, one);
+    } else {
+        MixVec<float, VEC>::st(scale + b * L + i, sc);
+    }
+}
+
+template <typename T, int VEC>
+__global__ void __launch_bounds__(kMixThreads) post_solo_kernel(const float *o, const float *g_out, float eps, int C, long long L, T *y)
+{
+    constexpr int U = 4;
+    const long long i = ((long long)blockIdx.x * kMixThreads + threadIdx.x) * VEC, base = (long long)blockIdx.y * C * L + i;
+    if (i >= L) return;
+    float s[VEC] = {};
+    auto sums = [&](int c, auto n) {
+        constexpr int N = decltype(n)::value;
+        float x[N][VEC];
+#pragma unroll
+        for (int u = 0; u < N; ++u) MixVec<float, VEC>::ld(o + base + (c + u) * L, x[u]);
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) s[e] = fmaf(x[u][e], x[u][e], s[e]);
+    };
+    auto write = [&](int c, auto n) {
+        constexpr int N = decltype(n)::value;
+        float x[N][VEC];
+#pragma unroll
+        for (int u = 0; u < N; ++u) MixVec<float, VEC>::ld(o + base + (c + u) * L, x[u]);
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            HN_G(g_out + c + u, 4);
+            const float g = __ldg(g_out + c + u);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) x[u][e] *= s[e] * g;
+            MixVec<T, VEC>::st(y + base + (c + u) * L, x[u]);
+        }
+    };
+    const std::integral_constant<int, U> several{};
+    const std::integral_constant<int, 1> one{};
+    int c = 0;
+    for (; c + U <= C; c += U) sums(c, several);
+    for (; c < C; ++c) sums(c, one);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) s[e] = rsqrtf(s[e] / (float)C + eps);
+    for (c = 0; c + U <= C; c += U) write(c, several);
+    for (; c < C; ++c) write(c, one);
+}
+
 template <typename T> __global__ void widen_kernel(const T *src, long long n, float *dst)
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -240,7 +350,11 @@ static int mix_grid(long long items)
 // Tiles of 32 tokens, or of 64 or 128 (two or four per lane) where rows divide that way and 1024 such tiles exist; the fewest
 // warps per tile that make 4096 warps in all, but no more than one per 8 channels or so.  Measured (bf16, scale + outer norm,
 // us): 512 tiles of 384 channels 29 with 8 warps, 34 with 16, 41 with 32; 42 tiles of 1170 channels 51, 31, 22.
-template <class F> static void mix_tiles(long long nb, long long L, int C, F go)
+// A thread per token (token_solo_kernel) takes few channels of many tokens, and rows that no vector of tokens divides, whose
+// tiles of 32 tokens start anywhere (operators, us, tiles -> solo: 8 x 511 x 511 tokens of 12 channels bf16 1292 -> 1106, of 48
+// 3995 -> 3490; fp32 of 24 2096 -> 1959, but 365 x 365 of 96 574 -> 604: few tokens or many fp32 channels stay with the tiles).
+constexpr int kSoloChannels = 16, kSoloOddF32 = 48;
+template <typename T, class F> static void mix_tiles(long long nb, long long L, int C, F go)
 {
     auto count = [&](int vec) { return nb * ((L + 32 * vec - 1) / (32 * vec)); };
     const int vec = L % 4 == 0 && count(4) >= 1024 ? 4 : L % 2 == 0 && count(2) >= 1024 ? 2 : 1;
@@ -248,10 +362,17 @@ template <class F> static void mix_tiles(long long nb, long long L, int C, F go)
     int nw = 4;
     while (nw < 32 && tiles * nw < 4096 && nw * 8 < C) nw *= 2;
     const dim3 grid((unsigned)((L + 32 * vec - 1) / (32 * vec)), (unsigned)nb);
-    if (vec == 4) return go(std::integral_constant<int, 4>{}, std::integral_constant<int, 4>{}, grid);      // (1024 tiles of 4 warps)
-    if (vec == 2) return go(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{}, grid);
+    const std::integral_constant<int, 0> solo{};
     const std::integral_constant<int, 1> one{};
-    if (nw == 4) go(one, std::integral_constant<int, 4>{}, grid);
+    const std::integral_constant<int, 2> two{};
+    const std::integral_constant<int, 4> four{};
+    if ((C <= kSoloChannels && tiles >= 1024) || (vec == 1 && tiles >= 4096 && (sizeof(T) == 2 || C <= kSoloOddF32))) {
+        const dim3 g((unsigned)((L + kMixThreads * vec - 1) / (kMixThreads * vec)), (unsigned)nb);
+        return vec == 4 ? go(four, solo, g) : vec == 2 ? go(two, solo, g) : go(one, solo, g);
+    }
+    if (vec == 4) return go(four, four, grid);               // (1024 tiles of 4 warps)
+    if (vec == 2) return go(two, four, grid);
+    if (nw == 4) go(one, four, grid);
     else if (nw == 8) go(one, std::integral_constant<int, 8>{}, grid);
     else if (nw == 16) go(one, std::integral_constant<int, 16>{}, grid);
     else go(one, std::integral_constant<int, 32>{}, grid);
@@ -261,8 +382,10 @@ template <typename T, bool GATES>
 static void token_scale_t(const T *q, const T *k, const T *v, const float *g_in, float eps, long long nb, int C, long long L, float *scale,
                           float *qz, float *kz, float *vz, cudaStream_t st)
 {
-    mix_tiles(nb, L, C, [&](auto vec, auto nw, dim3 grid) {
-        token_scale_kernel<T, decltype(vec)::value, decltype(nw)::value, GATES><<<grid, decltype(nw)::value * 32, 0, st>>>(q, k, v, g_in, eps, C, L, scale, qz, kz, vz);
+    mix_tiles<T>(nb, L, C, [&](auto vec, auto nw, dim3 grid) {
+        constexpr int VEC = decltype(vec)::value, NW = decltype(nw)::value;
+        if constexpr (NW == 0) token_solo_kernel<T, VEC, GATES><<<grid, kMixThreads, 0, st>>>(q, k, v, g_in, eps, C, L, scale, qz, kz, vz);
+        else token_scale_kernel<T, VEC, NW, GATES><<<grid, NW * 32, 0, st>>>(q, k, v, g_in, eps, C, L, scale, qz, kz, vz);
     });
 }
 
@@ -289,12 +412,16 @@ int launch_mixer_gates(const void *q, const void *k, const void *v, const float 
 
 template <typename T> static void mixer_post_t(const float *o, const float *g_out, float eps, long long nb, int C, long long L, T *y, cudaStream_t st)
 {
-    mix_tiles(nb, L, C, [&](auto vec, auto nw, dim3 grid) {
+    mix_tiles<T>(nb, L, C, [&](auto vec, auto nw, dim3 grid) {
         constexpr int VEC = decltype(vec)::value, NW = decltype(nw)::value;
-        const int per = (C + NW - 1) / NW;                   // channels per thread
-        if (per <= 4) mixer_post_kernel<T, VEC, NW, 4><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
-        else if (per <= 16) mixer_post_kernel<T, VEC, NW, 16><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
-        else mixer_post_kernel<T, VEC, NW, 0><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
+        if constexpr (NW == 0) {
+            post_solo_kernel<T, VEC><<<grid, kMixThreads, 0, st>>>(o, g_out, eps, C, L, y);
+        } else {
+            const int per = (C + NW - 1) / NW;               // channels per thread
+            if (per <= 4) mixer_post_kernel<T, VEC, NW, 4><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
+            else if (per <= 16) mixer_post_kernel<T, VEC, NW, 16><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
+            else mixer_post_kernel<T, VEC, NW, 0><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
+        }
     });
 }
 

@@ -104,3 +104,13 @@ def test_mixer_runs_in_several_passes_over_the_batch(dtype, shared, monkeypatch)
     monkeypatch.setenv("HYENAND_MIXER_MAX_BATCH", "2")
     w, (q, k, v, h) = W.random_problem((33, 20), B=5, C=4, dtype=dtype, h_shared=shared, seed=65)
     check_mixer(w, q, k, v, h, seed=65)
+
+
+# (many tokens of few channels, four, two and one per thread; one-kernel grids and the multi-kernel paths; rows that no vector of
+# tokens divides with more channels)
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("dims,B,C", [((256, 512), 1, 1), ((256, 512), 1, 5), ((362, 363), 1, 3), ((363, 363), 1, 2), ((363, 363), 1, 17),
+                                      ((15, 14), 700, 2), ((31, 33), 130, 1), ((16, 16), 513, 16)], ids=str)
+def test_mixer_many_tokens_of_few_channels(dims, B, C, dtype):
+    w, (q, k, v, h) = W.random_problem(dims, B=B, C=C, dtype=dtype, seed=66, h_shared=B > 1)
+    check_mixer(w, q, k, v, h, seed=66)
