@@ -231,11 +231,18 @@ struct RowsInvArgs {
 // idle SMs (calls of one small kernel 10.2 -> 8.5 us, of several 36.9 -> 34.4 and 28.4 -> 25.7).  Larger grids do not: blocks
 // that come in while others leave settle where there happens to be room, not evenly (with the early start everywhere a 1-D
 // grid of many slices takes 161 us instead of 149, a training step on 96^3 1848 instead of 1749).
+// Tensor memory is the one resource a CTA takes after its start: it is allocated between the wait and the trigger.  Allocated
+// before the wait, it could be what the preceding kernel's CTA on the same SM still waits for; triggered before, the following
+// kernel could take it first.  Either pair would wait for each other without end.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger()
+{
+    if (gridDim.x < 148) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
 __device__ __forceinline__ void pdl_join()
 {
     pdl_wait();
-    if (gridDim.x < 148) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    pdl_trigger();
 }
 
 template <typename... P, typename... A>

@@ -253,25 +253,26 @@ __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) hplane_kernel(PlaneArg
     static_assert(QP % C::NG == 0 || C::NG % QP == 0, "whole warps take part in the column loop");
     const int warp = tid >> 5;
     unsigned *tslot = reinterpret_cast<unsigned *>(smem + C::TMP + P);
-    if (warp == 0) tmem_alloc((unsigned)__cvta_generic_to_shared(tslot), TCOLS);
     load_plane_twiddles<LOG2P>(tw, twh, p.gtw, p.gtw_n, tid);
-    tmem_fence_before_sync();
     __syncthreads();
-    tmem_fence_after_sync();
-    const unsigned tbase = *tslot;
-    const unsigned tpark = tmem_addr(tbase, warp, (warp >> 2) * ROUNDS * NPT);
     PlaneTw<LOG2P, false> twp;
     twp.init(l, tw, twh + HP, tid, C::NT);
     PassTw<LOG2P - 1, false> twr;                            // half-length rows
     twr.base = twh + HP + P;
     PassTw<LOG2P - 1, false>::build(twh + HP + P, p.gtw, p.gtw_n, tid, C::NT);
+    pdl_wait();
+    if (warp == 0) tmem_alloc((unsigned)__cvta_generic_to_shared(tslot), TCOLS);       // (after the wait: see pdl_join)
+    tmem_fence_before_sync();
     __syncthreads();
+    tmem_fence_after_sync();
+    pdl_trigger();
+    const unsigned tbase = *tslot;
+    const unsigned tpark = tmem_addr(tbase, warp, (warp >> 2) * ROUNDS * NPT);
     const unsigned char *hb = (const unsigned char *)p.a;
     const int Lx = p.lx, Ly = p.ly, Kx = 2 * Lx - 1, Ky = 2 * Ly - 1;
     constexpr int R0 = PH0::R;
     const int J0 = HP + 1 - Lx;                              // window position of tap 0
     const int RU = (J0 * (int)sizeof(T) + 15) & ~15;         // bytes kept free before the first copied chunk
-    pdl_join();
     for (long long pl = blockIdx.x; pl < p.planes; pl += gridDim.x) {
         const long long ib = pl * (long long)Ky * Kx;
         float2 *dst = p.out + pl * (long long)C::XH * P;
@@ -673,22 +674,23 @@ __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) hplane_inv_kernel(Plan
     static_assert(QP % C::NG == 0 || C::NG % QP == 0, "whole warps take part in the column loop");
     const int warp = tid >> 5;
     unsigned *tslot = reinterpret_cast<unsigned *>(smem + C::TMP + P);
-    if (warp == 0) tmem_alloc((unsigned)__cvta_generic_to_shared(tslot), TCOLS);
     load_plane_twiddles<LOG2P>(tw, twh, p.gtw, p.gtw_n, tid);
-    tmem_fence_before_sync();
     __syncthreads();
-    tmem_fence_after_sync();
-    const unsigned tbase = *tslot;
-    const unsigned tpark = tmem_addr(tbase, warp, (warp >> 2) * ROUNDS * NPT);
     PlaneTw<LOG2P, true> twp;
     twp.init(l, tw, twh + HP, tid, C::NT);
     PassTw<LOG2P - 1, true> twr;                             // half-length rows
     twr.base = twh + HP + P;
     PassTw<LOG2P - 1, true>::build(twh + HP + P, p.gtw, p.gtw_n, tid, C::NT);
+    pdl_wait();
+    if (warp == 0) tmem_alloc((unsigned)__cvta_generic_to_shared(tslot), TCOLS);       // (after the wait: see pdl_join)
+    tmem_fence_before_sync();
     __syncthreads();
+    tmem_fence_after_sync();
+    pdl_trigger();
+    const unsigned tbase = *tslot;
+    const unsigned tpark = tmem_addr(tbase, warp, (warp >> 2) * ROUNDS * NPT);
     T *py = (T *)p.y;
     const int Lx = p.lx, Ly = p.ly, Kx = 2 * Lx - 1, Ky = 2 * Ly - 1, J0 = HP + 1 - Lx;
-    pdl_join();
     for (long long pl = blockIdx.x; pl < p.planes; pl += gridDim.x) {
         const float2 *src = p.in + pl * (long long)C::XH * P;
         T *out = py + pl * (long long)Ky * Kx;

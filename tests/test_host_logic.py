@@ -95,3 +95,20 @@ def test_every_kernel_source_registers_with_the_checked_build():
 
     units = [s for s in bld._sources() if includes_checks(s)]
     assert ctypes.CDLL(bld.build(debug=True))._ZN2hn9dbg_unitsEv() == len(units)
+
+
+def test_tensor_memory_is_taken_between_wait_and_trigger():
+    """Kernels started while their predecessor drains: tensor memory held during the wait, or taken after the successor may
+    start, could be what the other kernel's CTA on the same SM waits for."""
+    from paper_2607_19378_b200 import build as bld
+    kernels = 0
+    for name in bld._sources():
+        text = open(os.path.join(bld.CSRC, name)).read()
+        if "launch_pdl(" not in text:
+            continue
+        for body in re.split(r"\n__global__ ", text)[1:]:
+            if "tmem_alloc(" not in body:
+                continue
+            kernels += 1
+            assert 0 <= body.find("pdl_wait()") < body.find("tmem_alloc(") < body.find("pdl_trigger()") and "pdl_join()" not in body.split("\n}\n")[0]
+    assert kernels == 2
