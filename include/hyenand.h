@@ -218,7 +218,9 @@ void hyenand_mixer_destroy(hyenand_mixer *mixer);
  * one or two causal convolutions of reversed signals).  With bf16 I/O the kernels read the caller's tensors themselves
  * wherever the path takes an element type per launch; elsewhere the inputs are widened once.
  * The handle owns up to three plans and the scratch (about 4 GiB for the batch groups, 2 GiB for the dh groups; 2 GiB in all
- * where the spectra are formed once, and room for a shared filter's spectra from the first call that passes one).
+ * where the spectra are formed once).  The first call that passes a shared filter (h_batch_stride_elems = 0) allocates the room
+ * only such filters need (their fp32 tap gradients, their spectra where those are formed once): it may synchronise the device and
+ * may return HYENAND_ERR_ALLOC; inside a stream capture it does the same and captures nothing of it.
  * Limits: as the forward's; circular mode needs power-of-two grids.  Errors and stream semantics as hyenand_forward_ex.
  */
 typedef struct hyenand_grad hyenand_grad;

@@ -177,6 +177,7 @@ struct GuardedAllocs {
 };
 // cudaMalloc of bytes + two bands; *ptr is the first usable byte (256-byte aligned).  cudaSuccess or the error.
 cudaError_t guarded_alloc(GuardedAllocs *g, void **ptr, size_t bytes);
+cudaError_t guarded_alloc_in_call(GuardedAllocs *g, void **ptr, size_t bytes);      // the same inside a call that enqueues, captured or not
 void guarded_free_all(GuardedAllocs *g);
 long long guard_damage(const GuardedAllocs *g);       // damaged guard bytes, -1 if a copy failed
 

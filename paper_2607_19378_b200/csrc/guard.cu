@@ -69,7 +69,7 @@ DbgReport dbg_collect()
 void nvtx_push(const char *name) { nvtxRangePushA(name); }
 void nvtx_pop() { nvtxRangePop(); }
 
-cudaError_t guarded_alloc(GuardedAllocs *g, void **ptr, size_t bytes)
+static cudaError_t alloc_bands(GuardedAllocs *g, void **ptr, size_t bytes, cudaStream_t st)
 {
     *ptr = nullptr;
     if (g->n >= kMaxGuarded) return cudaErrorMemoryAllocation;
@@ -78,14 +78,35 @@ cudaError_t guarded_alloc(GuardedAllocs *g, void **ptr, size_t bytes)
     unsigned char *base = nullptr;
     cudaError_t e = cudaMalloc((void **)&base, body + 2 * kGuardBytes);
     if (e != cudaSuccess) return e;
-    e = cudaMemset(base, kGuardByte, kGuardBytes);
-    if (e == cudaSuccess) e = cudaMemset(base + kGuardBytes + bytes, kGuardByte, body - bytes + kGuardBytes);
+    auto fill = [&](unsigned char *p, size_t n) { return st ? cudaMemsetAsync(p, kGuardByte, n, st) : cudaMemset(p, kGuardByte, n); };
+    e = fill(base, kGuardBytes);
+    if (e == cudaSuccess) e = fill(base + kGuardBytes + bytes, body - bytes + kGuardBytes);
+    if (e == cudaSuccess && st) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { cudaFree(base); return e; }
     g->recs[g->n].base = base;
     g->recs[g->n].bytes = bytes;
     ++g->n;
     *ptr = base + kGuardBytes;
     return cudaSuccess;
+}
+
+cudaError_t guarded_alloc(GuardedAllocs *g, void **ptr, size_t bytes) { return alloc_bands(g, ptr, bytes, nullptr); }
+
+cudaError_t guarded_alloc_in_call(GuardedAllocs *g, void **ptr, size_t bytes)
+{
+    // An allocation is no stream operation, so it may happen while the caller's stream is captured as long as this thread's
+    // capture mode allows it; the bands are filled on a stream that belongs to no capture.
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    cudaStream_t st = nullptr;
+    e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) {
+        e = alloc_bands(g, ptr, bytes, st);
+        cudaStreamDestroy(st);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
 }
 
 void guarded_free_all(GuardedAllocs *g)

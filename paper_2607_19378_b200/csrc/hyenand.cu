@@ -201,10 +201,10 @@ static int len3_id(int need)
 
 static size_t elsize(int dtype) { return dtype == HYENAND_F32 ? 4 : 2; }
 
-static int dev_alloc(hyenand_plan *p, void **ptr, size_t bytes)
+static int dev_alloc(hyenand_plan *p, void **ptr, size_t bytes, bool in_call = false)
 {
     if (bytes == 0) bytes = 16;
-    cudaError_t e = guarded_alloc(&p->allocs, ptr, bytes);
+    cudaError_t e = in_call ? guarded_alloc_in_call(&p->allocs, ptr, bytes) : guarded_alloc(&p->allocs, ptr, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         *ptr = nullptr;
@@ -467,8 +467,8 @@ static int ensure_shared_filter_room(hyenand_plan *p)
     hyenand_plan::Lane &ln = p->lane[0];
     if (ln.wh_slices >= p->C) return 0;
     float2 *a = nullptr, *b = nullptr;
-    int e = dev_alloc(p, (void **)&a, sizeof(float2) * p->wh_a_slice * p->C);
-    if (!e && p->wh_b_slice) e = dev_alloc(p, (void **)&b, sizeof(float2) * p->wh_b_slice * p->C);
+    int e = dev_alloc(p, (void **)&a, sizeof(float2) * p->wh_a_slice * p->C, true);
+    if (!e && p->wh_b_slice) e = dev_alloc(p, (void **)&b, sizeof(float2) * p->wh_b_slice * p->C, true);
     if (e) return e;
     ln.wh_a = a; ln.wh_b = b; ln.wh_slices = p->C;       // (the smaller buffers stay with the plan until it is destroyed)
 #ifdef HYENAND_DEBUG
@@ -1656,23 +1656,25 @@ static bool spec_create(hyenand_grad *g)
     return true;
 }
 
-// room a filter shared over the batch needs, taken the first time one is used
-static int spec_shared_room(hyenand_grad *g)
+// Room a filter shared over the batch needs, taken the first time one is used (a handle for per-sample filters never pays for
+// it): fp32 taps of a pass on the one-kernel path, spectra as well where they are formed once.
+static int shared_room(hyenand_grad *g)
 {
-    if (g->maps_sh.valid) return HYENAND_OK;
-    const SpecGeo s = spec_geo(g->main);
+    if (!g->spec && !g->slice) return HYENAND_OK;
     cudaError_t e = cudaSuccess;
     auto get = [&](void **ptr, long long bytes) {
-        if (e == cudaSuccess && !*ptr) e = guarded_alloc(&g->allocs, ptr, (size_t)bytes);
+        if (e == cudaSuccess && !*ptr) e = guarded_alloc_in_call(&g->allocs, ptr, (size_t)bytes);
     };
-    get((void **)&g->fd, s.h * g->ns * 8); get((void **)&g->fhc, s.h * g->C * 8);
+    const SpecGeo s = g->spec ? spec_geo(g->main) : SpecGeo{};
+    if (g->spec) { get((void **)&g->fd, s.h * g->ns * 8); get((void **)&g->fhc, s.h * g->C * 8); }
     get((void **)&g->dhs, 4ll * g->nb * g->C * g->kvol);
     if (g->nb < g->B) get((void **)&g->dh32, 4ll * g->C * g->kvol);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(HYENAND_ERR_ALLOC, "scratch of the backward pass: %s", cudaGetErrorString(e));
     }
-    if (!core3_tma_make(&g->maps_sh, spec_core_args(g, true), g->ns, g->C)) return fail(HYENAND_ERR_CUDA, "tensor maps of the backward pass");
+    if (g->spec && !g->maps_sh.valid && !core3_tma_make(&g->maps_sh, spec_core_args(g, true), g->ns, g->C))
+        return fail(HYENAND_ERR_CUDA, "tensor maps of the backward pass");
     return HYENAND_OK;
 }
 
@@ -1810,22 +1812,14 @@ extern "C" hyenand_grad *hyenand_backward_create(int ndim, const int *dims, int 
                    !getenv("HYENAND_BACKWARD_RING_SLICES") && slice_geo(&g->sg, g->L, mode == HYENAND_MODE_CAUSAL, mode == HYENAND_MODE_CIRCULAR);
     }
     if (g->slice) {
-        // a plan for the twiddle table and the device, no workspace; the taps' gradients of a pass in fp32 (within 2 GiB) for
-        // a kernel shared over the batch
+        // a plan for the twiddle table and the device, no workspace; batch entries per pass of a kernel shared over the batch: the
+        // taps' gradients of a pass in fp32 within 2 GiB
         long long nb = (2ll << 30) / (4ll * C * g->kvol);
         if (const char *e = getenv("HYENAND_BACKWARD_MAX_BATCH")) { const long long v = atoll(e); if (v > 0 && v < nb) nb = v; }   // development aid
         g->nb = (int)(nb < 1 ? 1 : nb > B ? B : nb);
         g->main = create_plan(ndim, dims, 1, 1, mode, dtype, true, false);
         if (!g->main) { delete g; return nullptr; }
         g->adj = g->main;
-        cudaError_t ce = guarded_alloc(&g->allocs, (void **)&g->dhs, (size_t)g->nb * C * g->kvol * sizeof(float));
-        if (ce == cudaSuccess && g->nb < B) ce = guarded_alloc(&g->allocs, (void **)&g->dh32, (size_t)C * g->kvol * sizeof(float));
-        if (ce != cudaSuccess) {
-            cudaGetLastError();
-            fail(HYENAND_ERR_ALLOC, "scratch of the backward pass: %s", cudaGetErrorString(ce));
-            hyenand_backward_destroy(g);
-            return nullptr;
-        }
         return g;
     }
     if (spec_create(g)) {
@@ -1987,7 +1981,7 @@ extern "C" int hyenand_backward(hyenand_grad *g, const void *q, const void *k, c
                     return fail(HYENAND_ERR_INVALID_ARG, "output %d overlaps pointer %d", o, i);
             }
     }
-    if (g->spec && shared && (e = spec_shared_room(g))) return e;
+    if (shared && (e = shared_room(g))) return e;
     {
         DbgScope d;
         const size_t nbytes = (size_t)g->B * g->C * g->vol * elsize(g->dtype);
