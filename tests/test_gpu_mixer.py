@@ -114,3 +114,17 @@ def test_mixer_runs_in_several_passes_over_the_batch(dtype, shared, monkeypatch)
 def test_mixer_many_tokens_of_few_channels(dims, B, C, dtype):
     w, (q, k, v, h) = W.random_problem(dims, B=B, C=C, dtype=dtype, seed=66, h_shared=B > 1)
     check_mixer(w, q, k, v, h, seed=66)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("dims,B,C", [((40, 50), 2, 3), ((20, 30), 2, 3), ((20, 30), 2, 80), ((500,), 2, 4), ((40, 90), 2, 3), ((256, 512), 1, 2)],
+                         ids=str)
+def test_mixer_saturated_gates(dims, B, C, dtype):
+    """k and v far out where sigmoids saturate: exp(-x) overflows or is lost beside 1, in the gates of every path."""
+    w, (q, k, v, h) = W.random_problem(dims, B=B, C=C, dtype=dtype, seed=67)
+    g = torch.Generator().manual_seed(67)
+
+    def far(t):
+        mag = 80.0 + 40.0 * torch.rand(t.shape, generator=g)
+        return torch.where(torch.rand(t.shape, generator=g) < 0.2, t.float(), torch.sign(t.float()) * mag).to(t.dtype)
+    check_mixer(w, q, far(k), far(v), h, seed=67)
