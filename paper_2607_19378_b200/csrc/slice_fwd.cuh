@@ -292,13 +292,6 @@ __global__ void __launch_bounds__(SliceCta<SliceFft<L0, L1, L2>>::CT, SliceCta<S
         const long long u = u0 + grp;
         const bool live = u < units;
         const long long chan = shared ? u % p.C : 0, b0 = shared ? c_first + u / p.C * p.nb : 0;
-        if (!CT::WARP && shared) {
-            // A range that starts or ends inside a batch entry leaves units without a slice.  They are passed over whole
-            // (the same for the CTA): with the filter transformed and every entry skipped, no barrier would separate the
-            // last pass over bh from the next unit's first one.
-            const long long sf = b0 * p.C + chan, sl = sf < p.s0 ? sf + p.C : sf;      // first entry, first one in range
-            if (sl >= p.s1 || sl >= sf + (long long)p.nb * p.C) continue;
-        }
         {
             const long long hs = (shared ? chan : p.s0 + u) * g.kvol;
             auto taps = [&](const auto *h) {
@@ -415,8 +408,7 @@ template <typename T, int L0, int L1, int L2, bool FULL, bool EVEN, bool MIX> in
         const long long be = (a.s1 - 1) / a.C - a.s0 / a.C + 1;                  // batch entries touched
         long long best = -1;
         for (long long nb = 1; nb <= be && nb <= 64; ++nb) {
-            const long long un = (be + nb - 1) / nb * a.C, full = un < n ? un : n;     // (units without a slice cost nothing)
-            const long long cost = ((full + slots - 1) / slots) * (1 + 2 * nb);
+            const long long un = (be + nb - 1) / nb * a.C, cost = ((un + slots - 1) / slots) * (1 + 2 * nb);
             if (best < 0 || cost < best) { best = cost; a.nb = (int)nb; units = un; }
         }
     }
