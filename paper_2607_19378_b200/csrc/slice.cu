@@ -55,12 +55,38 @@ int launch_slice_bwd(const SliceBwdArgs &a, int dtype, cudaStream_t st)
     return dtype == 0 ? launch_slice_bwd_1d_f32(a, st) : launch_slice_bwd_1d_bf16(a, st);
 }
 
-int launch_slice(const SliceArgs &a, int dtype, cudaStream_t st)
+static int launch_range(const SliceArgs &a, int dtype, cudaStream_t st)
 {
     const bool f = dtype == 0, m = a.token_scale != nullptr;
     if (a.g.l0 > 0) return m ? (f ? launch_slice_mix_3d_f32(a, st) : launch_slice_mix_3d_bf16(a, st)) : (f ? launch_slice_3d_f32(a, st) : launch_slice_3d_bf16(a, st));
     if (a.g.l1 > 0) return m ? (f ? launch_slice_mix_2d_f32(a, st) : launch_slice_mix_2d_bf16(a, st)) : (f ? launch_slice_2d_f32(a, st) : launch_slice_2d_bf16(a, st));
     return m ? (f ? launch_slice_mix_1d_f32(a, st) : launch_slice_mix_1d_bf16(a, st)) : (f ? launch_slice_1d_f32(a, st) : launch_slice_1d_bf16(a, st));
+}
+
+// The kernel's units of a shared filter are channels by groups of whole batch entries.  A range that starts or ends inside an
+// entry (hyenand_forward_host above 64 MB) would leave it units without a slice, whose filter it transforms with no barrier
+// before the next unit writes the same buffer.  The partial entries run as slices with a filter each, the channel's own (tested
+// in the kernel instead, a batch of short sequences takes 147.6 us for 146.8).
+int launch_slice(const SliceArgs &a, int dtype, cudaStream_t st)
+{
+    if (a.C <= 0) return launch_range(a, dtype, st);
+    const long long C = a.C, first = (a.s0 + C - 1) / C * C, last = a.s1 / C * C;          // whole entries: [first, last)
+    int launches = 0;
+    auto run = [&](long long s0, long long s1, bool shared) {
+        if (launches < 0 || s0 >= s1) return;
+        SliceArgs r = a;
+        r.s0 = s0; r.s1 = s1;
+        if (!shared) {                                       // slice s of entry s0 / C takes filter s - s0 / C * C
+            r.C = 0;
+            r.h = (const char *)a.h - s0 / C * C * a.g.kvol * (a.h_bf16 ? 2 : 4);
+        }
+        const int n = launch_range(r, dtype, st);
+        launches = n < 0 ? n : launches + n;
+    };
+    run(a.s0, first < a.s1 ? first : a.s1, false);
+    run(first, last, true);
+    if (last >= first) run(last, a.s1, false);
+    return launches;
 }
 
 }  // namespace hn
