@@ -12,7 +12,7 @@
  * on the displacement i - j only (Definition A.2, Theorem A.5), q the outer
  * gate.  The sum is evaluated through FFTs on the zero-padded grid (Section
  * 3.2.1 "non-circular convolutions", Appendix B.1 Eq. 11-13): pad each axis to
- * P_n >= 2 L_n - 1 (a power of two), transform k*v and h, multiply the
+ * P_n >= 2 L_n - 1 points, transform k*v and h, multiply the
  * spectra, transform back, crop, apply q.  All arithmetic is fp32; bf16 is an
  * I/O format only (one round-to-nearest-even at the final store).
  *

@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) plane_inv_kernel(Plane
 // odd bins along x are brought back one after the other, each half through a store [bin][row pair y, y + P/2] of lines
 // G = A + iB that the column transforms leave behind (as in plane_inv_kernel), and a row of each half is one half-length
 // inverse: with E and O those of the even and of the odd bins, f[x] = E[x] + W_P^-x O[x], f[x + P/2] = E[x] - W_P^-x O[x].
-// E waits in tensor memory until O is there.  Bound by instruction issue and the phases' barriers like hplane_kernel (12 volumes
+// E waits in tensor memory until O is there.  Bound by the latency of its column loads and of the phases (issue slots 38 %; 12 volumes
 // of 96^3, bf16 taps: 329 us at 256 points, 285 at 192; its bytes alone need 78).
 template <typename T, int LOG2P>
 __global__ void __launch_bounds__(PlaneCfg<LOG2P>::NT, 1) hplane_inv_kernel(PlaneArgs p)

@@ -9,6 +9,7 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SUITES = ["tests/test_gpu_parity.py", "tests/test_gpu_mixer.py", "tests/test_gpu_synthesis.py", "tests/test_gpu_backward.py",
+          "tests/test_gpu_slice.py", "tests/test_gpu_core_lengths.py", "tests/test_gpu_backward_spectral.py", "tests/test_gpu_len3.py",
           "tests/test_zz_no_alloc.py"]
 # the largest long 1-D cases run for minutes under the checker and add no kernel the smaller ones leave out
 SKIP = "not large_padded_sizes and not above_2_pow_20 and not tensor_maps_follow"
