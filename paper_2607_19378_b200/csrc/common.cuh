@@ -186,6 +186,7 @@ constexpr int kMaxLineLog2 = 13;          // longest line transformed in shared 
 __host__ __device__ constexpr int len_of(int id) { return id < 16 ? 1 << id : 3 << (id - 16); }
 constexpr int kLen192 = 22, kLen384 = 23, kLen768 = 24;
 constexpr int kThreads = 256;             // threads per CTA of the generic kernels
+constexpr int kSms = 148;                 // SMs of the GPU this is built for; rules that use it pick the faster way there, either is right anywhere
 
 // ---- generic N-D path (nd_kernels.cu) ---------------------------------------------
 //
@@ -238,7 +239,7 @@ struct RowsInvArgs {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger()
 {
-    if (gridDim.x < 148) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (gridDim.x < kSms) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 __device__ __forceinline__ void pdl_join()
 {
@@ -247,10 +248,10 @@ __device__ __forceinline__ void pdl_join()
 }
 
 template <typename... P, typename... A>
-static inline void launch_pdl(void (*fn)(P...), dim3 grid, unsigned threads, size_t sm, cudaStream_t st, const A &...args)
+static inline void launch_pdl(void (*fn)(P...), unsigned grid, unsigned threads, size_t sm, cudaStream_t st, const A &...args)
 {
     cudaLaunchConfig_t c{};
-    c.gridDim = grid; c.blockDim = dim3(threads); c.dynamicSmemBytes = sm; c.stream = st;
+    c.gridDim = dim3(grid); c.blockDim = dim3(threads); c.dynamicSmemBytes = sm; c.stream = st;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;

@@ -119,7 +119,7 @@ extern "C" long long hyenand_debug_selftest(void)
 
 enum Path { PATH_ND_GENERIC = 0, PATH_CT1D = 1, PATH_PLANES3D = 2, PATH_FUSED2D = 3 };
 constexpr int kMaxLanes = 4;
-constexpr long long kFusedPlanesMax = 148;               // slices of 64-point planes that find an SM each
+constexpr long long kFusedPlanesMax = kSms;              // slices of 64-point planes that find an SM each
 
 struct hyenand_plan {
     int ndim, B, C, causal, dtype;
