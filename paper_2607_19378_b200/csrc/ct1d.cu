@@ -424,10 +424,10 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
     const TwoLevel twp{c->twp_coarse, c->twp_fine, c->lo};
     if (ct1d_uses_w(c)) {
         const bool staged_ok = c->causal != 0;
-        if (shared && c->r0 == 0 && !c->keep_filter && ct1d_w_filter(c, h, c->C, staged_ok, st, launches, prof, filter_pass)) return -1;
+        if (shared && c->r0 == 0 && !c->keep_filter && ct1d_w_filter(c, h, c->C, true, staged_ok, st, launches, prof, filter_pass)) return -1;
         for (long long s0 = c->r0; s0 < c->r1; s0 += c->slices_per_chunk) {
             const long long n = c->r1 - s0 < c->slices_per_chunk ? c->r1 - s0 : c->slices_per_chunk;
-            if (!shared && ct1d_w_filter(c, (const char *)h + (size_t)s0 * c->K * eh, n, staged_ok, st, launches, prof, filter_pass))
+            if (!shared && ct1d_w_filter(c, (const char *)h + (size_t)s0 * c->K * eh, n, false, staged_ok, st, launches, prof, filter_pass))
                 return -1;
             if (ct1d_w_body(c, (const char *)q + (size_t)s0 * c->L * eo, (const char *)k + (size_t)s0 * c->L * ei,
                             v ? (const char *)v + (size_t)s0 * c->L * ei : nullptr, n, shared, s0, (char *)y + (size_t)s0 * c->L * eo,
@@ -472,14 +472,14 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
 }
 
 // Both kernel families take either element type in every stage; the warp-engine kernels serve every length they have an
-// instance for (padded 2^14 .. 2^20), longer ones and the development switch take the block-wide kernels.
-bool ct1d_uses_w(const Ct1dPlan *c) { return !c->sw.force_generic && ct1d_w_supported(c->log2p1, c->log2p2); }
+// instance for (padded 2^14 .. 2^20), longer ones and the development switches take the block-wide kernels.
+bool ct1d_uses_w(const Ct1dPlan *c) { return !c->sw.force_generic && !c->sw.no_tma && ct1d_w_supported(c->log2p1, c->log2p2); }
 
 int ct1d_launches(const Ct1dPlan *c, bool shared)
 {
     const long long S = (long long)c->B * c->C;
     const long long chunks = (S + c->slices_per_chunk - 1) / c->slices_per_chunk;
-    if (ct1d_uses_w(c)) return (int)(shared ? 2 + 3 * chunks : 5 * chunks);
+    if (ct1d_uses_w(c)) return (int)(shared ? 1 + 3 * chunks : 5 * chunks);
     return (int)(shared ? 1 + 3 * chunks : 4 * chunks);
 }
 

@@ -24,7 +24,7 @@ struct Ct1dPlan {
     int dt_in, dt_out, dt_h;  // element types of k and v, of the gate q and the result y, of the taps h for the next forward
                               // (all equal to dtype unless the caller of ct1d_forward sets them: every stage takes its
                               // element type per launch)
-    int keep_filter;          // 1: the spectrum of the shared filter is still in wh from this plan's previous forward
+    int keep_filter;          // 1: the column transforms of the shared filter are still in wh from this plan's previous forward
                               // (same taps): the next forward does not transform it again
 };
 
@@ -38,7 +38,7 @@ bool ct1d_uses_w(const Ct1dPlan *c);
 
 // warp-engine kernels (ct1d_w.cu)
 bool ct1d_w_supported(int log2p1, int log2p2);
-int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
+int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool shared, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
                   int (*fallback)(Ct1dPlan *, const char *, long long, cudaStream_t, int *, Prof *));
 int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, long long s0,
                 void *y, cudaStream_t st, int *launches, Prof *prof);

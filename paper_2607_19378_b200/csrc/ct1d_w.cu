@@ -6,10 +6,11 @@
 //                one warp-group per column pair: transform along t1 (upper half of the
 //                padded input is zero), separate the two real columns, multiply by the
 //                inter-pass twiddle, coalesced store of [f1][t2].
-//   hspec_w      filter only: transform each kept row along t2 in place and fold in 1/P,
-//                so the filter spectrum is computed once per filter, not once per use.
+//   hspec_w      per-sample filters only: transform each kept row along t2 in place and fold in 1/P.
 //   core_w       one warp-group per row: transform along t2, multiply by the filter
-//                spectrum (Eq. 12), inverse transform chained in registers, undo twiddle.
+//                spectrum (Eq. 12), inverse transform chained in registers, undo twiddle.  The
+//                rows of a filter shared over the batch are transformed here, once per group of
+//                batch entries.
 //   cols_inv_w   rebuild the mirrored half, inverse along f1 keeping t < P/2, crop, gate
 //                with q, coalesced store.
 #include <type_traits>
@@ -19,25 +20,12 @@
 #include "tma_util.cuh"
 #include "ct1d.cuh"
 #include "plane_util.cuh"
+#include "tmem_util.cuh"
 
 namespace hn {
 
-constexpr int kCtThreads = 256;
-// column pairs per tile: at least 16 (64-byte rows of bf16), one or two lines per group of lanes
-// line stride of the column kernels: 16-byte aligned and = 2 (mod 16) complex numbers, so that the
-// 16-byte accesses of neighbouring lines (tile loads and stores run across lines) hit different banks
-__host__ __device__ constexpr int ct_ls(int n) { return (n + 15) / 16 * 16 + 2; }
-__host__ __device__ constexpr int ct_tx(int tpl) { return kCtThreads / tpl > 8 ? kCtThreads / tpl : 8; }
-// result tile of the forward column kernel as tensor copies: F1 rows in one box, or in two boxes whose
-// starts stay on 1024-byte boundaries (rows per box a multiple of 8)
-__host__ __device__ constexpr int ct_out_boxes(int f1) { return (f1 + 7) / 8 * 8 > 256 ? 2 : 1; }
-__host__ __device__ constexpr int ct_out_box_rows(int f1)
-{
-    return ct_out_boxes(f1) == 1 ? (f1 + 7) / 8 * 8 : ((f1 + 1) / 2 + 7) / 8 * 8;
-}
-// the inverse column kernel runs as CTAs of 4 warps: more, smaller tiles in flight per SM
-constexpr int kCtInvThreads = 128;
-__host__ __device__ constexpr int ct_inv_tx(int tpl) { return kCtInvThreads / tpl > 8 ? kCtInvThreads / tpl : 8; }
+// column kernels: CTAs of four warps, several per SM (they synchronise at barriers; more, smaller CTAs keep the schedulers busy)
+constexpr int kCtThreads = 128;
 
 template <int BYTES> __device__ __forceinline__ void cp_async_n(void *smem_dst, const void *gmem_src)
 {
@@ -66,158 +54,192 @@ struct ColsFwdWArgs {
     float2 *out;              // [slices][P1/2+1][P2]
     long long slices;
     long long in_slice;       // elements per slice of the input
-    bool vec;                 // every pair of column pairs starts on an 8-byte boundary; else element by element (lengths and
-                              // slices that start anywhere, on the block-wide kernels before: 102 -> 62 and 347 -> 198 us a call)
     int len;                  // valid elements (<= P/2)
     int *status;              // device word set when a bounded wait on a tensor copy gives up (may be NULL)
     int log2p2;
     const float2 *tw1;        // P1-point table
     TwoLevelW twp;
-    bool no_tma;              // development switch: per-thread copies even where tensor copies apply
 };
 
-// TMA = true: the tile (all rows t1 of TX column pairs, for k and for v) arrives as tensor copies into
-// row-major swizzled buffers, issued by one thread as soon as the previous tile has been read; false: 8-byte
-// asynchronous copies per thread into padded rows.
-// VEC: see ColsFwdWArgs::vec (a variant each: as a branch of one kernel the element loads cost the others 3 %)
-template <typename T, int LOG2P1, bool HAS_B, bool TMA, bool VEC>
-__global__ void __launch_bounds__(kCtThreads, (LOG2P1 >= 9 ? 2 : 4))
+// Tile geometry of the column kernels, one line (column pair) per group of lanes.  Spectra travel as NH halves of rows of ROWB bytes
+// (the swizzle span); the rows below P1/2 in boxes, the last one by an untiled copy of its own (a multiple of 8 rows in, where the
+// swizzle is the identity), so that the tile is no larger than its rows.
+template <typename T, int LOG2P1> struct CtGeo {
+    using F = WF<LOG2P1, false>;
+    using FI = WF<LOG2P1, true>;
+    static constexpr int P1 = 1 << LOG2P1, HP1 = P1 / 2, F1 = HP1 + 1, TPL = F::TPL;
+    static constexpr int TX = kCtThreads / TPL, TH = TX < 8 ? TX : 8, NH = TX / TH;           // pairs per tile and per half
+    static constexpr unsigned ROWB = TH * 16, HALFB_ALIGN = NH > 1 ? 1024 : 256,
+                              HALFB = (F1 * ROWB + HALFB_ALIGN - 1) / HALFB_ALIGN * HALFB_ALIGN;
+    static constexpr int BOXR = HP1 < 256 ? HP1 : 256, NB = HP1 / BOXR;                       // boxes of a tile
+    // tiles of the real tensors: HP1 rows of TX pairs
+    static constexpr unsigned QROW = TX * 2 * sizeof(T), QBYTES = HP1 * QROW;
+    static constexpr int QSW = QROW == 32 || QROW == 64 || QROW == 128 ? (int)QROW : 0;
+    static constexpr unsigned QMASK = QSW == 128 ? 0x70u : QSW == 64 ? 0x30u : QSW == 32 ? 0x10u : 0u;
+    static constexpr size_t QAL = QSW ? QSW * 8 : 128;       // the swizzle's period
+    // (groups of 16 lanes and more fill a half warp: any stride does)
+    static constexpr int PHN = F::ph(P1 - 1) > FI::ph(P1 - 1) ? F::ph(P1 - 1) : FI::ph(P1 - 1);
+    static constexpr int LS = TPL >= 16 ? (PHN + 2) / 2 * 2 : plane_ls(P1);
+    static constexpr size_t LINEB = sizeof(float2) * TX * LS;
+    static __host__ __device__ constexpr int fit(size_t total, int cap)
+    {
+        const int n = (int)(227 * 1024 / (total + 1024));
+        return n < cap ? n : cap;
+    }
+    // address of pair x of row t1 in a tile of a real tensor
+    static __device__ __forceinline__ unsigned at(int t1, int x)
+    {
+        const unsigned o = (unsigned)t1 * QROW + (unsigned)x * 2 * sizeof(T);
+        return o ^ ((o >> 3) & QMASK);
+    }
+};
+template <typename T, int LOG2P1, bool HAS_B> struct CtFwdGeo : CtGeo<T, LOG2P1> {
+    using B = CtGeo<T, LOG2P1>;
+    using Tw = PassTw<LOG2P1, false>;
+    // result tile over the lines, then the input tiles
+    static constexpr size_t OUTB = (size_t)B::NH * B::HALFB, LINES = 0, RAW = ((OUTB > B::LINEB ? OUTB : B::LINEB) + 1023) / 1024 * 1024,
+                            TW = RAW + (HAS_B ? 2 : 1) * (size_t)B::QBYTES, BARS = TW + sizeof(float2) * Tw::TOTAL, TOTAL = BARS + 8;
+    // by shared memory, and at 128 registers a thread for the long transforms, 80 for the short ones
+    static constexpr int PER_SM = B::fit(TOTAL, LOG2P1 >= 9 ? 4 : 6);
+};
+
+// A CTA of four warps works on a tile of TX column pairs; the next tile's inputs travel while this one is transformed.  IN: how
+// they come: 0 tensor copies, 1 asynchronous copies of 8 bytes, 2 element by element (slices that start
+// off 8-byte boundaries, eight loads in flight).
+// The separated bins leave as tensor copies from a swizzled tile over the lines.  262144 bf16 values, 512 rows: 383 us with two CTAs
+// of eight warps per SM, 348 with four of four (4.6 TB/s); the filter's rows 184, 168.  Bound by the shared-memory pipe (59 %) and
+// the barriers around the result tile.
+template <typename T, int LOG2P1, bool HAS_B, int IN>
+__global__ void __launch_bounds__(kCtThreads, (CtFwdGeo<T, LOG2P1, HAS_B>::PER_SM))
 ct_cols_fwd_w_kernel(ColsFwdWArgs p, const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                      const __grid_constant__ CUtensorMap map_o)
 {
-    using F = WF<LOG2P1, false>;
-    constexpr int P1 = 1 << LOG2P1, HP1 = P1 / 2, F1 = HP1 + 1, TPL = F::TPL;
-    constexpr int TX = ct_tx(TPL);                         // column pairs per tile
-    constexpr int NGRP = kCtThreads / TPL;                 // groups of lanes per CTA
-    constexpr int LS = ct_ls(phys_max(P1) + 2);                // room for the skewed line and for 2*(P1/2+1) bins
-    constexpr int PAIRB = 2 * (int)sizeof(T);              // bytes of one column pair of one row
-    extern __shared__ float2 smem[];
-    float2 *lines = smem;
-    float2 *twt = lines + TX * LS;
-    // staged inputs [tensor][row t1][pair x], fetched 8 bytes at a time; a row is padded by 8 bytes,
-    // which sends the lanes of a group (they differ in t1) to different banks
-    constexpr int PG = 8 / PAIRB;                          // column pairs per 8-byte copy
-    constexpr int RS = TX * PAIRB + 8;                     // bytes per staged row
-    unsigned char *raw = reinterpret_cast<unsigned char *>(twt + P1);
-    // tensor copies: rows of TX*PAIRB bytes (64 or 128: the swizzle span), 1024-byte aligned tile buffers
-    constexpr unsigned TROW = TX * PAIRB;
-    constexpr int TBOXR = HP1 < 256 ? HP1 : 256, TNB = HP1 / TBOXR;
-    constexpr unsigned TBYTES = HP1 * TROW;
-    static_assert(!TMA || TROW == 64 || TROW == 128, "tile rows match a swizzle span");
-    if constexpr (TMA) raw += (1024u - (smem_u32(raw) & 1023u)) & 1023u;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(raw + 2 * TBYTES);
-    // Result tile as tensor copies too (one line per group): the separated bins are written row-major
-    // [f1][pair] into a swizzled staging area that reuses the lines, as two halves of 8 pairs (128-byte rows);
-    // boxes of 136 rows keep every box start on a 1024-byte boundary.
-    constexpr bool TSTORE = TMA && TX == 16 && NGRP == 16;
-    constexpr int ONB = ct_out_boxes(F1), OBOXR = ct_out_box_rows(F1), OHALF = ONB * OBOXR * 128;   // boxes, rows per box, bytes per half
-    static_assert(!TSTORE || (F1 <= ONB * OBOXR && 2 * OHALF + 1024 <= TX * LS * 8), "result staging fits the lines");
-    unsigned char *to0 = reinterpret_cast<unsigned char *>(lines);
-    if constexpr (TSTORE) to0 += (1024u - (smem_u32(to0) & 1023u)) & 1023u;
-    const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL;
+    using G = CtFwdGeo<T, LOG2P1, HAS_B>;
+    using F = typename G::F;
+    constexpr int P1 = G::P1, HP1 = G::HP1, F1 = G::F1, TPL = G::TPL, TX = G::TX;
+    constexpr int NF = (F1 + TPL - 1) / TPL;               // bins of a lane
+    using P0 = typename F::template Pass<0>;
+    static_assert(F::NP == 2, "two passes");
+    extern __shared__ __align__(1024) unsigned char smem_dyn[];
+    if (smem_u32(smem_dyn) & 1023u) {                      // (aligned as declared: room to align it here would cost a CTA per SM)
+        if (threadIdx.x == 0 && p.status) atomicExch(p.status, 7);
+        return;
+    }
+    unsigned char *to = smem_dyn + G::LINES, *raw = smem_dyn + G::RAW;
+    float2 *twt = reinterpret_cast<float2 *>(smem_dyn + G::TW);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem_dyn + G::BARS);
+    const int tid = threadIdx.x, l = tid % TPL, x = tid / TPL;
     const unsigned m = F::group_mask(tid);
+    float2 *line = reinterpret_cast<float2 *>(to) + x * G::LS;
     PassTw<LOG2P1, false>::build(twt, p.tw1, P1, tid, kCtThreads);
     const PassTw<LOG2P1, false> tw{twt};
     const int P2 = 1 << p.log2p2;
     const int tpc = (P2 / 2) / TX;                         // tiles per slice (P2/2 is a multiple of TX)
     const long long tiles = p.slices * tpc;
-    const unsigned char *ab = (const unsigned char *)p.a, *bb = (const unsigned char *)p.b;
-    auto issue = [&](long long t) {                        // one thread
+    auto ask = [&](long long t) {                          // inputs of tile t: one thread, or all of them
         const long long s = t / tpc;
-        const int x = 2 * (int)(t % tpc) * TX;             // first column of the tile
-        mbar_expect_tx(bar, (HAS_B ? 2 : 1) * TBYTES);
+        const int c0 = (int)(t % tpc) * TX;
+        if constexpr (IN == 0) {
+            if (tid) return;
+            mbar_expect_tx(bar, (HAS_B ? 2 : 1) * G::QBYTES);
 #pragma unroll
-        for (int b = 0; b < TNB; ++b) {
-            tma_load_3d(raw + b * TBOXR * TROW, &map_a, bar, x, b * TBOXR, (int)s);
-            if (HAS_B) tma_load_3d(raw + TBYTES + b * TBOXR * TROW, &map_b, bar, x, b * TBOXR, (int)s);
+            for (int b = 0; b < G::NB; ++b) {
+                tma_load_3d(raw + b * G::BOXR * G::QROW, &map_a, bar, 2 * c0, b * G::BOXR, (int)s);
+                if (HAS_B) tma_load_3d(raw + G::QBYTES + b * G::BOXR * G::QROW, &map_b, bar, 2 * c0, b * G::BOXR, (int)s);
+            }
+        } else {
+            const T *ta = (const T *)p.a + s * p.in_slice, *tb = (const T *)p.b + s * p.in_slice;
+            if constexpr (IN == 1) {
+                constexpr int PG = 8 / (2 * sizeof(T));    // column pairs per copy
+                static_assert(HP1 * (TX / PG) % kCtThreads == 0, "whole rounds");
+#pragma unroll 4
+                for (int idx = tid; idx < HP1 * (TX / PG); idx += kCtThreads) {
+                    const int t1 = idx / (TX / PG), xg = idx % (TX / PG) * PG;
+                    const long long e0 = (long long)t1 * P2 + 2 * (c0 + xg);
+                    unsigned char *d = raw + G::at(t1, xg);
+                    if (e0 + 2 * PG <= p.len) {
+                        cp_async_n<8>(d, ta + e0);
+                        if (HAS_B) cp_async_n<8>(d + G::QBYTES, tb + e0);
+                    } else {
+                        for (int e = 0; e < 2 * PG; ++e) {
+                            const bool ok = e0 + e < p.len;
+                            if (ok) HN_G(ta + e0 + e, sizeof(T));
+                            if (ok && HAS_B) HN_G(tb + e0 + e, sizeof(T));
+                            reinterpret_cast<T *>(d)[e] = ok ? ta[e0 + e] : T(0.f);
+                            if (HAS_B) reinterpret_cast<T *>(d + G::QBYTES)[e] = ok ? tb[e0 + e] : T(0.f);
+                        }
+                    }
+                }
+            } else {
+                // neighbouring elements by neighbouring threads
+                constexpr int EPR = 2 * TX, U = 8;         // elements per row of the tile
+                static_assert(HP1 * EPR % (U * kCtThreads) == 0, "whole rounds");
+                for (int i0 = tid; i0 < HP1 * EPR; i0 += U * kCtThreads) {
+                    T va[U], vb[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int i = i0 + u * kCtThreads;
+                        const long long e = (long long)(i / EPR) * P2 + 2 * c0 + i % EPR;
+                        const bool ok = e < p.len;
+                        if (ok) HN_G(ta + e, sizeof(T));
+                        if (ok && HAS_B) HN_G(tb + e, sizeof(T));
+                        va[u] = ok ? __ldg(ta + e) : T(0.f);
+                        if (HAS_B) vb[u] = ok ? __ldg(tb + e) : T(0.f);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int i = i0 + u * kCtThreads;
+                        unsigned char *d = raw + G::at(i / EPR, i % EPR / 2) + (i & 1) * sizeof(T);
+                        *reinterpret_cast<T *>(d) = va[u];
+                        if (HAS_B) *reinterpret_cast<T *>(d + G::QBYTES) = vb[u];
+                    }
+                }
+            }
         }
     };
-    if constexpr (TMA) {
+    if constexpr (IN == 0) {
         if (tid == 0) {
             mbar_init(bar, 1);
             fence_mbar_init();
         }
-        __syncthreads();
-        if (tid == 0 && (long long)blockIdx.x < tiles) issue(blockIdx.x);
     }
+    __syncthreads();
+    long long t = blockIdx.x;
+    if (t < tiles) ask(t);
     unsigned phase = 0;
     int failed = 0;
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x, phase ^= 1u) {
-        const long long s = t / tpc;
+    for (; t < tiles; t += gridDim.x, phase ^= 1u) {
+        const long long tn = t + gridDim.x, s = t / tpc;
         const int c0 = (int)(t % tpc) * TX;
-        const long long base = s * p.in_slice;
-        if constexpr (TSTORE) { if (tid == 0) tma_wait_read0(); }   // the previous result tile has left the lines
-        __syncthreads();                                   // previous tile done with raw and lines
-        if constexpr (TMA) {
+        if constexpr (IN == 0) {
             if (!mbar_wait(bar, phase)) failed = 1;
         } else {
-        if constexpr (VEC) {
-        for (int idx = tid; idx < HP1 * (TX / PG); idx += kCtThreads) {
-            const int t1 = idx / (TX / PG), xg = idx % (TX / PG);
-            const long long e0 = (long long)t1 * P2 + 2 * (c0 + PG * xg);
-            unsigned char *d = raw + (size_t)t1 * RS + 8 * xg;
-            if (e0 + 2 * PG <= p.len) {
-                cp_async_n<8>(d, ab + (base + e0) * sizeof(T));
-                if (HAS_B) cp_async_n<8>(d + (size_t)HP1 * RS, bb + (base + e0) * sizeof(T));
-            } else {
-                for (int e = 0; e < 2 * PG; ++e) {
-                    const bool ok = e0 + e < p.len;
-                    if (ok) HN_G(reinterpret_cast<const T *>(ab) + base + e0 + e, sizeof(T));
-                    if (ok && HAS_B) HN_G(reinterpret_cast<const T *>(bb) + base + e0 + e, sizeof(T));
-                    reinterpret_cast<T *>(d)[e] = ok ? reinterpret_cast<const T *>(ab)[base + e0 + e] : T(0.f);
-                    if (HAS_B)
-                        reinterpret_cast<T *>(d + (size_t)HP1 * RS)[e] = ok ? reinterpret_cast<const T *>(bb)[base + e0 + e] : T(0.f);
-                }
-            }
+            cp_async_wait_all();
+            __syncthreads();
         }
-        } else {
-            // slices of any length: neighbouring elements by neighbouring threads, eight loads of each tensor in flight
-            constexpr int EPR = 2 * TX, U = 8;                 // elements per row of the tile
-            static_assert(HP1 * EPR % (U * kCtThreads) == 0, "whole rounds");
-            const T *ta = reinterpret_cast<const T *>(ab) + base, *tb = reinterpret_cast<const T *>(bb) + base;
-            for (int i0 = tid; i0 < HP1 * EPR; i0 += U * kCtThreads) {
-                T va[U], vb[U];
+        float2 keep[P0::IPL][P0::R];
+        F::template pass<0, PRUNE_IN>(l, tw,
+            [&](int, int, int idx) {
+                const unsigned char *d = raw + G::at(idx, x);
+                float a0 = staged<T>(d, 0, 0), a1 = staged<T>(d, 0, 1);
+                if (HAS_B) {
+                    a0 *= staged<T>(d + G::QBYTES, 0, 0);
+                    a1 *= staged<T>(d + G::QBYTES, 0, 1);
+                }
+                return make_float2(a0, a1);
+            },
+            [&](int i, int r, int, float2 v) { keep[i][r] = v; });
+        if (tid == 0) tma_wait_read0();                    // the previous result tile has left the lines
+        if (__syncthreads_or(failed)) break;               // and the input tile has been read
+        if (tn < tiles) ask(tn);
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int i = i0 + u * kCtThreads;
-                    const long long e = (long long)(i / EPR) * P2 + 2 * c0 + i % EPR;
-                    const bool ok = e < p.len;
-                    if (ok) HN_G(ta + e, sizeof(T));
-                    if (ok && HAS_B) HN_G(tb + e, sizeof(T));
-                    va[u] = ok ? __ldg(ta + e) : T(0.f);
-                    if (HAS_B) vb[u] = ok ? __ldg(tb + e) : T(0.f);
-                }
+        for (int i = 0; i < P0::IPL; ++i)
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int i = i0 + u * kCtThreads;
-                    unsigned char *d = raw + (size_t)(i / EPR) * RS + (i % EPR) * sizeof(T);
-                    *reinterpret_cast<T *>(d) = va[u];
-                    if (HAS_B) *reinterpret_cast<T *>(d + (size_t)HP1 * RS) = vb[u];
-                }
-            }
-        }
-        cp_async_wait_all();
-        __syncthreads();
-        }
-        float2 A0[(F1 + TPL - 1) / TPL], A1[(F1 + TPL - 1) / TPL];
-        for (int x = gid; x < TX; x += NGRP) {
-        float2 *line = lines + x * LS;
-        // TMA: the 16-byte chunk of pair x in row idx is XORed with a function of idx that the engine's strides
-        // (multiples of 8 rows) leave alone, so it depends on the lane only
-        constexpr unsigned RSTR = TMA ? TROW : (unsigned)RS;
-        const unsigned sw = TROW == 128 ? ((unsigned)l & 7u) : (((unsigned)l >> 1) & 3u);
-        const unsigned xo = TMA ? ((((unsigned)x * PAIRB >> 4) ^ sw) << 4) + (((unsigned)x * PAIRB) & 15u) : (unsigned)x * PAIRB;
-        const unsigned char *ra = raw + xo;
-        const unsigned char *rb = ra + (TMA ? (size_t)TBYTES : (size_t)HP1 * RS);
-        F::template run_to_line<PRUNE_IN>(l, m, tw, line, [&](int, int, int idx) {
-            float a0 = staged<T>(ra + (size_t)idx * RSTR, 0, 0), a1 = staged<T>(ra + (size_t)idx * RSTR, 0, 1);
-            if (HAS_B) {
-                a0 *= staged<T>(rb + (size_t)idx * RSTR, 0, 0);
-                a1 *= staged<T>(rb + (size_t)idx * RSTR, 0, 1);
-            }
-            return make_float2(a0, a1);
-        });
-        // separate the two real columns, apply W_P^(t2*f1), park both bins in the line
+            for (int r = 0; r < P0::R; ++r) line[F::ph((l + i * TPL) * P0::R + r)] = keep[i][r];
+        __syncwarp(m);
+        F::template mid<1, 2>(l, m, tw, line);             // (the last pass, line to line)
+        // separate the two real columns, apply W_P^(t2*f1)
+        float2 A0[NF], A1[NF];
         const unsigned t2 = 2u * (unsigned)(c0 + x);
         {
             // W_P^(t2*f1) with f1 = l + i*TPL is the product of a per-lane factor W_P^(t2*l) (one
@@ -228,7 +250,7 @@ ct_cols_fwd_w_kernel(ColsFwdWArgs p, const __grid_constant__ CUtensorMap map_a, 
             const float2 st0 = twp_w(p.twp, t2 * (unsigned)TPL), st1 = twp_w(p.twp, (t2 + 1u) * (unsigned)TPL);
             float2 w0 = cl0, w1 = cl1;
 #pragma unroll
-            for (int i = 0; i < (F1 + TPL - 1) / TPL; ++i) {
+            for (int i = 0; i < NF; ++i) {
                 const int f1 = l + i * TPL;
                 if (i > 0) {
                     if (i % 4 == 0) {
@@ -245,59 +267,39 @@ ct_cols_fwd_w_kernel(ColsFwdWArgs p, const __grid_constant__ CUtensorMap map_a, 
                     A1[i] = cmul(make_float2(0.5f * (z1.y + z2.y), 0.5f * (z2.x - z1.x)), w1);
                 }
             }
-            __syncwarp(m);
-            if constexpr (!TSTORE) {
+        }
+        __syncthreads();                                   // every line has been read
+        {
+            unsigned char *th = to + (x / G::TH) * G::HALFB;
+            const unsigned xi = (unsigned)(x % G::TH);
 #pragma unroll
-                for (int i = 0; i < (F1 + TPL - 1) / TPL; ++i) {
-                    const int f1 = l + i * TPL;
-                    if (f1 < F1) *reinterpret_cast<float4 *>(line + 2 * f1) = make_float4(A0[i].x, A0[i].y, A1[i].x, A1[i].y);
-                }
-            }
-        }
-        }
-        if constexpr (TMA) {
-            if (__syncthreads_or(failed)) break;           // the tile buffers are free again (and every line has been read)
-            if (tid == 0 && t + gridDim.x < tiles) issue(t + gridDim.x);
-        } else {
-            __syncthreads();
-        }
-        if constexpr (TSTORE) {
-            // group gid holds pair x = gid: rows f1 = l + i*TPL, 16 bytes each, chunk index XORed with (f1 & 7)
-            unsigned char *th = to0 + (gid >> 3) * OHALF;
-#pragma unroll
-            for (int i = 0; i < (F1 + TPL - 1) / TPL; ++i) {
+            for (int i = 0; i < NF; ++i) {
                 const int f1 = l + i * TPL;
-                if (f1 < F1)
-                    *reinterpret_cast<float4 *>(th + f1 * 128 + (((gid & 7) ^ (f1 & 7)) << 4)) = make_float4(A0[i].x, A0[i].y, A1[i].x, A1[i].y);
+                const unsigned sw = G::ROWB == 128 ? ((unsigned)f1 & 7u) : (((unsigned)f1 >> 1) & 3u);
+                if (f1 < F1) *reinterpret_cast<float4 *>(th + f1 * G::ROWB + ((xi ^ sw) << 4)) = make_float4(A0[i].x, A0[i].y, A1[i].x, A1[i].y);
             }
-            fence_async_smem();
-            __syncthreads();
-            if (tid == 0) {
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh)
-#pragma unroll
-                    for (int rb = 0; rb < ONB; ++rb)
-                        tma_store_3d(&map_o, to0 + hh * OHALF + rb * OBOXR * 128, 4 * c0 + 32 * hh, rb * OBOXR, (int)s);
-                tma_commit();
-            }
-            continue;
         }
-        float2 *dst = p.out + s * (long long)F1 * P2 + 2 * c0;
-        for (int idx = tid; idx < F1 * TX; idx += kCtThreads) {
-            const int f1 = idx / TX, x = idx % TX;
-            HN_G(dst + (long long)f1 * P2 + 2 * x, 16);
-            *reinterpret_cast<float4 *>(dst + (long long)f1 * P2 + 2 * x) =
-                *reinterpret_cast<const float4 *>(lines + x * LS + 2 * f1);
+        fence_async_smem();
+        __syncthreads();
+        if (tid == 0) {
+#pragma unroll
+            for (int hh = 0; hh < G::NH; ++hh) {
+                const unsigned char *th = to + hh * G::HALFB;
+#pragma unroll
+                for (int b = 0; b < G::NB; ++b) tma_store_3d(&map_o, th + b * G::BOXR * G::ROWB, 4 * (c0 + hh * G::TH), b * G::BOXR, (int)s);
+                float2 *last = p.out + (s * F1 + HP1) * (long long)P2 + 2 * (c0 + hh * G::TH);
+                HN_G(last, G::ROWB);
+                bulk_store(last, th + HP1 * G::ROWB, G::ROWB);
+            }
+            tma_commit();
         }
     }
-    if constexpr (TMA) {
-        if (failed) {
-            // a wait gave up: say so, then give the copy a bounded time to land before the buffers go away
-            if (p.status) atomicExch(p.status, 7);
-            mbar_wait(bar, phase);
-        }
+    if (failed) {
+        // a wait gave up: say so, then give the copy a bounded time to land before the buffers go away
+        if (p.status) atomicExch(p.status, 7);
+        mbar_wait(bar, phase);
     }
-    if constexpr (TSTORE) { if (tid == 0) tma_wait_all0(); }
+    if (tid == 0) tma_wait_all0();
 }
 
 // ---- filter rows: spectrum in place -----------------------------------------------------------------
@@ -335,92 +337,235 @@ __global__ void __launch_bounds__(256, 2) ct_hspec_w_kernel(HspecArgs p)
 
 struct CoreWArgs {
     float2 *u;                // [slices][F1][P2], in place
-    const float2 *hspec;      // [filters][F1][P2] spectra along t2 (scaled)
+    const float2 *h;          // [filters][F1][P2]: spectra along t2 (scaled), or with FILT the rows they are made from
     long long slices;
     int f1n;
     long long h_mod, h_off;
     const float2 *tw2;
     TwoLevelW twp;
+    // FILT only: a unit is one row of the filter of channel c and the same row of the batch entries it serves
+    int nb;                   // batch entries per unit
+    float scale;              // 1/P, folded into the filter's spectrum
 };
 
-template <int LOG2P2>
+// Twiddles of a pass from tensor memory (they depend on the lane only): 16 columns, 8 legs, at a time.
+struct TmemTw {
+    unsigned addr;
+    mutable float v[16];
+    template <int S> __device__ __forceinline__ float2 get(int, int r, int, int) const
+    {
+        if (r == 1 || (r & 7) == 0) {
+            TmemIO<16>::ld(v, addr + 16 * (r >> 3));
+            tmem_wait_ld();
+        }
+        return make_float2(v[2 * (r & 7)], v[2 * (r & 7) + 1]);
+    }
+};
+
+// FILT (a filter shared over the batch): a lane group transforms a row of the filter itself, parks the spectrum in its own
+// lanes of tensor memory and takes the row of nb batch entries through it, so the filter crosses HBM once and its spectrum
+// never.  In shared memory the spectra of 16 warps (8 KB each) do not fit beside their lines; in registers 64 more per thread
+// leave 8 warps per SM.  262144 bf16 values, 2 x 256 rows: 167 us in a kernel of the filter's own plus 525 here, now 600.  Bound by
+// instruction issue (60 % of the slots) and instruction fetch of the unrolled passes.  Three CTAs of four warps with twiddles in
+// registers and rows that travel ahead as untiled copies: 662.
+template <int LOG2P2, bool FILT>
 __global__ void __launch_bounds__(256, 2) ct_core_w_kernel(CoreWArgs p)
 {
     using F = WF<LOG2P2, false>;
     using FI = WF<LOG2P2, true>;
     constexpr int P2 = 1 << LOG2P2, TPL = F::TPL, NP = F::NP, G = 256 / TPL, LS = plane_ls(P2);
     using PL = typename F::LastPass;
+    constexpr int NV = PL::IPL * PL::R, NC = 2 * NV;       // points of a lane, tensor-memory columns of a warp
+    static_assert(NV % 16 == 0, "whole blocks of tensor memory");
     extern __shared__ float2 smem[];
+    __shared__ unsigned tm_slot;
     float2 *twt = smem + G * LS;
-    const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL;
+    const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL, warp = tid >> 5;
     const unsigned m = F::group_mask(tid);
     float2 *line = smem + gid * LS;
     PassTw<LOG2P2, false>::build(twt, p.tw2, P2, tid, 256);
     PassTw<LOG2P2, true>::build(twt + P2, p.tw2, P2, tid, 256);
+    // 1024 points: the twiddles of the forward passes sit in tensor memory too, beside the spectra (from shared memory they are a
+    // third of that pipe's work: 621 us)
+    constexpr bool TWTM = LOG2P2 == 10;
+    constexpr int TCOLS = (FILT ? 2 * NC : 0) + (TWTM ? 2 * PL::R : 0), TALLOC = TCOLS > 128 ? 256 : TCOLS > 64 ? 128 : 64;
+    if constexpr (TCOLS > 0) {
+        if (warp == 0) tmem_alloc(smem_u32(&tm_slot), TALLOC);
+        tmem_fence_before_sync();
+    }
     __syncthreads();
-    const PassTw<LOG2P2, false> tw{twt};
-    const PassTw<LOG2P2, true> twi{twt + P2};
-    const long long rows = p.slices * p.f1n;
-    for (long long r = (long long)blockIdx.x * G + gid; r < rows; r += (long long)gridDim.x * G) {
-        const long long s = r / p.f1n;
-        const int f1 = (int)(r % p.f1n);
-        const long long hs = p.h_mod ? (s + p.h_off) % p.h_mod : s;
-        float2 *row = p.u + r * P2;
-        const float2 *hrow = p.hspec + (hs * p.f1n + f1) * P2;
-        // the row is fetched with 16-byte asynchronous copies into the line (two bins per copy)
-        for (int c = l; c < P2 / 2; c += TPL) cp_async16(line + 2 * c, row + 2 * c);
-        cp_async_wait_all();
-        __syncwarp(m);
-        float2 Y[PL::IPL][PL::R];
-        {
-            // first pass reads the unskewed copy, then the usual skewed layout is used
-            using P0 = typename F::template Pass<0>;
-            float2 keep[P0::IPL][P0::R];
-            F::template pass<0, PRUNE_NONE>(l, tw,
-                [&](int, int, int idx) { return line[idx]; },
-                [&](int i, int rr, int, float2 v) { keep[i][rr] = v; });
-            __syncwarp(m);
+    if constexpr (TCOLS > 0) tmem_fence_after_sync();
+    const unsigned tm = FILT ? tmem_addr(tm_slot, warp, (warp >> 2) * NC) : 0u;
+    const unsigned tmt = TWTM ? tmem_addr(tm_slot, warp, FILT ? 2 * NC : 0) : 0u;
+    if constexpr (TWTM) {
+        if (warp < 4) {
 #pragma unroll
-            for (int i = 0; i < P0::IPL; ++i)
+            for (int b = 0; b < PL::R / 8; ++b) {
+                float v[16];
 #pragma unroll
-                for (int rr = 0; rr < P0::R; ++rr) line[F::ph((l + i * TPL) * P0::R + rr)] = keep[i][rr];
-            __syncwarp(m);
+                for (int e = 0; e < 8; ++e) {
+                    const float2 w = 8 * b + e == 0 ? make_float2(1.f, 0.f) : twt[(8 * b + e - 1) * PL::NS + l];
+                    v[2 * e] = w.x; v[2 * e + 1] = w.y;
+                }
+                TmemIO<16>::st(tmt + 16 * b, v);
+            }
+            tmem_wait_st();
         }
+        tmem_fence_before_sync();
+        __syncthreads();
+        tmem_fence_after_sync();
+    }
+    using TwT = typename std::conditional<TWTM, TmemTw, PassTw<LOG2P2, false>>::type;
+    TwT tw;
+    if constexpr (TWTM) tw.addr = tmt; else tw.base = twt;
+    const PassTw<LOG2P2, true> twi{twt + P2};
+
+    // Two equal passes: the inverse is the forward transform with real and imaginary parts exchanged on both ends, so one copy of
+    // the passes serves the filter's row, the forward and the inverse (three copies of 32-point butterflies are 70 KB of code,
+    // and every fifth cycle of a warp waited for instructions).
+    constexpr bool EQUAL = NP == 2 && F::radix(0) == F::radix(1);
+    using X = float2[PL::IPL][PL::R];
+
+    // x <- transform of x along t2; `in` fills the points of the first pass, in the order they also leave the last one
+    auto forward = [&](X &x, auto in) {
+        F::template pass<0, PRUNE_NONE>(l, tw, in, [&](int, int, int idx, float2 v) { line[F::ph(idx)] = v; });
+        __syncwarp(m);
         F::template mid<1, NP - 1, PRUNE_NONE>(l, m, tw, line);
         F::template pass<NP - 1, PRUNE_NONE>(l, tw,
             [&](int, int, int idx) { return line[F::ph(idx)]; },
-            [&](int i, int rr, int, float2 v) { Y[i][rr] = v; });
-        // spectral product with the precomputed filter spectrum (coalesced loads, no stores between)
+            [&](int i, int rr, int, float2 v) { x[i][rr] = v; });
+        __syncwarp(m);
+    };
+    // undo the inter-pass twiddle W_P^(t2*f1), t2 = l + TPL*q: per-lane factor W_P^(f1*l) times a
+    // per-row factor W_P^(f1*TPL*q) whose address is the same in all lanes
+    // (the per-row factor is looked up every fourth leg and advanced by one leg's step in between)
+    using PE = typename FI::LastPass;
+    struct Undo { float2 cl, stp, w; };
+    auto undo_init = [&](int f1) {
+        Undo t;
+        t.cl = twp_w(p.twp, (unsigned)f1 * (unsigned)l);
+        t.stp = twp_w(p.twp, (unsigned)f1 * (unsigned)(P2 / PE::R));
+        t.w = t.cl;
+        return t;
+    };
+    auto undo_store = [&](Undo &t, float2 *row, int f1, bool on, int r, int idx, float2 v) {
+        // legs of one item come in order r = 0, 1, ...: positions idx = l + i*TPL + r*(P2/R)
+        if (r % 4 == 0) t.w = cmul(t.cl, twp_w(p.twp, (unsigned)f1 * (unsigned)(idx - l)));
+        else t.w = cmul(t.w, t.stp);
+        if (on) { HN_G(row + idx, 8); row[idx] = cmulc(v, t.w); }
+    };
+    // one row of u: forward along t2, product(x) for every point, back, inter-pass twiddle undone.  first: it is the filter's row,
+    // whose spectrum goes to park(x) instead.
+    // (rows go from global memory straight to the first pass: through the line they cost two more trips of the shared-memory pipe)
+    auto row_through = [&](const float2 *src, float2 *row, int f1, bool on, bool first, auto park, auto product) {
+        X x;
+        if constexpr (EQUAL) {
 #pragma unroll
-        for (int i = 0; i < PL::IPL; ++i)
-#pragma unroll
-            for (int rr = 0; rr < PL::R; ++rr) {
-                HN_G(hrow + F::last_pos(l, i, rr), 8);
-                Y[i][rr] = cmul(Y[i][rr], __ldg(hrow + F::last_pos(l, i, rr)));
+            for (int r = 0; r < PL::R; ++r) {
+                if (on) HN_G(src + l + r * TPL, 8);
+                x[0][r] = on ? src[l + r * TPL] : make_float2(0.f, 0.f);
             }
-        __syncwarp(m);
-        FI::template pass<0, PRUNE_NONE>(l, twi,
-            [&](int i, int rr, int) { return Y[i][rr]; },
-            [&](int, int, int idx, float2 v) { line[FI::ph(idx)] = v; });
-        __syncwarp(m);
-        FI::template mid<1, NP - 1, PRUNE_NONE>(l, m, twi, line);
-        // undo the inter-pass twiddle W_P^(t2*f1), t2 = l + TPL*q: per-lane factor W_P^(f1*l) times a
-        // per-row factor W_P^(f1*TPL*q) whose address is the same in all lanes
-        // (the per-row factor is looked up every fourth leg and advanced by one leg's step in between)
-        const float2 cl = twp_w(p.twp, (unsigned)f1 * (unsigned)l);
-        using PE = typename FI::LastPass;
-        const float2 stp = twp_w(p.twp, (unsigned)f1 * (unsigned)(P2 / PE::R));
-        float2 w = cl;
-        FI::template pass<NP - 1, PRUNE_NONE>(l, twi,
-            [&](int, int, int idx) { return line[FI::ph(idx)]; },
-            [&](int, int r, int idx, float2 v) {
-                // legs of one item come in order r = 0, 1, ...: positions idx = l + i*TPL + r*(P2/R)
-                if (r % 4 == 0) w = cmul(cl, twp_w(p.twp, (unsigned)f1 * (unsigned)(idx - l)));
-                else w = cmul(w, stp);
-                HN_G(row + idx, 8);
-                row[idx] = cmulc(v, w);
+#pragma unroll 1
+            for (int way = 0;; ++way) {
+                forward(x, [&](int i, int r, int) { return x[i][r]; });
+                if (way) break;
+                if (first) { park(x); return; }
+                product(x);
+#pragma unroll
+                for (int r = 0; r < PL::R; ++r) x[0][r] = make_float2(x[0][r].y, x[0][r].x);
+            }
+            Undo t = undo_init(f1);
+#pragma unroll
+            for (int r = 0; r < PL::R; ++r) undo_store(t, row, f1, on, r, l + r * TPL, make_float2(x[0][r].y, x[0][r].x));
+        } else {
+            forward(x, [&](int, int, int idx) { if (on) HN_G(src + idx, 8); return on ? src[idx] : make_float2(0.f, 0.f); });
+            if (first) { park(x); return; }
+            product(x);
+            FI::template pass<0, PRUNE_NONE>(l, twi,
+                [&](int i, int rr, int) { return x[i][rr]; },
+                [&](int, int, int idx, float2 v) { line[FI::ph(idx)] = v; });
+            __syncwarp(m);
+            FI::template mid<1, NP - 1, PRUNE_NONE>(l, m, twi, line);
+            Undo t = undo_init(f1);
+            FI::template pass<NP - 1, PRUNE_NONE>(l, twi,
+                [&](int, int, int idx) { return line[FI::ph(idx)]; },
+                [&](int, int r, int idx, float2 v) { undo_store(t, row, f1, on, r, idx, v); });
+            __syncwarp(m);
+        }
+    };
+
+    if constexpr (!FILT) {
+        const long long rows = p.slices * p.f1n;
+        for (long long r = (long long)blockIdx.x * G + gid; r < rows; r += (long long)gridDim.x * G) {
+            const long long s = r / p.f1n;
+            const int f1 = (int)(r % p.f1n);
+            const long long hs = p.h_mod ? (s + p.h_off) % p.h_mod : s;
+            const float2 *hrow = p.h + (hs * p.f1n + f1) * P2;
+            row_through(p.u + r * P2, p.u + r * P2, f1, true, false, [](X &) {}, [&](X &Y) {
+                // product with the precomputed filter spectrum (coalesced loads, no stores between)
+#pragma unroll
+                for (int i = 0; i < PL::IPL; ++i)
+#pragma unroll
+                    for (int rr = 0; rr < PL::R; ++rr) {
+                        HN_G(hrow + F::last_pos(l, i, rr), 8);
+                        Y[i][rr] = cmul(Y[i][rr], __ldg(hrow + F::last_pos(l, i, rr)));
+                    }
             });
-        __syncwarp(m);
+        }
+    } else {
+        // slices [h_off, h_off + slices) of the batch counted from its first entry here: slice b * h_mod + c
+        const long long entries = (p.h_off + p.slices + p.h_mod - 1) / p.h_mod, chunks = (entries + p.nb - 1) / p.nb;
+        const long long per = p.h_mod * p.f1n, units = chunks * per;
+        constexpr int LPW = 32 / TPL;
+        // (a warp's groups go round together: tensor memory is reached by whole warps)
+        for (long long u0 = (long long)blockIdx.x * G + warp * LPW; u0 < units; u0 += (long long)gridDim.x * G) {
+            const long long u = u0 + (gid - warp * LPW);
+            const bool live = u < units;
+            const long long b0 = live ? u / per * p.nb : 0;
+            const int rc = live ? (int)(u % per) : 0, c = rc / p.f1n, f1 = rc % p.f1n;
+#pragma unroll 1
+            for (int j = -1; j < p.nb; ++j) {
+                const long long s = (b0 + j) * p.h_mod + c - p.h_off;
+                const bool first = j < 0, on = live && (first || (s >= 0 && s < p.slices));
+                float2 *row = p.u + (s * p.f1n + f1) * P2;
+                row_through(first ? p.h + (long long)rc * P2 : row, row, f1, on, first,
+                    [&](X &H) {
+                        __syncwarp();
+#pragma unroll
+                        for (int b = 0; b < NC / 32; ++b) {
+                            float Hc[32];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                const float2 v = H[(16 * b + e) / PL::R][(16 * b + e) % PL::R];
+                                Hc[2 * e] = v.x * p.scale;
+                                Hc[2 * e + 1] = v.y * p.scale;
+                            }
+                            TmemIO<32>::st(tm + 32 * b, Hc);
+                        }
+                        tmem_wait_st();
+                    },
+                    [&](X &Y) {
+                        __syncwarp();
+#pragma unroll
+                        for (int b = 0; b < NC / 32; ++b) {
+                            float Hc[32];
+                            TmemIO<32>::ld(Hc, tm + 32 * b);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                float2 &y = Y[(16 * b + e) / PL::R][(16 * b + e) % PL::R];
+                                y = cmul(y, make_float2(Hc[2 * e], Hc[2 * e + 1]));
+                            }
+                        }
+                    });
+            }
+        }
+    }
+    if constexpr (TCOLS > 0) {
+        tmem_fence_before_sync();
+        __syncthreads();
+        tmem_fence_after_sync();
+        if (warp == 0) tmem_dealloc(tm_slot, TALLOC);
     }
 }
 
@@ -432,174 +577,230 @@ struct ColsInvWArgs {
     void *y;
     long long slices;
     int len;                  // L
-    bool pair;                // slices of whole pairs: two elements per access
     int log2p2;
     const float2 *tw1;
     int *status;              // device word set when a bounded wait on a tensor copy gives up (may be NULL)
-    bool no_tma;              // development switch: per-thread copies even where tensor copies apply
 };
 
-// TMA = true: the gate tile q arrives, and the result tile y leaves, as tensor copies ([t1][pair] rows of
-// TX pairs, no swizzle: a warp touches whole consecutive rows); false: per-thread loads and stores.
-template <typename T, int LOG2P1, bool TMA, bool PAIR>
-__global__ void __launch_bounds__(kCtInvThreads, (LOG2P1 >= 9 ? 4 : 8))
-ct_cols_inv_w_kernel(ColsInvWArgs p, const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_y)
+// Gate and store of a tile of lines (`lines`: position t1 < P1/2 of line x holds the two real outputs of columns 2x, 2x+1).
+template <typename T, int LOG2P1, int TX, int LS, bool PAIR>
+__device__ __forceinline__ void ct_inv_epilogue(const ColsInvWArgs &p, const float2 *lines, long long s, int c0, int P2, int tid)
 {
     using FI = WF<LOG2P1, true>;
-    constexpr int P1 = 1 << LOG2P1, HP1 = P1 / 2, F1 = HP1 + 1, TPL = FI::TPL;
-    constexpr int TX = ct_inv_tx(TPL);
-    constexpr int NGRP = kCtInvThreads / TPL;
-    constexpr int LS = ct_ls(phys_max(P1) + 2);
-    extern __shared__ float2 smem[];
-    float2 *lines = smem;
-    float2 *twt = lines + TX * LS;
-    // gate and result tiles: HP1 rows of TX pairs
-    constexpr unsigned QROW = TX * 2 * sizeof(T), QBYTES = HP1 * QROW;
-    constexpr int QBOXR = HP1 < 256 ? HP1 : 256, QNB = HP1 / QBOXR;
-    unsigned char *tq = reinterpret_cast<unsigned char *>(twt + P1);
-    if constexpr (TMA) tq += (128u - (smem_u32(tq) & 127u)) & 127u;
-    unsigned char *ty = tq + QBYTES;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(ty + QBYTES);
-    const int tid = threadIdx.x, l = tid % TPL, gid = tid / TPL;
-    const unsigned m = FI::group_mask(tid);
-    if constexpr (TMA) {
-        if (tid == 0) {
-            mbar_init(bar, 1);
-            fence_mbar_init();
+    constexpr int HP1 = (1 << LOG2P1) / 2;
+    const T *pq = (const T *)p.q;
+    T *py = (T *)p.y;
+        const long long base = s * (long long)p.len + 2 * c0;
+    // a half warp takes 8 pairs of two neighbouring rows: line stride and skew then spread its
+    // 16 reads over all banks, and each row still receives whole 32-byte sectors
+    constexpr int NE = HP1 * TX / kCtThreads;
+    static_assert(HP1 * TX % kCtThreads == 0, "whole epilogue rounds");
+    constexpr int XB = TX >= 8 ? TX / 8 : 1;
+    const int x = TX < 8 ? tid % TX : (tid & 7) + 8 * ((tid >> 4) % XB);
+    const int tb = TX < 8 ? tid / TX : ((tid >> 3) & 1) + 2 * ((tid >> 4) / XB);
+    constexpr int TSTEP = kCtThreads / TX;
+    using Q2 = typename std::conditional<sizeof(T) == 4, float2, __nv_bfloat162>::type;
+    // gate values first (all requests in flight together), then products and stores
+    const long long ox = base + 2 * x;
+    if constexpr (!PAIR) {
+        T qa[NE], qb[NE];
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            const int t1 = tb + e * TSTEP;
+            const long long tt = (long long)t1 * P2 + 2 * (c0 + x), o = ox + (long long)t1 * P2;
+            if (tt < p.len) HN_G(pq + o, sizeof(T));
+            if (tt + 1 < p.len) HN_G(pq + o + 1, sizeof(T));
+            qa[e] = tt < p.len ? __ldg(pq + o) : T(0.f);
+            qb[e] = tt + 1 < p.len ? __ldg(pq + o + 1) : T(0.f);
+        }
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            const int t1 = tb + e * TSTEP;
+            const long long tt = (long long)t1 * P2 + 2 * (c0 + x), o = ox + (long long)t1 * P2;
+            const float2 z = lines[x * LS + FI::ph(t1)];
+            if (tt < p.len) IO<T>::st(py, o, z.x * (float)qa[e]);
+            if (tt + 1 < p.len) IO<T>::st(py, o + 1, z.y * (float)qb[e]);
+        }
+        return;
+    }
+    Q2 qv[NE];
+#pragma unroll
+    for (int e = 0; e < NE; ++e) {
+        const int t1 = tb + e * TSTEP;
+        const long long tt = (long long)t1 * P2 + 2 * (c0 + x);
+        if (tt < p.len) HN_G(pq + ox + (long long)t1 * P2, 2 * sizeof(T));
+        if (tt < p.len) qv[e] = __ldg(reinterpret_cast<const Q2 *>(pq + ox + (long long)t1 * P2));
+    }
+#pragma unroll
+    for (int e = 0; e < NE; ++e) {
+        const int t1 = tb + e * TSTEP;
+        const long long tt = (long long)t1 * P2 + 2 * (c0 + x);
+        if (tt < p.len) {
+            const float2 z = lines[x * LS + FI::ph(t1)];
+            const long long o = ox + (long long)t1 * P2;
+            HN_G(py + o, 2 * sizeof(T));
+            if constexpr (sizeof(T) == 4) {
+                *reinterpret_cast<float2 *>(py + o) = make_float2(z.x * qv[e].x, z.y * qv[e].y);
+            } else {
+                *reinterpret_cast<__nv_bfloat162 *>(py + o) =
+                    __floats2bfloat162_rn(z.x * __low2float(qv[e]), z.y * __high2float(qv[e]));
+            }
         }
     }
-    unsigned phase = 0;
-    int failed = 0;
-    PassTw<LOG2P1, true>::build(twt, p.tw1, P1, tid, kCtInvThreads);
-    const PassTw<LOG2P1, true> tw{twt};
+}
+
+template <typename T, int LOG2P1> struct CtInvGeo : CtGeo<T, LOG2P1> {
+    using B = CtGeo<T, LOG2P1>;
+    static constexpr size_t RAW = 0, Q = ((size_t)B::NH * B::HALFB + B::QAL - 1) / B::QAL * B::QAL, LINES = Q + B::QBYTES,
+                            BARS = LINES + B::LINEB, TOTAL = BARS + 16;
+    // by shared memory, and at 168 registers a thread for the long transforms, 96 for the short ones
+    static constexpr int PER_SM = B::fit(TOTAL, LOG2P1 >= 9 ? 3 : 5);
+};
+
+// Tensor copies bring the tile of the spectra while the tile before it is transformed, and the gate tile under the last pass; the
+// gated results take the gate's place and leave as a tensor copy.  QY: 0 gate and result as tensor copies, 1 pairs, 2 elements.
+// Twiddles of the second pass in registers.  Bound by HBM: 262144 bf16 values, 512 rows, 456 us with 16 warps per SM that fetched
+// their own tiles and waited for them, 267 with 12 warps here (6.0 TB/s).
+template <typename T, int LOG2P1, int QY>
+__global__ void __launch_bounds__(kCtThreads, (CtInvGeo<T, LOG2P1>::PER_SM))
+ct_cols_inv_w_kernel(ColsInvWArgs p, const __grid_constant__ CUtensorMap map_u, const __grid_constant__ CUtensorMap map_q,
+                     const __grid_constant__ CUtensorMap map_y)
+{
+    using G = CtInvGeo<T, LOG2P1>;
+    using FI = typename G::FI;
+    constexpr int P1 = G::P1, HP1 = G::HP1, F1 = G::F1, TPL = G::TPL, TX = G::TX;
+    using P0 = typename FI::template Pass<0>;
+    using PE = typename FI::LastPass;
+    static_assert(FI::NP == 2, "two passes");
+    using Q2 = typename std::conditional<sizeof(T) == 4, float2, __nv_bfloat162>::type;
+    extern __shared__ __align__(1024) unsigned char smem_dyn[];
+    unsigned char *base = smem_dyn;                        // (aligned as declared: room to align it here would cost a CTA per SM)
+    if (smem_u32(base) & 1023u) {
+        if (threadIdx.x == 0 && p.status) atomicExch(p.status, 8);
+        return;
+    }
+    unsigned char *raw = base + G::RAW, *tq = base + G::Q;
+    float2 *lines = reinterpret_cast<float2 *>(base + G::LINES);
+    uint64_t *bar_u = reinterpret_cast<uint64_t *>(base + G::BARS), *bar_q = bar_u + 1;
+    const int tid = threadIdx.x, l = tid % TPL, x = tid / TPL;
+    const unsigned m = FI::group_mask(tid);
+    float2 *line = lines + x * G::LS;
+    if (tid == 0) {
+        mbar_init(bar_u, 1);
+        mbar_init(bar_q, 1);
+        fence_mbar_init();
+    }
+    typename FI::template Hoist<1> tw;
+    for (int t = tid; t < P1; t += kCtThreads) { HN_G(p.tw1 + t, 8); lines[t] = p.tw1[t]; }
+    __syncthreads();
+    tw.load(l, lines);
+    __syncthreads();
     const int P2 = 1 << p.log2p2;
     const int tpc = (P2 / 2) / TX;
     const long long tiles = p.slices * tpc;
-    const T *pq = (const T *)p.q;
-    T *py = (T *)p.y;
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    auto issue_u = [&](long long t) {                      // one thread
         const long long s = t / tpc;
         const int c0 = (int)(t % tpc) * TX;
-        const float2 *src = p.in + s * (long long)F1 * P2 + 2 * c0;
-        if constexpr (TMA) { if (tid == 0) tma_wait_read0(); }        // the previous result tile has left its buffer
-        __syncthreads();
-        if constexpr (TMA) {
-            if (tid == 0) {
-                mbar_expect_tx(bar, QBYTES);
+        mbar_expect_tx(bar_u, G::NH * F1 * G::ROWB);
 #pragma unroll
-                for (int b = 0; b < QNB; ++b) tma_load_3d(tq + b * QBOXR * QROW, &map_q, bar, 2 * c0, b * QBOXR, (int)s);
-            }
+        for (int hh = 0; hh < G::NH; ++hh) {
+            unsigned char *d = raw + hh * G::HALFB;
+#pragma unroll
+            for (int b = 0; b < G::NB; ++b) tma_load_3d(d + b * G::BOXR * G::ROWB, &map_u, bar_u, 4 * (c0 + hh * G::TH), b * G::BOXR, (int)s);
+            const float2 *last = p.in + (s * F1 + HP1) * (long long)P2 + 2 * (c0 + hh * G::TH);
+            HN_G(last, G::ROWB);
+            bulk_load(d + HP1 * G::ROWB, last, G::ROWB, bar_u);
         }
-        // both bins of a column pair land side by side in slot f1 of that pair's line
-        for (int idx = tid; idx < F1 * TX; idx += kCtInvThreads) {
-            const int f1 = idx / TX, x = idx % TX;
-            cp_async16(lines + x * LS + 2 * f1, src + (long long)f1 * P2 + 2 * x);
-        }
-        cp_async_wait_all();
-        __syncthreads();
-        for (int x = gid; x < TX; x += NGRP) {
-            float2 *line = lines + x * LS;
-            // legs below half the first-pass radix read bins <= P1/2 directly, the others the mirrored bin
-            // conjugated: known per leg at compile time, except where a leg starts at bin P1/2 itself
-            constexpr int RH = FI::template Pass<0>::R / 2;
-            FI::template run_to_line<PRUNE_OUT, true>(l, m, tw, line, [&](int, int r, int idx) {
+    };
+    auto gate_boxes = [&](long long t, auto f) {
+        const long long s = t / tpc;
+        const int c0 = (int)(t % tpc) * TX;
+#pragma unroll
+        for (int b = 0; b < G::NB; ++b) f(tq + b * G::BOXR * G::QROW, 2 * c0, b * G::BOXR, (int)s);
+    };
+    long long t = blockIdx.x;
+    if (tid == 0 && t < tiles) {
+        issue_u(t);
+        if constexpr (QY == 0) gate_boxes(t, [&](void *, int cx, int cy, int cz) { tma_prefetch_3d(&map_q, cx, cy, cz); });
+    }
+    // pair x of a tile row: its 16-byte chunk, XORed with address bits 7 and up, which the engine's strides (multiples of 8 rows)
+    // leave alone, so it depends on the lane only; upwards for bins below P1/2, downwards for the mirrored ones
+    const int xi = x % G::TH;
+    const unsigned char *rx = raw + (x / G::TH) * G::HALFB;
+    auto chunk = [&](int row) {
+        const unsigned sw = G::ROWB == 128 ? ((unsigned)row & 7u) : (((unsigned)row >> 1) & 3u);
+        return *reinterpret_cast<const float4 *>(rx + (size_t)row * G::ROWB + (((unsigned)xi ^ sw) << 4));
+    };
+    unsigned phase = 0;
+    int failed = 0;
+    for (; t < tiles; t += gridDim.x, phase ^= 1u) {
+        const long long tn = t + gridDim.x, s = t / tpc;
+        const int c0 = (int)(t % tpc) * TX;
+        if (!mbar_wait(bar_u, phase)) failed = 1;
+        // legs below half the first-pass radix read bins <= P1/2 directly, the others the mirrored bin
+        // conjugated: known per leg at compile time, except where a leg starts at bin P1/2 itself
+        constexpr int RH = P0::R / 2;
+        FI::template pass<0, PRUNE_NONE>(l, tw,
+            [&](int, int r, int idx) {
                 if (r < RH) {
-                    const float4 ab = *reinterpret_cast<const float4 *>(line + 2 * idx);
+                    const float4 ab = chunk(idx);
                     return make_float2(ab.x - ab.w, ab.y + ab.z);
                 }
-                const float4 ab = *reinterpret_cast<const float4 *>(line + 2 * (P1 - idx));
+                const float4 ab = chunk(P1 - idx);
                 const float sg = (r == RH && idx == HP1) ? 1.f : -1.f;
                 return make_float2(fmaf(-sg, ab.w, ab.x), fmaf(sg, ab.y, ab.z));
-            });
-        }
-        __syncthreads();
-        // line x now holds, at position t1 < P1/2, the two real outputs of columns 2x, 2x+1
-        const long long base = s * (long long)p.len + 2 * c0;
-        // a half warp takes 8 pairs of two neighbouring rows: line stride and skew then spread its
-        // 16 reads over all banks, and each row still receives whole 32-byte sectors
-        constexpr int NE = HP1 * TX / kCtInvThreads;
-        static_assert(HP1 * TX % kCtInvThreads == 0, "whole epilogue rounds");
-        const int x = (tid & 7) + 8 * ((tid >> 4) % (TX / 8));
-        const int tb = ((tid >> 3) & 1) + 2 * ((tid >> 4) / (TX / 8));
-        constexpr int TSTEP = kCtInvThreads / TX;
-        using Q2 = typename std::conditional<sizeof(T) == 4, float2, __nv_bfloat162>::type;
-        if constexpr (TMA) {
-            // gate values from the tile that arrived during the transforms; results into the staging tile
-            if (!mbar_wait(bar, phase)) failed = 1;
-            phase ^= 1u;
-#pragma unroll
-            for (int e = 0; e < NE; ++e) {
-                const int t1 = tb + e * TSTEP;
-                const float2 z = lines[x * LS + FI::ph(t1)];
-                const Q2 qv = *reinterpret_cast<const Q2 *>(tq + t1 * QROW + x * sizeof(Q2));
-                Q2 *o = reinterpret_cast<Q2 *>(ty + t1 * QROW + x * sizeof(Q2));
-                if constexpr (sizeof(T) == 4) *o = make_float2(z.x * qv.x, z.y * qv.y);
-                else *o = __floats2bfloat162_rn(z.x * __low2float(qv), z.y * __high2float(qv));
+            },
+            [&](int, int, int idx, float2 v) { line[FI::ph(idx)] = v; });
+        if (__syncthreads_or(failed)) break;               // the tile buffer is free again
+        if (tid == 0) {
+            if (tn < tiles) issue_u(tn);
+            if constexpr (QY == 0) {
+                tma_wait_read0();                          // the results before these have left the gate's buffer
+                mbar_expect_tx(bar_q, G::QBYTES);
+                gate_boxes(t, [&](void *d, int cx, int cy, int cz) { tma_load_3d(d, &map_q, bar_q, cx, cy, cz); });
+                if (tn < tiles) gate_boxes(tn, [&](void *, int cx, int cy, int cz) { tma_prefetch_3d(&map_q, cx, cy, cz); });
             }
+        }
+        // at t1 < P1/2 the two real outputs of columns 2x, 2x+1
+        float2 z[PE::IPL][PE::R / 2];
+        FI::template pass<1, PRUNE_OUT>(l, tw, [&](int, int, int idx) { return line[FI::ph(idx)]; },
+                                        [&](int i, int r, int, float2 v) { z[i][r] = v; });
+        __syncwarp(m);
+        if constexpr (QY == 0) {
+            if (!mbar_wait(bar_q, phase)) failed = 2;
+#pragma unroll
+            for (int i = 0; i < PE::IPL; ++i)
+#pragma unroll
+                for (int r = 0; r < PE::R / 2; ++r) {
+                    Q2 *g = reinterpret_cast<Q2 *>(tq + G::at(l + i * TPL + r * (P1 / PE::R), x));
+                    const Q2 qv = *g;
+                    if constexpr (sizeof(T) == 4) *g = make_float2(z[i][r].x * qv.x, z[i][r].y * qv.y);
+                    else *g = __floats2bfloat162_rn(z[i][r].x * __low2float(qv), z[i][r].y * __high2float(qv));
+                }
             fence_async_smem();
             if (__syncthreads_or(failed)) break;
             if (tid == 0) {
-#pragma unroll
-                for (int b = 0; b < QNB; ++b) tma_store_3d(&map_y, ty + b * QBOXR * QROW, 2 * c0, b * QBOXR, (int)s);
+                gate_boxes(t, [&](void *d, int cx, int cy, int cz) { tma_store_3d(&map_y, d, cx, cy, cz); });
                 tma_commit();
             }
-            continue;
-        }
-        // gate values first (all requests in flight together), then products and stores
-        const long long ox = base + 2 * x;
-        if constexpr (!PAIR) {
-            T qa[NE], qb[NE];
+        } else {
 #pragma unroll
-            for (int e = 0; e < NE; ++e) {
-                const int t1 = tb + e * TSTEP;
-                const long long tt = (long long)t1 * P2 + 2 * (c0 + x), o = ox + (long long)t1 * P2;
-                if (tt < p.len) HN_G(pq + o, sizeof(T));
-                if (tt + 1 < p.len) HN_G(pq + o + 1, sizeof(T));
-                qa[e] = tt < p.len ? __ldg(pq + o) : T(0.f);
-                qb[e] = tt + 1 < p.len ? __ldg(pq + o + 1) : T(0.f);
-            }
+            for (int i = 0; i < PE::IPL; ++i)
 #pragma unroll
-            for (int e = 0; e < NE; ++e) {
-                const int t1 = tb + e * TSTEP;
-                const long long tt = (long long)t1 * P2 + 2 * (c0 + x), o = ox + (long long)t1 * P2;
-                const float2 z = lines[x * LS + FI::ph(t1)];
-                if (tt < p.len) IO<T>::st(py, o, z.x * (float)qa[e]);
-                if (tt + 1 < p.len) IO<T>::st(py, o + 1, z.y * (float)qb[e]);
-            }
-            continue;
-        }
-        Q2 qv[NE];
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            const int t1 = tb + e * TSTEP;
-            const long long tt = (long long)t1 * P2 + 2 * (c0 + x);
-            if (tt < p.len) HN_G(pq + ox + (long long)t1 * P2, 2 * sizeof(T));
-            if (tt < p.len) qv[e] = __ldg(reinterpret_cast<const Q2 *>(pq + ox + (long long)t1 * P2));
-        }
-#pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            const int t1 = tb + e * TSTEP;
-            const long long tt = (long long)t1 * P2 + 2 * (c0 + x);
-            if (tt < p.len) {
-                const float2 z = lines[x * LS + FI::ph(t1)];
-                const long long o = ox + (long long)t1 * P2;
-                HN_G(py + o, 2 * sizeof(T));
-                if constexpr (sizeof(T) == 4) {
-                    *reinterpret_cast<float2 *>(py + o) = make_float2(z.x * qv[e].x, z.y * qv[e].y);
-                } else {
-                    *reinterpret_cast<__nv_bfloat162 *>(py + o) =
-                        __floats2bfloat162_rn(z.x * __low2float(qv[e]), z.y * __high2float(qv[e]));
-                }
-            }
+                for (int r = 0; r < PE::R / 2; ++r) line[FI::ph(l + i * TPL + r * (P1 / PE::R))] = z[i][r];
+            __syncthreads();
+            ct_inv_epilogue<T, LOG2P1, TX, G::LS, QY == 1>(p, lines, s, c0, P2, tid);
+            __syncthreads();                               // the lines are free again
         }
     }
-    if constexpr (TMA) {
-        if (failed) {
-            if (p.status) atomicExch(p.status, 8);
-            mbar_wait(bar, phase ^ 1u);
-        }
-        if (tid == 0) tma_wait_all0();
+    if (failed) {
+        // a wait gave up: say so, then give copies that may still be in flight a bounded time to land
+        if (p.status) atomicExch(p.status, 8);
+        mbar_wait(bar_u, phase);
+        if (QY == 0 && failed == 2) mbar_wait(bar_q, phase);
+        if (t + gridDim.x < tiles && failed == 2) mbar_wait(bar_u, phase ^ 1u);
     }
+    if (tid == 0) tma_wait_all0();
 }
 
 // ---- launchers ----------------------------------------------------------------------------------------------
@@ -618,107 +819,91 @@ static int ctw_sms()
 
 bool ct1d_w_supported(int log2p1, int log2p2)
 {
-    if (log2p1 < 7 || log2p1 > 10 || log2p2 < 7 || log2p2 > 10) return false;
-    const int tx = ct_tx(log2p1 >= 10 ? 32 : (log2p1 >= 8 ? 16 : 8));
-    if (((1 << log2p2) / 2) % tx != 0) return false;
-    return true;
+    return log2p1 >= 7 && log2p1 <= 10 && log2p2 >= 7 && log2p2 <= 10 && tma_available();
 }
 
-template <typename T, int LOG2P1, bool HAS_B, bool TMA, bool VEC>
-static void launch_cols_fwd_w_tt(const ColsFwdWArgs &a, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, int grid,
-                                size_t sm, cudaStream_t st)
+// spectra [slice][P1/2+1][P2] complex, as fp32
+template <class G> static bool spectra_map(CUtensorMap *m, const float2 *base, int P2, long long slices)
 {
+    const unsigned long long dims[3] = {2ull * P2, (unsigned long long)G::F1, (unsigned long long)slices};
+    const unsigned long long strides[2] = {(unsigned long long)P2 * 8, (unsigned long long)G::F1 * P2 * 8};
+    const unsigned box[3] = {G::TH * 4, G::BOXR, 1};
+    return tma_encode_3d_cached(m, base, false, dims, strides, box, (int)G::ROWB);
+}
+
+// A tensor whose slices are whole numbers of rows of P2 elements, so that [slice][row][P2] is an exact view of it and rows past the
+// data read as zeros; false where tensor copies do not apply.
+template <class G, typename T> static bool rows_map(CUtensorMap *m, const void *base, int len, long long slice_elems, int P2, long long slices)
+{
+    if (len % P2 != 0 || G::QROW % 16 != 0) return false;
+    const unsigned long long dims[3] = {(unsigned long long)P2, (unsigned long long)(len / P2), (unsigned long long)slices};
+    const unsigned long long strides[2] = {(unsigned long long)P2 * sizeof(T), (unsigned long long)slice_elems * sizeof(T)};
+    const unsigned box[3] = {2 * G::TX, G::BOXR, 1};
+    return tma_encode_3d_cached(m, base, sizeof(T) == 2, dims, strides, box, G::QSW);
+}
+
+template <typename T, int LOG2P1, bool HAS_B, int IN>
+static void launch_cols_fwd_w_in(const ColsFwdWArgs &a, const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, long long pairs,
+                                 cudaStream_t st)
+{
+    using G = CtFwdGeo<T, LOG2P1, HAS_B>;
     static DevOnce attr;
     if (attr.first())
-        cudaFuncSetAttribute(ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, TMA, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, TMA, VEC><<<grid, kCtThreads, sm, st>>>(a, ma, mb, mo);
+        cudaFuncSetAttribute(ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, IN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::TOTAL);
+    const long long tiles = pairs / G::TX, res = (long long)G::PER_SM * ctw_sms();
+    ct_cols_fwd_w_kernel<T, LOG2P1, HAS_B, IN><<<(int)(tiles < res ? tiles : res), kCtThreads, G::TOTAL, st>>>(a, ma, mb, mo);
 }
 
-template <typename T, int LOG2P1> static int launch_cols_fwd_w_t(const ColsFwdWArgs &a0, cudaStream_t st)
+template <typename T, int LOG2P1, bool HAS_B> static int launch_cols_fwd_w_b(const ColsFwdWArgs &a, cudaStream_t st)
 {
-    ColsFwdWArgs a = a0;
-    a.vec = a.in_slice * sizeof(T) % 8 == 0 && (((uintptr_t)a.a | (uintptr_t)a.b) & 7) == 0;
-    using F = WF<LOG2P1, false>;
-    constexpr int P1 = 1 << LOG2P1, TX = ct_tx(F::TPL), LS = ct_ls(phys_max(P1) + 2);
-    const size_t sm = sizeof(float2) * ((size_t)TX * LS + P1) + (size_t)2 * (P1 / 2) * (2 * TX * sizeof(T) + 8);
+    using G = CtFwdGeo<T, LOG2P1, HAS_B>;
     const int P2 = 1 << a.log2p2;
-    const long long tiles = a.slices * ((P2 / 2) / TX);
-    const long long res = (LOG2P1 >= 9 ? 2ll : 4ll) * ctw_sms();   // resident CTAs
-    const int grid = (int)(tiles < res ? tiles : res);
-    if (grid <= 0) return 0;
-    // Tensor copies need the slice to be a whole number of rows of P2 elements (then [slice][row][P2] is an
-    // exact view of the input and rows past the data read as zeros) and tile rows of 64 or 128 bytes.
+    const long long pairs = a.slices * (P2 / 2);
+    if (pairs <= 0) return 0;
     alignas(64) CUtensorMap ma, mb, mo;
     memset(&ma, 0, sizeof(ma));
     memset(&mb, 0, sizeof(mb));
-    memset(&mo, 0, sizeof(mo));
-    constexpr unsigned TROW = TX * 2 * sizeof(T);
-    bool tma = (TROW == 64 || TROW == 128) && a.len % P2 == 0 && a.slices < (1ll << 31) && tma_available() && !a.no_tma;
-    if (tma) {
-        constexpr int HP1 = P1 / 2;
-        const unsigned long long dims[3] = {(unsigned long long)P2, (unsigned long long)(a.len / P2), (unsigned long long)a.slices};
-        const unsigned long long strides[2] = {(unsigned long long)P2 * sizeof(T), (unsigned long long)a.in_slice * sizeof(T)};
-        const unsigned box[3] = {2 * TX, (unsigned)(HP1 < 256 ? HP1 : 256), 1};
-        tma = tma_encode_3d_cached(&ma, a.a, sizeof(T) == 2, dims, strides, box, (int)TROW);
-        if (tma && a.b) tma = tma_encode_3d_cached(&mb, a.b, sizeof(T) == 2, dims, strides, box, (int)TROW);
-        // results [slice][P1/2+1][P2] complex, as fp32: boxes of 8 column pairs (32 floats) by 136 rows
-        const unsigned long long od[3] = {2ull * P2, (unsigned long long)(HP1 + 1), (unsigned long long)a.slices};
-        const unsigned long long os[2] = {(unsigned long long)P2 * 8, (unsigned long long)(HP1 + 1) * P2 * 8};
-        const unsigned ob[3] = {32, (unsigned)ct_out_box_rows(HP1 + 1), 1};
-        if (tma) tma = tma_encode_3d_cached(&mo, a.out, false, od, os, ob, 128);
-    }
-    if constexpr (TROW == 64 || TROW == 128) {
-        if (tma) {
-            if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, true, true>(a, ma, mb, mo, grid, sm, st);
-            else launch_cols_fwd_w_tt<T, LOG2P1, false, true, true>(a, ma, mb, mo, grid, sm, st);
-            return 1;
-        }
-    }
-    if (a.vec) {
-        if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, false, true>(a, ma, mb, mo, grid, sm, st);
-        else launch_cols_fwd_w_tt<T, LOG2P1, false, false, true>(a, ma, mb, mo, grid, sm, st);
-    } else if (a.b) launch_cols_fwd_w_tt<T, LOG2P1, true, false, false>(a, ma, mb, mo, grid, sm, st);
-    else launch_cols_fwd_w_tt<T, LOG2P1, false, false, false>(a, ma, mb, mo, grid, sm, st);
+    if (a.slices >= (1ll << 31) || !spectra_map<G>(&mo, a.out, P2, a.slices)) return -1;
+    const bool vec = a.in_slice * sizeof(T) % 8 == 0 && (((uintptr_t)a.a | (uintptr_t)a.b) & 7) == 0;
+    if (rows_map<G, T>(&ma, a.a, a.len, a.in_slice, P2, a.slices) && (!HAS_B || rows_map<G, T>(&mb, a.b, a.len, a.in_slice, P2, a.slices)))
+        launch_cols_fwd_w_in<T, LOG2P1, HAS_B, 0>(a, ma, mb, mo, pairs, st);
+    else if (vec) launch_cols_fwd_w_in<T, LOG2P1, HAS_B, 1>(a, ma, mb, mo, pairs, st);
+    else launch_cols_fwd_w_in<T, LOG2P1, HAS_B, 2>(a, ma, mb, mo, pairs, st);
     return 1;
 }
 
-template <typename T, int LOG2P1, bool TMA, bool PAIR>
-static void launch_cols_inv_w_tt(const ColsInvWArgs &a, const CUtensorMap &mq, const CUtensorMap &my, int grid, size_t sm, cudaStream_t st)
+template <typename T, int LOG2P1> static int launch_cols_fwd_w_t(const ColsFwdWArgs &a, cudaStream_t st)
 {
-    static DevOnce attr;
-    if (attr.first())
-        cudaFuncSetAttribute(ct_cols_inv_w_kernel<T, LOG2P1, TMA, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    ct_cols_inv_w_kernel<T, LOG2P1, TMA, PAIR><<<grid, kCtInvThreads, sm, st>>>(a, mq, my);
+    return a.b ? launch_cols_fwd_w_b<T, LOG2P1, true>(a, st) : launch_cols_fwd_w_b<T, LOG2P1, false>(a, st);
 }
 
-template <typename T, int LOG2P1> static int launch_cols_inv_w_t(const ColsInvWArgs &a0, cudaStream_t st)
+template <typename T, int LOG2P1, int QY>
+static void launch_cols_inv_w_qy(const ColsInvWArgs &a, const CUtensorMap &mu, const CUtensorMap &mq, const CUtensorMap &my, long long pairs,
+                                 cudaStream_t st)
 {
-    ColsInvWArgs a = a0;
-    a.pair = a.len % 2 == 0 && (((uintptr_t)a.q | (uintptr_t)a.y) & (2 * sizeof(T) - 1)) == 0;
-    using F = WF<LOG2P1, true>;
-    constexpr int P1 = 1 << LOG2P1, HP1 = P1 / 2, TX = ct_inv_tx(F::TPL), LS = ct_ls(phys_max(P1) + 2);
-    constexpr unsigned QROW = TX * 2 * sizeof(T);
-    // lines, twiddles, and (tensor-copy variant) gate tile, result tile, barrier, alignment slack
-    const size_t sm = sizeof(float2) * ((size_t)TX * LS + P1) + 2 * (size_t)HP1 * QROW + 8 + 128;
+    using G = CtInvGeo<T, LOG2P1>;
+    static DevOnce attr;
+    if (attr.first())
+        cudaFuncSetAttribute(ct_cols_inv_w_kernel<T, LOG2P1, QY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::TOTAL);
+    const long long tiles = pairs / G::TX, res = (long long)G::PER_SM * ctw_sms();
+    ct_cols_inv_w_kernel<T, LOG2P1, QY><<<(int)(tiles < res ? tiles : res), kCtThreads, G::TOTAL, st>>>(a, mu, mq, my);
+}
+
+template <typename T, int LOG2P1> static int launch_cols_inv_w_t(const ColsInvWArgs &a, cudaStream_t st)
+{
+    using G = CtInvGeo<T, LOG2P1>;
+    const bool pair = a.len % 2 == 0 && (((uintptr_t)a.q | (uintptr_t)a.y) & (2 * sizeof(T) - 1)) == 0;
     const int P2 = 1 << a.log2p2;
-    const long long tiles = a.slices * ((P2 / 2) / TX);
-    const long long res = (LOG2P1 >= 9 ? 4ll : 8ll) * ctw_sms();   // resident CTAs
-    const int grid = (int)(tiles < res ? tiles : res);
-    if (grid <= 0) return 0;
-    alignas(64) CUtensorMap mq, my;
+    const long long pairs = a.slices * (P2 / 2);
+    if (pairs <= 0) return 0;
+    alignas(64) CUtensorMap mu, mq, my;
     memset(&mq, 0, sizeof(mq));
     memset(&my, 0, sizeof(my));
-    // tensor copies need the slice to be a whole number of rows of P2 elements
-    bool tma = a.len % P2 == 0 && a.slices < (1ll << 31) && QROW % 16 == 0 && tma_available() && !a.no_tma;
-    if (tma) {
-        const unsigned long long dims[3] = {(unsigned long long)P2, (unsigned long long)(a.len / P2), (unsigned long long)a.slices};
-        const unsigned long long strides[2] = {(unsigned long long)P2 * sizeof(T), (unsigned long long)a.len * sizeof(T)};
-        const unsigned box[3] = {2 * TX, (unsigned)(HP1 < 256 ? HP1 : 256), 1};
-        tma = tma_encode_3d_cached(&mq, a.q, sizeof(T) == 2, dims, strides, box, 0) && tma_encode_3d_cached(&my, a.y, sizeof(T) == 2, dims, strides, box, 0);
-    }
-    if (tma) launch_cols_inv_w_tt<T, LOG2P1, true, true>(a, mq, my, grid, sm, st);
-    else if (a.pair) launch_cols_inv_w_tt<T, LOG2P1, false, true>(a, mq, my, grid, sm, st);
-    else launch_cols_inv_w_tt<T, LOG2P1, false, false>(a, mq, my, grid, sm, st);
+    if (a.slices >= (1ll << 31) || !spectra_map<G>(&mu, a.in, P2, a.slices)) return -1;
+    if (rows_map<G, T>(&mq, a.q, a.len, a.len, P2, a.slices) && rows_map<G, T>(&my, a.y, a.len, a.len, P2, a.slices))
+        launch_cols_inv_w_qy<T, LOG2P1, 0>(a, mu, mq, my, pairs, st);
+    else if (pair) launch_cols_inv_w_qy<T, LOG2P1, 1>(a, mu, mq, my, pairs, st);
+    else launch_cols_inv_w_qy<T, LOG2P1, 2>(a, mu, mq, my, pairs, st);
     return 1;
 }
 
@@ -730,14 +915,28 @@ template <int LOG2P2> static int launch_rows_w_t(const HspecArgs *hs, const Core
     static DevOnce attr;
     if (attr.first()) {
         cudaFuncSetAttribute(ct_hspec_w_kernel<LOG2P2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        cudaFuncSetAttribute(ct_core_w_kernel<LOG2P2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(ct_core_w_kernel<LOG2P2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(ct_core_w_kernel<LOG2P2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     }
-    const long long rows = hs ? hs->rows : co->slices * co->f1n;
-    const long long want = (rows + G - 1) / G;
+    const long long slots = (long long)ctw_sms() * 2 * G;
+    long long units = hs ? hs->rows : co->slices * co->f1n;
+    CoreWArgs c{};
+    if (co) c = *co;
+    if (co && c.scale != 0.f) {
+        // the count of batch entries per unit with the least work in the busiest slot: a transform for the filter, two per entry
+        const long long be = (c.h_off + c.slices + c.h_mod - 1) / c.h_mod;
+        long long best = -1;
+        for (long long nb = 1; nb <= be && nb <= 64; ++nb) {
+            const long long un = (be + nb - 1) / nb * c.h_mod * c.f1n, cost = ((un + slots - 1) / slots) * (1 + 2 * nb);
+            if (best < 0 || cost < best) { best = cost; c.nb = (int)nb; units = un; }
+        }
+    }
+    const long long want = (units + G - 1) / G;
     const int grid = (int)(want < (long long)ctw_sms() * 2 ? want : (long long)ctw_sms() * 2);
     if (grid <= 0) return 0;
     if (hs) ct_hspec_w_kernel<LOG2P2><<<grid, 256, sm, st>>>(*hs);
-    else ct_core_w_kernel<LOG2P2><<<grid, 256, sm, st>>>(*co);
+    else if (c.scale != 0.f) ct_core_w_kernel<LOG2P2, true><<<grid, 256, sm, st>>>(c);
+    else ct_core_w_kernel<LOG2P2, false><<<grid, 256, sm, st>>>(c);
     return 1;
 }
 
@@ -756,13 +955,13 @@ static int launch_rows_w(int log2p2, const HspecArgs *hs, const CoreWArgs *co, c
     return n;
 }
 
-int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
+int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool shared, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
                   int (*fallback)(Ct1dPlan *, const char *, long long, cudaStream_t, int *, Prof *))
 {
     const TwoLevelW twp{c->twp_coarse, c->twp_fine, c->lo};
     if (staged_ok) {
         ColsFwdWArgs a{};
-        a.a = h; a.b = nullptr; a.out = c->wh; a.slices = n; a.in_slice = c->K; a.len = c->K; a.status = c->status; a.no_tma = c->sw.no_tma;
+        a.a = h; a.b = nullptr; a.out = c->wh; a.slices = n; a.in_slice = c->K; a.len = c->K; a.status = c->status;
         a.log2p2 = c->log2p2; a.tw1 = c->tw1; a.twp = twp;
         prof->begin(KID_CT_COLS_H, st);
         int r = 0;
@@ -777,6 +976,7 @@ int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool staged_ok, cudaS
     } else if (fallback(c, (const char *)h, n, st, launches, prof)) {
         return -1;
     }
+    if (shared) return 0;                                  // the core transforms the rows of a shared filter itself
     HspecArgs hs{};
     hs.h = c->wh; hs.rows = n * ((1 << c->log2p1) / 2 + 1); hs.scale = (float)ldexp(1.0, -c->log2p); hs.tw2 = c->tw2;
     prof->begin(KID_CT_HSPEC, st);
@@ -792,7 +992,7 @@ int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long l
 {
     const TwoLevelW twp{c->twp_coarse, c->twp_fine, c->lo};
     ColsFwdWArgs a{};
-    a.a = k; a.b = v; a.out = c->wu; a.slices = n; a.in_slice = c->L; a.len = c->L; a.status = c->status; a.no_tma = c->sw.no_tma;
+    a.a = k; a.b = v; a.out = c->wu; a.slices = n; a.in_slice = c->L; a.len = c->L; a.status = c->status;
     a.log2p2 = c->log2p2; a.tw1 = c->tw1; a.twp = twp;
     prof->begin(KID_CT_COLS_U, st);
     int r = 0;
@@ -805,8 +1005,9 @@ int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long l
     if (r < 0) return -1;
     *launches += r;
     CoreWArgs co{};
-    co.u = c->wu; co.hspec = c->wh; co.slices = n; co.f1n = (1 << c->log2p1) / 2 + 1;
+    co.u = c->wu; co.h = c->wh; co.slices = n; co.f1n = (1 << c->log2p1) / 2 + 1;
     co.h_mod = shared ? c->C : 0; co.h_off = shared ? s0 % c->C : 0;
+    co.scale = shared ? (float)ldexp(1.0, -c->log2p) : 0.f;
     co.tw2 = c->tw2; co.twp = twp;
     prof->begin(KID_CT_CORE, st);
     r = launch_rows_w(c->log2p2, nullptr, &co, st);
@@ -814,7 +1015,7 @@ int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long l
     if (r < 0) return -1;
     *launches += r;
     ColsInvWArgs ci{};
-    ci.in = c->wu; ci.q = q; ci.y = y; ci.slices = n; ci.len = c->L; ci.log2p2 = c->log2p2; ci.tw1 = c->tw1; ci.status = c->status; ci.no_tma = c->sw.no_tma;
+    ci.in = c->wu; ci.q = q; ci.y = y; ci.slices = n; ci.len = c->L; ci.log2p2 = c->log2p2; ci.tw1 = c->tw1; ci.status = c->status;
     prof->begin(KID_CT_COLS_INV, st);
 #define CALLF(L) r = launch_cols_inv_w_t<float, L>(ci, st)
 #define CALLB(L) r = launch_cols_inv_w_t<bf16, L>(ci, st)
