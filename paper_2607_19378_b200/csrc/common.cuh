@@ -208,6 +208,7 @@ struct RowsArgs {
     int gtw_n;
     int full_in;          // 1: circular mode, k*v rows fill the whole line (len == P): nothing to prune
     int gtw_fresh;        // 1: the table was written by a kernel of the same call
+    int *status;          // device word set when a bounded wait on a copy gives up (may be NULL)
 };
 
 struct RowsInvArgs {

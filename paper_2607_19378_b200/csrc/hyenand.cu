@@ -587,6 +587,7 @@ static int filter_spectrum_generic(hyenand_plan *p, int l, const char *h, long l
     hyenand_plan::Lane &ln = p->lane[l];
     // rows of h, then (3-D) the middle axis
     RowsArgs r{};
+    r.status = p->dev_status;
     r.a = h; r.b = nullptr; r.out = ln.wh_a; r.pitch = p->XP;
     r.rows = n_slices * p->K[0] * p->K[1];
     r.len = p->K[2];
@@ -678,6 +679,7 @@ static int forward_generic(hyenand_plan *p, const char *q, const char *k, const 
                         const char *sq2, char *sy2) -> int {
             const size_t ei = elsize(dt_in), eo = elsize(dt_out);
             RowsArgs r{};
+            r.status = p->dev_status;
             r.a = sk + (size_t)s0 * p->vol * ei; r.b = sv ? sv + (size_t)s0 * p->vol * ei : nullptr; r.out = ln.ws_a; r.pitch = p->XP;
             r.rows = n * p->L[0] * p->L[1]; r.len = p->L[2]; r.shift = 0; r.log2p = p->log2p[2];
             r.prune_in = !p->circular; r.full_in = p->circular; r.gtw = p->gtw; r.gtw_n = p->gtw_n; r.gtw_fresh = p->gtw_fresh;
@@ -1515,6 +1517,7 @@ static int corr_dh(hyenand_grad *g, long long m, const void *gy, const void *gq,
     int c = 0;
     auto rows = [&](const void *a, const void *b, int dt, float2 *dst) {
         RowsArgs r{};
+        r.status = p->dev_status;
         r.a = a; r.b = b; r.out = dst; r.pitch = XP;
         r.rows = m * L[0] * L[1]; r.len = L[2]; r.shift = 0; r.log2p = p->log2p[2];
         r.prune_in = p->P[2] >= 2; r.full_in = 0; r.gtw = p->gtw; r.gtw_n = p->gtw_n;
@@ -1692,6 +1695,7 @@ static int backward_spectral(hyenand_grad *g, const void *q, const void *k, cons
     auto bad = [] { return fail(HYENAND_ERR_CUDA, "internal launch dispatch failed"); };
     auto rows = [&](const void *a, const void *b, long long n_rows, int len, int shift, bool prune, float2 *dst) {
         RowsArgs r{};
+        r.status = p->dev_status;
         r.a = a; r.b = b; r.out = dst; r.pitch = p->XP; r.rows = n_rows; r.len = len; r.shift = shift; r.log2p = p->log2p[2];
         r.prune_in = prune && !circ; r.full_in = circ; r.gtw = p->gtw; r.gtw_n = p->gtw_n;
         return (roww ? launch_rows_fwd_w(r, g->dtype, st) : launch_rows_fwd(r, g->dtype, st)) >= 0;
