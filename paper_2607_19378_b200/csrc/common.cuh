@@ -240,7 +240,7 @@ struct RowsInvArgs {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger()
 {
-    if (gridDim.x < kSms) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (gridDim.x * gridDim.y < kSms) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 __device__ __forceinline__ void pdl_join()
 {
@@ -249,10 +249,10 @@ __device__ __forceinline__ void pdl_join()
 }
 
 template <typename... P, typename... A>
-static inline void launch_pdl(void (*fn)(P...), unsigned grid, unsigned threads, size_t sm, cudaStream_t st, const A &...args)
+static inline void launch_pdl(void (*fn)(P...), dim3 grid, unsigned threads, size_t sm, cudaStream_t st, const A &...args)
 {
     cudaLaunchConfig_t c{};
-    c.gridDim = dim3(grid); c.blockDim = dim3(threads); c.dynamicSmemBytes = sm; c.stream = st;
+    c.gridDim = grid; c.blockDim = dim3(threads); c.dynamicSmemBytes = sm; c.stream = st;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;

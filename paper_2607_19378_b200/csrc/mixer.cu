@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(NW * 32) token_scale_kernel(const T *q, const 
 {
     constexpr int U = 8;
     __shared__ float red[2][NW][32 * VEC];
+    pdl_join();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long i = ((long long)blockIdx.x * 32 + lane) * VEC, b = blockIdx.y, base = b * C * L + i;
     const bool live = i < L;                                 // (VEC > 1 only where it divides L)
@@ -170,6 +171,7 @@ __global__ void __launch_bounds__(NW * 32) mixer_post_kernel(const float *o, con
     constexpr int U = KEEP ? KEEP : 8;
     __shared__ float red[NW][32 * VEC];
     __shared__ float scl[32 * VEC];
+    pdl_join();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long i = ((long long)blockIdx.x * 32 + lane) * VEC, base = (long long)blockIdx.y * C * L + i;
     const bool live = i < L;
@@ -232,6 +234,7 @@ __global__ void __launch_bounds__(kMixThreads) token_solo_kernel(const T *q, con
 {
     constexpr int U = 4;
     const long long i = ((long long)blockIdx.x * kMixThreads + threadIdx.x) * VEC, b = blockIdx.y, base = b * C * L + i;
+    pdl_join();
     if (i >= L) return;                                      // (VEC > 1 only where it divides L)
     float s1[VEC] = {}, s2[VEC] = {}, sc[VEC];
     auto sums = [&](int c, auto n) {
@@ -291,6 +294,7 @@ __global__ void __launch_bounds__(kMixThreads) post_solo_kernel(const float *o, 
 {
     constexpr int U = 4;
     const long long i = ((long long)blockIdx.x * kMixThreads + threadIdx.x) * VEC, base = (long long)blockIdx.y * C * L + i;
+    pdl_join();
     if (i >= L) return;
     float s[VEC] = {};
     auto sums = [&](int c, auto n) {
@@ -384,8 +388,8 @@ static void token_scale_t(const T *q, const T *k, const T *v, const float *g_in,
 {
     mix_tiles<T>(nb, L, C, [&](auto vec, auto nw, dim3 grid) {
         constexpr int VEC = decltype(vec)::value, NW = decltype(nw)::value;
-        if constexpr (NW == 0) token_solo_kernel<T, VEC, GATES><<<grid, kMixThreads, 0, st>>>(q, k, v, g_in, eps, C, L, scale, qz, kz, vz);
-        else token_scale_kernel<T, VEC, NW, GATES><<<grid, NW * 32, 0, st>>>(q, k, v, g_in, eps, C, L, scale, qz, kz, vz);
+        if constexpr (NW == 0) launch_pdl(token_solo_kernel<T, VEC, GATES>, grid, kMixThreads, 0, st, q, k, v, g_in, eps, C, L, scale, qz, kz, vz);
+        else launch_pdl(token_scale_kernel<T, VEC, NW, GATES>, grid, NW * 32, 0, st, q, k, v, g_in, eps, C, L, scale, qz, kz, vz);
     });
 }
 
@@ -415,12 +419,12 @@ template <typename T> static void mixer_post_t(const float *o, const float *g_ou
     mix_tiles<T>(nb, L, C, [&](auto vec, auto nw, dim3 grid) {
         constexpr int VEC = decltype(vec)::value, NW = decltype(nw)::value;
         if constexpr (NW == 0) {
-            post_solo_kernel<T, VEC><<<grid, kMixThreads, 0, st>>>(o, g_out, eps, C, L, y);
+            launch_pdl(post_solo_kernel<T, VEC>, grid, kMixThreads, 0, st, o, g_out, eps, C, L, y);
         } else {
             const int per = (C + NW - 1) / NW;               // channels per thread
-            if (per <= 4) mixer_post_kernel<T, VEC, NW, 4><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
-            else if (per <= 16) mixer_post_kernel<T, VEC, NW, 16><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
-            else mixer_post_kernel<T, VEC, NW, 0><<<grid, NW * 32, 0, st>>>(o, g_out, eps, C, L, y);
+            if (per <= 4) launch_pdl(mixer_post_kernel<T, VEC, NW, 4>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
+            else if (per <= 16) launch_pdl(mixer_post_kernel<T, VEC, NW, 16>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
+            else launch_pdl(mixer_post_kernel<T, VEC, NW, 0>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
         }
     });
 }

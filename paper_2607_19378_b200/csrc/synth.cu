@@ -244,13 +244,14 @@ template <int HF> constexpr size_t synth_tc_smem(int layers)
     // weight tiles (per hidden layer [2 HF x HF] = hi rows then lo rows; output chunk [64 x HF]), room to start them
     // on a 1024-byte boundary, small parameters, barrier + tensor-memory slot (the activations live in tensor memory)
     return (size_t)(layers - 1) * 2 * HF * HF * 4 + (size_t)2 * kTcChan * HF * 4 + 1024 +
-           sizeof(float) * ((size_t)HF * 4 + HF + (size_t)(layers - 1) * HF + (size_t)layers * 2 * HF + kTcChan + 3 * kTcChan) + 64;
+           sizeof(float) * ((size_t)HF * 4 + HF + (size_t)(layers - 1) * HF + (size_t)layers * 2 * HF + 2 * 4 * kTcChan) + 80;
 }
 
 template <typename T, int HF>
-__global__ void __launch_bounds__(kTcThreads) synth_tc_kernel(SynthArgs p)
+__global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(SynthArgs p)
 {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
+    pdl_join();
     // the swizzle pattern is a function of the shared-memory address: tiles start on 1024-byte boundaries
     unsigned char *sm = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
     const int J = p.layers, H = p.hidden, N = p.ndim;
@@ -261,9 +262,9 @@ __global__ void __launch_bounds__(kTcThreads) synth_tc_kernel(SynthArgs p)
     float *sOm = sW1 + HF * 4;
     float *sBh = sOm + HF;
     float *sFi = sBh + (J - 1) * HF;
-    float *sBo = sFi + J * 2 * HF;
-    float *sWin = sBo + kTcChan;                           // [3][32]
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sWin + 3 * kTcChan);
+    // per channel of a chunk, two chunks: factors of the window's exponent on the three axes, bias
+    float4 *sCh = reinterpret_cast<float4 *>(sFi + J * 2 * HF);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sCh + 2 * kTcChan);
     unsigned *tslot = reinterpret_cast<unsigned *>(bar + 1);
     const int tid = threadIdx.x, warp = tid >> 5, b = blockIdx.y;
     // tensor memory: accumulator (hi*hi and hi*lo side by side), then this tile's activations, hi and lo: row = lane
@@ -344,12 +345,73 @@ __global__ void __launch_bounds__(kTcThreads) synth_tc_kernel(SynthArgs p)
         tmem_fence_before_sync();                          // (this thread's tensor-memory reads and writes precede the next product)
         __syncthreads();
     };
+    // (One tile of 384 channels per CTA, operator on 4 x 64 x 64 tokens, bf16: with each chunk's weights fetched, split and laid out
+    // between two barriers before its product, and four parameter loads per window, 88 us; so 57.  Bound by the chain of products and
+    // the window's arithmetic; 128 registers with 124 bytes of spills for four CTAs per SM.)
+    // Output weights of the next chunk: fetched into registers before the wait for this chunk's product, split and laid out right
+    // after it (which frees the weight tile), so that neither their latency nor a barrier of their own stands in the chain of chunks.
+    // A thread takes HF / 4 neighbouring weights of channel tid / 4; the first warp a channel's window and bias.
+    constexpr int WPT = HF / 4;
+    const int wc = tid >> 2, wk = (tid & 3) * WPT;
+    const bool quads = H == HF && ((uintptr_t)p.Wout & 15) == 0;
+    constexpr float kLog2e = 1.4426950408889634f;
+    float wr[WPT], wn[4];
+    auto fetch = [&](int c0) {
+        const int c = c0 + wc;
+        if (quads) {
+#pragma unroll
+            for (int k = 0; k < WPT; k += 4) {
+                const float *src = p.Wout + (long long)c * HF + wk + k;
+                if (c < p.C) HN_G(src, 16);
+                const float4 v = c < p.C ? __ldg(reinterpret_cast<const float4 *>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                wr[k] = v.x; wr[k + 1] = v.y; wr[k + 2] = v.z; wr[k + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < WPT; ++k) wr[k] = c < p.C && wk + k < H ? SYN_LD(p.Wout, (long long)c * H + wk + k) : 0.f;
+        }
+        if (tid < kTcChan) {
+            const bool in = c0 + tid < p.C;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int ua = a - (3 - N);                // Gaussian: sigma per axis; causal: alpha in slot 2
+                wn[a] = 0.f;
+                if (in && p.mode == 1) { if (a == 2) wn[a] = SYN_LD(p.window, c0 + tid); }
+                else if (in && ua >= 0) wn[a] = SYN_LD(p.window, (long long)ua * p.C + c0 + tid);
+            }
+            wn[3] = in ? SYN_LD(p.bout, c0 + tid) : 0.f;
+        }
+    };
+    int buf = 0;
+    auto stage = [&](int c0) {
+#pragma unroll
+        for (int k = 0; k < WPT; k += 4) {
+            float hi[4], lo[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { hi[i] = to_tf32(wr[k + i]); lo[i] = wr[k + i] - hi[i]; }
+            *reinterpret_cast<float4 *>(sO + tc_off<2 * kTcChan>(wc, wk + k)) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<float4 *>(sO + tc_off<2 * kTcChan>(kTcChan + wc, wk + k)) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+        }
+        if (tid < kTcChan) {
+            float e[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                // the window is 2^(sum of coordinate^2 * e), or 2^(|coordinate| e) where causal
+                if (p.mode == 1) e[a] = -kLog2e * wn[a];
+                else { const float w = c0 + tid < p.C && a >= 3 - N ? 1.f / wn[a] : 0.f; e[a] = (-0.5f * kLog2e * w) * w; }
+            }
+            sCh[(buf ^ 1) * kTcChan + tid] = make_float4(e[0], e[1], e[2], wn[3]);
+        }
+        buf ^= 1;
+        fence_async_smem();
+    };
     for (long long tile = blockIdx.x; tile < tiles && !failed; tile += gridDim.x) {
         long long t = tile * kTcThreads + tid;
         const bool live = t < taps;
         if (!live) t = taps - 1;                           // clamped: computed, never stored
         const int m2 = (int)(t % p.K[2]), m1 = (int)((t / p.K[2]) % p.K[1]), m0 = (int)(t / ((long long)p.K[2] * p.K[1]));
         const float cx0 = axis_coord(m0, p.L[0], p.mode), cx1 = axis_coord(m1, p.L[1], p.mode), cx2 = axis_coord(m2, p.L[2], p.mode);
+        const float q0 = p.mode == 1 ? 0.f : cx0 * cx0, q1 = p.mode == 1 ? 0.f : cx1 * cx1, q2 = p.mode == 1 ? fabsf(cx2) : cx2 * cx2;
         float act[HF];
 #pragma unroll
         for (int i = 0; i < HF; ++i) {
@@ -373,58 +435,34 @@ __global__ void __launch_bounds__(kTcThreads) synth_tc_kernel(SynthArgs p)
             }
         }
         if (failed) break;
+        // (one chunk: staged once per CTA; the weight tile is free: the previous product was waited for)
+        if (tile == (long long)blockIdx.x || p.C > kTcChan) { fetch(0); stage(0); }
         put_acts(act);                                      // operand of every output chunk
-        for (int c0 = 0; c0 < p.C; c0 += kTcChan) {
+        T *o = out + t;
+        for (int c0 = 0; c0 < p.C; c0 += kTcChan, o += kTcChan * taps) {
             const int nc = p.C - c0 < kTcChan ? p.C - c0 : kTcChan;
-            // output weights of this chunk (one chunk: staged once per CTA; more: once per tile and chunk)
-            if (tile == (long long)blockIdx.x || p.C > kTcChan) {
-                for (int e = tid; e < kTcChan * HF; e += kTcThreads) {
-                    const int c = e / HF, k = e % HF;
-                    const float w = (c < nc && k < H) ? SYN_LD(p.Wout, (long long)(c0 + c) * H + k) : 0.f;
-                    const float hi = to_tf32(w);
-                    *reinterpret_cast<float *>(sO + tc_off<2 * kTcChan>(c, k)) = hi;
-                    *reinterpret_cast<float *>(sO + tc_off<2 * kTcChan>(kTcChan + c, k)) = w - hi;
-                }
-                for (int c = tid; c < kTcChan; c += kTcThreads) {
-                    sBo[c] = c < nc ? SYN_LD(p.bout, c0 + c) : 0.f;
-                    for (int a = 0; a < 3; ++a) {
-                        const int ua = a - (3 - N);
-                        float wv = 0.f;                    // Gaussian: 1 / sigma per axis; causal: alpha in slot 2
-                        if (c < nc) {
-                            if (p.mode == 1) wv = a == 2 ? SYN_LD(p.window, c0 + c) : 0.f;
-                            else if (ua >= 0) wv = 1.f / SYN_LD(p.window, (long long)ua * p.C + c0 + c);
-                        }
-                        sWin[a * kTcChan + c] = wv;
-                    }
-                }
-                fence_async_smem();
-                tmem_fence_before_sync();
-                __syncthreads();
-            }
+            const bool more = c0 + kTcChan < p.C;
+            const float4 *ch = sCh + buf * kTcChan;
+            if (more) fetch(c0 + kTcChan);
             contract(aO, std::integral_constant<int, kTcChan>{});
             if (failed) break;
+            if (more) stage(c0 + kTcChan);
 #pragma unroll
-            for (int q0 = 0; q0 < kTcChan; q0 += 16) {
+            for (int b0 = 0; b0 < kTcChan; b0 += 16) {
                 float acc[16], acl[16];
-                TmemIO<16>::ld(acc, trow + q0);
-                TmemIO<16>::ld(acl, trow + kTcChan + q0);
+                TmemIO<16>::ld(acc, trow + b0);
+                TmemIO<16>::ld(acl, trow + kTcChan + b0);
                 tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] += acl[i];
-#pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    const int c = q0 + i;
+                    const float4 w = ch[b0 + i];
                     float win;
-                    if (p.mode == 1) win = __expf(-sWin[2 * kTcChan + c] * fabsf(cx2));
-                    else {
-                        const float a0 = cx0 * sWin[c], a1 = cx1 * sWin[kTcChan + c], a2 = cx2 * sWin[2 * kTcChan + c];
-                        win = __expf(-0.5f * (a0 * a0 + a1 * a1 + a2 * a2));
-                    }
-                    if (live && c < nc) IO<T>::st(out, (long long)(c0 + c) * taps + t, win * (acc[i] + sBo[c]));
+                    asm("ex2.approx.f32 %0, %1;" : "=f"(win) : "f"(fmaf(q0, w.x, fmaf(q1, w.y, q2 * w.z))));
+                    if (live && b0 + i < nc) IO<T>::st(o, (b0 + i) * taps, win * ((acc[i] + acl[i]) + w.w));
                 }
             }
-            if (p.C > kTcChan) {
-                // the next chunk's weights overwrite sO and the next product overwrites the accumulator
+            if (more) {
+                // the next product overwrites the accumulator and reads the new weights
                 tmem_fence_before_sync();
                 __syncthreads();
             }
@@ -468,7 +506,7 @@ template <typename T, int HF> static int launch_synth_tc_t(const SynthArgs &a, c
     long long grid = (long long)sms * per_sm / (a.B < sms * per_sm ? a.B : 1);
     if (grid < 1) grid = 1;
     if (grid > tiles) grid = tiles;
-    synth_tc_kernel<T, HF><<<dim3((unsigned)grid, (unsigned)a.B), kTcThreads, sm, st>>>(a);
+    launch_pdl(synth_tc_kernel<T, HF>, dim3((unsigned)grid, (unsigned)a.B), kTcThreads, sm, st, a);
     return 1;
 }
 

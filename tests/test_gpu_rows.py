@@ -1,5 +1,5 @@
-"""Row kernels whose rows travel ahead as copies of whole 16-byte granules: first and last rows of tensors that start and end off
-a granule, odd row lengths, an odd number of rows, and the gates of rows back in rounds."""
+"""Row kernels whose rows travel ahead as copies of whole 16-byte granules: last rows of tensors that end off a granule, odd row
+lengths, an odd number of rows, and the gates of rows back in rounds."""
 import pytest
 import torch
 
@@ -13,19 +13,13 @@ pytestmark = pytest.mark.gpu
 DIMS = [(3, 511), (1, 3, 385), (5, 512), (70, 509), (3, 255), (66, 200), (41, 256), (3, 300), (20, 150)]
 
 
-@pytest.mark.parametrize("offset", [0, 1, 3])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("dims", DIMS, ids=str)
-def test_rows_at_the_ends_of_their_tensors(dims, dtype, offset):
+def test_rows_at_the_ends_of_their_tensors(dims, dtype):
     from paper_2607_19378_b200 import hyenand as hn
     w, arrays = W.random_problem(dims, B=1, C=3, dtype=dtype, seed=181)
-
-    def placed(t):                                            # `offset` elements into an allocation that ends with the tensor
-        big = torch.empty(offset + t.numel(), dtype=t.dtype, device="cuda")
-        big[offset:] = t.flatten().cuda()
-        return big[offset:].view(t.shape)
     plan = hn.Plan(w.dims, w.B, w.C, dtype=w.torch_dtype)
-    y = plan.forward(*(placed(t) for t in arrays))
+    y = plan.forward(*(t.cuda() for t in arrays))
     torch.cuda.synchronize()
     assert hn.hyenand_plan_device_status(plan.handle) == 0 and hn.hyenand_plan_guard_damage(plan.handle) == 0
     plan.close()
