@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int n = n0 + u * TPL;
-                    const bool oa = gq && n < p.len, ob = oa && has1;
+                    const bool oa = n < p.len, ob = oa && has1;
                     if (oa) HN_G(q0 + n, sizeof(T));
                     if (ob) HN_G(q1 + n, sizeof(T));
                     qa[u] = oa ? __ldg(q0 + n) : T(1.f);
@@ -340,8 +340,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) rows_inv_w_kernel(RowsInvArgs 
                 IO<T>::st(py, r0 * HP + l + t * TPL, z.x * qa[t]);
                 IO<T>::st(py, r1 * HP + l + t * TPL, z.y * qb[t]);
             }
+        } else if (pq) {
+            rows_out(pq, py);
         } else {
-            rows_out(pq, py);                              // (no gate tensor: the rows leave as they are)
+            // no gate tensor: the rows leave as they are
+            for (int n = l; n < p.len; n += TPL) {
+                const float2 z = at(n);
+                IO<T>::st(py, r0 * p.len + n, z.x);
+                if (has1) IO<T>::st(py, r1 * p.len + n, z.y);
+            }
         }
         if (p.y2) rows_out((const T *)p.q2, (T *)p.y2);    // second gate and result: the rows are still in the line
         __syncwarp(m);
