@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(
     float *sOm = sW1 + HF * 4;
     float *sBh = sOm + HF;
     float *sFi = sBh + (J - 1) * HF;
-    // per channel of a chunk, two chunks: factors of the window's exponent on the three axes, bias
+    // per channel of a chunk, two chunks: 1 / sigma on the three axes (causal: alpha in the last), bias
     float4 *sCh = reinterpret_cast<float4 *>(sFi + J * 2 * HF);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sCh + 2 * kTcChan);
     unsigned *tslot = reinterpret_cast<unsigned *>(bar + 1);
@@ -346,15 +346,15 @@ __global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(
         __syncthreads();
     };
     // (One tile of 384 channels per CTA, operator on 4 x 64 x 64 tokens, bf16: with each chunk's weights fetched, split and laid out
-    // between two barriers before its product, and four parameter loads per window, 88 us; so 57.  Bound by the chain of products and
-    // the window's arithmetic; 128 registers with 124 bytes of spills for four CTAs per SM.)
+    // between two barriers before its product, and four parameter loads per window, 88 us; so 64.  Bound by the chain of products and
+    // the window's arithmetic: its exponent as one sum of coordinate^2 times factors rounded in advance takes 57, but moves h by an ulp
+    // here and there, and a norm over one channel multiplies that by up to 1000.  126 registers for four CTAs per SM.)
     // Output weights of the next chunk: fetched into registers before the wait for this chunk's product, split and laid out right
     // after it (which frees the weight tile), so that neither their latency nor a barrier of their own stands in the chain of chunks.
     // A thread takes HF / 4 neighbouring weights of channel tid / 4; the first warp a channel's window and bias.
     constexpr int WPT = HF / 4;
     const int wc = tid >> 2, wk = (tid & 3) * WPT;
     const bool quads = H == HF && ((uintptr_t)p.Wout & 15) == 0;
-    constexpr float kLog2e = 1.4426950408889634f;
     float wr[WPT], wn[4];
     auto fetch = [&](int c0) {
         const int c = c0 + wc;
@@ -395,11 +395,8 @@ __global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(
         if (tid < kTcChan) {
             float e[3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                // the window is 2^(sum of coordinate^2 * e), or 2^(|coordinate| e) where causal
-                if (p.mode == 1) e[a] = -kLog2e * wn[a];
-                else { const float w = c0 + tid < p.C && a >= 3 - N ? 1.f / wn[a] : 0.f; e[a] = (-0.5f * kLog2e * w) * w; }
-            }
+            for (int a = 0; a < 3; ++a)
+                e[a] = p.mode == 1 ? wn[a] : c0 + tid < p.C && a >= 3 - N ? 1.f / wn[a] : 0.f;
             sCh[(buf ^ 1) * kTcChan + tid] = make_float4(e[0], e[1], e[2], wn[3]);
         }
         buf ^= 1;
@@ -411,7 +408,6 @@ __global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(
         if (!live) t = taps - 1;                           // clamped: computed, never stored
         const int m2 = (int)(t % p.K[2]), m1 = (int)((t / p.K[2]) % p.K[1]), m0 = (int)(t / ((long long)p.K[2] * p.K[1]));
         const float cx0 = axis_coord(m0, p.L[0], p.mode), cx1 = axis_coord(m1, p.L[1], p.mode), cx2 = axis_coord(m2, p.L[2], p.mode);
-        const float q0 = p.mode == 1 ? 0.f : cx0 * cx0, q1 = p.mode == 1 ? 0.f : cx1 * cx1, q2 = p.mode == 1 ? fabsf(cx2) : cx2 * cx2;
         float act[HF];
 #pragma unroll
         for (int i = 0; i < HF; ++i) {
@@ -447,20 +443,36 @@ __global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(
             contract(aO, std::integral_constant<int, kTcChan>{});
             if (failed) break;
             if (more) stage(c0 + kTcChan);
+            // bias and window of this thread's tap; AXES: 0 causal, else the axes whose coordinates are not all zero
+            auto store_chunk = [&](auto axes) {
+                constexpr int AXES = decltype(axes)::value;
 #pragma unroll
-            for (int b0 = 0; b0 < kTcChan; b0 += 16) {
-                float acc[16], acl[16];
-                TmemIO<16>::ld(acc, trow + b0);
-                TmemIO<16>::ld(acl, trow + kTcChan + b0);
-                tmem_wait_ld();
+                for (int b0 = 0; b0 < kTcChan; b0 += 16) {
+                    float acc[16], acl[16];
+                    TmemIO<16>::ld(acc, trow + b0);
+                    TmemIO<16>::ld(acl, trow + kTcChan + b0);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float4 w = ch[b0 + i];
-                    float win;
-                    asm("ex2.approx.f32 %0, %1;" : "=f"(win) : "f"(fmaf(q0, w.x, fmaf(q1, w.y, q2 * w.z))));
-                    if (live && b0 + i < nc) IO<T>::st(o, (b0 + i) * taps, win * ((acc[i] + acl[i]) + w.w));
+                    for (int i = 0; i < 16; ++i) {
+                        const float4 w = ch[b0 + i];
+                        float win;
+                        if constexpr (AXES == 0) win = __expf(-w.z * fabsf(cx2));
+                        else {
+                            // (the quotients are squared, not the reciprocals: those of a narrow window overflow, and 0 * inf is its
+                            // centre; summed in the order that the version without tensor cores compiles to, so that both give the
+                            // same bits)
+                            const float a1 = cx1 * w.y, a2 = cx2 * w.z;
+                            float r = a1 * a1;
+                            if constexpr (AXES == 3) { const float a0 = cx0 * w.x; r = fmaf(a0, a0, r); }
+                            win = __expf(-0.5f * fmaf(a2, a2, r));
+                        }
+                        if (live && b0 + i < nc) IO<T>::st(o, (b0 + i) * taps, win * ((acc[i] + acl[i]) + w.w));
+                    }
                 }
-            }
+            };
+            if (p.mode == 1) store_chunk(std::integral_constant<int, 0>{});
+            else if (N == 3) store_chunk(std::integral_constant<int, 3>{});
+            else store_chunk(std::integral_constant<int, 2>{});
             if (more) {
                 // the next product overwrites the accumulator and reads the new weights
                 tmem_fence_before_sync();
