@@ -251,7 +251,7 @@ template <typename T, int HF>
 __global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(SynthArgs p)
 {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    pdl_join();
+    pdl_wait();
     // the swizzle pattern is a function of the shared-memory address: tiles start on 1024-byte boundaries
     unsigned char *sm = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
     const int J = p.layers, H = p.hidden, N = p.ndim;
@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(kTcThreads, HF <= 32 ? 4 : 2) synth_tc_kernel(
     tmem_fence_before_sync();
     __syncthreads();
     tmem_fence_after_sync();
+    pdl_trigger();                                         // (after tensor memory: see pdl_join)
     const unsigned tbase = *tslot;
     const unsigned trow = tmem_addr(tbase, warp, 0);       // this thread's lane, column 0
     const unsigned aB = smem_u32(sB), aO = smem_u32(sO);
