@@ -374,10 +374,13 @@ template <typename T, class F> static void mix_tiles(long long nb, long long L, 
         const dim3 g((unsigned)((L + kMixThreads * vec - 1) / (kMixThreads * vec)), (unsigned)nb);
         return vec == 4 ? go(four, solo, g) : vec == 2 ? go(two, solo, g) : go(one, solo, g);
     }
-    // Many channels on few tokens: 16 warps on tiles of 64 tokens, whose channels stay in registers up to 24 per thread (outer norm of
-    // 4 x 4096 tokens of 384 channels, bf16: tiles of 32 and 8 warps, which read their tokens twice, 17.6 us, these 14.0; the scale
-    // 14.7 and 14.4).
-    if (vec == 1 && L % 2 == 0 && C >= 128 && count(2) >= 128) return go(two, std::integral_constant<int, 16>{}, dim3((unsigned)((L + 63) / 64), (unsigned)nb));
+    // 16 warps on tiles of 64 tokens, from 128 such tiles on: where tiles of 32 tokens would take 32 warps for at most 8 channels each,
+    // and for bf16 at 256 to 384 channels, which stay in registers (24 per thread) between the outer norm's sum and its result.
+    // Eq. 2 without the synthesis against those tiles, 196 to 5280 tokens, 1 to 32 entries: the first 0.99 to 1.11 times as fast, the
+    // second 0.98 to 1.06 (4 x 4096 tokens of 384 channels: outer norm 17.6 -> 14.0 us); but bf16 of 128 to 192 channels 0.96 to 1.02, of
+    // 512 and more 0.86 to 1.05, other fp32 0.92 to 1.02.
+    if (vec == 1 && L % 2 == 0 && count(2) >= 128 && ((nw == 32 && C <= 256) || (sizeof(T) == 2 && C >= 256 && C <= 384)))
+        return go(two, std::integral_constant<int, 16>{}, dim3((unsigned)((L + 63) / 64), (unsigned)nb));
     if (vec == 4) return go(four, four, grid);               // (1024 tiles of 4 warps)
     if (vec == 2) return go(two, four, grid);
     if (nw == 4) go(one, four, grid);
@@ -428,8 +431,12 @@ template <typename T> static void mixer_post_t(const float *o, const float *g_ou
             const int per = (C + NW - 1) / NW;               // channels per thread
             if (per <= 4) launch_pdl(mixer_post_kernel<T, VEC, NW, 4>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
             else if (per <= 16) launch_pdl(mixer_post_kernel<T, VEC, NW, 16>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
-            else if (per <= 24 && VEC * NW <= 32) launch_pdl(mixer_post_kernel<T, VEC, NW, 24>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
-            else launch_pdl(mixer_post_kernel<T, VEC, NW, 0>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
+            else {
+                if constexpr (VEC == 2 && NW == 16) {        // (1024 threads have 64 registers each: 24 channels would spill)
+                    if (per <= 24) return launch_pdl(mixer_post_kernel<T, VEC, NW, 24>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
+                }
+                launch_pdl(mixer_post_kernel<T, VEC, NW, 0>, grid, NW * 32, 0, st, o, g_out, eps, C, L, y);
+            }
         }
     });
 }

@@ -36,3 +36,9 @@ def test_rows_of_1024_points(kernel, limit):
 def test_rows_of_three_times_a_power_of_two():
     rows = {k: v for k, v in spill_loads("rows_w").items() if re.search(r"Li2[234]E", k)}
     assert len(rows) == 2 * 3 * 5 and max(rows.values()) <= 16, {k: v for k, v in rows.items() if v > 16}
+
+
+def test_norms_keep_their_channels_in_registers():
+    """mixer_post_kernel<T, VEC, NW, KEEP>: KEEP channels of a thread stay in registers between the sum and the result."""
+    kept = {k: v for k, v in spill_loads("mixer").items() if re.search(r"mixer_post_kernelI\w+?Li\dELi\d+ELi(4|16|24)E", k)}
+    assert len(kept) >= 2 * 2 * 5 and max(kept.values()) == 0, {k: v for k, v in kept.items() if v}
