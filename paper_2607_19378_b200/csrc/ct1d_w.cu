@@ -6,11 +6,12 @@
 //                one warp-group per column pair: transform along t1 (upper half of the
 //                padded input is zero), separate the two real columns, multiply by the
 //                inter-pass twiddle, coalesced store of [f1][t2].
-//   hspec_w      per-sample filters only: transform each kept row along t2 in place and fold in 1/P.
+//   hspec_w      per-sample filters, and shared ones where a group holds no whole batch entry: transform each kept
+//                row along t2 in place and fold in 1/P.
 //   core_w       one warp-group per row: transform along t2, multiply by the filter
 //                spectrum (Eq. 12), inverse transform chained in registers, undo twiddle.  The
 //                rows of a filter shared over the batch are transformed here, once per group of
-//                batch entries.
+//                the slices that it serves.
 //   cols_inv_w   rebuild the mirrored half, inverse along f1 keeping t < P/2, crop, gate
 //                with q, coalesced store.
 #include <type_traits>
@@ -343,9 +344,17 @@ struct CoreWArgs {
     long long h_mod, h_off;
     const float2 *tw2;
     TwoLevelW twp;
-    // FILT only: a unit is one row of the filter of channel c and the same row of the batch entries it serves
-    int nb;                   // batch entries per unit
+    // FILT only: a unit is one row of a channel's filter and the same row of the slices it serves
+    int nb;                   // slices per unit
     float scale;              // 1/P, folded into the filter's spectrum
+    // The slices are a range of the batch that need not be whole entries: slice s has the filter of channel (s + h_off) % h_mod, so
+    // the first `channels` of them have a filter each, and slice i + j * channels that of slice i.
+    __host__ __device__ long long channels() const { return slices < h_mod ? slices : h_mod; }
+    __host__ __device__ long long units(int n) const       // with n slices per unit; units of no slice come last and are left out
+    {
+        const long long c = channels(), step = c * n, full = (slices - 1) / step, rest = slices - full * step;
+        return (full * c + (rest < c ? rest : c)) * f1n;
+    }
 };
 
 // Twiddles of a pass from tensor memory (they depend on the lane only): 16 columns, 8 legs, at a time.
@@ -363,9 +372,9 @@ struct TmemTw {
 };
 
 // FILT (a filter shared over the batch): a lane group transforms a row of the filter itself, parks the spectrum in its own
-// lanes of tensor memory and takes the row of nb batch entries through it, so the filter crosses HBM once and its spectrum
+// lanes of tensor memory and takes the row of nb slices of its channel through it, so the filter crosses HBM once and its spectrum
 // never.  In shared memory the spectra of 16 warps (8 KB each) do not fit beside their lines; in registers 64 more per thread
-// leave 8 warps per SM.  262144 bf16 values, 2 x 256 rows: 167 us in a kernel of the filter's own plus 525 here, now 600.  Bound by
+// leave 8 warps per SM.  262144 bf16 values, 2 x 256 rows: 167 us in a kernel of the filter's own plus 525 here, now 595.  Bound by
 // instruction issue (60 % of the slots) and instruction fetch of the unrolled passes.  Three CTAs of four warps with twiddles in
 // registers and rows that travel ahead as untiled copies: 662.
 template <int LOG2P2, bool FILT>
@@ -513,22 +522,23 @@ __global__ void __launch_bounds__(256, 2) ct_core_w_kernel(CoreWArgs p)
             });
         }
     } else {
-        // slices [h_off, h_off + slices) of the batch counted from its first entry here: slice b * h_mod + c
-        const long long entries = (p.h_off + p.slices + p.h_mod - 1) / p.h_mod, chunks = (entries + p.nb - 1) / p.nb;
-        const long long per = p.h_mod * p.f1n, units = chunks * per;
+        const long long ch = p.channels(), per = ch * p.f1n, units = p.units(p.nb);
         constexpr int LPW = 32 / TPL;
         // (a warp's groups go round together: tensor memory is reached by whole warps)
         for (long long u0 = (long long)blockIdx.x * G + warp * LPW; u0 < units; u0 += (long long)gridDim.x * G) {
             const long long u = u0 + (gid - warp * LPW);
             const bool live = u < units;
-            const long long b0 = live ? u / per * p.nb : 0;
-            const int rc = live ? (int)(u % per) : 0, c = rc / p.f1n, f1 = rc % p.f1n;
+            const long long s0 = live ? u / per * p.nb * ch : 0;
+            const int rc = live ? (int)(u % per) : 0, i = rc / p.f1n, f1 = rc % p.f1n;
+            const float2 *hrow = p.h + ((i + p.h_off) % p.h_mod * p.f1n + f1) * P2;
+            float2 *const row0 = p.u + (s0 * p.f1n + rc) * P2;
+            const long long left = live ? p.slices - s0 - i : -ch;
 #pragma unroll 1
             for (int j = -1; j < p.nb; ++j) {
-                const long long s = (b0 + j) * p.h_mod + c - p.h_off;
-                const bool first = j < 0, on = live && (first || (s >= 0 && s < p.slices));
-                float2 *row = p.u + (s * p.f1n + f1) * P2;
-                row_through(first ? p.h + (long long)rc * P2 : row, row, f1, on, first,
+                const bool first = j < 0, on = j * ch < left;
+                if (!__any_sync(0xffffffffu, on)) break;
+                float2 *row = row0 + j * per * P2;
+                row_through(first ? hrow : row, row, f1, on, first,
                     [&](X &H) {
                         __syncwarp();
 #pragma unroll
@@ -923,12 +933,12 @@ template <int LOG2P2> static int launch_rows_w_t(const HspecArgs *hs, const Core
     CoreWArgs c{};
     if (co) c = *co;
     if (co && c.scale != 0.f) {
-        // the count of batch entries per unit with the least work in the busiest slot: a transform for the filter, two per entry
-        const long long be = (c.h_off + c.slices + c.h_mod - 1) / c.h_mod;
+        // the count of slices per unit with the least work in the busiest slot: a transform for the filter, two per slice
+        const long long most = (c.slices + c.channels() - 1) / c.channels();
         long long best = -1;
-        for (long long nb = 1; nb <= be && nb <= 64; ++nb) {
-            const long long un = (be + nb - 1) / nb * c.h_mod * c.f1n, cost = ((un + slots - 1) / slots) * (1 + 2 * nb);
-            if (best < 0 || cost < best) { best = cost; c.nb = (int)nb; units = un; }
+        for (int nb = 1; nb <= most && nb <= 64; ++nb) {
+            const long long un = c.units(nb), cost = ((un + slots - 1) / slots) * (1 + 2 * nb);
+            if (best < 0 || cost < best) { best = cost; c.nb = nb; units = un; }
         }
     }
     const long long want = (units + G - 1) / G;
@@ -955,7 +965,7 @@ static int launch_rows_w(int log2p2, const HspecArgs *hs, const CoreWArgs *co, c
     return n;
 }
 
-int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool shared, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
+int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool in_core, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
                   int (*fallback)(Ct1dPlan *, const char *, long long, cudaStream_t, int *, Prof *))
 {
     const TwoLevelW twp{c->twp_coarse, c->twp_fine, c->lo};
@@ -976,7 +986,7 @@ int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool shared, bool sta
     } else if (fallback(c, (const char *)h, n, st, launches, prof)) {
         return -1;
     }
-    if (shared) return 0;                                  // the core transforms the rows of a shared filter itself
+    if (in_core) return 0;                                 // the core transforms the rows of a shared filter itself
     HspecArgs hs{};
     hs.h = c->wh; hs.rows = n * ((1 << c->log2p1) / 2 + 1); hs.scale = (float)ldexp(1.0, -c->log2p); hs.tw2 = c->tw2;
     prof->begin(KID_CT_HSPEC, st);
@@ -987,7 +997,7 @@ int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool shared, bool sta
     return 0;
 }
 
-int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, long long s0,
+int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, bool in_core, long long s0,
                 void *y, cudaStream_t st, int *launches, Prof *prof)
 {
     const TwoLevelW twp{c->twp_coarse, c->twp_fine, c->lo};
@@ -1007,7 +1017,7 @@ int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long l
     CoreWArgs co{};
     co.u = c->wu; co.h = c->wh; co.slices = n; co.f1n = (1 << c->log2p1) / 2 + 1;
     co.h_mod = shared ? c->C : 0; co.h_off = shared ? s0 % c->C : 0;
-    co.scale = shared ? (float)ldexp(1.0, -c->log2p) : 0.f;
+    co.scale = in_core ? (float)ldexp(1.0, -c->log2p) : 0.f;
     co.tw2 = c->tw2; co.twp = twp;
     prof->begin(KID_CT_CORE, st);
     r = launch_rows_w(c->log2p2, nullptr, &co, st);
