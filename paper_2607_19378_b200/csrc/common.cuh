@@ -161,6 +161,7 @@ struct DevOnce {
 // created, and travel with the plan: a forward call never looks at the environment.
 struct Switches {
     bool force_generic, generic_rows, generic_core, no_tma;
+    bool refuse_maps;                 // HYENAND_REFUSE_MAPS: as if the driver took no tensor map of a long 1-D plan's workspace
     bool nvtx;                        // HYENAND_NVTX: name every kernel launch with an NVTX range
 };
 Switches read_switches();

@@ -399,6 +399,7 @@ int ct1d_init(Ct1dPlan *c, int L, int K, int log2p, int B, int C, int causal, in
     need = sizeof(float2) * per_slice * c->wh_slices;
     if (guarded_alloc(g, (void **)&c->wh, need) != cudaSuccess) { cudaGetLastError(); *bytes = need; return 3; }
     *bytes += need;
+    c->maps_ok = !sw.refuse_maps && ct1d_w_maps(c);
     return 0;
 }
 
@@ -472,8 +473,9 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
 }
 
 // Both kernel families take either element type in every stage; the warp-engine kernels serve every length they have an
-// instance for (padded 2^14 .. 2^20), longer ones and the development switches take the block-wide kernels.
-bool ct1d_uses_w(const Ct1dPlan *c) { return !c->sw.force_generic && !c->sw.no_tma && ct1d_w_supported(c->log2p1, c->log2p2); }
+// instance for (padded 2^14 .. 2^20); longer ones, a driver that takes no tensor maps of the workspace, and the development switches
+// leave the block-wide kernels.
+bool ct1d_uses_w(const Ct1dPlan *c) { return !c->sw.force_generic && !c->sw.no_tma && c->maps_ok; }
 
 // Where a group holds no whole batch entry and the batch has several, the core would transform every filter once per entry: there
 // the spectra are made once (3 x 800 rows of 262144 bf16 values in groups of 765: filters in the core 8619 us, spectra made once 6598).

@@ -19,6 +19,7 @@ struct Ct1dPlan {
     int lo;
     int *status;              // device word set when a bounded wait on a tensor copy gives up (owned by the plan)
     Switches sw;              // development switches, read when the plan was created
+    bool maps_ok;             // the driver takes tensor maps of wu and wh as the warp-engine kernels want them
     long long slices_per_chunk, wh_slices;
     long long r0, r1;         // slices [r0, r1) the next forward works on
     int dt_in, dt_out, dt_h;  // element types of k and v, of the gate q and the result y, of the taps h for the next forward
@@ -39,6 +40,7 @@ bool ct1d_filter_in_core(const Ct1dPlan *c);    // the core kernel transforms th
 
 // warp-engine kernels (ct1d_w.cu)
 bool ct1d_w_supported(int log2p1, int log2p2);
+bool ct1d_w_maps(const Ct1dPlan *c);
 int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool in_core, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
                   int (*fallback)(Ct1dPlan *, const char *, long long, cudaStream_t, int *, Prof *));
 int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, bool in_core, long long s0,

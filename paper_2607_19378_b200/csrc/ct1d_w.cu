@@ -841,6 +841,20 @@ template <class G> static bool spectra_map(CUtensorMap *m, const float2 *base, i
     return tma_encode_3d_cached(m, base, false, dims, strides, box, (int)G::ROWB);
 }
 
+// Whether the maps of a plan's workspace can be had.  They are made anew in each call, for the slices it works on; the address,
+// strides and box are these.
+bool ct1d_w_maps(const Ct1dPlan *c)
+{
+    if (!ct1d_w_supported(c->log2p1, c->log2p2)) return false;
+    const int P2 = 1 << c->log2p2;
+    alignas(64) CUtensorMap m;
+    bool ok = false;
+#define CALLM(L) ok = spectra_map<CtGeo<float, L>>(&m, c->wu, P2, c->slices_per_chunk) && spectra_map<CtGeo<float, L>>(&m, c->wh, P2, c->wh_slices)
+    switch (c->log2p1) { case 7: CALLM(7); break; case 8: CALLM(8); break; case 9: CALLM(9); break; case 10: CALLM(10); break; }
+#undef CALLM
+    return ok;
+}
+
 // A tensor whose slices are whole numbers of rows of P2 elements, so that [slice][row][P2] is an exact view of it and rows past the
 // data read as zeros; false where tensor copies do not apply.
 template <class G, typename T> static bool rows_map(CUtensorMap *m, const void *base, int len, long long slice_elems, int P2, long long slices)

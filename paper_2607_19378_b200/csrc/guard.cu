@@ -19,6 +19,7 @@ Switches read_switches()
     s.generic_rows = getenv("HYENAND_GENERIC_ROWS") != nullptr;
     s.generic_core = getenv("HYENAND_GENERIC_CORE") != nullptr;
     s.no_tma = getenv("HYENAND_NO_TMA") != nullptr;
+    s.refuse_maps = getenv("HYENAND_REFUSE_MAPS") != nullptr;
     s.nvtx = getenv("HYENAND_NVTX") != nullptr;
     return s;
 }

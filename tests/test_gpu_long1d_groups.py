@@ -67,3 +67,11 @@ def test_host_call_in_groups_has_the_same_bits(L, B, C):
     hn.hyenand_forward_host(plan.handle, hq, hk, hv, hh, 0, hy)
     plan.close()
     assert torch.equal(hy, y.cpu())
+
+
+@pytest.mark.parametrize("dtype,shared", [("f32", True), ("bf16", False)])
+def test_a_driver_that_takes_no_map_of_the_workspace(dtype, shared):
+    """Such a plan runs on the kernels without tensor copies; it is not an error."""
+    from parity_util import check
+    w, arrays = W.random_problem((20000,), B=2, C=2, dtype=dtype, causal=True, h_shared=shared, seed=222)
+    check(w, *arrays, env={"HYENAND_REFUSE_MAPS": "1"})
