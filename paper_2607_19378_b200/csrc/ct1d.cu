@@ -424,14 +424,14 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
     const size_t ei = c->dt_in == 0 ? 4 : 2, eo = c->dt_out == 0 ? 4 : 2, eh = c->dt_h == 0 ? 4 : 2;
     const TwoLevel twp{c->twp_coarse, c->twp_fine, c->lo};
     if (ct1d_uses_w(c)) {
-        const bool staged_ok = c->causal != 0, in_core = shared && ct1d_filter_in_core(c);
-        if (shared && c->r0 == 0 && !c->keep_filter && ct1d_w_filter(c, h, c->C, in_core, staged_ok, st, launches, prof, filter_pass)) return -1;
+        const bool staged_ok = c->causal != 0;
+        if (shared && c->r0 == 0 && !c->keep_filter && ct1d_w_filter(c, h, c->C, true, staged_ok, st, launches, prof, filter_pass)) return -1;
         for (long long s0 = c->r0; s0 < c->r1; s0 += c->slices_per_chunk) {
             const long long n = c->r1 - s0 < c->slices_per_chunk ? c->r1 - s0 : c->slices_per_chunk;
             if (!shared && ct1d_w_filter(c, (const char *)h + (size_t)s0 * c->K * eh, n, false, staged_ok, st, launches, prof, filter_pass))
                 return -1;
             if (ct1d_w_body(c, (const char *)q + (size_t)s0 * c->L * eo, (const char *)k + (size_t)s0 * c->L * ei,
-                            v ? (const char *)v + (size_t)s0 * c->L * ei : nullptr, n, shared, in_core, s0, (char *)y + (size_t)s0 * c->L * eo,
+                            v ? (const char *)v + (size_t)s0 * c->L * ei : nullptr, n, shared, s0, (char *)y + (size_t)s0 * c->L * eo,
                             st, launches, prof))
                 return -1;
         }
@@ -477,16 +477,11 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
 // leave the block-wide kernels.
 bool ct1d_uses_w(const Ct1dPlan *c) { return !c->sw.force_generic && !c->sw.no_tma && c->maps_ok; }
 
-// Where a group holds no whole batch entry and the batch has several, the core would transform every filter once per entry: there
-// the spectra are made once (3 x 800 rows of 262144 bf16 values in groups of 765: filters in the core 8619 us, spectra made once 6598).
-// A rule on the plan and not on the range of a call, whose bits it must not depend on.
-bool ct1d_filter_in_core(const Ct1dPlan *c) { return ct1d_uses_w(c) && (c->slices_per_chunk >= c->C || c->B == 1); }
-
 int ct1d_launches(const Ct1dPlan *c, bool shared)
 {
     const long long S = (long long)c->B * c->C;
     const long long chunks = (S + c->slices_per_chunk - 1) / c->slices_per_chunk;
-    if (ct1d_uses_w(c)) return (int)(shared ? (ct1d_filter_in_core(c) ? 1 : 2) + 3 * chunks : 5 * chunks);
+    if (ct1d_uses_w(c)) return (int)(shared ? 1 + 3 * chunks : 5 * chunks);
     return (int)(shared ? 1 + 3 * chunks : 4 * chunks);
 }
 

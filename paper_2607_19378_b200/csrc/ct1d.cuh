@@ -25,8 +25,8 @@ struct Ct1dPlan {
     int dt_in, dt_out, dt_h;  // element types of k and v, of the gate q and the result y, of the taps h for the next forward
                               // (all equal to dtype unless the caller of ct1d_forward sets them: every stage takes its
                               // element type per launch)
-    int keep_filter;          // 1: the column transforms (or spectra: ct1d_filter_in_core) of the shared filter are still in wh from
-                              // this plan's previous forward (same taps): the next forward does not transform it again
+    int keep_filter;          // 1: the column transforms of the shared filter are still in wh from this plan's previous forward
+                              // (same taps): the next forward does not transform it again
 };
 
 // allocations go on the plan's guarded list `g` and are freed with it
@@ -36,14 +36,13 @@ int ct1d_forward(Ct1dPlan *c, const void *q, const void *k, const void *v, const
                  void *y, cudaStream_t st, int *launches, Prof *prof);
 int ct1d_launches(const Ct1dPlan *c, bool shared);
 bool ct1d_uses_w(const Ct1dPlan *c);
-bool ct1d_filter_in_core(const Ct1dPlan *c);    // the core kernel transforms the rows of a filter shared over the batch itself
 
 // warp-engine kernels (ct1d_w.cu)
 bool ct1d_w_supported(int log2p1, int log2p2);
 bool ct1d_w_maps(const Ct1dPlan *c);
-int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool in_core, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
+int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool shared, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
                   int (*fallback)(Ct1dPlan *, const char *, long long, cudaStream_t, int *, Prof *));
-int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, bool in_core, long long s0,
+int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, long long s0,
                 void *y, cudaStream_t st, int *launches, Prof *prof);
 
 }  // namespace hn

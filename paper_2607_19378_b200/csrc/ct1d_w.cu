@@ -6,8 +6,7 @@
 //                one warp-group per column pair: transform along t1 (upper half of the
 //                padded input is zero), separate the two real columns, multiply by the
 //                inter-pass twiddle, coalesced store of [f1][t2].
-//   hspec_w      per-sample filters, and shared ones where a group holds no whole batch entry: transform each kept
-//                row along t2 in place and fold in 1/P.
+//   hspec_w      per-sample filters only: transform each kept row along t2 in place and fold in 1/P.
 //   core_w       one warp-group per row: transform along t2, multiply by the filter
 //                spectrum (Eq. 12), inverse transform chained in registers, undo twiddle.  The
 //                rows of a filter shared over the batch are transformed here, once per group of
@@ -376,7 +375,8 @@ struct TmemTw {
 // never.  In shared memory the spectra of 16 warps (8 KB each) do not fit beside their lines; in registers 64 more per thread
 // leave 8 warps per SM.  262144 bf16 values, 2 x 256 rows: 167 us in a kernel of the filter's own plus 525 here, now 595.  Bound by
 // instruction issue (60 % of the slots) and instruction fetch of the unrolled passes.  Three CTAs of four warps with twiddles in
-// registers and rows that travel ahead as untiled copies: 662.
+// registers and rows that travel ahead as untiled copies: 662.  Filters of which no group holds all (3 x 800 rows of 262144 values in groups
+// of 765, 2 x 390 of 524288 in groups of 383) are transformed once per slice; spectra made once and read here: 6517 -> 6567 us, 4894 -> 5079.
 template <int LOG2P2, bool FILT>
 __global__ void __launch_bounds__(256, 2) ct_core_w_kernel(CoreWArgs p)
 {
@@ -979,7 +979,7 @@ static int launch_rows_w(int log2p2, const HspecArgs *hs, const CoreWArgs *co, c
     return n;
 }
 
-int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool in_core, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
+int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool shared, bool staged_ok, cudaStream_t st, int *launches, Prof *prof,
                   int (*fallback)(Ct1dPlan *, const char *, long long, cudaStream_t, int *, Prof *))
 {
     const TwoLevelW twp{c->twp_coarse, c->twp_fine, c->lo};
@@ -1000,7 +1000,7 @@ int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool in_core, bool st
     } else if (fallback(c, (const char *)h, n, st, launches, prof)) {
         return -1;
     }
-    if (in_core) return 0;                                 // the core transforms the rows of a shared filter itself
+    if (shared) return 0;                                  // the core transforms the rows of a shared filter itself
     HspecArgs hs{};
     hs.h = c->wh; hs.rows = n * ((1 << c->log2p1) / 2 + 1); hs.scale = (float)ldexp(1.0, -c->log2p); hs.tw2 = c->tw2;
     prof->begin(KID_CT_HSPEC, st);
@@ -1011,7 +1011,7 @@ int ct1d_w_filter(Ct1dPlan *c, const void *h, long long n, bool in_core, bool st
     return 0;
 }
 
-int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, bool in_core, long long s0,
+int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long long n, bool shared, long long s0,
                 void *y, cudaStream_t st, int *launches, Prof *prof)
 {
     const TwoLevelW twp{c->twp_coarse, c->twp_fine, c->lo};
@@ -1031,7 +1031,7 @@ int ct1d_w_body(Ct1dPlan *c, const void *q, const void *k, const void *v, long l
     CoreWArgs co{};
     co.u = c->wu; co.h = c->wh; co.slices = n; co.f1n = (1 << c->log2p1) / 2 + 1;
     co.h_mod = shared ? c->C : 0; co.h_off = shared ? s0 % c->C : 0;
-    co.scale = in_core ? (float)ldexp(1.0, -c->log2p) : 0.f;
+    co.scale = shared ? (float)ldexp(1.0, -c->log2p) : 0.f;
     co.tw2 = c->tw2; co.twp = twp;
     prof->begin(KID_CT_CORE, st);
     r = launch_rows_w(c->log2p2, nullptr, &co, st);

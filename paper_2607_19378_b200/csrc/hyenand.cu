@@ -1116,15 +1116,15 @@ extern "C" int hyenand_plan_kernel_info(const hyenand_plan *p, int kid, int h_sh
             if (ct1d_uses_w(&c)) {
                 // (a shared filter's rows are read and transformed here, else its spectra are read)
                 *launches = chunks; *bytes = (2 * S + Sh) * F1 * P2 * c8;
-                *flops = 2 * fft_flops(S * F1, c.log2p2) + 12.0 * S * F1 * P2 + (h_shared && ct1d_filter_in_core(&c) ? fft_flops(Sh * F1, c.log2p2) : 0.0);
+                *flops = 2 * fft_flops(S * F1, c.log2p2) + 12.0 * S * F1 * P2 + (h_shared ? fft_flops(Sh * F1, c.log2p2) : 0.0);
             } else {
                 *launches = chunks; *bytes = S * 3 * F1 * P2 * c8;
                 *flops = 3 * fft_flops(S * F1, c.log2p2) + 12.0 * S * F1 * P2;
             }
             break;
         case KID_CT_HSPEC:
-            if (ct1d_uses_w(&c) && !(h_shared && ct1d_filter_in_core(&c))) {
-                *launches = h_shared ? 1 : chunks; *bytes = Sh * 2 * F1 * P2 * c8;
+            if (ct1d_uses_w(&c) && !h_shared) {
+                *launches = chunks; *bytes = Sh * 2 * F1 * P2 * c8;
                 *flops = fft_flops(Sh * F1, c.log2p2);
             }
             break;
