@@ -60,17 +60,17 @@ __device__ __forceinline__ void prefetch_rows_l2(const unsigned char *lo, const 
 // LATE: the twiddles a lane keeps in registers are read after the wait for the preceding kernel instead of before it.  The
 // compiler sinks such reads to where they are used when registers run out, but not past the wait: at 1024 points (32 x 32, 62
 // registers of twiddles, 128 in all) reading them early costs spills in every row pair (fp32, bytes of spill loads per thread:
-// k v rows 200 -> 256, rows back 136 -> 184; a forward of 512 x 512 grids 2654 -> 2701 us, late 2656).  Grids of fewer CTAs than SMs
+// staged k v rows 200 -> 256, rows back 136 -> 184; a forward of 512 x 512 grids 2654 -> 2701 us, late 2656).  Grids of fewer CTAs than SMs
 // start while their predecessor runs and gain more from early reads: one 500 x 500 grid 38.0 us late, 33.7 early.
 // AHEAD: a group's next rows travel by untiled copies into a buffer of its own while it works on the present ones; CTAs of four
 // warps, three per SM, with the twiddles of the second pass in registers.  Else the rows arrive in the group's line and the group
 // waits for them: CTAs of eight warps, two per SM.  Ahead at 1024 points (128 slices of 512x512, filter rows and k*v rows: fp32 206
 // and 102 us -> 184 and 91, bf16 190 and 94 -> 165 and 85) and for fp32 at 512 (57 and 32 -> 54 and 31); not for bf16 at 512 (52 and
 // 29 -> 53 and 32) and below (256 points: 63 and 35 -> 70 and 38), whose rows are a few hundred bytes and whose waits 16 warps cover.
-template <typename T, int LOG2P, int MODE> struct RowFwdGeo {
+template <typename T, int LOG2P, int MODE> constexpr bool kAheadRows = MODE != 3 && (LOG2P == 10 || (LOG2P == 9 && sizeof(T) == 4));
+template <typename T, int LOG2P, int MODE, bool AHEAD> struct RowFwdGeo {
     using F = WF<LOG2P, false>;
     static constexpr int P = len_of(LOG2P), HP = P / 2, TPL = F::TPL;
-    static constexpr bool AHEAD = MODE != 3 && (LOG2P == 10 || (LOG2P == 9 && sizeof(T) == 4));
     static constexpr int THREADS = AHEAD ? 128 : kRowThreads, PER_SM = AHEAD ? 3 : 2;
     static constexpr int G = THREADS / TPL, LS = plane_ls(P);
     static constexpr int NT = MODE == 0 ? 2 : 1;                                // tensors per row
@@ -83,13 +83,12 @@ template <typename T, int LOG2P, int MODE> struct RowFwdGeo {
     static_assert(G * LS >= P, "the lines hold the twiddle table at first");
 };
 
-template <typename T, int LOG2P, int MODE, bool LATE>
-__global__ void __launch_bounds__(RowFwdGeo<T, LOG2P, MODE>::THREADS, RowFwdGeo<T, LOG2P, MODE>::PER_SM) rows_fwd_w_kernel(RowsArgs p)
+template <typename T, int LOG2P, int MODE, bool LATE, bool AHEAD>
+__global__ void __launch_bounds__(RowFwdGeo<T, LOG2P, MODE, AHEAD>::THREADS, RowFwdGeo<T, LOG2P, MODE, AHEAD>::PER_SM) rows_fwd_w_kernel(RowsArgs p)
 {
-    using GE = RowFwdGeo<T, LOG2P, MODE>;
+    using GE = RowFwdGeo<T, LOG2P, MODE, AHEAD>;
     using F = typename GE::F;
     constexpr int P = GE::P, HP = GE::HP, TPL = GE::TPL, G = GE::G, LS = GE::LS, THREADS = GE::THREADS;
-    constexpr bool AHEAD = GE::AHEAD;
     constexpr int PR = (MODE == 1 || MODE == 3) ? PRUNE_NONE : PRUNE_IN;
     constexpr int NT = GE::NT, ROWMAX = GE::ROWMAX, SLOT = GE::SLOT;
     extern __shared__ __align__(128) unsigned char smem_dyn[];
@@ -114,7 +113,8 @@ __global__ void __launch_bounds__(RowFwdGeo<T, LOG2P, MODE>::THREADS, RowFwdGeo<
     const unsigned char *ab = (const unsigned char *)p.a, *bb = (const unsigned char *)p.b;
     const unsigned char *ahi = ab + p.rows * (long long)p.len * sizeof(T);
     const unsigned char *bhi = bb + p.rows * (long long)p.len * sizeof(T);
-    const long long pairs = (p.rows + 1) / 2, step = (long long)gridDim.x * G;
+    const long long pairs = (p.rows + 1) / 2;
+    auto after = [&](long long rp) { return rp + (long long)gridDim.x * G; };      // (a step held in registers costs 8 bytes of spills)
     const int rowb = p.len * (int)sizeof(T);
     // lane j < 2 NT fetches row j of the pair: a0, a1, b0, b1
     auto ask = [&](long long rp) {
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(RowFwdGeo<T, LOG2P, MODE>::THREADS, RowFwdGeo<
             F::template pass<0, PR>(l, tw, in, [&](int, int, int idx, float2 v) { line[F::ph(idx)] = v; });
             fence_async_smem();                            // (blanked and ragged elements, before the copies that follow)
             __syncwarp(m);
-            ask(rp + step);
+            ask(after(rp));
             F::template mid<1, F::NP>(l, m, tw, line);
         } else {
             F::template run_to_line<PR, MODE != 3>(l, m, tw, line, in);
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(RowFwdGeo<T, LOG2P, MODE>::THREADS, RowFwdGeo<
     int failed = 0;
     long long rp = (long long)blockIdx.x * G + gid;
     if constexpr (AHEAD) ask(rp);
-    for (; rp < pairs; rp += step, phase ^= 1u) {
+    for (; rp < pairs; rp = after(rp), phase ^= 1u) {
         const long long r0 = 2 * rp, r1 = r0 + 1;
         const bool has1 = r1 < p.rows;
         if constexpr (MODE == 3) {
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(RowFwdGeo<T, LOG2P, MODE>::THREADS, RowFwdGeo<
                 if (MODE != 1 && l == 0) {
                     // the k and v rows this group takes next travel to L2 while it works on these (measured: a gain for
                     // the short k*v rows, none for the long filter rows)
-                    const long long rn = 2 * (rp + step);
+                    const long long rn = 2 * after(rp);
                     if (rn + 1 < p.rows) {
                         prefetch_rows_l2(ab + rn * rowb, ab + (rn + 2) * rowb);
                         if (MODE == 0) prefetch_rows_l2(bb + rn * rowb, bb + (rn + 2) * rowb);
@@ -367,9 +367,9 @@ static int rows_sms()
     return n;
 }
 
-// length and grid size from which the kernels take their LATE variant
+// length and grid size from which the kernels take their LATE variant (rows ahead have none: no spills either way)
 template <int LOG2P> constexpr bool kLateRows = LOG2P == 10;
-static bool late_rows(int grid) { return grid >= rows_sms(); }
+static bool late_rows(long long ctas) { return ctas >= rows_sms(); }
 
 bool rows_w_supported(int log2p) { return (log2p >= 6 && log2p <= 10) || (log2p >= kLen192 && log2p <= kLen768); }
 
@@ -377,19 +377,25 @@ template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &
 {
     constexpr int P = len_of(LOG2P);
     if (a.rows <= 0) return 0;
-    auto go = [&](auto mode, auto late, int grid) {
-        using GE = RowFwdGeo<T, LOG2P, decltype(mode)::value>;
-        auto fn = rows_fwd_w_kernel<T, LOG2P, decltype(mode)::value, decltype(late)::value>;
+    auto go = [&](auto mode, auto late, auto ahead, long long want) {
+        using GE = RowFwdGeo<T, LOG2P, decltype(mode)::value, decltype(ahead)::value>;
+        auto fn = rows_fwd_w_kernel<T, LOG2P, decltype(mode)::value, decltype(late)::value, decltype(ahead)::value>;
         static DevOnce attr;
         if (attr.first()) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GE::TOTAL);
-        launch_pdl(fn, grid, GE::THREADS, GE::TOTAL, st, a);
+        const long long res = (long long)GE::PER_SM * rows_sms();
+        launch_pdl(fn, (unsigned)(want < res ? want : res), GE::THREADS, GE::TOTAL, st, a);
     };
     auto launch = [&](auto mode) {
-        using GE = RowFwdGeo<T, LOG2P, decltype(mode)::value>;
-        const long long want = ((a.rows + 1) / 2 + GE::G - 1) / GE::G, res = (long long)GE::PER_SM * rows_sms();
-        const int grid = (int)(want < res ? want : res);
-        if constexpr (kLateRows<LOG2P>) { if (late_rows(grid)) return go(mode, std::true_type{}, grid); }
-        go(mode, std::false_type{}, grid);
+        constexpr int M = decltype(mode)::value;
+        using GE = RowFwdGeo<T, LOG2P, M, false>;
+        const long long pairs = (a.rows + 1) / 2, want = (pairs + GE::G - 1) / GE::G;
+        if constexpr (kAheadRows<T, LOG2P, M>) {
+            // (a wait that gives up has to be reported: calls without a status word take the rows without such waits)
+            using GA = RowFwdGeo<T, LOG2P, M, true>;
+            if (a.status) return go(mode, std::false_type{}, std::true_type{}, (pairs + GA::G - 1) / GA::G);
+        }
+        if constexpr (kLateRows<LOG2P>) { if (late_rows(want)) return go(mode, std::true_type{}, std::false_type{}, want); }
+        go(mode, std::false_type{}, std::false_type{}, want);
     };
     if (a.full_in) {
         if constexpr ((P & (P - 1)) == 0) launch(std::integral_constant<int, 3>{}); else return -1;      // (periodic grids are powers of two)

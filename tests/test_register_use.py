@@ -42,3 +42,13 @@ def test_norms_keep_their_channels_in_registers():
     """mixer_post_kernel<T, VEC, NW, KEEP>: KEEP channels of a thread stay in registers between the sum and the result."""
     kept = {k: v for k, v in spill_loads("mixer").items() if re.search(r"mixer_post_kernelI\w+?Li\dELi\d+ELi(4|16|24)E", k)}
     assert len(kept) >= 2 * 2 * 5 and max(kept.values()) == 0, {k: v for k, v in kept.items() if v}
+
+
+def test_rows_that_travel_ahead_spill_nothing():
+    """rows_fwd_w_kernel<T, LOG2P, MODE, LATE, AHEAD>: four warps with 168 registers a thread.  Periodic rows, which have no such
+    variant, at what they have had from the start."""
+    rows = spill_loads("rows_w")
+    ahead = {k: v for k, v in rows.items() if re.search(r"rows_fwd_w_kernelI\w+?Li\d+ELi\dELb\dELb1E", k)}
+    assert len(ahead) == 3 * 3 and max(ahead.values()) == 0, ahead
+    periodic = {k: v for k, v in rows.items() if re.search(r"rows_fwd_w_kernelI\w+?Li10ELi3E", k)}
+    assert len(periodic) == 4 and max(periodic.values()) <= 232, periodic
