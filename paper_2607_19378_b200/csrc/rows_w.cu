@@ -64,10 +64,8 @@ __device__ __forceinline__ void prefetch_rows_l2(const unsigned char *lo, const 
 // start while their predecessor runs and gain more from early reads: one 500 x 500 grid 38.0 us late, 33.7 early.
 // AHEAD: a group's next rows travel by untiled copies into a buffer of its own while it works on the present ones; CTAs of four
 // warps, three per SM, with the twiddles of the second pass in registers.  Else the rows arrive in the group's line and the group
-// waits for them: CTAs of eight warps, two per SM.  Ahead at 1024 points (128 slices of 512x512, filter rows and k*v rows: fp32 206
-// and 102 us -> 184 and 91, bf16 190 and 94 -> 165 and 85) and for fp32 at 512 (57 and 32 -> 54 and 31); not for bf16 at 512 (52 and
-// 29 -> 53 and 32) and below (256 points: 63 and 35 -> 70 and 38), whose rows are a few hundred bytes and whose waits 16 warps cover.
-template <typename T, int LOG2P, int MODE> constexpr bool kAheadRows = MODE != 3 && (LOG2P == 10 || (LOG2P == 9 && sizeof(T) == 4));
+// waits for them: CTAs of eight warps, two per SM.  Where which is taken: ahead_rows below.
+template <typename T, int LOG2P, int MODE> constexpr bool kAheadRows = MODE != 3 && (LOG2P == 10 || (LOG2P == 9 && sizeof(T) == 4 && MODE == 1));
 template <typename T, int LOG2P, int MODE, bool AHEAD> struct RowFwdGeo {
     using F = WF<LOG2P, false>;
     static constexpr int P = len_of(LOG2P), HP = P / 2, TPL = F::TPL;
@@ -370,6 +368,23 @@ static int rows_sms()
 // length and grid size from which the kernels take their LATE variant (rows ahead have none: no spills either way)
 template <int LOG2P> constexpr bool kLateRows = LOG2P == 10;
 static bool late_rows(long long ctas) { return ctas >= rows_sms(); }
+// Rows ahead (GA) or staged (GS), for `pairs` pairs of rows.  1024 points: ahead (128 slices of 512x512, filter rows and k*v rows: fp32
+// 206 and 102 us -> 184 and 91, bf16 190 and 94 -> 165 and 85; passes of 11 to 62 slices 1.05 to 1.10 times as fast as with staged
+// rows), but for two ranges: pairs that are one round of the staged groups and more than one of those ahead (16 and 12 warps per SM),
+// and pairs whose staged CTAs, of twice as many groups, are fewer than the SMs, so that they let the next kernel in early, while the
+// CTAs ahead are not, or the rows are k*v rows, which the core waits for (staged / ahead: 10 slices of 100x400 fp32 28.3 and 29.2 us,
+// bf16 28.6 and 29.0; 20 of 40x511 fp32 27.3 and 28.4; 5 of 100x400 25.1 and 25.0; 4 of 512x512 fp32, in both ranges, 38.0 and 39.9).
+// 512 points: fp32 filter rows of three rounds and more (256x256, 70 to 257 slices: 1.01 to 1.09; 1788 to 9313 pairs 0.87 to 1.08,
+// mostly by the larger last round); k*v rows are faster staged (fp32 0.80 to
+// 0.95, bf16 52 and 29 us -> 53 and 32).  Shorter rows are a few hundred bytes, whose waits 16 warps cover (256 points: 63 and 35 ->
+// 70 and 38).
+template <int LOG2P, int MODE, class GA, class GS> static bool ahead_rows(long long pairs)
+{
+    const long long sms = rows_sms(), round_a = sms * GA::PER_SM * GA::G, round_s = sms * GS::PER_SM * GS::G;
+    if (LOG2P != 10) return pairs >= 3 * round_a;
+    const bool lets_in_early = pairs <= (sms - 1) * GS::G && (MODE == 0 || pairs > (sms - 1) * GA::G);
+    return !lets_in_early && (pairs <= round_a || pairs > round_s);
+}
 
 bool rows_w_supported(int log2p) { return (log2p >= 6 && log2p <= 10) || (log2p >= kLen192 && log2p <= kLen768); }
 
@@ -392,7 +407,7 @@ template <typename T, int LOG2P> static int launch_rows_fwd_w_t(const RowsArgs &
         if constexpr (kAheadRows<T, LOG2P, M>) {
             // (a wait that gives up has to be reported: calls without a status word take the rows without such waits)
             using GA = RowFwdGeo<T, LOG2P, M, true>;
-            if (a.status) return go(mode, std::false_type{}, std::true_type{}, (pairs + GA::G - 1) / GA::G);
+            if (a.status && ahead_rows<LOG2P, M, GA, GE>(pairs)) return go(mode, std::false_type{}, std::true_type{}, (pairs + GA::G - 1) / GA::G);
         }
         if constexpr (kLateRows<LOG2P>) { if (late_rows(want)) return go(mode, std::true_type{}, std::false_type{}, want); }
         go(mode, std::false_type{}, std::false_type{}, want);

@@ -1,5 +1,5 @@
 """Which of their two variants the forward row kernels take: rows that travel ahead wait for their copies, so a call takes them
-only where a wait that gives up has a status word to say so in."""
+only where a wait that gives up has a status word to say so in, and where they are the faster ones."""
 import pytest
 import torch
 
@@ -9,7 +9,7 @@ from paper_2607_19378_b200 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-STAGED = 256                                                   # threads per CTA
+AHEAD, STAGED = 128, 256                                       # threads per CTA
 
 
 def row_kernels(call):
@@ -46,6 +46,31 @@ def test_calls_without_a_status_word_make_no_wait_for_copies(dims, dtype):
     found = row_kernels(lambda: hn.hyenand_forward_noalloc(w.dims, 1, 2, 0, code, *dev, dev[3][0].numel(), y))
     assert found and set(found) == {STAGED}, found
     assert_parity(y.cpu(), oracle.conv_fft(q, k, v, h, "linear"), q, w)
+
+
+# filter rows, k*v rows.  fp32 of 512 points: ahead for the filter's alone, from three rounds of the GPU's groups on; 1024 points:
+# ahead, but for rows that are one round of the staged groups and more than one of those, or that let the next kernel in early
+ROUTES = [((256, 256), 16, "f32", STAGED, STAGED), ((70, 199), 160, "f32", AHEAD, STAGED), ((70, 199), 160, "bf16", STAGED, STAGED),
+          ((300, 512), 3, "f32", STAGED, STAGED), ((512, 512), 4, "f32", STAGED, STAGED), ((300, 512), 4, "bf16", AHEAD, STAGED),
+          ((300, 511), 8, "bf16", AHEAD, AHEAD), ((40, 511), 5, "f32", AHEAD, STAGED)]
+
+
+@pytest.mark.parametrize("dims,C,dtype,h_rows,kv_rows", ROUTES, ids=str)
+def test_rows_ahead_where_they_are_the_faster_ones(dims, C, dtype, h_rows, kv_rows):
+    from paper_2607_19378_b200 import hyenand as hn
+    w, (q, k, v, h) = W.random_problem(dims, B=1, C=C, dtype=dtype, seed=232)
+    dev = [t.cuda() for t in (q, k, v, h)]
+    plan = hn.Plan(w.dims, 1, C, dtype=w.torch_dtype)
+    y = torch.empty_like(dev[0])
+    found = row_kernels(lambda: plan.forward(*dev, y))
+    status, damage = hn.hyenand_plan_device_status(plan.handle), hn.hyenand_plan_guard_damage(plan.handle)
+    plan.close()
+    assert (status, damage) == (0, 0)
+    assert sorted(found) == sorted((h_rows, kv_rows)), found
+    for c in sorted({0, 1, C - 1}):
+        one = [t[:, c:c + 1] for t in (q, k, v, h)]
+        ws = W.Workload("one", w.dims, 1, 1, dtype)
+        assert_parity(y[:, c:c + 1].cpu(), oracle.conv_fft(*one, "linear"), one[0], ws, what=f"channel {c}")
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
