@@ -519,7 +519,8 @@ template <typename T, int HF> static int launch_synth_tc_t(const SynthArgs &a, c
     long long grid = (long long)sms * per_sm / (a.B < sms * per_sm ? a.B : 1);
     if (grid < 1) grid = 1;
     if (grid > tiles) grid = tiles;
-    launch_pdl(synth_tc_kernel<T, HF>, dim3((unsigned)grid, (unsigned)a.B), kTcThreads, sm, st, a);
+    // (a plain launch: its own wait returns at once; the kernel after it may still be let in early)
+    synth_tc_kernel<T, HF><<<dim3((unsigned)grid, (unsigned)a.B), kTcThreads, sm, st>>>(a);
     return 1;
 }
 
