@@ -107,7 +107,7 @@ template <typename T, int LOG2P1, bool HAS_B> struct CtFwdGeo : CtGeo<T, LOG2P1>
 // they come: 0 tensor copies, 1 asynchronous copies of 8 bytes, 2 element by element (slices that start
 // off 8-byte boundaries, eight loads in flight).
 // The separated bins leave as tensor copies from a swizzled tile over the lines.  262144 bf16 values, 512 rows: 383 us with two CTAs
-// of eight warps per SM, 348 with four of four (4.6 TB/s); the filter's rows 184, 168.  Bound by the shared-memory pipe (59 %) and
+// of eight warps per SM, 348 with four of four (4.6 TB/s); the filter's rows 184, 168.  Bound by the shared-memory pipe (75 %) and
 // the barriers around the result tile.
 template <typename T, int LOG2P1, bool HAS_B, int IN>
 __global__ void __launch_bounds__(kCtThreads, (CtFwdGeo<T, LOG2P1, HAS_B>::PER_SM))
@@ -374,7 +374,7 @@ struct TmemTw {
 // lanes of tensor memory and takes the row of nb slices of its channel through it, so the filter crosses HBM once and its spectrum
 // never.  In shared memory the spectra of 16 warps (8 KB each) do not fit beside their lines; in registers 64 more per thread
 // leave 8 warps per SM.  262144 bf16 values, 2 x 256 rows: 167 us in a kernel of the filter's own plus 525 here, now 595.  Bound by
-// instruction issue (60 % of the slots) and instruction fetch of the unrolled passes.  Three CTAs of four warps with twiddles in
+// instruction issue (64 % of the slots) and instruction fetch of the unrolled passes.  Three CTAs of four warps with twiddles in
 // registers and rows that travel ahead as untiled copies: 662.  Filters of which no group holds all (3 x 800 rows of 262144 values in groups
 // of 765, 2 x 390 of 524288 in groups of 383) are transformed once per slice; spectra made once and read here: 6517 -> 6567 us, 4894 -> 5079.
 template <int LOG2P2, bool FILT>
